@@ -237,7 +237,8 @@ def oracle_sample_text(spec, n_images=REF_IMAGES, wl_name=None):
 
 # the files that define the iteration's kernels (the host-side API and the no-allocation entry point
 # launch them but do not change their code)
-KERNEL_SOURCES = ("ss_fft.cuh", "ss_internal.h", "ss_kernels.cuh", "ss_kernels_f32.cu", "ss_kernels_f64.cu")
+KERNEL_SOURCES = ("ss_fft.cuh", "ss_internal.h", "ss_kernels.cuh", "ss_kernels_f32.cu", "ss_kernels_f64.cu", "ss_twopass.cuh",
+                  "ss_twopass.cu")
 
 
 def kernel_source_hash():

@@ -1,7 +1,7 @@
 """Builds libss.so (the C-ABI library) in-tree for sm_103a with nvcc.
 
-Three translation units compile in parallel (FP32 kernels, FP64 kernels, host runtime) and link
-into ``paper_1804_07135_gb300/libss.so`` against the shared CUDA runtime.
+The translation units (FP32 kernels, FP64 kernels, host runtime, one unit per length of the two-pass
+transforms) compile in parallel and link into ``paper_1804_07135_gb300/libss.so`` against the shared CUDA runtime.
 """
 from __future__ import annotations
 
@@ -17,6 +17,8 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libss.so")
 SOURCES = ("ss_kernels_f32.cu", "ss_kernels_f64.cu", "ss_api.cu", "ss_noalloc.cu")
+# lengths of the two-pass transforms (SS_T2_LENGTHS of csrc/ss_internal.h)
+T2_LENGTHS = (32, 48, 64, 80, 96, 112, 128, 144, 160, 192, 224, 256, 288, 320, 384, 448, 512)
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -58,9 +60,10 @@ def build(force: bool = False, verbose: bool = False) -> str:
     cc = nvcc()
     common = [cc, *ARCH, "-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", CSRC]
 
-    def compile_one(src: str) -> str:
-        obj = os.path.join(BUILD, src.replace(".cu", ".o"))
-        cmd = common + ["-c", os.path.join(CSRC, src), "-o", obj]
+    def compile_one(unit) -> str:
+        src, defines = unit
+        obj = os.path.join(BUILD, "_".join([src[:-3], *(str(v) for v in defines.values())]) + ".o")
+        cmd = common + [f"-D{k}={v}" for k, v in defines.items()] + ["-c", os.path.join(CSRC, src), "-o", obj]
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError(f"nvcc failed on {src}:\n{r.stdout}\n{r.stderr}")
@@ -68,8 +71,10 @@ def build(force: bool = False, verbose: bool = False) -> str:
             print(r.stderr)
         return obj
 
-    with cf.ThreadPoolExecutor(len(SOURCES)) as ex:
-        objs = list(ex.map(compile_one, SOURCES))
+    units = [(src, {}) for src in SOURCES]
+    units += [("ss_twopass.cu", {"SS_T2_P": P}) for P in reversed(T2_LENGTHS)]  # the long ones first
+    with cf.ThreadPoolExecutor(min(len(units), os.cpu_count() or 8)) as ex:
+        objs = list(ex.map(compile_one, units))
     tmp = LIB + f".tmp{os.getpid()}"
     libdir = cuda_lib_dir()
     cmd = [cc, *ARCH, "-shared", "-o", tmp, *objs, "-cudart", "shared", "-L", libdir,

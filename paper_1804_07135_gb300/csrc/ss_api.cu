@@ -25,22 +25,16 @@ namespace {
 thread_local std::string g_create_error;
 
 // ---- small helpers --------------------------------------------------------------------------------
-bool is_smooth23(int m) {
-    while (m % 2 == 0) m /= 2;
-    while (m % 3 == 0) m /= 3;
-    return m == 1;
-}
-
-// Padded transform length: the smallest 2^a 3^b >= 2n - 1, enough for the linear (non-circular)
-// convolution of n sites with offsets -(n-1)..(n-1) (Sec. II-A, the zero-padded kernel).
-// Padded transform length for n sites: the smallest 2^a 3^b >= 2n - 1, or the power of two >= 2n - 1
-// when that is at most 1/8 longer (its transforms need no radix-3 stages: 112 sites pad to 256, not 243).
-int padded_len(int n) {
-    int m = std::max(1, 2 * n - 1);
-    while (!is_smooth23(m)) ++m;
-    int p2 = 1;
-    while (p2 < 2 * n - 1) p2 <<= 1;
-    return 8 * p2 <= 9 * m ? p2 : m;
+// Padded transform length for n sites, enough for the linear (non-circular) convolution with offsets
+// -(n-1)..(n-1) (Sec. II-A, the zero-padded kernel): padded_smooth(n), except that an FP32 length without
+// two-pass kernels is exchanged for the next one that has them (two_pass: the kernels along this axis have a
+// two-pass form at all).  Lattices of up to 12 sites a side keep the short length: one CTA transforms all of
+// their lines at once either way.
+int padded_len(int n, bool two_pass) {
+    const int m = padded_smooth(n);
+    if (!two_pass || n <= 12 || t2_length(m)) return m;
+    const int t = t2_length_from(2 * n - 1);
+    return t ? t : m;
 }
 
 FftPlan make_plan(int P) { return fft_make_plan(P); }
@@ -113,7 +107,6 @@ struct Group {
     int n_eblk = 0;
     // device
     void *s = nullptr, *sp = nullptr, *spec = nullptr, *dhat = nullptr, *twx = nullptr, *twy = nullptr;
-    void *twxs = nullptr, *twys = nullptr;
     void *t2x = nullptr, *t2y = nullptr;  // two-pass twiddle tables (2 Px, 2 Py entries)
     void *prm = nullptr, *hout = nullptr;
     InterpEntry* interp = nullptr;
@@ -262,8 +255,6 @@ template <typename T> GroupArgs<T> group_args(const ss_ctx* c, const Group& g) {
     a.dhat = (const T*)g.dhat;
     a.twx = (const cplx<T>*)g.twx;
     a.twy = (const cplx<T>*)g.twy;
-    a.twxs = (const cplx<T>*)g.twxs;
-    a.twys = (const cplx<T>*)g.twys;
     a.t2x = (const cplx<T>*)g.t2x;
     a.t2y = (const cplx<T>*)g.t2y;
     a.planx = g.planx;
@@ -306,7 +297,7 @@ void set_rows(Group& g, int ty_a, int ty_c, int thr_a = 256, int thr_c = 256) {
         g.smem_c = f128_x_smem(ty_c);
     }
     if (x2) {
-        g.thr_a = g.thr_c = kX2Threads;
+        g.thr_a = g.thr_c = x2_threads(g.Px);
         g.smem_a = x2_smem(g.Px, false);
         g.smem_c = x2_smem(g.Px, true);
     }
@@ -403,8 +394,6 @@ template <typename T> ss_status setup_group(ss_ctx* c, Group& g) {
     TRY(dalloc(c, (void**)&g.epart, (size_t)g.n_img * kEvalTerms * g.nz * g.ny * sizeof(double)));  // any rows per CTA
     TRY(dalloc(c, &g.twx, g.Px * sizeof(C)));
     TRY(dalloc(c, &g.twy, g.Py * sizeof(C)));
-    TRY(dalloc(c, &g.twxs, g.Px * sizeof(C)));
-    TRY(dalloc(c, &g.twys, g.Py * sizeof(C)));
     TRY(dalloc(c, &g.t2x, 2 * g.Px * sizeof(C)));
     TRY(dalloc(c, &g.t2y, 2 * g.Py * sizeof(C)));
     if (g.direct) TRY(dalloc(c, &g.hdir, (size_t)g.n_img * 3 * g.N * sizeof(T)));
@@ -434,11 +423,6 @@ template <typename T> ss_status setup_group(ss_ctx* c, Group& g) {
     for (int i = 0; i < g.Py; ++i) ty[i] = C{T(twy[i].x), T(twy[i].y)};
     CUDA_TRY(c, cudaMemcpyAsync(g.twx, tx.data(), g.Px * sizeof(C), cudaMemcpyHostToDevice, c->cs));
     CUDA_TRY(c, cudaMemcpyAsync(g.twy, ty.data(), g.Py * sizeof(C), cudaMemcpyHostToDevice, c->cs));
-    std::vector<C> sx(g.Px, C{T(0), T(0)}), sy(g.Py, C{T(0), T(0)});
-    fft_stage_twiddles(g.planx, twx.data(), sx.data());
-    fft_stage_twiddles(g.plany, twy.data(), sy.data());
-    CUDA_TRY(c, cudaMemcpyAsync(g.twxs, sx.data(), g.Px * sizeof(C), cudaMemcpyHostToDevice, c->cs));
-    CUDA_TRY(c, cudaMemcpyAsync(g.twys, sy.data(), g.Py * sizeof(C), cudaMemcpyHostToDevice, c->cs));
     std::vector<C> t2x(2 * g.Px), t2y(2 * g.Py);
     two_pass_twiddles(g.Px, twx, t2x.data());
     two_pass_twiddles(g.Py, twy, t2y.data());
@@ -527,7 +511,7 @@ template <typename T> ss_status tune_group(ss_ctx* c, Group& g) {
     const size_t cs = 2 * real_size(c);
     std::vector<std::pair<int, int>> cands;  // (threads, rows)
     if (g.dipole && x2p_ok((int)real_size(c), g.Px)) {
-        cands.push_back({kX2Threads, kX2Rows});  // one shape: nothing to tune
+        cands.push_back({x2_threads(g.Px), kX2Rows});  // one shape: nothing to tune
     } else if (g.dipole && f128_x((int)real_size(c), g.Px)) {
         for (int ty : {2, 4, 8})  // 48 threads per row; row counts that divide 16 keep the passes conflict-free
             cands.push_back({f128_x_threads(ty), ty});
@@ -1001,17 +985,17 @@ ss_status ensure_ev64(ss_ctx* c) {
         e.ny = g.ny;
         e.nz = g.nz;
         e.N = g.N;
-        e.Px = g.Px;
-        e.Py = g.Py;
+        e.dipole = g.dipole;
+        e.Px = e.dipole ? padded_len(e.nx, false) : 1;
+        e.Py = e.dipole ? padded_len(e.ny, false) : 1;
         e.n_img = g.n_img;
         e.n_pairs = g.n_pairs;
         e.strs = g.strs;
         e.str_img0 = g.str_img0;
         e.str_K = g.str_K;
-        e.dipole = g.dipole;
         e.direct = g.direct;
-        e.planx = g.planx;
-        e.plany = g.plany;
+        e.planx = make_plan(e.Px);
+        e.plany = make_plan(e.Py);
         configure_group(e);
         if (e.smem_a > 227 * 1024 || e.smem_b > 227 * 1024 || e.smem_c > 227 * 1024)
             return fail(c, SS_ERR_INVALID_ARG, "lattice %d x %d x %d: the FP64 evaluation needs more shared memory than a CTA has",
@@ -1308,8 +1292,8 @@ ss_status ss_create_batch(int n_strings, const ss_string_desc* descs, const ss_o
     size_t stage = 0;
     for (Group& g : c->groups) {
         g.n_pairs = (g.n_img + 1) / 2;
-        g.Px = g.dipole ? padded_len(g.nx) : 1;
-        g.Py = g.dipole ? padded_len(g.ny) : 1;
+        g.Px = g.dipole ? padded_len(g.nx, !use_fp64(c)) : 1;
+        g.Py = g.dipole ? padded_len(g.ny, !use_fp64(c) && g.nz <= kT2MaxNz) : 1;
         g.planx = make_plan(g.Px);
         g.plany = make_plan(g.Py);
         g.rbytes = (int)real_size(c);
@@ -1322,8 +1306,11 @@ ss_status ss_create_batch(int n_strings, const ss_string_desc* descs, const ss_o
     }
     if (use_fp64(c))
         set_smem_limits<double>(227 * 1024);
-    else
+    else {
         set_smem_limits<float>(227 * 1024);
+        for (Group& g : c->groups)
+            if (g.dipole) set_t2_smem_limits(g.Px, g.Py, 227 * 1024);
+    }
     {
         ss_status st = dalloc(c, (void**)&c->d_err, sizeof(int));
         if (st != SS_OK) return bail(st);

@@ -132,50 +132,143 @@ template <typename C> struct Dft<12, C> {
     }
 };
 
-// Size-R DFTs whose inputs R/2..R-1 are zero (the zero-padded half of a forward transform).
-template <int R, typename C> struct DftHalfIn;
-template <typename C> struct DftHalfIn<2, C> {
-    static __device__ __forceinline__ void run(C* v) { v[1] = v[0]; }
+// ---- further DFT sizes of the two-pass transforms: primes 5 and 7, and composites by Cooley-Tukey -------
+// cos(2 pi k / n) and sin(2 pi k / n) at compile time: the angle reduced exactly to [0, pi/4] in integers,
+// then the Taylor series (its terms fall below 1e-19 well before the loop ends).
+struct CxCs {
+    double c, s;
 };
-template <typename C> struct DftHalfIn<4, C> {
-    static __device__ __forceinline__ void run(C* v) {
-        const C a = v[0], b = v[1], mb = cmi(v[1]);
-        v[0] = cadd(a, b);
-        v[1] = cadd(a, mb);
-        v[2] = csub(a, b);
-        v[3] = csub(a, mb);
+__host__ __device__ constexpr CxCs cx_cos_sin(int k, int n) {
+    long m = 4L * (((k % n) + n) % n);  // angle = 2 pi m / D, D = 4 n
+    const long D = 4L * n;
+    bool neg_s = false, neg_c = false, swap = false;
+    if (2 * m > D) m = D - m, neg_s = true;
+    if (4 * m > D) m = D / 2 - m, neg_c = true;
+    if (8 * m > D) m = D / 4 - m, swap = true;
+    const double x = 6.283185307179586476925286766559 * (double)m / (double)D;
+    double c = 0.0, s = 0.0, t = 1.0;
+    for (int i = 0; i < 24; ++i) {  // t = x^i / i! with the sign of the series' pairs
+        if (i % 2 == 0)
+            c += (i % 4 == 0) ? t : -t;
+        else
+            s += (i % 4 == 1) ? t : -t;
+        t *= x / (double)(i + 1);
     }
+    const double cc = swap ? s : c, ss = swap ? c : s;
+    return CxCs{neg_c ? -cc : cc, neg_s ? -ss : ss};
+}
+// y + a x with a real
+template <typename C> __device__ __forceinline__ C caxpy(decltype(C{}.x) a, C x, C y) {
+    return C{y.x + a * x.x, y.y + a * x.y};
+}
+__device__ __forceinline__ float2 caxpy(float a, float2 x, float2 y) { return __ffma2_rn(make_float2(a, a), x, y); }
+
+template <int I> struct ic {
+    static constexpr int v = I;
 };
-template <typename C> struct DftHalfIn<8, C> {
-    static __device__ __forceinline__ void run(C* v) {
-        using R = decltype(v[0].x);
-        const R q = R(0.7071067811865475244008443621048490);
-        // even part DFT4(x0, x2, 0, 0), odd part DFT4(x1, x3, 0, 0)
-        const C x0 = v[0], x1 = v[1], x2 = v[2], x3 = v[3];
-        const C m2 = cmi(x2), m3 = cmi(x3);
-        const C e0 = cadd(x0, x2), e1 = cadd(x0, m2), e2 = csub(x0, x2), e3 = csub(x0, m2);
-        const C o0 = cadd(x1, x3), o1 = cadd(x1, m3), o2 = csub(x1, x3), o3 = csub(x1, m3);
-        const C t1 = C{q * (o1.x + o1.y), q * (o1.y - o1.x)};
-        const C t2 = cmi(o2);
-        const C t3 = C{q * (o3.y - o3.x), -q * (o3.x + o3.y)};
-        v[0] = cadd(e0, o0);
-        v[4] = csub(e0, o0);
-        v[1] = cadd(e1, t1);
-        v[5] = csub(e1, t1);
-        v[2] = cadd(e2, t2);
-        v[6] = csub(e2, t2);
-        v[3] = cadd(e3, t3);
-        v[7] = csub(e3, t3);
+template <int I, int N, typename F> __device__ __forceinline__ void static_for(F f) {
+    if constexpr (I < N) {
+        f(ic<I>{});
+        static_for<I + 1, N>(f);
     }
+}
+// a * W_N^K, W_N = exp(-2 pi i / N)
+template <int K, int N, typename C> __device__ __forceinline__ C mul_w(C a) {
+    using R = decltype(a.x);
+    constexpr int k = K % N;
+    if constexpr (k == 0) {
+        return a;
+    } else if constexpr (4 * k == N) {
+        return cmi(a);
+    } else if constexpr (2 * k == N) {
+        return C{-a.x, -a.y};
+    } else if constexpr (4 * k == 3 * N) {
+        return C{-a.y, a.x};
+    } else {
+        constexpr CxCs w = cx_cos_sin(k, N);
+        return cmul(a, C{R(w.c), R(-w.s)});
+    }
+}
+
+template <typename C> struct Dft<1, C> {
+    static __device__ __forceinline__ void run(C*) {}
 };
 
-// Host-side plan: radices 8, 4, 2 first (largest first), then 3s.
+// Odd prime R: with s_j = v_j + v_{R-j} and d_j = v_j - v_{R-j}, X_k and X_{R-k} are
+// v_0 + sum_j s_j cos(2 pi j k / R) -+ i sum_j d_j sin(2 pi j k / R), 1 <= j, k <= (R-1)/2.
+template <int R, typename C> struct DftPrime {
+    static __device__ __forceinline__ void run(C* v) {
+        using Re = decltype(v[0].x);
+        constexpr int M = (R - 1) / 2;
+        C s[M], d[M];
+#pragma unroll
+        for (int j = 0; j < M; ++j) {
+            s[j] = cadd(v[1 + j], v[R - 1 - j]);
+            d[j] = csub(v[1 + j], v[R - 1 - j]);
+        }
+        const C v0 = v[0];
+#pragma unroll
+        for (int j = 0; j < M; ++j) v[0] = cadd(v[0], s[j]);
+        static_for<1, M + 1>([&](auto kk) {
+            constexpr int k = decltype(kk)::v;
+            C a = v0, b = C{Re(0), Re(0)};
+            static_for<1, M + 1>([&](auto jj) {
+                constexpr int j = decltype(jj)::v;
+                constexpr CxCs w = cx_cos_sin(j * k, R);
+                a = caxpy(Re(w.c), s[j - 1], a);
+                b = caxpy(Re(w.s), d[j - 1], b);
+            });
+            const C r = cmi(b);
+            v[k] = cadd(a, r);
+            v[R - k] = csub(a, r);
+        });
+    }
+};
+template <typename C> struct Dft<5, C> : DftPrime<5, C> {};
+template <typename C> struct Dft<7, C> : DftPrime<7, C> {};
+
+// N = N1 N2 by Cooley-Tukey (n = N2 n1 + n2, k = k1 + N1 k2): N1-point DFTs over n1 for each n2, the
+// twiddles W_N^{n2 k1}, then N2-point DFTs over n2.
+template <int N1, int N2, typename C> struct DftCt {
+    static __device__ __forceinline__ void run(C* v) {
+        constexpr int N = N1 * N2;
+        C a[N2][N1];
+        static_for<0, N2>([&](auto nn) {
+            constexpr int n2 = decltype(nn)::v;
+#pragma unroll
+            for (int n1 = 0; n1 < N1; ++n1) a[n2][n1] = v[N2 * n1 + n2];
+            Dft<N1, C>::run(a[n2]);
+            static_for<0, N1>([&](auto kk) {
+                constexpr int k1 = decltype(kk)::v;
+                a[n2][k1] = mul_w<n2 * k1, N>(a[n2][k1]);
+            });
+        });
+#pragma unroll
+        for (int k1 = 0; k1 < N1; ++k1) {
+            C q[N2];
+#pragma unroll
+            for (int n2 = 0; n2 < N2; ++n2) q[n2] = a[n2][k1];
+            Dft<N2, C>::run(q);
+#pragma unroll
+            for (int k2 = 0; k2 < N2; ++k2) v[k1 + N1 * k2] = q[k2];
+        }
+    }
+};
+template <typename C> struct Dft<9, C> : DftCt<3, 3, C> {};
+template <typename C> struct Dft<10, C> : DftCt<5, 2, C> {};
+template <typename C> struct Dft<14, C> : DftCt<7, 2, C> {};
+template <typename C> struct Dft<16, C> : DftCt<4, 4, C> {};
+
+// Host-side plan: radices 8, 4, 2 first (largest first), then 3s, 5s and 7s (the last two only in the setup
+// transforms of the tensor spectrum: a length with those factors has two-pass kernels).
 inline FftPlan fft_make_plan(int P) {
     FftPlan p{};
     p.P = P;
-    int a = 0, b = 0, q = P;
+    int a = 0, b = 0, c5 = 0, c7 = 0, q = P;
     while (q % 2 == 0) q /= 2, ++a;
     while (q % 3 == 0) q /= 3, ++b;
+    while (q % 5 == 0) q /= 5, ++c5;
+    while (q % 7 == 0) q /= 7, ++c7;
     int n = 0;
     const int n8 = a / 3, rem = a % 3;
     if (rem == 1 && n8 == 0) {
@@ -190,6 +283,8 @@ inline FftPlan fft_make_plan(int P) {
         if (rem == 2) p.radix[n++] = 4;
     }
     for (int i = 0; i < b; ++i) p.radix[n++] = 3;
+    for (int i = 0; i < c5; ++i) p.radix[n++] = 5;
+    for (int i = 0; i < c7; ++i) p.radix[n++] = 7;
     p.nstages = n;
     int ns = 1;
     for (int s = 0; s < n; ++s) {
@@ -206,7 +301,7 @@ inline FftPlan fft_make_plan(int P) {
 // Elements each thread holds in registers per stage: 8 (9 for radix 3).  Lines are transformed in
 // passes of fft_lines_per_pass() lines, so any block of at least P/8 threads can transform any number
 // of lines.
-template <int R> struct StageCap { static constexpr int B = R == 2 ? 4 : R == 3 ? 3 : R == 4 ? 2 : 1; };
+template <int R> struct StageCap { static constexpr int B = R == 2 ? 4 : R == 3 ? 3 : R == 8 ? 1 : 2; };
 constexpr int kFftElemsPerThread = 8;
 
 __host__ __device__ inline int fft_lines_per_pass(int nthr, int P) { return (nthr * kFftElemsPerThread) / P; }
@@ -259,8 +354,9 @@ __device__ __forceinline__ void fft_stage(C* buf, const C* tw, int LS, int L, in
 }
 
 // Forward FFT of L lines (stride LS, elements at fft_pad positions) in shared memory.  Must be called
-// by every thread of the block, with blockDim.x >= fft_min_threads(P).  Ends synchronised.
-template <typename C>
+// by every thread of the block, with blockDim.x >= fft_min_threads(P).  Ends synchronised.  R57: the plan
+// may hold radices 5 and 7.
+template <bool R57 = false, typename C>
 __device__ __forceinline__ void fft_lines(C* buf, const C* tw, const FftPlan& plan, int LS, int L, int tid, int nthr) {
     const int lpp = max(1, fft_lines_per_pass(nthr, plan.P));  // the host guarantees >= 1; never loop forever
     for (int l0 = 0; l0 < L; l0 += lpp) {
@@ -272,144 +368,15 @@ __device__ __forceinline__ void fft_lines(C* buf, const C* tw, const FftPlan& pl
                 case 8: fft_stage<8>(b, tw, LS, nl, Q, Ns, tws, msk, tid, nthr); break;
                 case 4: fft_stage<4>(b, tw, LS, nl, Q, Ns, tws, msk, tid, nthr); break;
                 case 3: fft_stage<3>(b, tw, LS, nl, Q, Ns, tws, msk, tid, nthr); break;
+                case 5:
+                    if constexpr (R57) fft_stage<5>(b, tw, LS, nl, Q, Ns, tws, msk, tid, nthr);
+                    break;
+                case 7:
+                    if constexpr (R57) fft_stage<7>(b, tw, LS, nl, Q, Ns, tws, msk, tid, nthr);
+                    break;
                 default: fft_stage<2>(b, tw, LS, nl, Q, Ns, tws, msk, tid, nthr); break;
             }
         }
-    }
-}
-
-// ---- compile-time plans for the padded lengths the workloads use --------------------------------
-// Same radix order and stage constants as fft_make_plan, but known to the compiler, so every index
-// of a butterfly is a shift, mask or constant multiply.
-__host__ __device__ constexpr int cx_pow(int P, int f) { return P % f == 0 ? 1 + cx_pow(P / f, f) : 0; }
-__host__ __device__ constexpr int cx_nstages(int P) {
-    return (cx_pow(P, 2) % 3 == 1 && cx_pow(P, 2) / 3 == 0 ? 1
-            : cx_pow(P, 2) % 3 == 1                        ? cx_pow(P, 2) / 3 + 1
-            : cx_pow(P, 2) % 3 == 2                        ? cx_pow(P, 2) / 3 + 1
-                                                           : cx_pow(P, 2) / 3) +
-           cx_pow(P, 3);
-}
-// radix of stage s
-__host__ __device__ constexpr int cx_radix(int P, int s) {
-    return (cx_pow(P, 2) % 3 == 1 && cx_pow(P, 2) / 3 == 0)
-               ? (s == 0 ? 2 : 3)
-               : (cx_pow(P, 2) % 3 == 1
-                      ? (s < cx_pow(P, 2) / 3 - 1 ? 8 : s < cx_pow(P, 2) / 3 + 1 ? 4 : 3)
-                      : (cx_pow(P, 2) % 3 == 2 ? (s < cx_pow(P, 2) / 3 ? 8 : s == cx_pow(P, 2) / 3 ? 4 : 3)
-                                               : (s < cx_pow(P, 2) / 3 ? 8 : 3)));
-}
-__host__ __device__ constexpr int cx_ns(int P, int s) { return s == 0 ? 1 : cx_ns(P, s - 1) * cx_radix(P, s - 1); }
-
-// Offset of stage s's twiddles in the per-stage table: stage s (with ns > 1) holds W_P^{jm*r*tw} at
-// [jm][r-1], jm < ns, 1 <= r < R, so a butterfly reads its R-1 twiddles at base + constants.  The
-// table has P - radix(0) entries in all (fewer than P).
-__host__ __device__ constexpr int cx_tw_off(int P, int s) {
-    return s == 0 ? 0 : cx_tw_off(P, s - 1) + (cx_ns(P, s - 1) > 1 ? cx_ns(P, s - 1) * (cx_radix(P, s - 1) - 1) : 0);
-}
-// True when fft_pad(j + r*Q) - fft_pad(j) does not depend on j (loads at base + constants).
-__host__ __device__ constexpr bool cx_load_linear(int Q, int R) {
-    for (int j = 0; j < Q; ++j)
-        for (int r = 0; r < R; ++r)
-            if (fft_pad(j + r * Q) - fft_pad(j) != fft_pad(r * Q)) return false;
-    return true;
-}
-// True when fft_pad(e0 + r*NS) - fft_pad(e0) does not depend on the butterfly (stores at base + constants).
-__host__ __device__ constexpr bool cx_store_linear(int P, int R, int NS) {
-    for (int j = 0; j < P / R; ++j) {
-        const int jm = j % NS, e0 = (j - jm) * R + jm;
-        for (int r = 0; r < R; ++r)
-            if (fft_pad(e0 + r * NS) - fft_pad(e0) != fft_pad(r * NS)) return false;
-    }
-    return true;
-}
-
-// PIN: inputs r >= R/2 of this stage are zero (first stage of a zero-padded forward transform).
-// POUT: only outputs r < R/2 are stored (last stage of a transform read below P/2).
-template <int P, int S, bool PIN, bool POUT, int R = cx_radix(P, S), int NS = cx_ns(P, S), typename C>
-__device__ __forceinline__ void fft_stage_c(C* buf, const C* tws, int LS, int L, int tid, int nthr) {
-    constexpr int B = StageCap<R>::B;
-    constexpr int RIN = PIN ? R / 2 : R;    // inputs read
-    constexpr int ROUT = POUT ? R / 2 : R;  // outputs stored
-    constexpr int Q = P / R;
-    constexpr bool LIN_LD = cx_load_linear(Q, R);
-    constexpr bool LIN_ST = cx_store_linear(P, R, NS);
-    constexpr int TWO = cx_tw_off(P, S);
-    C v[B][R];
-    int dline[B], de[B];
-#pragma unroll
-    for (int i = 0; i < B; ++i) {
-        const int b = tid + i * nthr;
-        const int line = b / Q, j = b % Q;
-        dline[i] = -1;
-        de[i] = 0;
-        if (line < L) {
-            const int jm = j % NS;
-            const C* src = buf + line * LS;
-            const C* s0 = src + fft_pad(j);
-            const C* w = tws + TWO + jm * (R - 1);
-#pragma unroll
-            for (int r = 0; r < RIN; ++r) {
-                C x = LIN_LD ? s0[fft_pad(r * Q)] : src[fft_pad(j + r * Q)];
-                if (NS > 1 && r > 0) x = cmul(x, w[r - 1]);
-                v[i][r] = x;
-            }
-            if constexpr (PIN)
-                DftHalfIn<R, C>::run(v[i]);
-            else
-                Dft<R, C>::run(v[i]);
-            dline[i] = line * LS;
-            de[i] = (j - jm) * R + jm;
-        }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < B; ++i) {
-        if (dline[i] >= 0) {
-            C* d0 = buf + dline[i] + fft_pad(de[i]);
-#pragma unroll
-            for (int r = 0; r < ROUT; ++r) {
-                if (LIN_ST)
-                    d0[fft_pad(r * NS)] = v[i][r];
-                else
-                    buf[dline[i] + fft_pad(de[i] + r * NS)] = v[i][r];
-            }
-        }
-    }
-    __syncthreads();
-}
-
-template <int P, int S, bool ZERO_HI_IN, bool HI_OUT_UNUSED, typename C>
-__device__ __forceinline__ void fft_stages_c(C* buf, const C* tws, int LS, int L, int tid, int nthr) {
-    if constexpr (S < cx_nstages(P)) {
-        constexpr int R = cx_radix(P, S);
-        constexpr bool pin = ZERO_HI_IN && S == 0 && R != 3;
-        constexpr bool pout = HI_OUT_UNUSED && S == cx_nstages(P) - 1 && R != 3;
-        fft_stage_c<P, S, pin, pout>(buf, tws, LS, L, tid, nthr);
-        fft_stages_c<P, S + 1, ZERO_HI_IN, HI_OUT_UNUSED>(buf, tws, LS, L, tid, nthr);
-    }
-}
-
-// Forward FFT of L lines of compile-time length P; tws is the per-stage twiddle table.
-// ZERO_HI_IN: elements P/2..P-1 of every line are zero on entry (their loads are skipped).
-// HI_OUT_UNUSED: only elements 0..P/2-1 of the result are read afterwards (the rest is left stale).
-template <int P, bool ZERO_HI_IN = false, bool HI_OUT_UNUSED = false, typename C>
-__device__ __forceinline__ void fft_lines_c(C* buf, const C* tws, int LS, int L, int tid, int nthr) {
-    const int lpp = max(1, fft_lines_per_pass(nthr, P));
-    for (int l0 = 0; l0 < L; l0 += lpp)
-        fft_stages_c<P, 0, ZERO_HI_IN, HI_OUT_UNUSED>(buf + l0 * LS, tws, LS, min(lpp, L - l0), tid, nthr);
-}
-
-// Host: per-stage twiddle table (see cx_tw_off) of a plan from its flat table w[k] = W_P^k.
-template <typename C, typename W> inline void fft_stage_twiddles(const FftPlan& p, const W* w, C* out) {
-    int o = 0;
-    for (int s = 0; s < p.nstages; ++s) {
-        const int R = p.radix[s], Ns = p.ns[s];
-        if (Ns == 1) continue;
-        for (int jm = 0; jm < Ns; ++jm)
-            for (int r = 1; r < R; ++r) {
-                const W x = w[(jm * r * p.tw[s]) % p.P];
-                out[o++] = C{decltype(C{}.x)(x.x), decltype(C{}.x)(x.y)};
-            }
     }
 }
 
@@ -490,7 +457,7 @@ template <typename C> __device__ __forceinline__ void f128_pass2(C (&v)[8], cons
     Dft<8, C>::run(v);
 }
 
-// ---- lengths P = 16 R2 (R2 = 12, 16, 24: 192, 256, 384) in two register passes ------------------------
+// ---- lengths P = 16 R2 (R2 = 2..32: 32 to 512) in two register passes ------------------------------------
 // A line of P elements is held in shared memory as R2 rows of 16 at row stride kT2Row = 17 (element
 // (r, c) at r * 17 + c; a line takes kT2Row * R2 slots).  With n = R2 n1 + n2, k = k1 + 16 k2 (n1, k1 < 16;
 // n2, k2 < R2) the forward transform is
@@ -507,7 +474,8 @@ template <typename C> __device__ __forceinline__ void f128_pass2(C (&v)[8], cons
 // pass A, role (k1, par2), column k1: the R2/2-point DFTs as in pass 2, times W_P^{k1 y2}, back into column k1
 //   (row y2);
 // pass B, role (y2, par), row y2: an 8-point DFT of (T[j][y2] +- T[j+8][y2]) W_16^{j par} -> Y[y2 + R2 (2m + par)];
-// an inverse read below P/2 keeps m < 4.  The twiddles of pass 1 and pass A come from the tables of
+// an inverse read below P/2 keeps m < 4.  For odd R2 (48, 80, 112, 144) passes 2 and A take one role per column
+// k1 with the whole R2-point DFT (t2_col_vals with H = R2 and no split).  The twiddles of pass 1 and pass A come from the tables of
 // GroupArgs::t2x / t2y (t1 = the pass-1 half, ta = the pass-A half, indexed so that a warp's lanes read
 // consecutive entries); the ramp W_R2^j = W_P^{16 j} from the flat table tw (the same entry across a warp).
 __device__ __forceinline__ int t2_at(int r, int c) { return r * kT2Row + c; }
@@ -523,40 +491,50 @@ __device__ __forceinline__ void t2_pass1(C (&u)[8], int n2, int par, const C* __
         line[t2_at(n2, 2 * m + par)] = cmul(u[m], t1[(2 * m + par) * (P / 16) + n2]);  // W_P^{n2 (2m + par)}
 }
 
-// The R2/2-point DFTs of pass 2 (TW_OUT = false) or pass A (TW_OUT = true) for column k1 and parity par2:
-// a[m] = the output of row 2m + par2 (times W_P^{k1 (2m + par2)} in pass A).  col(j) returns the column's
+// Roles per column of passes 2 and A (2: the output rows split by parity; 1: odd R2) and outputs per role.
+template <int P> struct T2 {
+    static constexpr int R2 = P / 16, NP = R2 % 2 == 0 ? 2 : 1, H = R2 / NP;
+};
+
+// The H-point DFTs of pass 2 (TW_OUT = false) or pass A (TW_OUT = true) for column k1 and parity par2:
+// a[m] = the output of row NP m + par2 (times W_P^{k1 (NP m + par2)} in pass A).  col(j) returns the column's
 // row j (from shared or global memory).
 template <int P, bool TW_OUT, typename C, typename Col>
-__device__ __forceinline__ void t2_col_vals(C (&a)[P / 32], Col col, int k1, int par2, const C* __restrict__ tw,
+__device__ __forceinline__ void t2_col_vals(C (&a)[T2<P>::H], Col col, int k1, int par2, const C* __restrict__ tw,
                                             const C* __restrict__ ta) {
-    constexpr int R2 = P / 16, H = R2 / 2;
+    constexpr int H = T2<P>::H, NP = T2<P>::NP;
+    if constexpr (NP == 2) {
 #pragma unroll
-    for (int j = 0; j < H; ++j) {
-        const C lo = col(j), hi = col(j + H);
-        a[j] = par2 ? csub(lo, hi) : cadd(lo, hi);
-    }
-    if (par2) {
+        for (int j = 0; j < H; ++j) {
+            const C lo = col(j), hi = col(j + H);
+            a[j] = par2 ? csub(lo, hi) : cadd(lo, hi);
+        }
+        if (par2) {
 #pragma unroll
-        for (int j = 1; j < H; ++j) a[j] = cmul(a[j], tw[16 * j]);  // W_R2^j
+            for (int j = 1; j < H; ++j) a[j] = cmul(a[j], tw[16 * j]);  // W_R2^j
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < H; ++j) a[j] = col(j);
     }
     Dft<H, C>::run(a);
     if constexpr (TW_OUT) {
 #pragma unroll
-        for (int m = 0; m < H; ++m) a[m] = cmul(a[m], ta[(2 * m + par2) * 16 + k1]);  // W_P^{k1 (2m + par2)}
+        for (int m = 0; m < H; ++m) a[m] = cmul(a[m], ta[(NP * m + par2) * 16 + k1]);  // W_P^{k1 (NP m + par2)}
     }
 }
 
-// Pass 2 / pass A in place on a shared line: reads column k1, writes rows 2m + par2 of the same column.
+// Pass 2 / pass A in place on a shared line: reads column k1, writes rows NP m + par2 of the same column.
 // The caller pairs the roles par2 = 0 and 1 of a column in one warp; the column is read whole before
 // either writes (a __syncwarp between the reads and the writes).
 template <int P, bool TW_OUT, typename C>
 __device__ __forceinline__ void t2_cols(C* line, int k1, int par2, const C* __restrict__ tw, const C* __restrict__ ta) {
-    constexpr int H = P / 32;
+    constexpr int H = T2<P>::H, NP = T2<P>::NP;
     C a[H];
     t2_col_vals<P, TW_OUT>(a, [&](int j) { return line[t2_at(j, k1)]; }, k1, par2, tw, ta);
-    __syncwarp();
+    if constexpr (NP == 2) __syncwarp();
 #pragma unroll
-    for (int m = 0; m < H; ++m) line[t2_at(2 * m + par2, k1)] = a[m];
+    for (int m = 0; m < H; ++m) line[t2_at(NP * m + par2, k1)] = a[m];
 }
 
 // Pass B of row y2: v[m] = Y[y2 + R2 (2m + par)] for m < 4 (the outputs below P/2).
@@ -569,18 +547,6 @@ __device__ __forceinline__ void t2_passB(C (&v)[8], const C* line, int y2, int p
     }
     if (par) mul_w16_ramp(v);
     Dft<8, C>::run(v);
-}
-
-// Dispatch: compile-time plan when PC > 0 (tw = per-stage table), the runtime plan otherwise (tw =
-// flat table).
-// The pruning flags apply to the compile-time path only; they require the zero padding / the unread
-// outputs to cover at least the upper half of the line (true for padded length 2n when n <= P/2).
-template <int PC, bool ZERO_HI_IN = false, bool HI_OUT_UNUSED = false, typename C>
-__device__ __forceinline__ void fft_lines_any(C* buf, const C* tw, const FftPlan& plan, int LS, int L, int tid, int nthr) {
-    if constexpr (PC > 0)
-        fft_lines_c<PC, ZERO_HI_IN, HI_OUT_UNUSED>(buf, tw, LS, L, tid, nthr);
-    else
-        fft_lines(buf, tw, plan, LS, L, tid, nthr);
 }
 
 }  // namespace ss

@@ -24,7 +24,6 @@ constexpr int kMaxThreadsX = 512;   // largest block of the x-transform kernels 
 constexpr int kMinBlocksX = 2;      // resident 512-thread blocks per SM they are compiled for (64 registers)
 constexpr int kMaxThreadsYz = 384;  // block size of the y/z kernel (3 x 128: one z-convolution row per warp)
 constexpr int kMinBlocksYz = 2;
-constexpr int kYzKxb1 = 4;          // kx columns per CTA of the y/z kernel for single-layer films
 constexpr int kMaxThreads128 = 384;  // length-128 x kernels: at most 8 rows of 48 threads
 constexpr int kMinBlocks128 = 3;     // resident 384-thread blocks per SM of the length-128 kernels (56 registers)
 constexpr int kArcMaxChunk = 8;     // image differences one arc CTA accumulates
@@ -75,11 +74,9 @@ template <typename T> struct GroupArgs {
     T* sp;
     cplx<T>* spec;
     const T* dhat;
-    const cplx<T>* twx;   // flat twiddle tables W_P^k (runtime plans)
+    const cplx<T>* twx;   // flat twiddle tables W_P^k
     const cplx<T>* twy;
-    const cplx<T>* twxs;  // per-stage twiddle tables (compile-time plans), P entries each
-    const cplx<T>* twys;
-    // two-pass transforms (P = 128, 192, 256, 384), 2P entries each, laid out so that the lanes of a warp
+    // two-pass transforms (P a multiple of 16), 2P entries each, laid out so that the lanes of a warp
     // read consecutive entries: [0, P) pass 1, W_P^{n2 (2m + par)} at (2m + par) * P/16 + n2; [P, 2P) pass A,
     // W_P^{k1 (2m + par2)} at P + (2m + par2) * 16 + k1
     const cplx<T>* t2x;
@@ -203,18 +200,37 @@ inline size_t f128_yz_smem(int nz, int Py, bool* stage_dhat) {
 }
 
 
-// Lengths 192, 256 and 384 in two register passes (FP32, ss_fft.cuh): a line is R2 = P/16 rows of 16 at
-// row stride kT2Row; the y/z kernel for those Py with 1, 4 or 8 layers (24 lines per CTA: 8, 2 or 1 kx
-// columns), the x kernels for those Px with kX2Rows rows per CTA.
+// Lengths P = 16 R2 in two register passes (FP32, ss_fft.cuh, ss_twopass.cuh): a line is R2 = P/16 rows of 16
+// at row stride kT2Row; the y/z kernel for those Py with 1 to 8 layers, the x kernels for those Px with
+// kX2Rows rows per CTA.  The list covers lattices of up to 256 sites a side; each length is a multiple of 16
+// whose passes need DFTs of at most 16 points.
+#define SS_T2_LENGTHS(X) \
+    X(32) X(48) X(64) X(80) X(96) X(112) X(128) X(144) X(160) X(192) X(224) X(256) X(288) X(320) X(384) X(448) X(512)
+inline bool t2_length(int P) {
+    switch (P) {
+#define SS_CASE(L) case L:
+        SS_T2_LENGTHS(SS_CASE)
+#undef SS_CASE
+        return true;
+        default: return false;
+    }
+}
+// The smallest two-pass length >= m, or 0.
+inline int t2_length_from(int m) {
+    for (int P = (m + 15) / 16 * 16; P <= 512; P += 16)
+        if (t2_length(P)) return P;
+    return 0;
+}
 constexpr int kT2Row = 17;
+constexpr int kT2MaxNz = 8;
 __host__ __device__ constexpr int t2_line(int P) { return kT2Row * (P / 16); }
 constexpr int kYz2Threads = 384;
-// kx columns per CTA: the default (24 lines) and the alternative the autotuner also times (12 lines for
+// kx columns per CTA: the default (15 to 24 lines) and the alternative the autotuner also times (12 lines for
 // one or four layers); 0 when nz has no two-pass kernel
-inline int yz2p_kxb(int nz) { return nz == 1 ? 8 : nz == 4 ? 2 : nz == 8 ? 1 : 0; }
+inline int yz2p_kxb(int nz) { return nz == 1 ? 8 : nz == 2 ? 4 : nz <= 4 ? 2 : nz <= kT2MaxNz ? 1 : 0; }
 inline int yz2p_kxb_alt(int nz) { return nz == 1 ? 4 : nz == 4 ? 1 : 0; }
 inline bool yz2p_ok(int real_bytes, int Py, int nz, int Px) {
-    if (real_bytes != 4 || !(Py == 192 || Py == 256 || Py == 384)) return false;
+    if (real_bytes != 4 || !t2_length(Py) || f128_yz(real_bytes, Py, nz)) return false;
     const int kxb = yz2p_kxb(nz);
     return kxb > 0 && Px % kxb == 0;
 }
@@ -222,13 +238,28 @@ inline bool yz2p_ok(int real_bytes, int Py, int nz, int Px) {
 inline int yz2p_kxb_use(int nz, int tuned) { return tuned > 0 && (tuned == yz2p_kxb(nz) || tuned == yz2p_kxb_alt(nz)) ? tuned : yz2p_kxb(nz); }
 inline size_t yz2p_smem(int Py, int nz, int kxb) { return (size_t)3 * nz * kxb * t2_line(Py) * 8; }
 constexpr int kX2Rows = 4;
-constexpr int kX2Threads = 384;
+// threads of an x CTA: short lines have fewer roles than 384 threads would take
+__host__ __device__ constexpr int x2_threads(int P) { return P <= 48 ? 128 : P <= 80 ? 192 : P <= 160 ? 256 : 384; }
 __host__ __device__ constexpr int x2_round(int v) { return v + ((16 / kX2Rows - v % 16) + 16) % 16; }
 __host__ __device__ constexpr int x2_lsx(int P) { return x2_round(t2_line(P) - 1); }  // transform lines
 __host__ __device__ constexpr int x2_lb(int P) { return x2_round(fft_pad(P / 2 - 1) + 1); }  // x-space lines
-inline bool x2p_ok(int real_bytes, int Px) { return real_bytes == 4 && (Px == 192 || Px == 256 || Px == 384); }
+inline bool x2p_ok(int real_bytes, int Px) { return real_bytes == 4 && t2_length(Px) && !f128_x(real_bytes, Px); }
 inline size_t x2_smem(int P, bool inverse) {
     return (size_t)3 * kX2Rows * (x2_lsx(P) + x2_lb(P)) * 8 + (inverse ? 32 * 2 * kEvalTerms * 8 : 0);
+}
+// Padded transform length for n sites: the smallest 2^a 3^b >= 2n - 1, or the power of two >= 2n - 1 when that
+// is at most 1/8 longer.
+inline int padded_smooth(int n) {
+    auto smooth = [](int m) {
+        while (m % 2 == 0) m /= 2;
+        while (m % 3 == 0) m /= 3;
+        return m == 1;
+    };
+    int m = n > 1 ? 2 * n - 1 : 1;
+    while (!smooth(m)) ++m;
+    int p2 = 1;
+    while (p2 < 2 * n - 1) p2 <<= 1;
+    return 8 * p2 <= 9 * m ? p2 : m;
 }
 
 
@@ -265,6 +296,15 @@ template <typename T, typename Tin>
 void launch_aos_to_soa(const Tin* src, T* dst, int K, int N, int* err, cudaStream_t st);
 template <typename T, typename Tout>
 void launch_soa_to_aos(const T* src, Tout* dst, int K, int N, Tout scale, cudaStream_t st);
+// Two-pass kernels of one length P (ss_twopass.cuh, one translation unit per length): the x kernels for
+// g.Px = P (the x-inverse kernel in the given mode of xinv_sites), the y/z kernel for g.Py = P, and the
+// dynamic shared-memory limit of all of them.
+template <typename T, int P> void t2_xfwd(const GroupArgs<T>& g, cudaStream_t st);
+template <typename T, int P> void t2_xinv(const GroupArgs<T>& g, int mode, T dt, T* hout, bool pdl, cudaStream_t st);
+template <typename T, int P> void t2_yz(const GroupArgs<T>& g, cudaStream_t st);
+template <typename T, int P> void t2_smem_limits(int bytes);
+// The limits of the two-pass kernels of lengths Px and Py (those that have some).
+void set_t2_smem_limits(int Px, int Py, int bytes);
 void launch_interp_identity(InterpEntry* tab, int img0, int K, cudaStream_t st);
 // the FP32 state [K][3][N] handed to the FP64 energy evaluation: every spin renormalised in FP64
 void launch_widen_unit(const float* src, double* dst, int K, int N, const int* pair_on, cudaStream_t st);

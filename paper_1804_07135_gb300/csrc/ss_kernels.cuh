@@ -220,7 +220,7 @@ __device__ __forceinline__ void xfwd_gather(const GroupArgs<T>& g, cplx<T>* buf,
 // images of pair p: s[img] = normalise((1-t) sp[src0] + t sp[src1]) (or a copy), written back to s,
 // packed as re/im of 3*rows complex lines, zero-padded to Px and transformed along x.
 // Output spec[p][kx][c][z][y].
-template <typename T, bool DO_FFT, int PX>
+template <typename T, bool DO_FFT>
 __global__ void __launch_bounds__(kMaxThreadsX, kMinBlocksX) xfwd_kernel(GroupArgs<T> g) {
     using C = cplx<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(kMaxThreadsX, kMinBlocksX) xfwd_kernel(GroupAr
     const int nx = g.nx;
     if (g.pair_on && !g.pair_on[p]) return;  // uniform over the CTA
     if (DO_FFT)
-        for (int i = tid; i < g.Px; i += nthr) tw[i] = PX > 0 ? g.twxs[i] : g.twx[i];
+        for (int i = tid; i < g.Px; i += nthr) tw[i] = g.twx[i];
     griddep_wait();
     griddep_launch_dependents();
     xfwd_gather(g, DO_FFT ? buf : (C*)nullptr, g.lsx, rows, p, z, y0, rows, tid, nthr);
@@ -243,9 +243,9 @@ __global__ void __launch_bounds__(kMaxThreadsX, kMinBlocksX) xfwd_kernel(GroupAr
         buf[line * g.lsx + fft_pad(x)] = C{T(0), T(0)};
     }
     __syncthreads();
-    fft_lines_any<PX, true, false>(buf, tw, g.planx, g.lsx, 3 * rows, tid, nthr);
+    fft_lines(buf, tw, g.planx, g.lsx, 3 * rows, tid, nthr);
     // transpose out: each thread writes the rows of one (kx, c), contiguous in y
-    const int Px = PX > 0 ? PX : g.Px;
+    const int Px = g.Px;
     C* outp = g.spec + (size_t)p * Px * 3 * g.nz * g.ny;
     for (int kc = tid; kc < Px * 3; kc += nthr) {
         const int kx = kc / 3, c = kc - 3 * kx;
@@ -492,21 +492,19 @@ __device__ __forceinline__ void zconv_any(C* A, int lsy, int Py, int nz, int kx,
     }
 }
 
-// KXB > 1 (single-layer films): KXB consecutive kx columns per CTA (their spectra are contiguous), so
-// the short per-column work is amortised over more lines per barrier; the tensor slab is then read
-// through L1 (stage_dhat is ignored).
-template <typename T, int PY, int NZ, int KXB = 1>
+// The y/z kernel of the lengths without two-pass kernels (runtime plan); NZ > 0: that many layers, unrolled.
+template <typename T, int NZ>
 __global__ void __launch_bounds__(kMaxThreadsYz, kMinBlocksYz) yz_kernel(GroupArgs<T> g, int stage_dhat) {
     using C = cplx<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* tw = reinterpret_cast<C*>(smem_raw);
-    C* A = tw + g.Py;  // KXB*3*nz lines of stride lsy
+    C* A = tw + g.Py;  // 3*nz lines of stride lsy
     const int tid = threadIdx.x, nthr = blockDim.x;
-    const int kx = blockIdx.x * KXB, p = blockIdx.y;
+    const int kx = blockIdx.x, p = blockIdx.y;
     if (g.pair_on && !g.pair_on[p]) return;  // uniform over the CTA
-    const int Py = PY > 0 ? PY : g.Py;
+    const int Py = g.Py;
     const int nz = NZ > 0 ? NZ : g.nz;
-    const int ny = g.ny, L = 3 * nz * KXB;
+    const int ny = g.ny, L = 3 * nz;
     const int hy = Py / 2;
     const int kxo = min(kx, g.Px - kx);
     C* blk = g.spec + ((size_t)p * g.Px + kx) * 3 * nz * ny;
@@ -515,33 +513,24 @@ __global__ void __launch_bounds__(kMaxThreadsYz, kMinBlocksYz) yz_kernel(GroupAr
     const T* dslab = g.dhat + (size_t)kxo * (hy + 1) * nz * 6;
     const int dk = 1, dq = hy + 1;  // strides of kyo and of (|dz|*6 + comp)
     T* dsm = reinterpret_cast<T*>(A + L * g.lsy);
-    if (KXB == 1 && stage_dhat) {
+    if (stage_dhat) {
         for (int i = tid; i < (hy + 1) * nz * 6; i += nthr) dsm[i] = dslab[i];
         dslab = dsm;
     }
-    for (int i = tid; i < Py; i += nthr) tw[i] = PY > 0 ? g.twys[i] : g.twy[i];
+    for (int i = tid; i < Py; i += nthr) tw[i] = g.twy[i];
     griddep_wait();
     griddep_launch_dependents();
     for (int it = tid; it < L * Py; it += nthr) {
-        const int line = it / Py, y = it - line * Py;  // Py is a constant in the specialised variants
+        const int line = it / Py, y = it - line * Py;
         A[line * g.lsy + fft_pad(y)] = (y < ny) ? blk[line * ny + y] : C{T(0), T(0)};
     }
     __syncthreads();
-    fft_lines_any<PY, true, false>(A, tw, g.plany, g.lsy, L, tid, nthr);
-    if constexpr (KXB == 1) {
-        if constexpr (NZ > 0)
-            zconv_c<NZ>(A, A, g.lsy, Py, kx, g.Px, dslab, dk, dq, tid, nthr);
-        else
-            zconv_any(A, g.lsy, Py, nz, kx, g.Px, dslab, dk, dq, tid, nthr);
-    } else {
-        static_assert(NZ > 0, "several kx per CTA only with a compile-time layer count");
-        for (int b = 0; b < KXB; ++b) {
-            const int kxb = kx + b, kxob = min(kxb, g.Px - kxb);
-            zconv_c<NZ>(A + (size_t)b * 3 * NZ * g.lsy, A + (size_t)b * 3 * NZ * g.lsy, g.lsy, Py, kxb, g.Px,
-                        g.dhat + (size_t)kxob * (hy + 1) * NZ * 6, dk, dq, tid, nthr);
-        }
-    }
-    fft_lines_any<PY, false, true>(A, tw, g.plany, g.lsy, L, tid, nthr);
+    fft_lines(A, tw, g.plany, g.lsy, L, tid, nthr);
+    if constexpr (NZ > 0)
+        zconv_c<NZ>(A, A, g.lsy, Py, kx, g.Px, dslab, dk, dq, tid, nthr);
+    else
+        zconv_any(A, g.lsy, Py, nz, kx, g.Px, dslab, dk, dq, tid, nthr);
+    fft_lines(A, tw, g.plany, g.lsy, L, tid, nthr);
     for (int it = tid; it < L * ny; it += nthr) {
         const int line = it / ny, y = it - line * ny;
         blk[line * ny + y] = cconj(A[line * g.lsy + fft_pad(y)]);
@@ -617,140 +606,6 @@ __global__ void __launch_bounds__(kMaxThreadsYz, kMinBlocks128) yz128_kernel(Gro
 #pragma unroll
         for (int k2 = 0; k2 < 4; ++k2)
             if (k1 + 16 * k2 < ny) dst[16 * k2] = cconj(v[k2]);
-    }
-}
-
-// yz for Py = P in {192, 256, 384} (ny <= P/2), FP32, NZ layers, KXB kx columns per CTA: the y-transforms
-// in two register passes each way (t2_pass1 / t2_cols / t2_passB, ss_fft.cuh) on lines held in the
-// 17-strided row layout, the z-convolution in place between them.  One shared line per (column, component,
-// layer): 3 NZ KXB lines of t2_line(P) complex elements, read from the spectrum in pass 1 and written back
-// (rows y < ny) in pass B; one shared-memory round trip per pass instead of one per Stockham stage.
-// 384 threads; pass 2 and pass A take one warp per line (16 columns x 2 parities).  Three CTAs per SM,
-// two at P = 384 (its 78 KB lines; there the kernel keeps 80 registers, which runs a batch of size groups
-// faster than three CTAs of 56 registers would, although one group alone runs faster with three).
-template <int NZ, int P>
-__device__ __forceinline__ void zconv_t2(float2* A, int kx, int Px, const float* dslab, int tid, int nthr) {
-    constexpr int LS = t2_line(P), hy = P / 2, dq = P / 2 + 1;
-    const float sxg = kx > Px / 2 ? -1.f : 1.f;
-    const int nk = nthr / 3;
-    // rounds of nk frequencies; a round reads and writes only its own ky, so one barrier (between its
-    // reads and its writes) orders it against every other round
-    for (int k0 = 0; k0 < P; k0 += nk) {
-        const int a = tid / nk;
-        const int ky = k0 + (tid - a * nk);
-        const bool act = a < 3 && ky < P;
-        float2 out[NZ];
-        int pky = 0;
-        if (act) {
-            const int kyo = min(ky, P - ky);
-            const float syg = ky > hy ? -1.f : 1.f;
-            const float* d = dslab + kyo;
-            pky = t2_pos(ky);
-            const int i0 = a == 0 ? 0 : (a == 1 ? 3 : 4);
-            const int i1 = a == 0 ? 3 : (a == 1 ? 1 : 5);
-            const int i2 = a == 0 ? 4 : (a == 1 ? 5 : 2);
-            const float f0 = a == 0 ? 1.f : (a == 1 ? sxg * syg : sxg);
-            const float f1 = a == 0 ? sxg * syg : (a == 1 ? 1.f : syg);
-            const float f2 = a == 0 ? sxg : (a == 1 ? syg : 1.f);
-            float e0[NZ], e1[NZ], e2[NZ];
-#pragma unroll
-            for (int q = 0; q < NZ; ++q) {
-                e0[q] = d[(q * 6 + i0) * dq] * f0;
-                e1[q] = d[(q * 6 + i1) * dq] * f1;
-                e2[q] = d[(q * 6 + i2) * dq] * f2;
-            }
-#pragma unroll
-            for (int z = 0; z < NZ; ++z) out[z] = make_float2(0.f, 0.f);
-            // paired FP32 form as in zconv_c: out += (e, e) * S and (g, g) * (i S), i S = (-S.y, S.x)
-            if (a < 2) {
-#pragma unroll
-                for (int zp = 0; zp < NZ; ++zp) {
-                    const float2 sx = A[(0 * NZ + zp) * LS + pky];
-                    const float2 sy = A[(1 * NZ + zp) * LS + pky];
-                    const float2 sz = A[(2 * NZ + zp) * LS + pky];
-                    const float2 isz = make_float2(-sz.y, sz.x), nisz = make_float2(sz.y, -sz.x);
-#pragma unroll
-                    for (int z = 0; z < NZ; ++z) {
-                        const int q = z >= zp ? z - zp : zp - z;
-                        out[z] = __ffma2_rn(make_float2(e0[q], e0[q]), sx, out[z]);
-                        out[z] = __ffma2_rn(make_float2(e1[q], e1[q]), sy, out[z]);
-                        out[z] = __ffma2_rn(make_float2(e2[q], e2[q]), z >= zp ? isz : nisz, out[z]);
-                    }
-                }
-            } else {
-#pragma unroll
-                for (int zp = 0; zp < NZ; ++zp) {
-                    const float2 sx = A[(0 * NZ + zp) * LS + pky];
-                    const float2 sy = A[(1 * NZ + zp) * LS + pky];
-                    const float2 sz = A[(2 * NZ + zp) * LS + pky];
-                    const float2 isx = make_float2(-sx.y, sx.x), nisx = make_float2(sx.y, -sx.x);
-                    const float2 isy = make_float2(-sy.y, sy.x), nisy = make_float2(sy.y, -sy.x);
-#pragma unroll
-                    for (int z = 0; z < NZ; ++z) {
-                        const int q = z >= zp ? z - zp : zp - z;
-                        out[z] = __ffma2_rn(make_float2(e0[q], e0[q]), z >= zp ? isx : nisx, out[z]);
-                        out[z] = __ffma2_rn(make_float2(e1[q], e1[q]), z >= zp ? isy : nisy, out[z]);
-                        out[z] = __ffma2_rn(make_float2(e2[q], e2[q]), sz, out[z]);
-                    }
-                }
-            }
-        }
-        __syncthreads();
-        if (act) {
-#pragma unroll
-            for (int z = 0; z < NZ; ++z) A[(a * NZ + z) * LS + pky] = cconj(out[z]);
-        }
-    }
-}
-
-template <int P, int NZ, int KXB>
-__global__ void __launch_bounds__(kYz2Threads, P == 384 ? 2 : 3) yz2p_kernel(GroupArgs<float> g) {
-    using C = float2;
-    constexpr int R2 = P / 16, LS = t2_line(P), L = 3 * NZ * KXB;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* A = reinterpret_cast<C*>(smem_raw);
-    const int tid = threadIdx.x, nthr = blockDim.x;
-    const int kx = blockIdx.x * KXB, p = blockIdx.y;
-    const int ny = g.ny;
-    C* blk = g.spec + ((size_t)p * g.Px + kx) * 3 * NZ * ny;  // KXB consecutive columns are contiguous
-    const C* __restrict__ tw = g.twy;                         // W_P^k
-    const C* __restrict__ t1 = g.t2y;                         // pass 1
-    const C* __restrict__ ta = g.t2y + P;                     // pass A
-    griddep_wait();
-    griddep_launch_dependents();
-    // pass 1, role (n2, line, par), n2 fastest: the zero-padded spectrum lines in, rows of Z out
-    for (int r = tid; r < 2 * R2 * L; r += nthr) {
-        const int n2 = r % R2, q = r / R2, line = q % L, par = q / L;
-        const C* src = blk + (size_t)line * ny + n2;
-        C u[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) u[j] = R2 * j + n2 < ny ? src[R2 * j] : make_float2(0.f, 0.f);
-        t2_pass1<P>(u, n2, par, t1, A + line * LS);
-    }
-    __syncthreads();
-    // pass 2: one warp per line (lanes = 16 columns x 2 parities)
-    for (int r = tid; r < 32 * L; r += nthr) t2_cols<P, false>(A + (r >> 5) * LS, r & 15, (r >> 4) & 1, tw, ta);
-    __syncthreads();
-#pragma unroll 1
-    for (int b = 0; b < KXB; ++b) {
-        const int kxb = kx + b, kxo = min(kxb, g.Px - kxb);
-        zconv_t2<NZ, P>(A + b * 3 * NZ * LS, kxb, g.Px, g.dhat + (size_t)kxo * (P / 2 + 1) * NZ * 6, tid, nthr);
-    }
-    __syncthreads();
-    // pass A (the inverse transform of the conjugated field spectra, in place by columns)
-    for (int r = tid; r < 32 * L; r += nthr) t2_cols<P, true>(A + (r >> 5) * LS, r & 15, (r >> 4) & 1, tw, ta);
-    __syncthreads();
-    // pass B, role (y2, line, par): rows y < ny back to the spectrum, conjugated
-    for (int r = tid; r < 2 * R2 * L; r += nthr) {
-        const int y2 = r % R2, q = r / R2, line = q % L, par = q / L;
-        C v[8];
-        t2_passB(v, A + line * LS, y2, par);
-        C* dst = blk + (size_t)line * ny;
-#pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            const int y = y2 + R2 * (2 * m + par);
-            if (y < ny) dst[y] = cconj(v[m]);
-        }
     }
 }
 
@@ -1027,6 +882,8 @@ __device__ __forceinline__ void xinv_sites(const GroupArgs<T>& g, T dt, T* hout,
     }
     if constexpr (MODE == 2 || MODE == 5)
         if (dt == T(0)) return;  // uniform over the grid: no energy partials wanted
+    if constexpr (MODE == 1)
+        if (!g.epart) return;  // the field alone
     if constexpr (MODE != 1)
         block_reduce_t2d<2>(eacc, acc, red);
     else if constexpr (std::is_same<T, float>::value)
@@ -1058,7 +915,7 @@ __device__ __forceinline__ void xinv_sites(const GroupArgs<T>& g, T dt, T* hout,
 // MODE 1 (eval): FP64 energy terms of the FP64-renormalised spins, bonds to +x, +y, +z counted once
 //                (Eq. 1): tJ = -sum s_i.s_j, tD = sum (r_ij x z).(s_i x s_j), tK = -sum s_z^2,
 //                tw = -(1/2) sum conv.s; optionally the field h.
-template <typename T, bool DO_FFT, int MODE, int PX>
+template <typename T, bool DO_FFT, int MODE>
 __global__ void __launch_bounds__(kMaxThreadsX, kMinBlocksX) xinv_kernel(GroupArgs<T> g, T dt, T* hout) {
     using C = cplx<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1071,11 +928,11 @@ __global__ void __launch_bounds__(kMaxThreadsX, kMinBlocksX) xinv_kernel(GroupAr
     const int ny = g.ny, nz = g.nz;
     if (g.pair_on && !g.pair_on[p]) return;  // uniform over the CTA
     if (DO_FFT)
-        for (int i = tid; i < g.Px; i += nthr) tw[i] = PX > 0 ? g.twxs[i] : g.twx[i];
+        for (int i = tid; i < g.Px; i += nthr) tw[i] = g.twx[i];
     griddep_wait();
     griddep_launch_dependents();
     if (DO_FFT) {
-        const int Px = PX > 0 ? PX : g.Px;
+        const int Px = g.Px;
         const C* inp = g.spec + (size_t)p * Px * 3 * nz * ny;
         for (int kc = tid; kc < Px * 3; kc += nthr) {
             const int kx = kc / 3, c = kc - 3 * kx;
@@ -1084,7 +941,7 @@ __global__ void __launch_bounds__(kMaxThreadsX, kMinBlocksX) xinv_kernel(GroupAr
             for (int yy = 0; yy < rows; ++yy) b[yy * g.lsx] = cconj(s[yy]);
         }
         __syncthreads();
-        fft_lines_any<PX, false, true>(buf, tw, g.planx, g.lsx, 3 * rows, tid, nthr);
+        fft_lines(buf, tw, g.planx, g.lsx, 3 * rows, tid, nthr);
     }
     xinv_sites<T, DO_FFT, MODE>(g, dt, hout, buf, g.lsx, red, p, z, y0, rows, tid, nthr);
 }
@@ -1138,104 +995,6 @@ __global__ void __launch_bounds__(kMaxThreads128, kMinBlocks128) xinv128_kernel(
     }
     __syncthreads();
     xinv_sites<T, true, MODE>(g, dt, hout, buf, kF128Buf, red, p, z, y0, rows, tid, nthr);
-}
-
-// ------------------------------------------------------------------------------------------------
-// x kernels for Px = P in {192, 256, 384} (nx <= P/2), FP32: the x-transforms in two register passes
-// (ss_fft.cuh) on kX2Rows rows of one layer of an image pair per CTA.  Every role order puts the rows
-// fastest across a warp: the spectrum's rows of one (kx, c) are contiguous in global memory, and with
-// line strides = 16 / kX2Rows (mod 16) the lanes of a half-warp (kX2Rows rows x 16 / kX2Rows consecutive
-// columns or rows of a line) hit distinct shared-memory banks.
-// xfwd: the gather (Eq. 12) into x-space lines, pass 1 into the transform lines, pass 2 straight to the
-// spectrum spec[p][kx][c][z][y].
-template <int P>
-__global__ void __launch_bounds__(kX2Threads, 3) xfwd2p_kernel(GroupArgs<float> g) {
-    using C = float2;
-    constexpr int R2 = P / 16, H = R2 / 2, ROWS = kX2Rows, L = 3 * ROWS, LSX = x2_lsx(P), LB = x2_lb(P);
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* xb = reinterpret_cast<C*>(smem_raw);  // line c * ROWS + yy: the pair at x, fft_pad positions
-    C* A = xb + L * LB;                       // line c * ROWS + yy: rows of Z
-    const int tid = threadIdx.x, nthr = blockDim.x;
-    const int p = blockIdx.z, z = blockIdx.y, y0 = blockIdx.x * ROWS;
-    const int rows = min(ROWS, g.ny - y0), nx = g.nx;
-    const C* __restrict__ tw = g.twx;  // W_P^k
-    const C* __restrict__ t1 = g.t2x;  // pass 1
-    griddep_wait();
-    griddep_launch_dependents();
-    xfwd_gather(g, xb, LB, ROWS, p, z, y0, rows, tid, nthr);
-    __syncthreads();
-    // pass 1, role (yy, n2, c, par)
-    for (int r = tid; r < 2 * R2 * L; r += nthr) {
-        const int yy = r % ROWS, q = r / ROWS, n2 = q % R2, q2 = q / R2, c = q2 % 3, par = q2 / 3;
-        if (yy >= rows) continue;
-        const C* b = xb + (c * ROWS + yy) * LB;
-        C u[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) u[j] = R2 * j + n2 < nx ? b[fft_pad(R2 * j + n2)] : make_float2(0.f, 0.f);
-        t2_pass1<P>(u, n2, par, t1, A + (c * ROWS + yy) * LSX);
-    }
-    __syncthreads();
-    // pass 2, role (yy, k1, par2, c): X[k1 + 16 (2m + par2)] to the spectrum
-    const size_t kstride = (size_t)3 * g.nz * g.ny;  // between consecutive kx
-    C* outp = g.spec + (size_t)p * P * kstride + (size_t)z * g.ny + y0;
-    for (int r = tid; r < 32 * L; r += nthr) {
-        const int yy = r % ROWS, q = r / ROWS, k1 = q & 15, par2 = (q >> 4) & 1, c = q >> 5;
-        if (yy >= rows) continue;
-        const C* col = A + (c * ROWS + yy) * LSX + k1;
-        C a[H];
-        t2_col_vals<P, false>(a, [&](int j) { return col[j * kT2Row]; }, k1, par2, tw, tw);
-        C* o = outp + (size_t)c * g.nz * g.ny + yy;
-#pragma unroll
-        for (int m = 0; m < H; ++m) o[(size_t)(k1 + 16 * (2 * m + par2)) * kstride] = a[m];
-    }
-}
-
-// xinv: pass A straight from the spectrum (conjugated) into the transform lines, pass B into x-space
-// lines (fft_pad positions, line c * rows + yy), then the per-site work of xinv_sites in mode MODE.
-template <int P, int MODE>
-__global__ void __launch_bounds__(kX2Threads, 3) xinv2p_kernel(GroupArgs<float> g, float dt, float* hout) {
-    using C = float2;
-    constexpr int R2 = P / 16, H = R2 / 2, ROWS = kX2Rows, L = 3 * ROWS, LSX = x2_lsx(P), LB = x2_lb(P);
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* A = reinterpret_cast<C*>(smem_raw);  // line c * ROWS + yy: columns of T
-    C* xb = A + L * LSX;                     // line c * rows + yy: the field convolution at x
-    double* red = reinterpret_cast<double*>(xb + L * LB);
-    const int tid = threadIdx.x, nthr = blockDim.x;
-    const int p = blockIdx.z, z = blockIdx.y, y0 = blockIdx.x * ROWS;
-    const int rows = min(ROWS, g.ny - y0), nx = g.nx;
-    const size_t kstride = (size_t)3 * g.nz * g.ny;
-    const C* inp = g.spec + (size_t)p * P * kstride + (size_t)z * g.ny + y0;
-    const C* __restrict__ tw = g.twx;
-    const C* __restrict__ ta = g.t2x + P;  // pass A
-    griddep_wait();
-    griddep_launch_dependents();
-    // pass A, role (yy, k1, par2, c): column k1 of the conjugated spectrum line (c, yy)
-    for (int r = tid; r < 32 * L; r += nthr) {
-        const int yy = r % ROWS, q = r / ROWS, k1 = q & 15, par2 = (q >> 4) & 1, c = q >> 5;
-        if (yy >= rows) continue;
-        const C* sc = inp + (size_t)c * g.nz * g.ny + yy + (size_t)k1 * kstride;
-        C a[H];
-        t2_col_vals<P, true>(a, [&](int j) { return cconj(sc[(size_t)16 * j * kstride]); }, k1, par2, tw, ta);
-        C* o = A + (c * ROWS + yy) * LSX + k1 + par2 * kT2Row;
-#pragma unroll
-        for (int m = 0; m < H; ++m) o[2 * m * kT2Row] = a[m];
-    }
-    __syncthreads();
-    // pass B, role (yy, y2, c, par): x = y2 + R2 (2m + par) < nx
-    for (int r = tid; r < 2 * R2 * L; r += nthr) {
-        const int yy = r % ROWS, q = r / ROWS, y2 = q % R2, q2 = q / R2, c = q2 % 3, par = q2 / 3;
-        if (yy >= rows) continue;
-        C v[8];
-        t2_passB(v, A + (c * ROWS + yy) * LSX, y2, par);
-        C* b = xb + (c * rows + yy) * LB;
-#pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            const int x = y2 + R2 * (2 * m + par);
-            if (x < nx) b[fft_pad(x)] = v[m];
-        }
-    }
-    __syncthreads();
-    xinv_sites<float, true, MODE>(g, dt, hout, xb, LB, red, p, z, y0, rows, tid, nthr);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -2204,7 +1963,7 @@ __global__ void __launch_bounds__(256) fft_strided_f64_kernel(double2* data, con
         buf[i * LS + fft_pad(e)] = data[base + e * elem_stride];
     }
     __syncthreads();
-    fft_lines(buf, tw, plan, LS, L, tid, nthr);
+    fft_lines<true>(buf, tw, plan, LS, L, tid, nthr);
     for (int it = tid; it < L * P; it += nthr) {
         const int i = it / P, e = it - i * P;
         const int l = l0 + i;
@@ -2307,11 +2066,12 @@ static inline void launch_ex(void (*kernel)(KArgs...), dim3 grid, dim3 block, si
 template <int MODE>
 static inline bool launch_xinv2p(const GroupArgs<float>& g, float dt, float* hout, bool pdl, cudaStream_t st) {
     if (!x2p_ok(4, g.Px)) return false;
-    const dim3 grid((g.ny + g.ty_c - 1) / g.ty_c, g.nz, g.n_pairs), blk(kX2Threads);
-    const size_t sm = x2_smem(g.Px, true);
-    if (g.Px == 192) launch_ex(xinv2p_kernel<192, MODE>, grid, blk, sm, st, pdl, g, dt, hout);
-    else if (g.Px == 256) launch_ex(xinv2p_kernel<256, MODE>, grid, blk, sm, st, pdl, g, dt, hout);
-    else launch_ex(xinv2p_kernel<384, MODE>, grid, blk, sm, st, pdl, g, dt, hout);
+    switch (g.Px) {
+#define SS_CASE(P) \
+    case P: t2_xinv<float, P>(g, MODE, dt, hout, pdl, st); break;
+        SS_T2_LENGTHS(SS_CASE)
+#undef SS_CASE
+    }
     return true;
 }
 
@@ -2321,24 +2081,24 @@ static inline int grid1d(size_t n, int thr) {
     return (int)(b ? b : 1);
 }
 
-// Compile-time padded lengths and (Py, nz) pairs of the workloads (FP32 only; the FP64 path and any
-// other size use the runtime plans).
-#define SS_FOR_PX(X) X(32) X(128) X(192) X(256) X(384)
-#define SS_FOR_PYNZ(X) X(32, 1) X(128, 4) X(128, 8) X(192, 4) X(256, 1) X(256, 4) X(256, 8) X(384, 8)
+// Layer counts with an unrolled z-convolution in the runtime-plan y/z kernel (FP32; the FP64 path and any
+// other count use the loop over layers).
 #define SS_FOR_NZ(X) X(1) X(4) X(8)
 
 template <typename T> void launch_xfwd(const GroupArgs<T>& g, bool do_fft, int nthr, size_t smem, cudaStream_t st) {
     dim3 grid((g.ny + g.ty_a - 1) / g.ty_a, g.nz, g.n_pairs);
     if (!do_fft) {
-        launch_pdl(xfwd_kernel<T, false, 0>, grid, dim3(nthr), 0, st, g);
+        launch_pdl(xfwd_kernel<T, false>, grid, dim3(nthr), 0, st, g);
         return;
     }
     if constexpr (std::is_same<T, float>::value) {
-        if (x2p_ok(4, g.Px)) {  // rows per CTA are kX2Rows (set by the host)
-            const size_t sm = x2_smem(g.Px, false);
-            if (g.Px == 192) launch_pdl(xfwd2p_kernel<192>, grid, dim3(kX2Threads), sm, st, g);
-            else if (g.Px == 256) launch_pdl(xfwd2p_kernel<256>, grid, dim3(kX2Threads), sm, st, g);
-            else launch_pdl(xfwd2p_kernel<384>, grid, dim3(kX2Threads), sm, st, g);
+        if (x2p_ok(4, g.Px)) {
+            switch (g.Px) {
+#define SS_CASE(P) \
+    case P: t2_xfwd<float, P>(g, st); break;
+                SS_T2_LENGTHS(SS_CASE)
+#undef SS_CASE
+            }
             return;
         }
         if (f128_x(4, g.Px)) {
@@ -2349,17 +2109,8 @@ template <typename T> void launch_xfwd(const GroupArgs<T>& g, bool do_fft, int n
             else launch_pdl(xfwd128_kernel<T, 8>, grid, blk, sm, st, g);  // rows per CTA are 2, 4 or 8
             return;
         }
-        switch (g.Px) {
-#define SS_CASE(P)                                                \
-    case P:                                                       \
-        launch_pdl(xfwd_kernel<T, true, P>, grid, dim3(nthr), smem, st, g); \
-        return;
-            SS_FOR_PX(SS_CASE)
-#undef SS_CASE
-            default: break;
-        }
     }
-    launch_pdl(xfwd_kernel<T, true, 0>, grid, dim3(nthr), smem, st, g);
+    launch_pdl(xfwd_kernel<T, true>, grid, dim3(nthr), smem, st, g);
 }
 
 template <typename T> void launch_yz(const GroupArgs<T>& g, int nthr, size_t smem, cudaStream_t st) {
@@ -2367,21 +2118,14 @@ template <typename T> void launch_yz(const GroupArgs<T>& g, int nthr, size_t sme
     const size_t base = (size_t)(g.Py + 3 * g.nz * g.lsy) * sizeof(cplx<T>);
     const int stage = smem >= base + (size_t)(g.Py / 2 + 1) * g.nz * 6 * sizeof(T);
     if constexpr (std::is_same<T, float>::value) {
-        if (yz2p_ok(4, g.Py, g.nz, g.Px) && g.Px % yz2p_kxb_use(g.nz, g.yz_kxb) == 0) {
-            const int kxb = yz2p_kxb_use(g.nz, g.yz_kxb);
-            const size_t sm = yz2p_smem(g.Py, g.nz, kxb);
-            const dim3 blk(kYz2Threads), gr(g.Px / kxb, g.n_pairs);
-#define SS_CASE(P)                                                                         \
-    if (g.Py == P) {                                                                       \
-        if (g.nz == 1 && kxb == 8) launch_pdl(yz2p_kernel<P, 1, 8>, gr, blk, sm, st, g);      \
-        else if (g.nz == 1) launch_pdl(yz2p_kernel<P, 1, 4>, gr, blk, sm, st, g);             \
-        else if (g.nz == 4 && kxb == 2) launch_pdl(yz2p_kernel<P, 4, 2>, gr, blk, sm, st, g); \
-        else if (g.nz == 4) launch_pdl(yz2p_kernel<P, 4, 1>, gr, blk, sm, st, g);             \
-        else launch_pdl(yz2p_kernel<P, 8, 1>, gr, blk, sm, st, g);                            \
-        return;                                                                            \
-    }
-            SS_CASE(192) SS_CASE(256) SS_CASE(384)
+        if (yz2p_ok(4, g.Py, g.nz, g.Px)) {
+            switch (g.Py) {
+#define SS_CASE(P) \
+    case P: t2_yz<float, P>(g, st); break;
+                SS_T2_LENGTHS(SS_CASE)
 #undef SS_CASE
+            }
+            return;
         }
         if (f128_yz(4, g.Py, g.nz)) {
             bool st128 = false;
@@ -2392,50 +2136,22 @@ template <typename T> void launch_yz(const GroupArgs<T>& g, int nthr, size_t sme
                 launch_pdl(yz128_kernel<T, 4>, grid, dim3(f128_yz_threads(4)), sm128, st, g, (int)st128);
             return;
         }
-        if (g.nz == 1 && g.Px % kYzKxb1 == 0) {  // single layer: several kx columns per CTA
-            const dim3 gridb(g.Px / kYzKxb1, g.n_pairs);
-            const size_t smb = (size_t)(g.Py + 3 * kYzKxb1 * g.lsy) * sizeof(cplx<T>);
-            if (g.Py == 256) {
-                launch_pdl(yz_kernel<T, 256, 1, kYzKxb1>, gridb, dim3(nthr), smb, st, g, 0);
-                return;
-            }
-            if (g.Py == 32) {
-                launch_pdl(yz_kernel<T, 32, 1, kYzKxb1>, gridb, dim3(nthr), smb, st, g, 0);
-                return;
-            }
-        }
-        if (g.nz == 4 && g.Px % 2 == 0 && (g.Py == 192 || g.Py == 256)) {  // four layers: two kx columns
-            const dim3 gridb(g.Px / 2, g.n_pairs);
-            const size_t smb = (size_t)(g.Py + 3 * 4 * 2 * g.lsy) * sizeof(cplx<T>);
-            if (g.Py == 192)
-                launch_pdl(yz_kernel<T, 192, 4, 2>, gridb, dim3(nthr), smb, st, g, 0);
-            else
-                launch_pdl(yz_kernel<T, 256, 4, 2>, gridb, dim3(nthr), smb, st, g, 0);
-            return;
-        }
-#define SS_CASE(P, Z)                                                   \
-    if (g.Py == P && g.nz == Z) {                                       \
-        launch_pdl(yz_kernel<T, P, Z>, grid, dim3(nthr), smem, st, g, stage); \
-        return;                                                         \
-    }
-        SS_FOR_PYNZ(SS_CASE)
-#undef SS_CASE
 #define SS_CASE(Z)                                                      \
     if (g.nz == Z) {                                                    \
-        launch_pdl(yz_kernel<T, 0, Z>, grid, dim3(nthr), smem, st, g, stage); \
+        launch_pdl(yz_kernel<T, Z>, grid, dim3(nthr), smem, st, g, stage); \
         return;                                                         \
     }
         SS_FOR_NZ(SS_CASE)
 #undef SS_CASE
     }
-    launch_pdl(yz_kernel<T, 0, 0>, grid, dim3(nthr), smem, st, g, stage);
+    launch_pdl(yz_kernel<T, 0>, grid, dim3(nthr), smem, st, g, stage);
 }
 
 template <typename T>
 void launch_xinv_step(const GroupArgs<T>& g, bool do_fft, T dt, int nthr, size_t smem, cudaStream_t st) {
     dim3 grid((g.ny + g.ty_c - 1) / g.ty_c, g.nz, g.n_pairs);
     if (!do_fft) {
-        launch_pdl(xinv_kernel<T, false, 0, 0>, grid, dim3(nthr), smem, st, g, dt, (T*)nullptr);
+        launch_pdl(xinv_kernel<T, false, 0>, grid, dim3(nthr), smem, st, g, dt, (T*)nullptr);
         return;
     }
     if constexpr (std::is_same<T, float>::value) {
@@ -2448,17 +2164,8 @@ void launch_xinv_step(const GroupArgs<T>& g, bool do_fft, T dt, int nthr, size_t
             else launch_pdl(xinv128_kernel<T, 0, 8>, grid, blk, sm, st, g, dt, (T*)nullptr);
             return;
         }
-        switch (g.Px) {
-#define SS_CASE(P)                                                            \
-    case P:                                                                   \
-        launch_pdl(xinv_kernel<T, true, 0, P>, grid, dim3(nthr), smem, st, g, dt, (T*)nullptr); \
-        return;
-            SS_FOR_PX(SS_CASE)
-#undef SS_CASE
-            default: break;
-        }
     }
-    launch_pdl(xinv_kernel<T, true, 0, 0>, grid, dim3(nthr), smem, st, g, dt, (T*)nullptr);
+    launch_pdl(xinv_kernel<T, true, 0>, grid, dim3(nthr), smem, st, g, dt, (T*)nullptr);
 }
 
 template <typename T>
@@ -2476,9 +2183,9 @@ void launch_xinv_eval(const GroupArgs<T>& g, bool do_fft, T* hout, int nthr, siz
         }
     }
     if (do_fft) {
-        xinv_kernel<T, true, 1, 0><<<grid, nthr, smem, st>>>(g, T(0), hout);
+        xinv_kernel<T, true, 1><<<grid, nthr, smem, st>>>(g, T(0), hout);
     } else {
-        xinv_kernel<T, false, 1, 0><<<grid, nthr, smem, st>>>(g, T(0), hout);
+        xinv_kernel<T, false, 1><<<grid, nthr, smem, st>>>(g, T(0), hout);
     }
 }
 
@@ -2498,9 +2205,9 @@ static void launch_xinv_force_mode(const GroupArgs<T>& g, bool do_fft, T* kout, 
         }
     }
     if (do_fft)
-        xinv_kernel<T, true, MODE, 0><<<grid, nthr, smem, st>>>(g, flag, kout);
+        xinv_kernel<T, true, MODE><<<grid, nthr, smem, st>>>(g, flag, kout);
     else
-        xinv_kernel<T, false, MODE, 0><<<grid, nthr, smem, st>>>(g, flag, kout);
+        xinv_kernel<T, false, MODE><<<grid, nthr, smem, st>>>(g, flag, kout);
 }
 
 template <typename T>
@@ -2528,9 +2235,9 @@ void launch_xinv_step_llg(const GroupArgs<T>& g, bool do_fft, T dt, int nthr, si
         }
     }
     if (do_fft)
-        launch_pdl(xinv_kernel<T, true, 4, 0>, grid, dim3(nthr), smem, st, g, dt, (T*)nullptr);
+        launch_pdl(xinv_kernel<T, true, 4>, grid, dim3(nthr), smem, st, g, dt, (T*)nullptr);
     else
-        launch_pdl(xinv_kernel<T, false, 4, 0>, grid, dim3(nthr), smem, st, g, dt, (T*)nullptr);
+        launch_pdl(xinv_kernel<T, false, 4>, grid, dim3(nthr), smem, st, g, dt, (T*)nullptr);
 }
 
 template <typename T>
@@ -2548,9 +2255,9 @@ void launch_xinv_step_climb(const GroupArgs<T>& g, bool do_fft, T dt, T* hc, int
         }
     }
     if (do_fft)
-        launch_pdl(xinv_kernel<T, true, 3, 0>, grid, dim3(nthr), smem, st, g, dt, hc);
+        launch_pdl(xinv_kernel<T, true, 3>, grid, dim3(nthr), smem, st, g, dt, hc);
     else
-        launch_pdl(xinv_kernel<T, false, 3, 0>, grid, dim3(nthr), smem, st, g, dt, hc);
+        launch_pdl(xinv_kernel<T, false, 3>, grid, dim3(nthr), smem, st, g, dt, hc);
 }
 
 template <typename T> void launch_dipole_direct(const GroupArgs<T>& g, T* hdir, cudaStream_t st) {
@@ -2639,20 +2346,20 @@ template <typename F> static inline void set_dyn_smem(F* kernel, int bytes) {
     cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes - (int)fa.sharedSizeBytes);
 }
 template <typename T> void set_smem_limits(int bytes) {
-    set_dyn_smem(xfwd_kernel<T, true, 0>, bytes);
-    set_dyn_smem(yz_kernel<T, 0, 0>, bytes);
-    set_dyn_smem(xinv_kernel<T, true, 0, 0>, bytes);
-    set_dyn_smem(xinv_kernel<T, true, 1, 0>, bytes);
-    set_dyn_smem(xinv_kernel<T, false, 0, 0>, bytes);
-    set_dyn_smem(xinv_kernel<T, false, 1, 0>, bytes);
-    set_dyn_smem(xinv_kernel<T, true, 2, 0>, bytes);
-    set_dyn_smem(xinv_kernel<T, false, 2, 0>, bytes);
-    set_dyn_smem(xinv_kernel<T, true, 3, 0>, bytes);
-    set_dyn_smem(xinv_kernel<T, false, 3, 0>, bytes);
-    set_dyn_smem(xinv_kernel<T, true, 4, 0>, bytes);
-    set_dyn_smem(xinv_kernel<T, false, 4, 0>, bytes);
-    set_dyn_smem(xinv_kernel<T, true, 5, 0>, bytes);
-    set_dyn_smem(xinv_kernel<T, false, 5, 0>, bytes);
+    set_dyn_smem(xfwd_kernel<T, true>, bytes);
+    set_dyn_smem(yz_kernel<T, 0>, bytes);
+    set_dyn_smem(xinv_kernel<T, true, 0>, bytes);
+    set_dyn_smem(xinv_kernel<T, true, 1>, bytes);
+    set_dyn_smem(xinv_kernel<T, false, 0>, bytes);
+    set_dyn_smem(xinv_kernel<T, false, 1>, bytes);
+    set_dyn_smem(xinv_kernel<T, true, 2>, bytes);
+    set_dyn_smem(xinv_kernel<T, false, 2>, bytes);
+    set_dyn_smem(xinv_kernel<T, true, 3>, bytes);
+    set_dyn_smem(xinv_kernel<T, false, 3>, bytes);
+    set_dyn_smem(xinv_kernel<T, true, 4>, bytes);
+    set_dyn_smem(xinv_kernel<T, false, 4>, bytes);
+    set_dyn_smem(xinv_kernel<T, true, 5>, bytes);
+    set_dyn_smem(xinv_kernel<T, false, 5>, bytes);
     set_dyn_smem(spline_apply_kernel<T>, 200 * 1024);
     set_dyn_smem(arc_kernel<T>, bytes);
     if constexpr (std::is_same<T, float>::value) {
@@ -2668,40 +2375,26 @@ template <typename T> void set_smem_limits(int bytes) {
 #undef SS_CASE
         set_dyn_smem(yz128_kernel<T, 4>, bytes);
         set_dyn_smem(yz128_kernel<T, 8>, bytes);
-#define SS_CASE(P)                                 \
-    set_dyn_smem(xfwd2p_kernel<P>, bytes);         \
-    set_dyn_smem(xinv2p_kernel<P, 0>, bytes);      \
-    set_dyn_smem(xinv2p_kernel<P, 1>, bytes);      \
-    set_dyn_smem(xinv2p_kernel<P, 2>, bytes);      \
-    set_dyn_smem(xinv2p_kernel<P, 3>, bytes);      \
-    set_dyn_smem(xinv2p_kernel<P, 4>, bytes);      \
-    set_dyn_smem(xinv2p_kernel<P, 5>, bytes);      \
-    set_dyn_smem(yz2p_kernel<P, 1, 4>, bytes);     \
-    set_dyn_smem(yz2p_kernel<P, 4, 1>, bytes);     \
-    set_dyn_smem(yz2p_kernel<P, 1, 8>, bytes);     \
-    set_dyn_smem(yz2p_kernel<P, 4, 2>, bytes);     \
-    set_dyn_smem(yz2p_kernel<P, 8, 1>, bytes);
-        SS_CASE(192) SS_CASE(256) SS_CASE(384)
-#undef SS_CASE
-#define SS_CASE(P)                                  \
-    set_dyn_smem(xfwd_kernel<T, true, P>, bytes);   \
-    set_dyn_smem(xinv_kernel<T, true, 0, P>, bytes);
-        SS_FOR_PX(SS_CASE)
-#undef SS_CASE
-        set_dyn_smem(yz_kernel<T, 256, 1, kYzKxb1>, bytes);
-        set_dyn_smem(yz_kernel<T, 32, 1, kYzKxb1>, bytes);
-        set_dyn_smem(yz_kernel<T, 192, 4, 2>, bytes);
-        set_dyn_smem(yz_kernel<T, 256, 4, 2>, bytes);
-#define SS_CASE(P, Z) set_dyn_smem(yz_kernel<T, P, Z>, bytes);
-        SS_FOR_PYNZ(SS_CASE)
-#undef SS_CASE
-#define SS_CASE(Z) set_dyn_smem(yz_kernel<T, 0, Z>, bytes);
+#define SS_CASE(Z) set_dyn_smem(yz_kernel<T, Z>, bytes);
         SS_FOR_NZ(SS_CASE)
 #undef SS_CASE
     }
 }
 
 #ifdef SS_COMMON_LAUNCHERS
+void set_t2_smem_limits(int Px, int Py, int bytes) {
+    for (int P : {Px, Py}) {
+        switch (P) {
+#define SS_CASE(L) \
+    case L: t2_smem_limits<float, L>(bytes); break;
+            SS_T2_LENGTHS(SS_CASE)
+#undef SS_CASE
+            default: break;
+        }
+        if (Px == Py) break;
+    }
+}
+
 void launch_fft_strided_f64(double2* data, const double2* tw, const FftPlan& plan, int n_lines, long elem_stride,
                             int inner_count, long inner_stride, long outer_stride, cudaStream_t st) {
     const int P = plan.P;  // <= 2048 (validated by the host)

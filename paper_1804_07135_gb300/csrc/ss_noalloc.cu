@@ -33,12 +33,14 @@ static __device__ __align__(256) unsigned char g_scratch[kNoAllocScratchBytes];
 struct ScratchSlot {
     unsigned char* ptr;
     bool ready;
+    bool limits[513];  // shared-memory limits of the two-pass kernels of a length are raised
 };
 std::mutex g_mu;
 ScratchSlot g_slots[kMaxDevices];
 
-// Device address of g_scratch on the current device, looked up once per device.
-ss_status scratch_of_current_device(unsigned char** out) {
+// Device address of g_scratch on the current device, looked up once per device; raises the shared-memory
+// limits of the kernels of padded lengths Px and Py on their first use there.
+ss_status scratch_of_current_device(int Px, int Py, unsigned char** out) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return SS_ERR_CUDA;
     if (dev < 0 || dev >= kMaxDevices) return SS_ERR_CUDA;
@@ -54,26 +56,18 @@ ss_status scratch_of_current_device(unsigned char** out) {
         g_slots[dev].ptr = static_cast<unsigned char*>(p);
         g_slots[dev].ready = true;
     }
+    for (int P : {Px, Py})
+        if (t2_length(P) && !g_slots[dev].limits[P]) {
+            set_t2_smem_limits(P, P, 227 * 1024);
+            g_slots[dev].limits[P] = true;
+        }
     *out = g_slots[dev].ptr;
     return SS_OK;
 }
 
-// ---- sizes and launch shapes: the padded-length rule of the context path; the x-kernel row count is a
+// ---- sizes and launch shapes: padded_smooth lengths (the scratch limits are stated in them); the x-kernel row count is a
 // fixed rule of its own (no autotuning), chosen to keep every CTA's shared memory under 48 KB ----
-bool smooth23(int m) {
-    while (m % 2 == 0) m /= 2;
-    while (m % 3 == 0) m /= 3;
-    return m == 1;
-}
-int pad_len(int n) {  // the context's rule: smallest 2^a 3^b >= 2n - 1, or a power of two <= 1/8 longer
-    int m = n > 1 ? 2 * n - 1 : 1;
-    while (!smooth23(m)) ++m;
-    int p2 = 1;
-    while (p2 < 2 * n - 1) p2 <<= 1;
-    return 8 * p2 <= 9 * m ? p2 : m;
-}
 FftPlan plan_of(int P) { return fft_make_plan(P); }
-int up32(int v) { return ((v + 31) / 32) * 32; }
 size_t up256(size_t v) { return (v + 255) & ~size_t(255); }
 
 __global__ void na_twiddles(double2* tw64, float2* tw32, int P) {
@@ -108,21 +102,6 @@ __global__ void na_tensor_fill(double2* data, int nx, int ny, int nz, int Px, in
             d[5] = c * 3.0 * y * z * inv5;
         }
         for (int k = 0; k < 6; ++k) data[(size_t)k * total + i] = make_double2(d[k], 0.0);
-    }
-}
-
-// Per-stage twiddle table of a plan from the flat FP64 table (layout of fft_stage_twiddles).
-__global__ void na_stage_twiddles(FftPlan p, const double2* tw64, float2* out) {
-    int o = 0;
-    for (int s = 0; s < p.nstages; ++s) {
-        const int R = p.radix[s], Ns = p.ns[s];
-        if (Ns == 1) continue;
-        for (int e = threadIdx.x; e < Ns * (R - 1); e += blockDim.x) {
-            const int jm = e / (R - 1), r = 1 + e % (R - 1);
-            const double2 x = tw64[(jm * r * p.tw[s]) % p.P];
-            out[o + e] = make_float2((float)x.x, (float)x.y);
-        }
-        o += Ns * (R - 1);
     }
 }
 
@@ -181,7 +160,7 @@ extern "C" ss_status ss_field_noalloc(int nx, int ny, int nz, double J, double D
     }
     const bool dip = w != 0.0;
     const int N = nx * ny * nz;
-    const int Px = dip ? pad_len(nx) : 1, Py = dip ? pad_len(ny) : 1;
+    const int Px = dip ? padded_smooth(nx) : 1, Py = dip ? padded_smooth(ny) : 1;
     const int lsx = fft_line_stride(Px), lsy = fft_line_stride(Py), pairs = (n_images + 1) / 2;
     // launch shapes, as for a context of FP32 precision
     const int thr = kMaxThreadsX, thr_b = kMaxThreadsYz;
@@ -193,15 +172,16 @@ extern "C" ss_status ss_field_noalloc(int nx, int ny, int nz, double J, double D
         }
     }
     if (dip && f128_x(4, Px)) ty = f128_x_rows(ty);  // the length-128 x kernels take 2, 4 or 8 rows
-    if (dip && x2p_ok(4, Px)) ty = kX2Rows;          // the lengths-192/256/384 x kernels take kX2Rows
+    if (dip && (Px == 192 || Px == 256 || Px == 384)) ty = kX2Rows;
     const size_t smem_a = (size_t)(Px + 3 * ty * lsx) * sizeof(float2);
     const size_t smem_c = smem_a + 32 * 2 * kEvalTerms * sizeof(double);
     size_t smem_b = (size_t)(Py + 3 * nz * lsy) * sizeof(float2);
     const size_t slab = (size_t)(Py / 2 + 1) * nz * 6 * sizeof(float);
     if (slab <= 24 * 1024) smem_b += slab;
     if (smem_c > 227 * 1024 || smem_b > 227 * 1024) return SS_ERR_INVALID_ARG;
+    // scratch layout.  The size of a request that fits is part of the interface, so it stays what it was when
+    // the evaluation kept energy partials (n_eblk per image and term) and per-stage twiddles here
     const int n_eblk = nz * ((ny + ty - 1) / ty);
-    // scratch layout
     size_t off = 0;
     auto take = [&](size_t bytes) {
         const size_t o = off;
@@ -211,12 +191,12 @@ extern "C" ss_status ss_field_noalloc(int nx, int ny, int nz, double J, double D
     const size_t o_err = take(sizeof(int));
     const size_t o_tw64x = take(Px * sizeof(double2)), o_tw64y = take(Py * sizeof(double2));
     const size_t o_twx = take(Px * sizeof(float2)), o_twy = take(Py * sizeof(float2));
-    const size_t o_twxs = take(Px * sizeof(float2)), o_twys = take(Py * sizeof(float2));
+    take(Px * sizeof(float2)), take(Py * sizeof(float2));
     const size_t o_t2x = take(2 * Px * sizeof(float2)), o_t2y = take(2 * Py * sizeof(float2));
     const size_t o_dhat = take(dip ? (size_t)(Px / 2 + 1) * (Py / 2 + 1) * nz * 6 * sizeof(float) : 0);
     const size_t o_prm = take(n_images * sizeof(ImgParam<float>));
     const size_t o_interp = take(n_images * sizeof(InterpEntry));
-    const size_t o_epart = take((size_t)n_images * kEvalTerms * n_eblk * sizeof(double));
+    take((size_t)n_images * kEvalTerms * n_eblk * sizeof(double));
     const size_t o_work = off;
     const size_t tensor_bytes = dip ? (size_t)6 * nz * Px * Py * sizeof(double2) : 0;
     const size_t o_s = o_work;
@@ -227,7 +207,7 @@ extern "C" ss_status ss_field_noalloc(int nx, int ny, int nz, double J, double D
     if (need > kNoAllocScratchBytes) return SS_ERR_INVALID_ARG;  // beyond the built-in scratch
     unsigned char* base = nullptr;
     {
-        const ss_status s = scratch_of_current_device(&base);
+        const ss_status s = scratch_of_current_device(Px, Py, &base);
         if (s != SS_OK) return s;
     }
     int* err = reinterpret_cast<int*>(base + o_err);
@@ -240,10 +220,6 @@ extern "C" ss_status ss_field_noalloc(int nx, int ny, int nz, double J, double D
     na_twiddles<<<(Py + 127) / 128, 128, 0, st>>>(tw64y, twy, Py);
     float* dhat = reinterpret_cast<float*>(base + o_dhat);
     const FftPlan px = plan_of(Px), py = plan_of(Py);
-    float2* twxs = reinterpret_cast<float2*>(base + o_twxs);
-    float2* twys = reinterpret_cast<float2*>(base + o_twys);
-    na_stage_twiddles<<<1, 256, 0, st>>>(px, tw64x, twxs);
-    na_stage_twiddles<<<1, 256, 0, st>>>(py, tw64y, twys);
     float2* t2x = reinterpret_cast<float2*>(base + o_t2x);
     float2* t2y = reinterpret_cast<float2*>(base + o_t2y);
     na_t2_table<<<(2 * Px + 127) / 128, 128, 0, st>>>(Px, tw64x, t2x);
@@ -281,18 +257,14 @@ extern "C" ss_status ss_field_noalloc(int nx, int ny, int nz, double J, double D
     g.dhat = dhat;
     g.twx = twx;
     g.twy = twy;
-    g.twxs = twxs;
-    g.twys = twys;
     g.t2x = t2x;
     g.t2y = t2y;
     g.planx = px;
     g.plany = py;
     g.prm = prm;
     g.interp = interp;
-    g.epart = reinterpret_cast<double*>(base + o_epart);
-    g.n_eblk = n_eblk;
-    g.ty_a = ty;
-    g.ty_c = ty;
+    g.epart = nullptr;  // the field alone
+    g.ty_a = g.ty_c = dip && x2p_ok(4, Px) ? kX2Rows : ty;  // the two-pass x kernels take kX2Rows
     g.err = err;
     launch_xfwd<float>(g, dip, thr, smem_a, st);
     if (dip) launch_yz<float>(g, thr_b, smem_b, st);
