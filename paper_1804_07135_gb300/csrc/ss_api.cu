@@ -99,6 +99,7 @@ struct Group {
     bool dipole = false;  // FFT dipole convolution (SS_DIPOLE_FFT and some w != 0)
     bool direct = false;  // direct dipole sums (SS_DIPOLE_DIRECT and some w != 0)
     void* hdir = nullptr; // [image][3][N] direct sums
+    void* dtab = nullptr; // [6][N] tensor table of the direct sums
     FftPlan planx{}, plany{};
     int lsx = 1, lsy = 1;
     int ty_a = 1, ty_c = 1, thr_a = 128, thr_b = 128, thr_c = 128, thr_arc = 256;
@@ -396,7 +397,18 @@ template <typename T> ss_status setup_group(ss_ctx* c, Group& g) {
     TRY(dalloc(c, &g.twy, g.Py * sizeof(C)));
     TRY(dalloc(c, &g.t2x, 2 * g.Px * sizeof(C)));
     TRY(dalloc(c, &g.t2y, 2 * g.Py * sizeof(C)));
-    if (g.direct) TRY(dalloc(c, &g.hdir, (size_t)g.n_img * 3 * g.N * sizeof(T)));
+    if (g.direct) {
+        TRY(dalloc(c, &g.hdir, (size_t)g.n_img * 3 * g.N * sizeof(T)));
+        TRY(dalloc(c, &g.dtab, (size_t)6 * g.N * sizeof(T)));
+        std::vector<T> tab((size_t)6 * g.N, T(0));  // [component][(|dz| ny + |dy|) nx + |dx|]
+        for (int i = 1; i < g.N; ++i) {
+            double d[6];
+            dipole_tensor_at(i % g.nx, (i / g.nx) % g.ny, i / (g.nx * g.ny), d);
+            for (int k = 0; k < 6; ++k) tab[(size_t)k * g.N + i] = T(4.0 * M_PI * d[k]);
+        }
+        CUDA_TRY(c, cudaMemcpyAsync(g.dtab, tab.data(), tab.size() * sizeof(T), cudaMemcpyHostToDevice, c->cs));
+        CUDA_TRY(c, cudaStreamSynchronize(c->cs));
+    }
     if (g.dipole) {
         TRY(dalloc(c, &g.spec, (size_t)g.n_pairs * g.Px * 3 * g.nz * g.ny * sizeof(C)));
         TRY(dalloc(c, &g.dhat, (size_t)(g.Px / 2 + 1) * (g.Py / 2 + 1) * g.nz * 6 * sizeof(T)));
@@ -614,7 +626,7 @@ template <typename T> int time_entries(ss_ctx* c, Group& g, int which_only) {
     };
     entry(true, [&] { launch_xfwd<T>(a, g.dipole, g.thr_a, g.smem_a, c->cs); });
     entry(g.dipole, [&] { launch_yz<T>(a, g.thr_b, g.smem_b, c->cs); });
-    entry(g.direct, [&] { launch_dipole_direct<T>(a, (T*)g.hdir, c->cs); });
+    entry(g.direct, [&] { launch_dipole_direct<T>(a, (T*)g.hdir, (const T*)g.dtab, c->cs); });
     entry(true, [&] {
         if (c->dynamics == SS_DYN_LLG)
             launch_xinv_step_llg<T>(a, g.dipole, dt, g.thr_c, g.smem_c, c->cs);
@@ -727,7 +739,7 @@ template <typename T> void issue_rk_round(ss_ctx* c, Group& g, bool first, cudaS
         launch_rk_assemble<T>(ai, r, s, st);
         launch_xfwd<T>(ai, g.dipole, g.thr_a, g.smem_a, st);
         if (g.dipole) launch_yz<T>(ai, g.thr_b, g.smem_b, st);
-        if (g.direct) launch_dipole_direct<T>(ai, (T*)g.hdir, st);
+        if (g.direct) launch_dipole_direct<T>(ai, (T*)g.hdir, (const T*)g.dtab, st);
         launch_xinv_force<T>(ai, g.dipole, r.k + s * stride, first && s == 0, c->dynamics == SS_DYN_LLG, g.thr_c,
                              g.smem_c_eval, st);
     }
@@ -810,7 +822,7 @@ template <typename T> int rk_time_entries(ss_ctx* c, Group& g, int which_only) {
         entry(true, [&] { launch_rk_assemble<T>(ai, r, st, c->cs); });
         entry(true, [&] { launch_xfwd<T>(ai, g.dipole, g.thr_a, g.smem_a, c->cs); });
         entry(g.dipole, [&] { launch_yz<T>(ai, g.thr_b, g.smem_b, c->cs); });
-        entry(g.direct, [&] { launch_dipole_direct<T>(ai, (T*)g.hdir, c->cs); });
+        entry(g.direct, [&] { launch_dipole_direct<T>(ai, (T*)g.hdir, (const T*)g.dtab, c->cs); });
         entry(true, [&] {
             launch_xinv_force<T>(ai, g.dipole, r.k + st * stride, st == 0, c->dynamics == SS_DYN_LLG, g.thr_c,
                                  g.smem_c_eval, c->cs);
@@ -862,7 +874,7 @@ template <typename T> void issue_group_iteration(ss_ctx* c, Group& g, cudaStream
         GroupArgs<T> a = group_args<T>(c, g);
         launch_xfwd<T>(a, g.dipole, g.thr_a, g.smem_a, st);
         if (g.dipole) launch_yz<T>(a, g.thr_b, g.smem_b, st);
-        if (g.direct) launch_dipole_direct<T>(a, (T*)g.hdir, st);
+        if (g.direct) launch_dipole_direct<T>(a, (T*)g.hdir, (const T*)g.dtab, st);
         if (c->dynamics == SS_DYN_LLG) {
             launch_xinv_step_llg<T>(a, g.dipole, dt, g.thr_c, g.smem_c, st);
         } else if (c->climb) {
@@ -883,7 +895,7 @@ template <typename T> void issue_eval(ss_ctx* c, Group& g, T* hout, cudaStream_t
     a.pair_on = pair_on;
     launch_xfwd<T>(a, g.dipole, g.thr_a, g.smem_a, st);
     if (g.dipole) launch_yz<T>(a, g.thr_b, g.smem_b, st);
-    if (g.direct) launch_dipole_direct<T>(a, (T*)g.hdir, st);
+    if (g.direct) launch_dipole_direct<T>(a, (T*)g.hdir, (const T*)g.dtab, st);
     launch_xinv_eval<T>(a, g.dipole, hout, g.thr_c, g.smem_c_eval, st);
     launch_eval_reduce<T>(a, g.arc, g.eval_terms, g.eval_E, g.eval_cn, st);
 }

@@ -279,7 +279,8 @@ template <typename T> void launch_xinv_step_climb(const GroupArgs<T>& g, bool do
                                                   cudaStream_t st);
 template <typename T> void launch_xinv_step_llg(const GroupArgs<T>& g, bool do_fft, T dt, int nthr, size_t smem,
                                                 cudaStream_t st);
-template <typename T> void launch_dipole_direct(const GroupArgs<T>& g, T* hdir, cudaStream_t st);
+// dtab: the tensor table of the direct sum, [6][N] over (|dz|, |dy|, |dx|)
+template <typename T> void launch_dipole_direct(const GroupArgs<T>& g, T* hdir, const T* dtab, cudaStream_t st);
 template <typename T> void launch_climb(const GroupArgs<T>& g, const ArcArgs& a, T dt, const T* hc, cudaStream_t st);
 template <typename T> void launch_spline_apply(const GroupArgs<T>& g, const ArcArgs& a, int maxK, cudaStream_t st);
 template <typename T> void launch_rk_assemble(const GroupArgs<T>& g, const RkArgs<T>& r, int stage, cudaStream_t st);

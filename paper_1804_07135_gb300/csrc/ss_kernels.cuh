@@ -1720,46 +1720,84 @@ __global__ void __launch_bounds__(256) rk_commit_kernel(GroupArgs<T> g, RkArgs<T
 // ---- direct dipole sum (SS_DIPOLE_DIRECT) -------------------------------------------------------------
 // conv_i = sum_{j != i} (3 (r.s_j) r / r^5 - s_j / r^3), r = r_j - r_i in lattice units: Eq. 6 with the
 // tensor of Eq. 7 (its 1/(4 pi) cancels against the 4 pi of w's definition); the x-inverse kernel
-// multiplies by w.  grid (ceil(N / 128), n_img), 128 threads, one site i each; the image's spins (from s,
-// the gathered state) and their coordinates stream through shared memory in tiles of 128 sites.
-template <typename T>
-__global__ void __launch_bounds__(128) dipole_direct_kernel(GroupArgs<T> g, T* hdir) {
-    __shared__ T sj[3][128];
-    __shared__ int xj[128], yj[128], zj[128];
-    const int im = blockIdx.y, tid = threadIdx.x, N = g.N, nx = g.nx, ny = g.ny;
-    const int i = blockIdx.x * 128 + tid;
-    const T* s = g.s + (size_t)im * 3 * N;
+// multiplies by w.  The six tensor components come from a table over |dx|, |dy|, |dz| (dtab: [component][N],
+// the octant's values, zero at the origin, so j = i needs no test), with the signs of the off-diagonal ones
+// applied as sign bits.  A CTA takes 32 sites (a warp's lanes) of M images; its 8 warps share the sum over j,
+// 32 of each 256-site tile staged in shared memory, and their partial sums are added in warp order at the
+// end.  FP64 is bound by the FP64 pipe (two lane-operations per clock and SM): nine multiply-adds per pair
+// of sites, five for a single layer (xz and yz vanish), instead of a square root and a division per pair
+// and image as the sum was first written: 16x16x1 x 16 images 352 -> 16.0 us on one GB300.
+// M (images that share a table load) is 4 while the grid still fills the chip twice, fewer on small
+// lattices, where CTAs are what is missing.
+constexpr int kDirTile = 256, kDirWarps = 8;
+__device__ __forceinline__ float flip_sign(float v, unsigned s) { return __uint_as_float(__float_as_uint(v) ^ s); }
+__device__ __forceinline__ double flip_sign(double v, unsigned s) {
+    return __hiloint2double(__double2hiint(v) ^ (int)s, __double2loint(v));
+}
+template <typename T, int M, bool FILM>
+__global__ void __launch_bounds__(32 * kDirWarps) dipole_direct_kernel(GroupArgs<T> g, T* hdir, const T* __restrict__ dtab) {
+    constexpr int Q = 3 * M;
+    // the tile's spins [j][component * M + image]; after the sum the warps' partials [warp][q][lane]
+    __shared__ __align__(16) T sm[kDirTile * Q];
+    __shared__ int cj[kDirTile];  // x | y << 10 | z << 20
+    static_assert(kDirWarps * 32 == kDirTile, "one staged site per thread, one partial slot per (warp, q, lane)");
+    const int im0 = blockIdx.y * M, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int N = g.N, nx = g.nx, ny = g.ny;
+    const int i = min(blockIdx.x * 32 + lane, N - 1);
     const int xi = i % nx, yi = (i / nx) % ny, zi = i / (nx * ny);
-    T a0 = T(0), a1 = T(0), a2 = T(0);
-    for (int t0 = 0; t0 < N; t0 += 128) {
+    T acc[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) acc[q] = T(0);
+    for (int t0 = 0; t0 < N; t0 += kDirTile) {
         const int j = t0 + tid;
         __syncthreads();  // the previous tile is consumed
-        if (j < N) {
-            sj[0][tid] = s[j];
-            sj[1][tid] = s[N + j];
-            sj[2][tid] = s[2 * N + j];
-            xj[tid] = j % nx;
-            yj[tid] = (j / nx) % ny;
-            zj[tid] = j / (nx * ny);
+#pragma unroll
+        for (int m = 0; m < M; ++m) {
+            const bool in = j < N && im0 + m < g.n_img;
+            const T* s = g.s + (size_t)(im0 + m) * 3 * N + j;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) sm[tid * Q + c * M + m] = in ? s[(size_t)c * N] : T(0);
         }
+        cj[tid] = j < N ? (j % nx) | ((j / nx) % ny) << 10 | (j / (nx * ny)) << 20 : 0;  // past N: spin zero
         __syncthreads();
-        const int nt = min(128, N - t0);
-        for (int q = 0; q < nt; ++q) {
-            const T dx = T(xj[q] - xi), dy = T(yj[q] - yi), dz = T(zj[q] - zi);
-            const T r2 = dx * dx + dy * dy + dz * dz;
-            if (r2 == T(0)) continue;  // j == i
-            const T ir = rsqrt_t<T>(r2), ir3 = ir * ir * ir, ir5 = ir3 * ir * ir;
-            const T rs3 = T(3) * (dx * sj[0][q] + dy * sj[1][q] + dz * sj[2][q]) * ir5;
-            a0 += rs3 * dx - sj[0][q] * ir3;
-            a1 += rs3 * dy - sj[1][q] * ir3;
-            a2 += rs3 * dz - sj[2][q] * ir3;
+#pragma unroll 2
+        for (int q = 0; q < 32; ++q) {
+            const int jj = warp * 32 + q, p = cj[jj];
+            const int dx = (p & 1023) - xi, dy = (p >> 10 & 1023) - yi, dz = (p >> 20) - zi;
+            const T* d = dtab + ((size_t)(abs(dz) * ny + abs(dy)) * nx + abs(dx));
+            const T dxx = d[0], dyy = d[N], dzz = d[2 * (size_t)N];
+            const T dxy = flip_sign(d[3 * (size_t)N], (unsigned)(dx ^ dy) & 0x80000000u);
+            const T dxz = FILM ? T(0) : flip_sign(d[4 * (size_t)N], (unsigned)(dx ^ dz) & 0x80000000u);
+            const T dyz = FILM ? T(0) : flip_sign(d[5 * (size_t)N], (unsigned)(dy ^ dz) & 0x80000000u);
+            const T* s = sm + jj * Q;
+#pragma unroll
+            for (int m = 0; m < M; ++m) {
+                const T sx = s[m], sy = s[M + m], sz = s[2 * M + m];
+                acc[m] += dxx * sx;
+                acc[M + m] += dxy * sx;
+                acc[2 * M + m] += dzz * sz;
+                acc[m] += dxy * sy;
+                acc[M + m] += dyy * sy;
+                if (!FILM) {
+                    acc[2 * M + m] += dxz * sx;
+                    acc[m] += dxz * sz;
+                    acc[M + m] += dyz * sz;
+                    acc[2 * M + m] += dyz * sy;
+                }
+            }
         }
     }
-    if (i < N) {
-        T* o = hdir + (size_t)im * 3 * N + i;
-        o[0] = a0;
-        o[N] = a1;
-        o[2 * N] = a2;
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < Q; ++q) sm[(warp * Q + q) * 32 + lane] = acc[q];
+    __syncthreads();
+    for (int o = tid; o < Q * 32; o += 32 * kDirWarps) {
+        const int q = o >> 5, l = o & 31, c = q / M, im = im0 + q % M, site = blockIdx.x * 32 + l;
+        if (site >= N || im >= g.n_img) continue;
+        T v = T(0);
+#pragma unroll
+        for (int w = 0; w < kDirWarps; ++w) v += sm[(w * Q + q) * 32 + l];
+        hdir[(size_t)im * 3 * N + (size_t)c * N + site] = v;
     }
 }
 
@@ -2260,8 +2298,19 @@ void launch_xinv_step_climb(const GroupArgs<T>& g, bool do_fft, T dt, T* hc, int
         launch_pdl(xinv_kernel<T, false, 3>, grid, dim3(nthr), smem, st, g, dt, hc);
 }
 
-template <typename T> void launch_dipole_direct(const GroupArgs<T>& g, T* hdir, cudaStream_t st) {
-    dipole_direct_kernel<T><<<dim3((g.N + 127) / 128, g.n_img), 128, 0, st>>>(g, hdir);
+template <typename T> void launch_dipole_direct(const GroupArgs<T>& g, T* hdir, const T* dtab, cudaStream_t st) {
+    const int sites = (g.N + 31) / 32;
+    const bool film = g.nz == 1;
+    int M = 4;
+    while (M > 1 && (long)sites * ((g.n_img + M - 1) / M) < 2 * 152) M /= 2;
+    const dim3 grid(sites, (g.n_img + M - 1) / M), blk(32 * kDirWarps);
+#define SS_CASE(m)                                                                             \
+    if (M == m) {                                                                              \
+        if (film) dipole_direct_kernel<T, m, true><<<grid, blk, 0, st>>>(g, hdir, dtab);       \
+        else dipole_direct_kernel<T, m, false><<<grid, blk, 0, st>>>(g, hdir, dtab);           \
+    }
+    SS_CASE(1) SS_CASE(2) SS_CASE(4)
+#undef SS_CASE
 }
 
 template <typename T> void launch_climb(const GroupArgs<T>& g, const ArcArgs& a, T dt, const T* hc, cudaStream_t st) {
@@ -2427,7 +2476,7 @@ void launch_widen_unit(const float* src, double* dst, int K, int N, const int* p
     template void launch_xinv_step_llg<T>(const GroupArgs<T>&, bool, T, int, size_t, cudaStream_t);             \
     template void launch_xinv_step_climb<T>(const GroupArgs<T>&, bool, T, T*, int, size_t, cudaStream_t);       \
     template void launch_climb<T>(const GroupArgs<T>&, const ArcArgs&, T, const T*, cudaStream_t);             \
-    template void launch_dipole_direct<T>(const GroupArgs<T>&, T*, cudaStream_t);                              \
+    template void launch_dipole_direct<T>(const GroupArgs<T>&, T*, const T*, cudaStream_t);                    \
     template void launch_spline_apply<T>(const GroupArgs<T>&, const ArcArgs&, int, cudaStream_t);              \
     template DpCoef<T> dp_coefficients<T>(int);                                                               \
     template void launch_rk_assemble<T>(const GroupArgs<T>&, const RkArgs<T>&, int, cudaStream_t);             \
