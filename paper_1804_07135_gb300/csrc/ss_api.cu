@@ -330,13 +330,8 @@ void configure_group(Group& g) {
     g.smem_b = (size_t)(g.Py + 3 * g.nz * g.lsy) * cs;
     const size_t slab = (size_t)(g.Py / 2 + 1) * g.nz * 6 * (size_t)g.rbytes;
     if (slab <= 24 * 1024) g.smem_b += slab;
-    if (g.dipole && f128_yz(g.rbytes, g.Py, g.nz)) {
-        bool stage = false;
-        g.thr_b = f128_yz_threads(g.nz);
-        g.smem_b = f128_yz_smem(g.nz, g.Py, &stage);
-    }
     if (g.dipole && yz2p_ok(g.rbytes, g.Py, g.nz, g.Px)) {
-        g.thr_b = kYz2Threads;
+        g.thr_b = yz2p_threads(g.Py, g.nz);
         g.smem_b = yz2p_smem(g.Py, g.nz, yz2p_kxb_use(g.nz, g.yz_kxb));
     }
 }
@@ -374,7 +369,8 @@ template <typename T> ss_status build_tensor_spectrum(ss_ctx* c, Group& g) {
         launch_fft_strided_f64(d_data, d_twx, px, 6 * nz * Py, 1, 1, 0, Px, c->cs);
         // y: columns of length Py, stride Px
         launch_fft_strided_f64(d_data, d_twy, py, 6 * nz * Px, Px, Px, 1, (long)plane, c->cs);
-        launch_extract_octant<T>(d_data, (T*)g.dhat, Px, Py, nz, 4.0 * M_PI / ((double)Px * Py), c->cs);
+        launch_extract_octant<T>(d_data, (T*)g.dhat, Px, Py, nz,
+                                 dhat_factor(g.rbytes, Py, nz, Px) * 4.0 * M_PI / ((double)Px * Py), c->cs);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->cs);
@@ -1051,7 +1047,8 @@ ss_status evaluate_energies(ss_ctx* c, int gi, const Group** out) {
 // every string of size group gi, for the group's current state, into *out ([image], NaN for the others).
 // The FP32 evaluation gives each image's energy E_k with a round-off bound B_k: its local terms are FP32
 // per site and summed in FP32 per thread and warp (bounded below), and the dipole term's FFT round-off
-// obeys ||d conv||_2 <= eps ||conv||_2, eps = u (2 log2(Px Py) + 3 nz + 4), so |dE_k| <= w (1/2) eps
+// obeys ||d conv||_2 <= eps ||conv||_2, eps = u (2 log2(Px Py) + 3 nz + 6) (2 of it for the sums and
+// differences of mirrored layers), so |dE_k| <= w (1/2) eps
 // ||conv_k||_2 sqrt(N), plus 1e-9 + 1e-13 |E_k| for the FP64 sums.  An image whose upper bound E_k + B_k lies below the
 // largest lower bound max_j (E_j - B_j) of its string cannot be the highest one, so only image 0 and the
 // remaining images are evaluated in FP64 -- the pairs holding them, on the FP64 evaluation copy.
@@ -1075,7 +1072,7 @@ ss_status barrier_energies(ss_ctx* c, int gi, const std::vector<double>** out) {
         CUDA_TRY(c, cudaMemcpyAsync(buf.data(), g.eval_E, buf.size() * sizeof(double), cudaMemcpyDeviceToHost, c->cs));
         CUDA_TRY(c, cudaMemcpyAsync(cn.data(), g.eval_cn, cn.size() * sizeof(double), cudaMemcpyDeviceToHost, c->cs));
         TRY(sync_check(c));
-        const double eps = std::ldexp(1.0, -24) * (2.0 * std::log2((double)g.Px * g.Py) + 3.0 * g.nz + 4.0);
+        const double eps = std::ldexp(1.0, -24) * (2.0 * std::log2((double)g.Px * g.Py) + 3.0 * g.nz + 6.0);
         std::vector<int> on(g.n_pairs, 0);
         for (int i = 0; i < nstr; ++i) {
             const ss_string_desc& d = c->strs[g.strs[i]].d;

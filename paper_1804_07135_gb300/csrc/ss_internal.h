@@ -175,13 +175,11 @@ template <typename T> struct RkArgs {
 
 enum { kErrInvalidSpin = 1, kErrNonFinite = 2, kErrStepCollapse = 4 };
 
-// Length-128 transforms in two register passes (FP32): the x kernels when Px = 128, the y/z kernel
-// when Py = 128 and nz is 4 or 8.  16 threads per line; their launch shapes follow from the rows per
-// CTA (x kernels) or from nz (y/z kernel), whatever block size and shared memory the caller passes.
+// Length-128 transforms in two register passes (FP32): the x kernels when Px = 128.  16 threads per line;
+// their launch shapes follow from the rows per CTA, whatever block size and shared memory the caller passes.
 constexpr int kF128Line = 145;  // line stride of their exchange buffers (complex elements, 1 mod 16)
 constexpr int kF128Buf = 72;    // line stride of the x kernels' 64-point lines (fft_pad positions, 8 mod 16)
 inline bool f128_x(int real_bytes, int Px) { return real_bytes == 4 && Px == 128; }
-inline bool f128_yz(int real_bytes, int Py, int nz) { return real_bytes == 4 && Py == 128 && (nz == 4 || nz == 8); }
 // rows per CTA of the x kernels: 2, 4 or 8 (compile-time); anything else is taken as 8
 inline int f128_x_rows(int ty) { return ty == 2 || ty == 4 ? ty : 8; }
 inline int f128_x_threads(int rows) { return 48 * rows; }
@@ -189,16 +187,6 @@ inline size_t f128_x_smem(int rows) {
     // line buffer, exchange buffer (lines rounded up to a multiple of 4), reduction scratch
     return (size_t)(3 * rows * kF128Buf + (3 * rows + 3) / 4 * 4 * kF128Line) * 8 + 32 * 2 * kEvalTerms * sizeof(double);
 }
-inline int f128_yz_threads(int nz) { return 48 * nz; }
-// The length-128 y/z kernel reads its tensor slab through L1 rather than staging it in shared memory
-// (measured faster: the 16 pairs of one kx would otherwise each copy the same slab, and the smaller
-// shared footprint leaves more L1).
-inline size_t f128_yz_smem(int nz, int Py, bool* stage_dhat) {
-    (void)Py;
-    *stage_dhat = false;
-    return (size_t)2 * 3 * nz * kF128Line * 8;
-}
-
 
 // Lengths P = 16 R2 in two register passes (FP32, ss_fft.cuh, ss_twopass.cuh): a line is R2 = P/16 rows of 16
 // at row stride kT2Row; the y/z kernel for those Py with 1 to 8 layers, the x kernels for those Px with
@@ -224,19 +212,27 @@ inline int t2_length_from(int m) {
 constexpr int kT2Row = 17;
 constexpr int kT2MaxNz = 8;
 __host__ __device__ constexpr int t2_line(int P) { return kT2Row * (P / 16); }
-constexpr int kYz2Threads = 384;
 // kx columns per CTA: the default (15 to 24 lines) and the alternative the autotuner also times (12 lines for
 // one or four layers); 0 when nz has no two-pass kernel
 inline int yz2p_kxb(int nz) { return nz == 1 ? 8 : nz == 2 ? 4 : nz <= 4 ? 2 : nz <= kT2MaxNz ? 1 : 0; }
 inline int yz2p_kxb_alt(int nz) { return nz == 1 ? 4 : nz == 4 ? 1 : 0; }
 inline bool yz2p_ok(int real_bytes, int Py, int nz, int Px) {
-    if (real_bytes != 4 || !t2_length(Py) || f128_yz(real_bytes, Py, nz)) return false;
+    if (real_bytes != 4 || !t2_length(Py)) return false;
     const int kxb = yz2p_kxb(nz);
     return kxb > 0 && Px % kxb == 0;
 }
+// threads and resident CTAs of the y/z kernel: with four or more layers the z-convolution wants 64 registers
+// (four to six layers) or 80 (seven, eight); as many CTAs as registers and shared memory allow
+__host__ __device__ constexpr int yz2p_threads(int P, int nz) { return nz <= 3 || P > 320 ? 384 : nz >= 7 || P <= 256 ? 256 : 384; }
+__host__ __device__ constexpr int yz2p_blocks(int P, int nz) { return P > 320 ? 2 : nz >= 4 && nz <= 6 && P <= 256 ? 4 : 3; }
 // columns per CTA a launch uses: the tuned choice when it is one of the two, else the default
 inline int yz2p_kxb_use(int nz, int tuned) { return tuned > 0 && (tuned == yz2p_kxb(nz) || tuned == yz2p_kxb_alt(nz)) ? tuned : yz2p_kxb(nz); }
 inline size_t yz2p_smem(int Py, int nz, int kxb) { return (size_t)3 * nz * kxb * t2_line(Py) * 8; }
+// Factor of the stored tensor spectrum besides 4 pi / (Px Py): the two-pass y/z kernel convolves sums and
+// differences of mirrored layers, which leaves a factor 2 to be taken out (exact)
+inline double dhat_factor(int real_bytes, int Py, int nz, int Px) {
+    return nz > 1 && yz2p_ok(real_bytes, Py, nz, Px) ? 0.5 : 1.0;
+}
 constexpr int kX2Rows = 4;
 // threads of an x CTA: short lines have fewer roles than 384 threads would take
 __host__ __device__ constexpr int x2_threads(int P) { return P <= 48 ? 128 : P <= 80 ? 192 : P <= 160 ? 256 : 384; }

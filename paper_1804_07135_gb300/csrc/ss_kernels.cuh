@@ -319,10 +319,9 @@ constexpr int kYzItems = 4;
 // across a warp (nthr/3 a multiple of 32), both z loops unrolled so |z - z'| and the z-parity sign are
 // constants.  Row a of the tensor: a = x: (xx, xy, i xz); a = y: (xy, yy, i yz); a = z: (i xz, i yz, zz).
 // dslab holds the coefficient (kyo, |dz|, comp) at dslab[kyo*dk + (|dz|*6 + comp)*dq].
-// INPLACE: lines of A (stride lsy, fft_pad positions) are overwritten with the conjugated result;
-// otherwise the result goes to the lines of B (same stride, plain positions) and A is only read.
-template <int NZ, bool INPLACE = true, typename T, typename C>
-__device__ __forceinline__ void zconv_c(const C* A, C* B, int lsy, int Py, int kx, int Px, const T* dslab, int dk,
+// The lines of A (stride lsy, fft_pad positions) are overwritten with the conjugated result.
+template <int NZ, typename T, typename C>
+__device__ __forceinline__ void zconv_c(C* A, int lsy, int Py, int kx, int Px, const T* dslab, int dk,
                                         int dq, int tid, int nthr) {
     const int hx = Px / 2, hy = Py / 2;
     const T sxg = kx > hx ? T(-1) : T(1);
@@ -337,7 +336,7 @@ __device__ __forceinline__ void zconv_c(const C* A, C* B, int lsy, int Py, int k
             const int kyo = min(ky, Py - ky);
             const T syg = ky > hy ? T(-1) : T(1);
             const T* d = dslab + (size_t)kyo * dk;
-            pky = INPLACE ? fft_pad(ky) : ky;
+            pky = fft_pad(ky);
             // coefficient slots (xx 0, yy 1, zz 2, xy 3, xz 4, yz 5) and x/y parity signs of row a
             const int i0 = a == 0 ? 0 : (a == 1 ? 3 : 4);
             const int i1 = a == 0 ? 3 : (a == 1 ? 1 : 5);
@@ -420,13 +419,13 @@ __device__ __forceinline__ void zconv_c(const C* A, C* B, int lsy, int Py, int k
                 }
             }
         }
-        if constexpr (INPLACE) __syncthreads();
+        __syncthreads();
         if (act) {
             // conjugated: the inverse transform is the conjugate of the forward transform of the conjugate
 #pragma unroll
-            for (int z = 0; z < NZ; ++z) B[(a * NZ + z) * lsy + pky] = cconj(out[z]);
+            for (int z = 0; z < NZ; ++z) A[(a * NZ + z) * lsy + pky] = cconj(out[z]);
         }
-        if constexpr (INPLACE) __syncthreads();
+        __syncthreads();
     }
 }
 
@@ -527,85 +526,13 @@ __global__ void __launch_bounds__(kMaxThreadsYz, kMinBlocksYz) yz_kernel(GroupAr
     __syncthreads();
     fft_lines(A, tw, g.plany, g.lsy, L, tid, nthr);
     if constexpr (NZ > 0)
-        zconv_c<NZ>(A, A, g.lsy, Py, kx, g.Px, dslab, dk, dq, tid, nthr);
+        zconv_c<NZ>(A, g.lsy, Py, kx, g.Px, dslab, dk, dq, tid, nthr);
     else
         zconv_any(A, g.lsy, Py, nz, kx, g.Px, dslab, dk, dq, tid, nthr);
     fft_lines(A, tw, g.plany, g.lsy, L, tid, nthr);
     for (int it = tid; it < L * ny; it += nthr) {
         const int line = it / ny, y = it - line * ny;
         blk[line * ny + y] = cconj(A[line * g.lsy + fft_pad(y)]);
-    }
-}
-
-// yz for Py = 128 (ny <= 64), NZ layers: the y-transforms in two register passes each way
-// (f128_pass1/2, 16 roles per line, 16 * 3 * NZ threads) around the z-convolution.  Two shared
-// regions of 3*NZ lines alternate: R1 = forward exchange, then the z-convolution output; R2 = forward
-// output (z-convolution input, stride kLz), then the inverse exchange.
-constexpr int kLz = 136;  // line stride of the z-convolution input/output ([line][ky], 8 mod 16)
-template <typename T, int NZ>
-__global__ void __launch_bounds__(kMaxThreadsYz, kMinBlocks128) yz128_kernel(GroupArgs<T> g, int stage_dhat) {
-    using C = cplx<T>;
-    constexpr int L = 3 * NZ, hy = 64;
-    static_assert(L % 4 == 0, "pass-1 roles take lines in groups of four");
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* R1 = reinterpret_cast<C*>(smem_raw);
-    C* R2 = R1 + L * kF128Line;
-    T* dsm = reinterpret_cast<T*>(R2 + L * kF128Line);
-    const int tid = threadIdx.x, nthr = blockDim.x;
-    const int kx = blockIdx.x, p = blockIdx.y;
-    const int ny = g.ny;
-    const int kxo = min(kx, g.Px - kx);
-    C* blk = g.spec + ((size_t)p * g.Px + kx) * L * ny;
-    const T* dslab = g.dhat + (size_t)kxo * (hy + 1) * NZ * 6;
-    if (stage_dhat) {
-        for (int i = tid; i < (hy + 1) * NZ * 6; i += nthr) dsm[i] = dslab[i];
-        dslab = dsm;
-    }
-    const C* __restrict__ tw = g.t2y;  // pass-1 twiddles of length 128
-    griddep_wait();
-    griddep_launch_dependents();
-    for (int r = tid; r < 16 * L; r += nthr) {
-        int line, n2, par;
-        f128_role1(r, line, n2, par);
-        const C* src = blk + (size_t)line * ny + n2;
-        C u[8];
-#pragma unroll
-        for (int n1 = 0; n1 < 8; ++n1) u[n1] = 8 * n1 + n2 < ny ? src[8 * n1] : C{T(0), T(0)};
-        f128_pass1<false>(u, u, n2, par, tw, R1 + line * kF128Line);
-    }
-    __syncthreads();
-    for (int r = tid; r < 16 * L; r += nthr) {
-        const int k1 = r & 15, line = r >> 4;
-        C v[8];
-        f128_pass2(v, R1 + line * kF128Line, k1);
-        C* a = R2 + line * kLz + k1;
-#pragma unroll
-        for (int k2 = 0; k2 < 8; ++k2) a[16 * k2] = v[k2];
-    }
-    __syncthreads();
-    zconv_c<NZ, false>(R2, R1, kLz, 128, kx, g.Px, dslab, 1, hy + 1, tid, nthr);
-    __syncthreads();
-    for (int r = tid; r < 16 * L; r += nthr) {
-        int line, n2, par;
-        f128_role1(r, line, n2, par);
-        const C* b = R1 + line * kLz + n2;
-        C u[8], hi[8];
-#pragma unroll
-        for (int n1 = 0; n1 < 8; ++n1) {
-            u[n1] = b[8 * n1];
-            hi[n1] = b[8 * n1 + 64];
-        }
-        f128_pass1<true>(u, hi, n2, par, tw, R2 + line * kF128Line);
-    }
-    __syncthreads();
-    for (int r = tid; r < 16 * L; r += nthr) {
-        const int k1 = r & 15, line = r >> 4;
-        C v[8];
-        f128_pass2(v, R2 + line * kF128Line, k1);
-        C* dst = blk + (size_t)line * ny + k1;
-#pragma unroll
-        for (int k2 = 0; k2 < 4; ++k2)
-            if (k1 + 16 * k2 < ny) dst[16 * k2] = cconj(v[k2]);
     }
 }
 
@@ -2165,15 +2092,6 @@ template <typename T> void launch_yz(const GroupArgs<T>& g, int nthr, size_t sme
             }
             return;
         }
-        if (f128_yz(4, g.Py, g.nz)) {
-            bool st128 = false;
-            const size_t sm128 = f128_yz_smem(g.nz, g.Py, &st128);
-            if (g.nz == 8)
-                launch_pdl(yz128_kernel<T, 8>, grid, dim3(f128_yz_threads(8)), sm128, st, g, (int)st128);
-            else
-                launch_pdl(yz128_kernel<T, 4>, grid, dim3(f128_yz_threads(4)), sm128, st, g, (int)st128);
-            return;
-        }
 #define SS_CASE(Z)                                                      \
     if (g.nz == Z) {                                                    \
         launch_pdl(yz_kernel<T, Z>, grid, dim3(nthr), smem, st, g, stage); \
@@ -2422,8 +2340,6 @@ template <typename T> void set_smem_limits(int bytes) {
     set_dyn_smem(xinv128_kernel<T, 5, R>, bytes);
         SS_CASE(2) SS_CASE(4) SS_CASE(8)
 #undef SS_CASE
-        set_dyn_smem(yz128_kernel<T, 4>, bytes);
-        set_dyn_smem(yz128_kernel<T, 8>, bytes);
 #define SS_CASE(Z) set_dyn_smem(yz_kernel<T, Z>, bytes);
         SS_FOR_NZ(SS_CASE)
 #undef SS_CASE

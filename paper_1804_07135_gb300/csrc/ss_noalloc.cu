@@ -231,7 +231,7 @@ extern "C" ss_status ss_field_noalloc(int nx, int ny, int nz, double J, double D
         na_tensor_fill<<<(int)((cells + 255) / 256 < 4096 ? (cells + 255) / 256 : 4096), 256, 0, st>>>(tens, nx, ny, nz, Px, Py);
         launch_fft_strided_f64(tens, tw64x, px, 6 * nz * Py, 1, 1, 0, Px, st);
         launch_fft_strided_f64(tens, tw64y, py, 6 * nz * Px, Px, Px, 1, (long)Px * Py, st);
-        launch_extract_octant<float>(tens, dhat, Px, Py, nz, 4.0 * M_PI / ((double)Px * Py), st);
+        launch_extract_octant<float>(tens, dhat, Px, Py, nz, dhat_factor(4, Py, nz, Px) * 4.0 * M_PI / ((double)Px * Py), st);
     }
     ImgParam<float>* prm = reinterpret_cast<ImgParam<float>*>(base + o_prm);
     InterpEntry* interp = reinterpret_cast<InterpEntry*>(base + o_interp);

@@ -11,92 +11,178 @@ namespace ss {
 // 17-strided row layout, the z-convolution in place between them.  One shared line per (column, component,
 // layer): 3 NZ KXB lines of t2_line(P) complex elements, read from the spectrum in pass 1 and written back
 // (rows y < ny) in pass B; one shared-memory round trip per pass instead of one per Stockham stage.
-// 384 threads; pass 2 and pass A take one warp per line (16 columns x 2 parities), or half a warp (odd P/16).
-// Three CTAs per SM, two from P = 384 on (its 78 KB lines; there the kernel keeps 80 registers, which runs a
-// batch of size groups faster than three CTAs of 56 registers would, although one group alone runs faster
-// with three).
+// Pass 2 and pass A take one warp per line (16 columns x 2 parities), or half a warp (odd P/16).
+//
+// The z-convolution works on sums and differences of mirrored layers.  A component of the tensor is even
+// in z (t) or odd (G), so with n = NZ, e_i = s_i + s_{n-1-i}, o_i = s_i - s_{n-1-i} (i < n/2; the middle layer
+// of an odd n is an e of its own) and the same for the field (a factor 2, taken into dhat), even components
+// map e to e and o to o, odd ones e to o and o to e: two independent systems, (x, y in e; z in o) and
+// (x, y in o; z in e), each a real symmetric matrix of a quarter of the elements.  With sg = +1 or -1 for the
+// two, its blocks are t(|i-j|) + sg t(n-1-i-j) between x and y, t(|i-j|) - sg t(n-1-i-j) for zz, and
+// G(i-j) + sg G(n-1-i-j) between x or y (row i) and i times z (row j), so every product is a real
+// coefficient times a complex number.  Half the multiply-adds of the direct sum (144 instead of 192 + 96 per
+// frequency and system at 8 layers), and each spectrum element is read from shared memory once instead of
+// three times; the transforms are linear, so e and o are formed when pass 1 reads the layers and undone
+// when pass B writes them.  Kernel times on one GB300 before and after: 192x192x8 x 128 images 1420 -> 1214 us,
+// 128x128x8 x 192 788 -> 703, 128x128x4 x 384 733 -> 610, 100x100x5 x 32 79 -> 67, 112x112x1 x 60 (xz = yz = 0
+// left out) 40.5 -> 28.6.  What bounds it now (ncu, 192x192x8): no pipe (L1/shared 66%, FMA 45%, issue 54%);
+// 24 warps per SM wait for barriers and shared memory.
+template <int NZ, int PAR> struct ZSys {  // PAR 0: (x, y in e; z in o), 1: (x, y in o; z in e)
+    static constexpr int ME = (NZ + 1) / 2, MO = NZ / 2;
+    static constexpr int NXY = PAR == 0 ? ME : MO, NZC = PAR == 0 ? MO : ME;  // elements of x (and y), and of z
+};
+
+// One system at one frequency: A points at the frequency's element of line 0 (line stride LS), d at its
+// coefficients (component c, |dz| at d[(|dz| * 6 + c) * DQ]); par the system; fx, fy the parity signs of kx, ky
+// (the tensor's xy, xz, yz are odd in them: flip x and y going in and coming out).  The result replaces the
+// inputs, conjugated (the inverse transform is the conjugate of the forward transform of the conjugate).
+template <int NZ, int PAR, int LS, int DQ>
+__device__ __forceinline__ void zconv_sys(float2* A, const float* __restrict__ d, int par, float fx, float fy) {
+    using S = ZSys<NZ, PAR>;  // the shape; for even NZ both systems share it and par picks one at run time
+    constexpr int NA = S::NXY, NB = S::NZC;
+    constexpr int NA1 = NA > 0 ? NA : 1, NB1 = NB > 0 ? NB : 1;
+    const float sg = par ? -1.f : 1.f;
+    float2* Ax = A + (par ? S::ME : 0) * LS;
+    float2* Ay = Ax + NZ * LS;
+    float2* Az = A + (2 * NZ + (par ? 0 : S::ME)) * LS;
+    float2 X[NA1], Y[NA1], Z[NB1], HX[NA1], HY[NA1], W[NB1];
+    const float2 fx2 = make_float2(fx, fx), fy2 = make_float2(fy, fy), zero = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < NA; ++i) {
+        X[i] = __fmul2_rn(fx2, Ax[i * LS]);
+        Y[i] = __fmul2_rn(fy2, Ay[i * LS]);
+        HX[i] = HY[i] = zero;
+    }
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+        const float2 z = Az[i * LS];
+        Z[i] = make_float2(-z.y, z.x);  // i z
+        W[i] = zero;
+    }
+    auto load = [&](int c, float (&t)[NZ]) {
+#pragma unroll
+        for (int q = 0; q < NZ; ++q) t[q] = d[(q * 6 + c) * DQ];
+    };
+    auto dup = [](float a) { return make_float2(a, a); };
+    // t(|i-j|) + s t(n-1-i-j) for an even component
+    auto even = [&](const float (&t)[NZ], float s, int i, int j) {
+        return dup(fmaf(s, t[NZ - 1 - i - j], t[i > j ? i - j : j - i]));
+    };
+    float t[NZ];
+    if constexpr (NA > 0) {
+        load(0, t);  // xx
+#pragma unroll
+        for (int i = 0; i < NA; ++i)
+#pragma unroll
+            for (int j = 0; j <= i; ++j) {
+                const float2 c = even(t, sg, i, j);
+                HX[i] = __ffma2_rn(c, X[j], HX[i]);
+                if (j < i) HX[j] = __ffma2_rn(c, X[i], HX[j]);
+            }
+        load(3, t);  // xy
+#pragma unroll
+        for (int i = 0; i < NA; ++i)
+#pragma unroll
+            for (int j = 0; j <= i; ++j) {
+                const float2 c = even(t, sg, i, j);
+                HX[i] = __ffma2_rn(c, Y[j], HX[i]);
+                HY[i] = __ffma2_rn(c, X[j], HY[i]);
+                if (j < i) {
+                    HX[j] = __ffma2_rn(c, Y[i], HX[j]);
+                    HY[j] = __ffma2_rn(c, X[i], HY[j]);
+                }
+            }
+        load(1, t);  // yy
+#pragma unroll
+        for (int i = 0; i < NA; ++i)
+#pragma unroll
+            for (int j = 0; j <= i; ++j) {
+                const float2 c = even(t, sg, i, j);
+                HY[i] = __ffma2_rn(c, Y[j], HY[i]);
+                if (j < i) HY[j] = __ffma2_rn(c, Y[i], HY[j]);
+            }
+    }
+    if constexpr (NA > 0 && NB > 0) {
+        // G(i-j) + sg G(n-1-i-j), G(0) = 0: xz, then yz
+        auto odd = [&](const float (&t)[NZ], int i, int j) {
+            const int p = NZ - 1 - i - j;
+            const float hank = p > 0 ? t[p] : p < 0 ? -t[-p] : 0.f;
+            return dup(i == j ? sg * hank : fmaf(sg, hank, i > j ? t[i - j] : -t[j - i]));
+        };
+        load(4, t);
+#pragma unroll
+        for (int i = 0; i < NA; ++i)
+#pragma unroll
+            for (int j = 0; j < NB; ++j) {
+                const float2 c = odd(t, i, j);
+                HX[i] = __ffma2_rn(c, Z[j], HX[i]);
+                W[j] = __ffma2_rn(c, X[i], W[j]);
+            }
+        load(5, t);
+#pragma unroll
+        for (int i = 0; i < NA; ++i)
+#pragma unroll
+            for (int j = 0; j < NB; ++j) {
+                const float2 c = odd(t, i, j);
+                HY[i] = __ffma2_rn(c, Z[j], HY[i]);
+                W[j] = __ffma2_rn(c, Y[i], W[j]);
+            }
+    }
+    const float2 cx = make_float2(fx, -fx), cy = make_float2(fy, -fy);
+#pragma unroll
+    for (int i = 0; i < NA; ++i) {
+        Ax[i * LS] = __fmul2_rn(cx, HX[i]);
+        Ay[i * LS] = __fmul2_rn(cy, HY[i]);
+    }
+    if constexpr (NB > 0) {
+        load(2, t);  // zz
+#pragma unroll
+        for (int i = 0; i < NB; ++i)
+#pragma unroll
+            for (int j = 0; j <= i; ++j) {
+                const float2 c = even(t, -sg, i, j);
+                W[i] = __ffma2_rn(c, Z[j], W[i]);
+                if (j < i) W[j] = __ffma2_rn(c, Z[i], W[j]);
+            }
+#pragma unroll
+        for (int i = 0; i < NB; ++i) Az[i * LS] = make_float2(W[i].y, W[i].x);  // conj(-i W)
+    }
+}
+
+// The z-convolution of one column: one item per (frequency, system), reading and writing its own elements.
 template <int NZ, int P>
 __device__ __forceinline__ void zconv_t2(float2* A, int kx, int Px, const float* dslab, int tid, int nthr) {
-    constexpr int LS = t2_line(P), hy = P / 2, dq = P / 2 + 1;
-    const float sxg = kx > Px / 2 ? -1.f : 1.f;
-    const int nk = nthr / 3;
-    // rounds of nk frequencies; a round reads and writes only its own ky, so one barrier (between its
-    // reads and its writes) orders it against every other round
-    for (int k0 = 0; k0 < P; k0 += nk) {
-        const int a = tid / nk;
-        const int ky = k0 + (tid - a * nk);
-        const bool act = a < 3 && ky < P;
-        float2 out[NZ];
-        int pky = 0;
-        if (act) {
-            const int kyo = min(ky, P - ky);
-            const float syg = ky > hy ? -1.f : 1.f;
-            const float* d = dslab + kyo;
-            pky = t2_pos(ky);
-            const int i0 = a == 0 ? 0 : (a == 1 ? 3 : 4);
-            const int i1 = a == 0 ? 3 : (a == 1 ? 1 : 5);
-            const int i2 = a == 0 ? 4 : (a == 1 ? 5 : 2);
-            const float f0 = a == 0 ? 1.f : (a == 1 ? sxg * syg : sxg);
-            const float f1 = a == 0 ? sxg * syg : (a == 1 ? 1.f : syg);
-            const float f2 = a == 0 ? sxg : (a == 1 ? syg : 1.f);
-            float e0[NZ], e1[NZ], e2[NZ];
-#pragma unroll
-            for (int q = 0; q < NZ; ++q) {
-                e0[q] = d[(q * 6 + i0) * dq] * f0;
-                e1[q] = d[(q * 6 + i1) * dq] * f1;
-                e2[q] = d[(q * 6 + i2) * dq] * f2;
-            }
-#pragma unroll
-            for (int z = 0; z < NZ; ++z) out[z] = make_float2(0.f, 0.f);
-            // paired FP32 form as in zconv_c: out += (e, e) * S and (g, g) * (i S), i S = (-S.y, S.x)
-            if (a < 2) {
-#pragma unroll
-                for (int zp = 0; zp < NZ; ++zp) {
-                    const float2 sx = A[(0 * NZ + zp) * LS + pky];
-                    const float2 sy = A[(1 * NZ + zp) * LS + pky];
-                    const float2 sz = A[(2 * NZ + zp) * LS + pky];
-                    const float2 isz = make_float2(-sz.y, sz.x), nisz = make_float2(sz.y, -sz.x);
-#pragma unroll
-                    for (int z = 0; z < NZ; ++z) {
-                        const int q = z >= zp ? z - zp : zp - z;
-                        out[z] = __ffma2_rn(make_float2(e0[q], e0[q]), sx, out[z]);
-                        out[z] = __ffma2_rn(make_float2(e1[q], e1[q]), sy, out[z]);
-                        out[z] = __ffma2_rn(make_float2(e2[q], e2[q]), z >= zp ? isz : nisz, out[z]);
-                    }
-                }
-            } else {
-#pragma unroll
-                for (int zp = 0; zp < NZ; ++zp) {
-                    const float2 sx = A[(0 * NZ + zp) * LS + pky];
-                    const float2 sy = A[(1 * NZ + zp) * LS + pky];
-                    const float2 sz = A[(2 * NZ + zp) * LS + pky];
-                    const float2 isx = make_float2(-sx.y, sx.x), nisx = make_float2(sx.y, -sx.x);
-                    const float2 isy = make_float2(-sy.y, sy.x), nisy = make_float2(sy.y, -sy.x);
-#pragma unroll
-                    for (int z = 0; z < NZ; ++z) {
-                        const int q = z >= zp ? z - zp : zp - z;
-                        out[z] = __ffma2_rn(make_float2(e0[q], e0[q]), z >= zp ? isx : nisx, out[z]);
-                        out[z] = __ffma2_rn(make_float2(e1[q], e1[q]), z >= zp ? isy : nisy, out[z]);
-                        out[z] = __ffma2_rn(make_float2(e2[q], e2[q]), sz, out[z]);
-                    }
-                }
-            }
-        }
-        __syncthreads();
-        if (act) {
-#pragma unroll
-            for (int z = 0; z < NZ; ++z) A[(a * NZ + z) * LS + pky] = cconj(out[z]);
+    constexpr int LS = t2_line(P), DQ = P / 2 + 1;
+    const float fx = kx > Px / 2 ? -1.f : 1.f;
+    for (int it = tid; it < (NZ == 1 ? P : 2 * P); it += nthr) {
+        const int par = it >= P ? 1 : 0, ky = it - par * P;
+        const float fy = ky > P / 2 ? -1.f : 1.f;
+        const float* d = dslab + min(ky, P - ky);
+        float2* a = A + t2_pos(ky);
+        if constexpr (NZ == 1) {  // xz and yz vanish
+            const float2 X = a[0], Y = a[LS], Z = a[2 * LS];
+            const float xx = d[0], yy = d[DQ], zz = d[2 * DQ], xy = fx * fy * d[3 * DQ];
+            a[0] = make_float2(xx * X.x + xy * Y.x, -(xx * X.y + xy * Y.y));
+            a[LS] = make_float2(xy * X.x + yy * Y.x, -(xy * X.y + yy * Y.y));
+            a[2 * LS] = make_float2(zz * Z.x, -zz * Z.y);
+        } else if constexpr (NZ % 2 == 0) {  // the two systems have the same shape
+            zconv_sys<NZ, 0, LS, DQ>(a, d, par, fx, fy);
+        } else if (par == 0) {
+            zconv_sys<NZ, 0, LS, DQ>(a, d, 0, fx, fy);
+        } else {
+            zconv_sys<NZ, 1, LS, DQ>(a, d, 1, fx, fy);
         }
     }
 }
 
 template <int P, int NZ, int KXB>
-__global__ void __launch_bounds__(kYz2Threads, P >= 384 ? 2 : 3) yz2p_kernel(GroupArgs<float> g) {
+__global__ void __launch_bounds__(yz2p_threads(P, NZ), yz2p_blocks(P, NZ)) yz2p_kernel(GroupArgs<float> g) {
     using C = float2;
     constexpr int R2 = P / 16, LS = t2_line(P), L = 3 * NZ * KXB, RC = 16 * T2<P>::NP;  // RC: roles per line
+    constexpr int ME = (NZ + 1) / 2, MO = NZ / 2, LP = 3 * ME * KXB;                    // LP: pairs of mirrored layers
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* A = reinterpret_cast<C*>(smem_raw);
-    const int tid = threadIdx.x, nthr = blockDim.x;
+    C* A = reinterpret_cast<C*>(smem_raw);  // line (b * 3 + c) * NZ + q: e_q for q < ME, o_{q - ME} above
+    const int tid = threadIdx.x, nthr = yz2p_threads(P, NZ);
     const int kx = blockIdx.x * KXB, p = blockIdx.y;
     const int ny = g.ny;
     C* blk = g.spec + ((size_t)p * g.Px + kx) * 3 * NZ * ny;  // KXB consecutive columns are contiguous
@@ -105,14 +191,34 @@ __global__ void __launch_bounds__(kYz2Threads, P >= 384 ? 2 : 3) yz2p_kernel(Gro
     const C* __restrict__ ta = g.t2y + P;                     // pass A
     griddep_wait();
     griddep_launch_dependents();
-    // pass 1, role (n2, line, par), n2 fastest: the zero-padded spectrum lines in, rows of Z out
-    for (int r = tid; r < 2 * R2 * L; r += nthr) {
-        const int n2 = r % R2, q = r / R2, line = q % L, par = q / L;
-        const C* src = blk + (size_t)line * ny + n2;
+    // pass 1, role (n2, mirrored pair of lines, par), n2 fastest: the zero-padded spectrum lines in, rows of
+    // Z of their sum and difference out
+    for (int r = tid; r < 2 * R2 * LP; r += nthr) {
+        const int n2 = r % R2, q = r / R2, lp = q % LP, par = q / LP;
+        const int bc = lp / ME, i = lp % ME;
+        const C* src = blk + (size_t)(bc * NZ + i) * ny + n2;
         C u[8];
+        if (MO == ME || i < MO) {
+            const C* src2 = blk + (size_t)(bc * NZ + NZ - 1 - i) * ny + n2;
+            C v[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) u[j] = R2 * j + n2 < ny ? src[R2 * j] : make_float2(0.f, 0.f);
-        t2_pass1<P>(u, n2, par, t1, A + line * LS);
+            for (int j = 0; j < 8; ++j) {
+                const bool in = R2 * j + n2 < ny;
+                u[j] = in ? src[R2 * j] : make_float2(0.f, 0.f);
+                v[j] = in ? src2[R2 * j] : make_float2(0.f, 0.f);
+            }
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const C a = u[j];
+                u[j] = cadd(a, v[j]);
+                v[j] = csub(a, v[j]);
+            }
+            t2_pass1<P>(v, n2, par, t1, A + (bc * NZ + ME + i) * LS);
+        } else {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) u[j] = R2 * j + n2 < ny ? src[R2 * j] : make_float2(0.f, 0.f);
+        }
+        t2_pass1<P>(u, n2, par, t1, A + (bc * NZ + i) * LS);
     }
     __syncthreads();
     // pass 2: one warp per line (lanes = 16 columns x 2 parities; half a warp for odd P/16)
@@ -127,16 +233,31 @@ __global__ void __launch_bounds__(kYz2Threads, P >= 384 ? 2 : 3) yz2p_kernel(Gro
     // pass A (the inverse transform of the conjugated field spectra, in place by columns)
     for (int r = tid; r < RC * L; r += nthr) t2_cols<P, true>(A + r / RC * LS, r & 15, r % RC / 16, tw, ta);
     __syncthreads();
-    // pass B, role (y2, line, par): rows y < ny back to the spectrum, conjugated
-    for (int r = tid; r < 2 * R2 * L; r += nthr) {
-        const int y2 = r % R2, q = r / R2, line = q % L, par = q / L;
+    // pass B, role (y2, mirrored pair of lines, par): rows y < ny of both layers back to the spectrum, conjugated
+    for (int r = tid; r < 2 * R2 * LP; r += nthr) {
+        const int y2 = r % R2, q = r / R2, lp = q % LP, par = q / LP;
+        const int bc = lp / ME, i = lp % ME;
         C v[8];
-        t2_passB(v, A + line * LS, y2, par);
-        C* dst = blk + (size_t)line * ny;
+        t2_passB(v, A + (bc * NZ + i) * LS, y2, par);
+        C* dst = blk + (size_t)(bc * NZ + i) * ny;
+        if (MO == ME || i < MO) {
+            C w[8];
+            t2_passB(w, A + (bc * NZ + ME + i) * LS, y2, par);
+            C* dst2 = blk + (size_t)(bc * NZ + NZ - 1 - i) * ny;
 #pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            const int y = y2 + R2 * (2 * m + par);
-            if (y < ny) dst[y] = cconj(v[m]);
+            for (int m = 0; m < 4; ++m) {
+                const int y = y2 + R2 * (2 * m + par);
+                if (y < ny) {
+                    dst[y] = cconj(cadd(v[m], w[m]));
+                    dst2[y] = cconj(csub(v[m], w[m]));
+                }
+            }
+        } else {
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                const int y = y2 + R2 * (2 * m + par);
+                if (y < ny) dst[y] = cconj(v[m]);
+            }
         }
     }
 }
@@ -266,9 +387,9 @@ template <typename T, int P> void t2_yz(const GroupArgs<T>& g, cudaStream_t st) 
     int kxb = yz2p_kxb_use(g.nz, g.yz_kxb);
     if (g.Px % kxb) kxb = yz2p_kxb(g.nz);
     const size_t sm = yz2p_smem(P, g.nz, kxb);
-    const dim3 grid(g.Px / kxb, g.n_pairs), blk(kYz2Threads);
+    const dim3 grid(g.Px / kxb, g.n_pairs);
 #define SS_CASE(Z, B) \
-    if (g.nz == Z && kxb == B) launch_pdl(yz2p_kernel<P, Z, B>, grid, blk, sm, st, g);
+    if (g.nz == Z && kxb == B) launch_pdl(yz2p_kernel<P, Z, B>, grid, dim3(yz2p_threads(P, Z)), sm, st, g);
     SS_T2_YZ(SS_CASE)
 #undef SS_CASE
 }
