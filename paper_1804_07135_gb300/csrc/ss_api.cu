@@ -279,10 +279,6 @@ template <typename T> GroupArgs<T> group_args(const ss_ctx* c, const Group& g) {
 // they need.
 void set_rows(Group& g, int ty_a, int ty_c, int thr_a = 256, int thr_c = 256) {
     const size_t cs = 2 * (size_t)g.rbytes;
-    if (g.dipole && f128_x(g.rbytes, g.Px)) {
-        ty_a = f128_x_rows(ty_a);
-        ty_c = f128_x_rows(ty_c);
-    }
     const bool x2 = g.dipole && x2p_ok(g.rbytes, g.Px);  // two-pass x kernels: fixed rows per CTA
     if (x2) ty_a = ty_c = kX2Rows;
     g.ty_a = ty_a;
@@ -291,14 +287,8 @@ void set_rows(Group& g, int ty_a, int ty_c, int thr_a = 256, int thr_c = 256) {
     g.thr_c = thr_c;
     g.smem_a = (size_t)(g.Px + 3 * g.ty_a * g.lsx) * cs;
     g.smem_c = (size_t)(g.Px + 3 * g.ty_c * g.lsx) * cs + 32 * 2 * kEvalTerms * sizeof(double);
-    if (g.dipole && f128_x(g.rbytes, g.Px)) {  // the launchers derive these shapes themselves
-        g.thr_a = f128_x_threads(ty_a);
-        g.thr_c = f128_x_threads(ty_c);
-        g.smem_a = f128_x_smem(ty_a);
-        g.smem_c = f128_x_smem(ty_c);
-    }
     if (x2) {
-        g.thr_a = g.thr_c = x2_threads(g.Px);
+        g.thr_a = g.thr_c = x2_launch_threads(g.Px, g.nx, (long)((g.ny + kX2Rows - 1) / kX2Rows) * g.nz * g.n_pairs);
         g.smem_a = x2_smem(g.Px, false);
         g.smem_c = x2_smem(g.Px, true);
     }
@@ -322,7 +312,6 @@ void configure_group(Group& g) {
             break;
         }
     }
-    if (g.dipole && f128_x(g.rbytes, g.Px)) ty = 8;  // 384 threads
     set_rows(g, ty, ty, 512, 512);
     // y/z kernel: all 3*nz lines of one (pair, kx) in shared memory, plus the kx slab of the tensor
     // spectrum when it is small enough to stage
@@ -331,7 +320,7 @@ void configure_group(Group& g) {
     const size_t slab = (size_t)(g.Py / 2 + 1) * g.nz * 6 * (size_t)g.rbytes;
     if (slab <= 24 * 1024) g.smem_b += slab;
     if (g.dipole && yz2p_ok(g.rbytes, g.Py, g.nz, g.Px)) {
-        g.thr_b = yz2p_threads(g.Py, g.nz);
+        g.thr_b = yz2p_threads(g.Py);
         g.smem_b = yz2p_smem(g.Py, g.nz, yz2p_kxb_use(g.nz, g.yz_kxb));
     }
 }
@@ -494,10 +483,9 @@ template <typename T> ss_status tune_group(ss_ctx* c, Group& g) {
     // kernel's columns per CTA (e.g. to profile the tuned shapes, or to compare both column counts)
     if (const char* env = getenv("SS_X_CONFIG")) {
         int ta = 0, ya = 0, tc = 0, yc = 0, kxb = 0;
-        const bool f128 = g.dipole && f128_x((int)real_size(c), g.Px);  // block size follows the rows
         const int n = sscanf(env, "%d:%d:%d:%d:%d", &ta, &ya, &tc, &yc, &kxb);
-        if (n >= 4 && (f128 || ((ta == 256 || ta == 512) && (tc == 256 || tc == 512))) && ya >= 1 && yc >= 1 &&
-            ya <= g.ny && yc <= g.ny) {  // the x kernels for Px = 128 take 2, 4 or 8 rows (others become 8)
+        if (n >= 4 && (ta == 256 || ta == 512) && (tc == 256 || tc == 512) && ya >= 1 && yc >= 1 && ya <= g.ny &&
+            yc <= g.ny) {
             g.yz_kxb = n == 5 ? kxb : 0;  // a count the kernel does not take falls back to the default
             set_rows(g, ya, yc, ta, tc);
             configure_yz_smem(g);
@@ -520,9 +508,6 @@ template <typename T> ss_status tune_group(ss_ctx* c, Group& g) {
     std::vector<std::pair<int, int>> cands;  // (threads, rows)
     if (g.dipole && x2p_ok((int)real_size(c), g.Px)) {
         cands.push_back({x2_threads(g.Px), kX2Rows});  // one shape: nothing to tune
-    } else if (g.dipole && f128_x((int)real_size(c), g.Px)) {
-        for (int ty : {2, 4, 8})  // 48 threads per row; row counts that divide 16 keep the passes conflict-free
-            cands.push_back({f128_x_threads(ty), ty});
     } else {
         for (int thr : {256, 512})
             for (int ty : {1, 2, 4, 5, 8, 10, 16})

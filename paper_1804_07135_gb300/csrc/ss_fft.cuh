@@ -258,6 +258,9 @@ template <typename C> struct Dft<9, C> : DftCt<3, 3, C> {};
 template <typename C> struct Dft<10, C> : DftCt<5, 2, C> {};
 template <typename C> struct Dft<14, C> : DftCt<7, 2, C> {};
 template <typename C> struct Dft<16, C> : DftCt<4, 4, C> {};
+template <typename C> struct Dft<18, C> : DftCt<3, 6, C> {};
+template <typename C> struct Dft<20, C> : DftCt<5, 4, C> {};
+template <typename C> struct Dft<24, C> : DftCt<3, 8, C> {};
 
 // Host-side plan: radices 8, 4, 2 first (largest first), then 3s, 5s and 7s (the last two only in the setup
 // transforms of the tensor spectrum: a length with those factors has two-pass kernels).
@@ -380,28 +383,7 @@ __device__ __forceinline__ void fft_lines(C* buf, const C* tw, const FftPlan& pl
     }
 }
 
-// ---- length 128 in two register passes -----------------------------------------------------------
-// With n = 8 n1 + n2 and k = k1 + 16 k2 (n1, k1 < 16; n2, k2 < 8) and W = W_128,
-//   X[k1 + 16 k2] = sum_{n2} W_8^{n2 k2} W^{n2 k1} Y[n2][k1],   Y[n2][k1] = sum_{n1} W_16^{n1 k1} x[8 n1 + n2].
-// Split by the parity of k1 = 2 m + par, the 16-point inner DFT is an 8-point DFT over n1 < 8 of
-//   u[n1] = (x[8 n1 + n2] + (-1)^par x[8 n1 + 64 + n2]) W_16^{par n1},
-// so a line takes two passes of 8-point DFTs in registers with one exchange through shared memory:
-// pass 1, role (n2, par): Z[n2][2m + par] = W^{n2 (2m + par)} DFT8(u)[m];
-// pass 2, role k1:        X[k1 + 16 k2] = DFT8(Z[.][k1])[k2].
-// A line with a zero upper half (x[n] = 0 for n >= 64) drops the second term of u; a transform read
-// only below 64 evaluates k2 < 4 in pass 2 (the other outputs are dead code).
-// Exchange buffer Z[line][n2][k1] at line * kF128Line + n2 * kF128N2 + k1 (kF128Line = 1 mod 16, in
-// ss_internal.h): the 16 lanes of a half-warp reading 16 consecutive k1 of one line, or writing 8 n2 of
-// two consecutive lines (pass-1 roles below), touch 16 distinct bank pairs.
-constexpr int kF128N2 = 18;
-// Pass-1 role r -> (line, n2, par): n2 = r & 7, then four consecutive lines, then par, so par is uniform
-// across a warp; lines are taken in groups of four (callers skip line >= their count).
-__device__ __forceinline__ void f128_role1(int r, int& line, int& n2, int& par) {
-    n2 = r & 7;
-    par = (r >> 5) & 1;
-    line = ((r >> 6) << 2) | ((r >> 3) & 3);
-}
-
+// ---- multiplications by 16th roots of unity
 // a * W_16^J for a compile-time J < 8, W_16 = exp(-2 pi i / 16)
 template <int J, typename C> __device__ __forceinline__ C mul_w16(C a) {
     using R = decltype(a.x);
@@ -432,68 +414,50 @@ template <typename C> __device__ __forceinline__ void mul_w16_ramp(C (&u)[8]) {
     u[7] = mul_w16<7>(u[7]);
 }
 
-// Pass 1 for role (n2, par) of one line.  u holds x[8 n1 + n2] for n1 < 8 on entry; hi (when given)
-// holds x[8 n1 + 64 + n2].  Writes Z[n2][2m + par] of the line at zl = exchange buffer + line offset.
-// t1: the pass-1 twiddle table (GroupArgs::t2x / t2y), W_128^{n2 (2m + par)} at (2m + par) * 8 + n2.
-template <bool HAS_HI, typename C>
-__device__ __forceinline__ void f128_pass1(C (&u)[8], const C (&hi)[8], int n2, int par, const C* __restrict__ t1,
-                                           C* zl) {
-    if constexpr (HAS_HI) {
-#pragma unroll
-        for (int j = 0; j < 8; ++j) u[j] = par ? csub(u[j], hi[j]) : cadd(u[j], hi[j]);
-    }
-    if (par) mul_w16_ramp(u);
-    Dft<8, C>::run(u);
-    C* z = zl + n2 * kF128N2 + par;
-#pragma unroll
-    for (int m = 0; m < 8; ++m) z[2 * m] = cmul(u[m], t1[(2 * m + par) * 8 + n2]);  // W_128^{n2 (2m + par)}
-}
-
-// Pass 2 for role k1 of one line: v[k2] = X[k1 + 16 k2] (k2 < KOUT) from Z[.][k1] at zl + k1.
-template <typename C> __device__ __forceinline__ void f128_pass2(C (&v)[8], const C* zl, int k1) {
-    const C* z = zl + k1;
-#pragma unroll
-    for (int n2 = 0; n2 < 8; ++n2) v[n2] = z[n2 * kF128N2];
-    Dft<8, C>::run(v);
-}
-
 // ---- lengths P = 16 R2 (R2 = 2..32: 32 to 512) in two register passes ------------------------------------
 // A line of P elements is held in shared memory as R2 rows of 16 at row stride kT2Row = 17 (element
 // (r, c) at r * 17 + c; a line takes kT2Row * R2 slots).  With n = R2 n1 + n2, k = k1 + 16 k2 (n1, k1 < 16;
 // n2, k2 < R2) the forward transform is
-//   X[k1 + 16 k2] = sum_{n2} W_R2^{n2 k2} Z[n2][k1],   Z[n2][k1] = W_P^{n2 k1} sum_{n1} W_16^{n1 k1} x[R2 n1 + n2],
-// both sums split by the parity of their output index into half-size DFTs (W = W_P, as for length 128):
-// pass 1, role (n2, par), inputs x[R2 n1 + n2]: an 8-point DFT of (x[R2 j + n2] +- x[R2 (j+8) + n2]) W_16^{j par}
-//   -> row n2 of Z (k1 = 2m + par);
-// pass 2, role (k1, par2), column k1 of Z: an R2/2-point DFT of (Z[j][k1] +- Z[j + R2/2][k1]) W_R2^{j par2}
-//   -> X[k1 + 16 (2m + par2)], written back in place into column k1 (row k2), so X[ky] sits at
-//   (ky >> 4) * 17 + (ky & 15).
+//   X[k1 + 16 k2] = sum_{n2} W_R2^{n2 k2} Z[n2][k1],   Z[n2][k1] = W_P^{n2 k1} sum_{n1} W_16^{n1 k1} x[R2 n1 + n2]:
+// pass 1, role n2, inputs x[R2 j + n2], j < 8 (the upper half of the line is zero): the 16-point DFT as two
+//   8-point ones of x W_16^{j par}, par = 0, 1 -> row n2 of Z (k1 = 2m + par);
+// pass 2, role k1, column k1 of Z: the R2-point DFT -> X[k1 + 16 k2], written back in place into column k1
+//   (row k2), so X[ky] sits at (ky >> 4) * 17 + (ky & 15).
 // The inverse direction (a forward transform of the conjugate) starts from that column layout: with
 // y = y2 + R2 y1,
 //   Y[y2 + R2 y1] = sum_{k1} W_16^{k1 y1} T[k1][y2],   T[k1][y2] = W_P^{k1 y2} sum_{k2} W_R2^{k2 y2} V[k1 + 16 k2];
-// pass A, role (k1, par2), column k1: the R2/2-point DFTs as in pass 2, times W_P^{k1 y2}, back into column k1
-//   (row y2);
-// pass B, role (y2, par), row y2: an 8-point DFT of (T[j][y2] +- T[j+8][y2]) W_16^{j par} -> Y[y2 + R2 (2m + par)];
-// an inverse read below P/2 keeps m < 4.  For odd R2 (48, 80, 112, 144) passes 2 and A take one role per column
-// k1 with the whole R2-point DFT (t2_col_vals with H = R2 and no split).  The twiddles of pass 1 and pass A come from the tables of
-// GroupArgs::t2x / t2y (t1 = the pass-1 half, ta = the pass-A half, indexed so that a warp's lanes read
-// consecutive entries); the ramp W_R2^j = W_P^{16 j} from the flat table tw (the same entry across a warp).
+// pass A, role k1, column k1: the R2-point DFT as in pass 2, times W_P^{k1 y2}, back into column k1 (row y2);
+// pass B, role y2, row y2: the outputs below P/2, Y[y2 + R2 y1], y1 = 2m + par < 8, from 8-point DFTs of
+//   (T[j][y2] +- T[j+8][y2]) W_16^{j par}.
+// So every element crosses shared memory once per pass.  (Roles of one parity each, with half the registers,
+// read every element twice: the y/z kernel of 64x64x8 spent 75% of its time's L1 wavefronts there.)  From
+// R2 = 28 on a whole column takes too many registers, and passes 2 and A take two roles per column, par2 = 0
+// and 1, with the R2/2-point DFTs of the outputs of one parity.  The twiddles of pass 1 and pass A come from
+// the tables of GroupArgs::t2x / t2y (t1 = the pass-1 half, ta = the pass-A half, indexed so that a warp's lanes
+// read consecutive entries); the ramp W_R2^j = W_P^{16 j} of the split columns from the flat table tw (the
+// same entry across a warp).
 __device__ __forceinline__ int t2_at(int r, int c) { return r * kT2Row + c; }
 __device__ __forceinline__ int t2_pos(int ky) { return t2_at(ky >> 4, ky & 15); }
 
 // Pass 1 of a line whose upper half is zero: u[j] = x[R2 j + n2] (j < 8) on entry; writes row n2 of Z.
 template <int P, typename C>
-__device__ __forceinline__ void t2_pass1(C (&u)[8], int n2, int par, const C* __restrict__ t1, C* line) {
-    if (par) mul_w16_ramp(u);
+__device__ __forceinline__ void t2_pass1(C (&u)[8], int n2, const C* __restrict__ t1, C* line) {
+    C w[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) w[j] = u[j];
+    mul_w16_ramp(w);
     Dft<8, C>::run(u);
 #pragma unroll
+    for (int m = 0; m < 8; ++m) line[t2_at(n2, 2 * m)] = cmul(u[m], t1[2 * m * (P / 16) + n2]);  // W_P^{2 m n2}
+    Dft<8, C>::run(w);
+#pragma unroll
     for (int m = 0; m < 8; ++m)
-        line[t2_at(n2, 2 * m + par)] = cmul(u[m], t1[(2 * m + par) * (P / 16) + n2]);  // W_P^{n2 (2m + par)}
+        line[t2_at(n2, 2 * m + 1)] = cmul(w[m], t1[(2 * m + 1) * (P / 16) + n2]);  // W_P^{(2 m + 1) n2}
 }
 
-// Roles per column of passes 2 and A (2: the output rows split by parity; 1: odd R2) and outputs per role.
+// Roles per column of passes 2 and A (2: the output rows split by parity) and outputs per role.
 template <int P> struct T2 {
-    static constexpr int R2 = P / 16, NP = R2 % 2 == 0 ? 2 : 1, H = R2 / NP;
+    static constexpr int R2 = P / 16, NP = R2 > 24 ? 2 : 1, H = R2 / NP;
 };
 
 // The H-point DFTs of pass 2 (TW_OUT = false) or pass A (TW_OUT = true) for column k1 and parity par2:
@@ -537,16 +501,24 @@ __device__ __forceinline__ void t2_cols(C* line, int k1, int par2, const C* __re
     for (int m = 0; m < H; ++m) line[t2_at(NP * m + par2, k1)] = a[m];
 }
 
-// Pass B of row y2: v[m] = Y[y2 + R2 (2m + par)] for m < 4 (the outputs below P/2).
+// Pass B of row y2: v[y1] = Y[y2 + R2 y1] for y1 < 8 (the outputs below P/2).
 template <typename C>
-__device__ __forceinline__ void t2_passB(C (&v)[8], const C* line, int y2, int par) {
+__device__ __forceinline__ void t2_passB(C (&v)[8], const C* line, int y2) {
+    C s[8], d[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
         const C lo = line[t2_at(y2, j)], hi = line[t2_at(y2, j + 8)];
-        v[j] = par ? csub(lo, hi) : cadd(lo, hi);
+        s[j] = cadd(lo, hi);
+        d[j] = csub(lo, hi);
     }
-    if (par) mul_w16_ramp(v);
-    Dft<8, C>::run(v);
+    Dft<8, C>::run(s);
+    mul_w16_ramp(d);
+    Dft<8, C>::run(d);
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+        v[2 * m] = s[m];
+        v[2 * m + 1] = d[m];
+    }
 }
 
 }  // namespace ss

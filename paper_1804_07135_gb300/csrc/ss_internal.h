@@ -24,8 +24,6 @@ constexpr int kMaxThreadsX = 512;   // largest block of the x-transform kernels 
 constexpr int kMinBlocksX = 2;      // resident 512-thread blocks per SM they are compiled for (64 registers)
 constexpr int kMaxThreadsYz = 384;  // block size of the y/z kernel (3 x 128: one z-convolution row per warp)
 constexpr int kMinBlocksYz = 2;
-constexpr int kMaxThreads128 = 384;  // length-128 x kernels: at most 8 rows of 48 threads
-constexpr int kMinBlocks128 = 3;     // resident 384-thread blocks per SM of the length-128 kernels (56 registers)
 constexpr int kArcMaxChunk = 8;     // image differences one arc CTA accumulates
 constexpr int kArcMaxK = 1024;      // images per string
 
@@ -175,19 +173,6 @@ template <typename T> struct RkArgs {
 
 enum { kErrInvalidSpin = 1, kErrNonFinite = 2, kErrStepCollapse = 4 };
 
-// Length-128 transforms in two register passes (FP32): the x kernels when Px = 128.  16 threads per line;
-// their launch shapes follow from the rows per CTA, whatever block size and shared memory the caller passes.
-constexpr int kF128Line = 145;  // line stride of their exchange buffers (complex elements, 1 mod 16)
-constexpr int kF128Buf = 72;    // line stride of the x kernels' 64-point lines (fft_pad positions, 8 mod 16)
-inline bool f128_x(int real_bytes, int Px) { return real_bytes == 4 && Px == 128; }
-// rows per CTA of the x kernels: 2, 4 or 8 (compile-time); anything else is taken as 8
-inline int f128_x_rows(int ty) { return ty == 2 || ty == 4 ? ty : 8; }
-inline int f128_x_threads(int rows) { return 48 * rows; }
-inline size_t f128_x_smem(int rows) {
-    // line buffer, exchange buffer (lines rounded up to a multiple of 4), reduction scratch
-    return (size_t)(3 * rows * kF128Buf + (3 * rows + 3) / 4 * 4 * kF128Line) * 8 + 32 * 2 * kEvalTerms * sizeof(double);
-}
-
 // Lengths P = 16 R2 in two register passes (FP32, ss_fft.cuh, ss_twopass.cuh): a line is R2 = P/16 rows of 16
 // at row stride kT2Row; the y/z kernel for those Py with 1 to 8 layers, the x kernels for those Px with
 // kX2Rows rows per CTA.  The list covers lattices of up to 256 sites a side; each length is a multiple of 16
@@ -221,10 +206,13 @@ inline bool yz2p_ok(int real_bytes, int Py, int nz, int Px) {
     const int kxb = yz2p_kxb(nz);
     return kxb > 0 && Px % kxb == 0;
 }
-// threads and resident CTAs of the y/z kernel: with four or more layers the z-convolution wants 64 registers
-// (four to six layers) or 80 (seven, eight); as many CTAs as registers and shared memory allow
-__host__ __device__ constexpr int yz2p_threads(int P, int nz) { return nz <= 3 || P > 320 ? 384 : nz >= 7 || P <= 256 ? 256 : 384; }
-__host__ __device__ constexpr int yz2p_blocks(int P, int nz) { return P > 320 ? 2 : nz >= 4 && nz <= 6 && P <= 256 ? 4 : 3; }
+// threads and resident CTAs of the y/z kernel: small CTAs, so that several per SM are in different passes, of
+// 80 registers per thread (64 spill in the z-convolution and the mirrored pass 1); as many as registers and
+// shared memory (24 lines: 26 KB at 128, 78 KB at 384) allow
+__host__ __device__ constexpr int yz2p_threads(int P) { return P <= 128 ? 128 : P <= 256 ? 192 : P <= 320 ? 256 : 384; }
+__host__ __device__ constexpr int yz2p_blocks(int P) {
+    return P <= 128 ? 6 : P <= 256 ? 4 : P <= 320 ? 3 : 2;
+}
 // columns per CTA a launch uses: the tuned choice when it is one of the two, else the default
 inline int yz2p_kxb_use(int nz, int tuned) { return tuned > 0 && (tuned == yz2p_kxb(nz) || tuned == yz2p_kxb_alt(nz)) ? tuned : yz2p_kxb(nz); }
 inline size_t yz2p_smem(int Py, int nz, int kxb) { return (size_t)3 * nz * kxb * t2_line(Py) * 8; }
@@ -234,14 +222,24 @@ inline double dhat_factor(int real_bytes, int Py, int nz, int Px) {
     return nz > 1 && yz2p_ok(real_bytes, Py, nz, Px) ? 0.5 : 1.0;
 }
 constexpr int kX2Rows = 4;
-// threads of an x CTA: short lines have fewer roles than 384 threads would take
-__host__ __device__ constexpr int x2_threads(int P) { return P <= 48 ? 128 : P <= 80 ? 192 : P <= 160 ? 256 : 384; }
+// x CTAs: pass 2 has 192 roles (up to P = 384), pass 1 has 12 P/16, the sites take 4 nx (even nx) or 8 nx items.
+// The kernels are compiled for up to x2_threads threads in x2_blocks CTAs per SM (64 registers, 80 from P = 288
+// on) and launched with x2_launch_threads of them: on a grid of many waves the smaller block, of which more fit
+// on an SM (128x128x4 x 384 images: step kernel 311 us with 192 threads, 333 with 256); on a small grid the
+// larger one where it takes fewer rounds over the sites (112x112x1 x 60: iteration 56.2 us with 192, 53.7 with
+// 256).
+__host__ __device__ constexpr int x2_threads(int P) { return P <= 64 ? 128 : P <= 128 ? 192 : 256; }
+__host__ __device__ constexpr int x2_blocks(int P) { return P <= 64 ? 8 : P <= 128 ? 5 : P <= 256 ? 4 : 3; }
+inline int x2_launch_threads(int P, int nx, long ctas) {
+    const int hi = x2_threads(P), lo = P > 64 && P <= 256 ? hi - 64 : hi;
+    const int items = nx % 2 == 0 ? 4 * nx : 8 * nx;
+    return ctas < 10L * 152 && (items + hi - 1) / hi < (items + lo - 1) / lo ? hi : lo;
+}
 __host__ __device__ constexpr int x2_round(int v) { return v + ((16 / kX2Rows - v % 16) + 16) % 16; }
 __host__ __device__ constexpr int x2_lsx(int P) { return x2_round(t2_line(P) - 1); }  // transform lines
-__host__ __device__ constexpr int x2_lb(int P) { return x2_round(fft_pad(P / 2 - 1) + 1); }  // x-space lines
-inline bool x2p_ok(int real_bytes, int Px) { return real_bytes == 4 && t2_length(Px) && !f128_x(real_bytes, Px); }
+inline bool x2p_ok(int real_bytes, int Px) { return real_bytes == 4 && t2_length(Px); }
 inline size_t x2_smem(int P, bool inverse) {
-    return (size_t)3 * kX2Rows * (x2_lsx(P) + x2_lb(P)) * 8 + (inverse ? 32 * 2 * kEvalTerms * 8 : 0);
+    return (size_t)3 * kX2Rows * x2_lsx(P) * 8 + (inverse ? 32 * 2 * kEvalTerms * 8 : 0);
 }
 // Padded transform length for n sites: the smallest 2^a 3^b >= 2n - 1, or the power of two >= 2n - 1 when that
 // is at most 1/8 longer.

@@ -111,12 +111,21 @@ __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wa
 __device__ __forceinline__ void griddep_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 
 // ------------------------------------------------------------------------------------------------
+// Position of x within a line of the x kernels: fft_pad (runtime plans), or row x mod R2, column x / R2 of the
+// two-pass lines (where pass 1 reads its inputs and pass B leaves its outputs in place).
+struct PadPos {
+    __device__ __forceinline__ int operator()(int x) const { return fft_pad(x); }
+};
+template <int R2> struct T2Pos {
+    __device__ __forceinline__ int operator()(int x) const { return t2_at((unsigned)x % R2, (unsigned)x / R2); }
+};
+
 // Gather of rows [y0, y0+rows) of layer z for pair p: s[img] = normalise((1-t) sp[src0] + t sp[src1])
-// (or a copy), written back to s and, when buf is given, to line c*lrows + yy of buf (stride ls,
-// fft_pad positions) as re/im of the pair.
-template <typename T>
+// (or a copy), written back to s and, when buf is given, to line c*lrows + yy of buf (stride ls, x at pos(x))
+// as re/im of the pair.
+template <typename T, typename Pos>
 __device__ __forceinline__ void xfwd_gather(const GroupArgs<T>& g, cplx<T>* buf, int ls, int lrows, int p, int z,
-                                            int y0, int rows, int tid, int nthr) {
+                                            int y0, int rows, int tid, int nthr, Pos pos) {
     using C = cplx<T>;
     const int nx = g.nx, N = g.N;
     const int ia = 2 * p;
@@ -170,7 +179,7 @@ __device__ __forceinline__ void xfwd_gather(const GroupArgs<T>& g, cplx<T>* buf,
                     for (int c = 0; c < 3; ++c)
 #pragma unroll
                         for (int k = 0; k < 2; ++k)
-                            buf[(c * lrows + yy) * ls + fft_pad(x + k)] = C{out[0][k][c], out[1][k][c]};
+                            buf[(c * lrows + yy) * ls + pos(x + k)] = C{out[0][k][c], out[1][k][c]};
                 }
             }
             return;
@@ -211,7 +220,7 @@ __device__ __forceinline__ void xfwd_gather(const GroupArgs<T>& g, cplx<T>* buf,
         }
         if (buf) {
 #pragma unroll
-            for (int c = 0; c < 3; ++c) buf[(c * lrows + yy) * ls + fft_pad(x)] = C{out[0][c], out[1][c]};
+            for (int c = 0; c < 3; ++c) buf[(c * lrows + yy) * ls + pos(x)] = C{out[0][c], out[1][c]};
         }
     }
 }
@@ -235,7 +244,7 @@ __global__ void __launch_bounds__(kMaxThreadsX, kMinBlocksX) xfwd_kernel(GroupAr
         for (int i = tid; i < g.Px; i += nthr) tw[i] = g.twx[i];
     griddep_wait();
     griddep_launch_dependents();
-    xfwd_gather(g, DO_FFT ? buf : (C*)nullptr, g.lsx, rows, p, z, y0, rows, tid, nthr);
+    xfwd_gather(g, DO_FFT ? buf : (C*)nullptr, g.lsx, rows, p, z, y0, rows, tid, nthr, PadPos{});
     if (!DO_FFT) return;
     const int padw = g.Px - nx;
     for (int it = tid; it < 3 * rows * padw; it += nthr) {
@@ -252,55 +261,6 @@ __global__ void __launch_bounds__(kMaxThreadsX, kMinBlocksX) xfwd_kernel(GroupAr
         C* o = outp + ((size_t)kc * g.nz + z) * g.ny + y0;
         const C* b = buf + c * rows * g.lsx + fft_pad(kx);
         for (int yy = 0; yy < rows; ++yy) o[yy] = b[yy * g.lsx];
-    }
-}
-
-// xfwd for Px = 128 (nx <= 64), ROWS (2, 4 or 8) rows per CTA: the same gather, then the x-transform of
-// the 3*ROWS lines in two register passes (f128_pass1/2) with 16 roles per line; the second pass writes
-// the spectrum straight to global memory, rows fastest across a warp (the rows of one (kx, c) are
-// contiguous there).  Rows past ny (last CTA) are skipped.
-template <typename T, int ROWS>
-__global__ void __launch_bounds__(kMaxThreadsX, kMinBlocksX) xfwd128_kernel(GroupArgs<T> g) {
-    using C = cplx<T>;
-    static_assert(16 % ROWS == 0, "the pass-2 role permutation needs ROWS | 16");
-    constexpr int L = 3 * ROWS, NQ = 16 / ROWS;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* buf = reinterpret_cast<C*>(smem_raw);  // L lines of kF128Buf, fft_pad positions
-    C* zx = buf + L * kF128Buf;                // exchange buffer
-    const int tid = threadIdx.x, nthr = blockDim.x;
-    const int p = blockIdx.z, z = blockIdx.y, y0 = blockIdx.x * ROWS;
-    const int rows = min(ROWS, g.ny - y0);
-    const int nx = g.nx;
-    const C* __restrict__ tw = g.t2x;  // pass-1 twiddles of length 128
-    griddep_wait();
-    griddep_launch_dependents();
-    xfwd_gather(g, buf, kF128Buf, ROWS, p, z, y0, rows, tid, nthr);
-    __syncthreads();
-    for (int r = tid; r < 16 * ((L + 3) & ~3); r += nthr) {
-        int line, n2, par;
-        f128_role1(r, line, n2, par);
-        if (line >= L || line % ROWS >= rows) continue;
-        const C* b = buf + line * kF128Buf;
-        C u[8];
-#pragma unroll
-        for (int n1 = 0; n1 < 8; ++n1) u[n1] = 8 * n1 + n2 < nx ? b[fft_pad(8 * n1 + n2)] : C{T(0), T(0)};
-        f128_pass1<false>(u, u, n2, par, tw, zx + line * kF128Line);
-    }
-    __syncthreads();
-    // pass 2: role (c, j, yy), yy fastest; k1 = a permutation of j that puts a half-warp's 16 reads (rows
-    // yy, k1 spaced by ROWS) in distinct banks
-    const size_t kstride = (size_t)3 * g.nz * g.ny;  // between consecutive kx
-    C* outp = g.spec + (size_t)p * 128 * kstride + (size_t)z * g.ny + y0;
-    for (int r = tid; r < 16 * L; r += nthr) {
-        const int c = r / (16 * ROWS), rem = r % (16 * ROWS);
-        const int j = rem / ROWS, yy = rem % ROWS;
-        if (yy >= rows) continue;
-        const int k1 = (j % NQ) * ROWS + j / NQ;
-        C v[8];
-        f128_pass2(v, zx + (c * ROWS + yy) * kF128Line, k1);
-        C* o = outp + (size_t)k1 * kstride + (size_t)c * g.nz * g.ny + yy;
-#pragma unroll
-        for (int k2 = 0; k2 < 8; ++k2) o[(size_t)16 * k2 * kstride] = v[k2];
     }
 }
 
@@ -566,10 +526,10 @@ __device__ __forceinline__ T step_site(const T* s0, const T* hf, T dt, T* un) {
 // Step modes (0, 3, 4 of xinv_sites), FP32, even nx: two adjacent sites (x even, x + 1) per thread and
 // pass, so the spin planes move as float2 (one load serves both sites' y and z neighbours, and the inner
 // x neighbours come from the pair itself).  eacc[h] accumulates the energy terms of image 2p + h.
-template <int MODE>
+template <int MODE, typename Pos>
 __device__ __forceinline__ void xinv_sites_step2(const GroupArgs<float>& g, float dt, float* hout, const float2* buf,
-                                                 int ls, int p, int z, int y0, int rows, int tid, int nthr,
-                                                 const int (&climbs)[2], float (&eacc)[2]) {
+                                                 int ls, int lrows, int p, int z, int y0, int rows, int tid, int nthr,
+                                                 const int (&climbs)[2], float (&eacc)[2], Pos pos) {
     const int nx = g.nx, ny = g.ny, nz = g.nz, N = g.N, hx = nx >> 1;
     const int ia = 2 * p;
     const float2 zero = make_float2(0.f, 0.f);
@@ -611,7 +571,7 @@ __device__ __forceinline__ void xinv_sites_step2(const GroupArgs<float>& g, floa
                 d[c] = k ? ym[c].y : ym[c].x;
                 e[c] = k ? zp[c].y : zp[c].x;
                 f[c] = k ? zm[c].y : zm[c].x;
-                const float2 v = buf[(c * rows + yy) * ls + fft_pad(x + k)];
+                const float2 v = buf[(c * lrows + yy) * ls + pos(x + k)];
                 conv[c] = h == 0 ? v.x : -v.y;  // conjugate of the forward transform of the conjugate
             }
             local_field(pr, s0, a, b, cc, d, e, f, conv, hf);
@@ -643,16 +603,16 @@ __device__ __forceinline__ void xinv_sites_step2(const GroupArgs<float>& g, floa
 
 // ------------------------------------------------------------------------------------------------
 // Per-site work of the x-inverse kernels on rows [y0, y0+rows) of layer z, pair p; buf holds the
-// forward transforms of the conjugated field spectra (line c*rows + yy, fft_pad positions) when
+// forward transforms of the conjugated field spectra (line c*lrows + yy, x at pos(x)) when
 // HAS_CONV.  MODE 0: projected Euler step into sp and energy partials.  MODE 1: FP64 energy terms (and
 // the field into hout when given).  MODE 3: MODE 0, except that the image flagged in g.climb_img writes
 // its force F = h - (s.h) s into hout instead of stepping (the climbing-image kernels step it).
 // MODE 2 (a Runge-Kutta stage): the force F = h - (s.h) s of Eq. 13
 // into hout, s as stored (not renormalised); energy partials only when dt != 0.  MODES 4 and 5: as 0 and 2
 // with the right-hand side of Eq. 9 (precession and damping, prefactors g.llg_a and g.llg_b).
-template <typename T, bool HAS_CONV, int MODE>
-__device__ __forceinline__ void xinv_sites(const GroupArgs<T>& g, T dt, T* hout, const cplx<T>* buf, int ls,
-                                           double* red, int p, int z, int y0, int rows, int tid, int nthr) {
+template <typename T, bool HAS_CONV, int MODE, typename Pos>
+__device__ __forceinline__ void xinv_sites(const GroupArgs<T>& g, T dt, T* hout, const cplx<T>* buf, int ls, int lrows,
+                                           double* red, int p, int z, int y0, int rows, int tid, int nthr, Pos pos) {
     using C = cplx<T>;
     const int nx = g.nx, ny = g.ny, nz = g.nz, N = g.N;
     const int ia = 2 * p;
@@ -671,7 +631,7 @@ __device__ __forceinline__ void xinv_sites(const GroupArgs<T>& g, T dt, T* hout,
     }
     if constexpr ((MODE == 0 || MODE == 3 || MODE == 4) && HAS_CONV && std::is_same<T, float>::value) {
         if ((nx & 1) == 0) {  // uniform over the grid
-            xinv_sites_step2<MODE>(g, dt, hout, buf, ls, p, z, y0, rows, tid, nthr, climbs, eacc);
+            xinv_sites_step2<MODE>(g, dt, hout, buf, ls, lrows, p, z, y0, rows, tid, nthr, climbs, eacc, pos);
             done = true;
         }
     }
@@ -704,7 +664,7 @@ __device__ __forceinline__ void xinv_sites(const GroupArgs<T>& g, T dt, T* hout,
         if (HAS_CONV) {
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                const C v = buf[(c * rows + yy) * ls + fft_pad(x)];
+                const C v = buf[(c * lrows + yy) * ls + pos(x)];
                 conv[c] = h == 0 ? v.x : -v.y;  // conjugate of the forward transform of the conjugate
             }
         } else if (g.hdir) {  // direct dipole sums
@@ -870,58 +830,7 @@ __global__ void __launch_bounds__(kMaxThreadsX, kMinBlocksX) xinv_kernel(GroupAr
         __syncthreads();
         fft_lines(buf, tw, g.planx, g.lsx, 3 * rows, tid, nthr);
     }
-    xinv_sites<T, DO_FFT, MODE>(g, dt, hout, buf, g.lsx, red, p, z, y0, rows, tid, nthr);
-}
-
-// xinv for Px = 128 (nx <= 64), ROWS (2, 4 or 8) rows per CTA: the inverse x-transform (a forward
-// transform of the conjugate) of the 3*ROWS lines in two register passes, inputs read straight from the
-// spectrum (rows fastest across a warp), outputs x < 64 into buf; then the same per-site work as
-// xinv_kernel.  Rows past ny (last CTA) are skipped.
-template <typename T, int MODE, int ROWS>
-__global__ void __launch_bounds__(kMaxThreads128, kMinBlocks128) xinv128_kernel(GroupArgs<T> g, T dt, T* hout) {
-    using C = cplx<T>;
-    static_assert(16 % ROWS == 0 && ROWS >= 2, "the pass-1 role permutation needs ROWS in {2, 4, 8, 16}");
-    constexpr int L = 3 * ROWS, NQ = 16 / ROWS;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* buf = reinterpret_cast<C*>(smem_raw);  // L lines of kF128Buf, fft_pad positions
-    C* zx = buf + L * kF128Buf;                // exchange buffer
-    double* red = reinterpret_cast<double*>(zx + (L + 3) / 4 * 4 * kF128Line);
-    const int tid = threadIdx.x, nthr = blockDim.x;
-    const int p = blockIdx.z, z = blockIdx.y, y0 = blockIdx.x * ROWS;
-    const int rows = min(ROWS, g.ny - y0);
-    const size_t kstride = (size_t)3 * g.nz * g.ny;  // between consecutive kx
-    const C* inp = g.spec + (size_t)p * 128 * kstride + (size_t)z * g.ny + y0;
-    const C* __restrict__ tw = g.t2x;  // pass-1 twiddles of length 128
-    griddep_wait();
-    griddep_launch_dependents();
-    // pass 1: role (c, par, j, yy), yy fastest, then j (n2 a permutation of j that puts a half-warp's
-    // stores in distinct banks), so par is uniform across a warp for ROWS >= 4
-    for (int r = tid; r < 16 * L; r += nthr) {
-        const int t = r / ROWS, yy = r % ROWS;
-        if (yy >= rows) continue;
-        const int j = t & 7, par = (t >> 3) & 1, c = t >> 4;
-        const int n2 = (j % NQ) * (8 / NQ) + j / NQ;
-        const C* s = inp + (size_t)n2 * kstride + (size_t)c * g.nz * g.ny + yy;  // kx = 8 n1 + n2
-        C u[8], hi[8];
-#pragma unroll
-        for (int n1 = 0; n1 < 8; ++n1) {
-            u[n1] = cconj(s[(size_t)8 * n1 * kstride]);
-            hi[n1] = cconj(s[(size_t)(8 * n1 + 64) * kstride]);
-        }
-        f128_pass1<true>(u, hi, n2, par, tw, zx + (c * ROWS + yy) * kF128Line);
-    }
-    __syncthreads();
-    for (int r = tid; r < 16 * L; r += nthr) {
-        const int k1 = r & 15, line = r >> 4;
-        if (line % ROWS >= rows) continue;
-        C v[8];
-        f128_pass2(v, zx + line * kF128Line, k1);
-        C* b = buf + (line / ROWS * rows + line % ROWS) * kF128Buf;  // xinv_sites reads line c*rows + yy
-#pragma unroll
-        for (int k2 = 0; k2 < 4; ++k2) b[fft_pad(k1 + 16 * k2)] = v[k2];
-    }
-    __syncthreads();
-    xinv_sites<T, true, MODE>(g, dt, hout, buf, kF128Buf, red, p, z, y0, rows, tid, nthr);
+    xinv_sites<T, DO_FFT, MODE>(g, dt, hout, buf, g.lsx, rows, red, p, z, y0, rows, tid, nthr, PadPos{});
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -2066,14 +1975,6 @@ template <typename T> void launch_xfwd(const GroupArgs<T>& g, bool do_fft, int n
             }
             return;
         }
-        if (f128_x(4, g.Px)) {
-            const dim3 blk(f128_x_threads(g.ty_a));
-            const size_t sm = f128_x_smem(g.ty_a);
-            if (g.ty_a == 2) launch_pdl(xfwd128_kernel<T, 2>, grid, blk, sm, st, g);
-            else if (g.ty_a == 4) launch_pdl(xfwd128_kernel<T, 4>, grid, blk, sm, st, g);
-            else launch_pdl(xfwd128_kernel<T, 8>, grid, blk, sm, st, g);  // rows per CTA are 2, 4 or 8
-            return;
-        }
     }
     launch_pdl(xfwd_kernel<T, true>, grid, dim3(nthr), smem, st, g);
 }
@@ -2112,14 +2013,6 @@ void launch_xinv_step(const GroupArgs<T>& g, bool do_fft, T dt, int nthr, size_t
     }
     if constexpr (std::is_same<T, float>::value) {
         if (launch_xinv2p<0>(g, dt, nullptr, true, st)) return;
-        if (f128_x(4, g.Px)) {
-            const dim3 blk(f128_x_threads(g.ty_c));
-            const size_t sm = f128_x_smem(g.ty_c);
-            if (g.ty_c == 2) launch_pdl(xinv128_kernel<T, 0, 2>, grid, blk, sm, st, g, dt, (T*)nullptr);
-            else if (g.ty_c == 4) launch_pdl(xinv128_kernel<T, 0, 4>, grid, blk, sm, st, g, dt, (T*)nullptr);
-            else launch_pdl(xinv128_kernel<T, 0, 8>, grid, blk, sm, st, g, dt, (T*)nullptr);
-            return;
-        }
     }
     launch_pdl(xinv_kernel<T, true, 0>, grid, dim3(nthr), smem, st, g, dt, (T*)nullptr);
 }
@@ -2129,14 +2022,6 @@ void launch_xinv_eval(const GroupArgs<T>& g, bool do_fft, T* hout, int nthr, siz
     dim3 grid((g.ny + g.ty_c - 1) / g.ty_c, g.nz, g.n_pairs);
     if constexpr (std::is_same<T, float>::value) {
         if (do_fft && launch_xinv2p<1>(g, T(0), hout, false, st)) return;
-        if (do_fft && f128_x(4, g.Px)) {
-            const int nt = f128_x_threads(g.ty_c);
-            const size_t sm = f128_x_smem(g.ty_c);
-            if (g.ty_c == 2) xinv128_kernel<T, 1, 2><<<grid, nt, sm, st>>>(g, T(0), hout);
-            else if (g.ty_c == 4) xinv128_kernel<T, 1, 4><<<grid, nt, sm, st>>>(g, T(0), hout);
-            else xinv128_kernel<T, 1, 8><<<grid, nt, sm, st>>>(g, T(0), hout);
-            return;
-        }
     }
     if (do_fft) {
         xinv_kernel<T, true, 1><<<grid, nthr, smem, st>>>(g, T(0), hout);
@@ -2151,14 +2036,6 @@ static void launch_xinv_force_mode(const GroupArgs<T>& g, bool do_fft, T* kout, 
     dim3 grid((g.ny + g.ty_c - 1) / g.ty_c, g.nz, g.n_pairs);
     if constexpr (std::is_same<T, float>::value) {
         if (do_fft && launch_xinv2p<MODE>(g, flag, kout, false, st)) return;
-        if (do_fft && f128_x(4, g.Px)) {
-            const int nt = f128_x_threads(g.ty_c);
-            const size_t sm = f128_x_smem(g.ty_c);
-            if (g.ty_c == 2) xinv128_kernel<T, MODE, 2><<<grid, nt, sm, st>>>(g, flag, kout);
-            else if (g.ty_c == 4) xinv128_kernel<T, MODE, 4><<<grid, nt, sm, st>>>(g, flag, kout);
-            else xinv128_kernel<T, MODE, 8><<<grid, nt, sm, st>>>(g, flag, kout);
-            return;
-        }
     }
     if (do_fft)
         xinv_kernel<T, true, MODE><<<grid, nthr, smem, st>>>(g, flag, kout);
@@ -2181,14 +2058,6 @@ void launch_xinv_step_llg(const GroupArgs<T>& g, bool do_fft, T dt, int nthr, si
     dim3 grid((g.ny + g.ty_c - 1) / g.ty_c, g.nz, g.n_pairs);
     if constexpr (std::is_same<T, float>::value) {
         if (do_fft && launch_xinv2p<4>(g, dt, nullptr, true, st)) return;
-        if (do_fft && f128_x(4, g.Px)) {
-            const dim3 blk(f128_x_threads(g.ty_c));
-            const size_t sm = f128_x_smem(g.ty_c);
-            if (g.ty_c == 2) launch_pdl(xinv128_kernel<T, 4, 2>, grid, blk, sm, st, g, dt, (T*)nullptr);
-            else if (g.ty_c == 4) launch_pdl(xinv128_kernel<T, 4, 4>, grid, blk, sm, st, g, dt, (T*)nullptr);
-            else launch_pdl(xinv128_kernel<T, 4, 8>, grid, blk, sm, st, g, dt, (T*)nullptr);
-            return;
-        }
     }
     if (do_fft)
         launch_pdl(xinv_kernel<T, true, 4>, grid, dim3(nthr), smem, st, g, dt, (T*)nullptr);
@@ -2201,14 +2070,6 @@ void launch_xinv_step_climb(const GroupArgs<T>& g, bool do_fft, T dt, T* hc, int
     dim3 grid((g.ny + g.ty_c - 1) / g.ty_c, g.nz, g.n_pairs);
     if constexpr (std::is_same<T, float>::value) {
         if (do_fft && launch_xinv2p<3>(g, dt, hc, true, st)) return;
-        if (do_fft && f128_x(4, g.Px)) {
-            const dim3 blk(f128_x_threads(g.ty_c));
-            const size_t sm = f128_x_smem(g.ty_c);
-            if (g.ty_c == 2) launch_pdl(xinv128_kernel<T, 3, 2>, grid, blk, sm, st, g, dt, hc);
-            else if (g.ty_c == 4) launch_pdl(xinv128_kernel<T, 3, 4>, grid, blk, sm, st, g, dt, hc);
-            else launch_pdl(xinv128_kernel<T, 3, 8>, grid, blk, sm, st, g, dt, hc);
-            return;
-        }
     }
     if (do_fft)
         launch_pdl(xinv_kernel<T, true, 3>, grid, dim3(nthr), smem, st, g, dt, hc);
@@ -2306,12 +2167,22 @@ void launch_extract_octant(const double2* spec, T* dhat, int Px, int Py, int nz,
 }
 
 // Raises the dynamic shared-memory limit of every kernel that stages lines in shared memory to
-// `bytes` less the kernel's static shared memory (the two together may not exceed `bytes`).
-template <typename F> static inline void set_dyn_smem(F* kernel, int bytes) {
+// `bytes` less the kernel's static shared memory (the two together may not exceed `bytes`).  carve_kb > 0 also
+// asks for that split of the SM's 256 KB between shared memory and L1 (the sizes are 100, 132, 164, 196 and
+// 228 KB; the percentage is rounded down so that the next size up is not taken).
+template <typename F> static inline void set_dyn_smem(F* kernel, int bytes, int carve_kb = 0) {
     cudaFuncAttributes fa{};
     if (cudaFuncGetAttributes(&fa, kernel) != cudaSuccess) return;
     cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes - (int)fa.sharedSizeBytes);
+    if (carve_kb) cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, carve_kb * 100 / 228);
 }
+// One split for every kernel of an iteration (two-pass kernels of up to 384 points, arc, climbing image,
+// spline): an SM changes its split only when it is empty, and with programmatic dependent launch and graph
+// branches it never is, so a kernel that starts on SMs split for another one keeps that split -- the y/z kernel
+// of 384 points ran with one resident CTA behind an x kernel that had asked for less shared memory.  164 KB
+// hold two y/z CTAs of 384 points or three of 256 and leave 92 KB of L1 to the stencil.  The 20-string study on
+// one GB300: 4078 us per iteration with each kernel's own split, 3526 with this one.
+constexpr int kCarveKb = 164;
 template <typename T> void set_smem_limits(int bytes) {
     set_dyn_smem(xfwd_kernel<T, true>, bytes);
     set_dyn_smem(yz_kernel<T, 0>, bytes);
@@ -2327,19 +2198,11 @@ template <typename T> void set_smem_limits(int bytes) {
     set_dyn_smem(xinv_kernel<T, false, 4>, bytes);
     set_dyn_smem(xinv_kernel<T, true, 5>, bytes);
     set_dyn_smem(xinv_kernel<T, false, 5>, bytes);
-    set_dyn_smem(spline_apply_kernel<T>, 200 * 1024);
-    set_dyn_smem(arc_kernel<T>, bytes);
+    set_dyn_smem(spline_apply_kernel<T>, 200 * 1024, kCarveKb);
+    set_dyn_smem(arc_kernel<T>, bytes, kCarveKb);
+    set_dyn_smem(climb_dot_kernel<T>, bytes, kCarveKb);
+    set_dyn_smem(climb_apply_kernel<T>, bytes, kCarveKb);
     if constexpr (std::is_same<T, float>::value) {
-#define SS_CASE(R)                                  \
-    set_dyn_smem(xfwd128_kernel<T, R>, bytes);      \
-    set_dyn_smem(xinv128_kernel<T, 0, R>, bytes);   \
-    set_dyn_smem(xinv128_kernel<T, 1, R>, bytes);   \
-    set_dyn_smem(xinv128_kernel<T, 2, R>, bytes);   \
-    set_dyn_smem(xinv128_kernel<T, 3, R>, bytes);   \
-    set_dyn_smem(xinv128_kernel<T, 4, R>, bytes);   \
-    set_dyn_smem(xinv128_kernel<T, 5, R>, bytes);
-        SS_CASE(2) SS_CASE(4) SS_CASE(8)
-#undef SS_CASE
 #define SS_CASE(Z) set_dyn_smem(yz_kernel<T, Z>, bytes);
         SS_FOR_NZ(SS_CASE)
 #undef SS_CASE

@@ -171,7 +171,7 @@ extern "C" ss_status ss_field_noalloc(int nx, int ny, int nz, double J, double D
             break;
         }
     }
-    if (dip && f128_x(4, Px)) ty = f128_x_rows(ty);  // the length-128 x kernels take 2, 4 or 8 rows
+    if (dip && Px == 128 && ty != 2 && ty != 4) ty = 8;
     if (dip && (Px == 192 || Px == 256 || Px == 384)) ty = kX2Rows;
     const size_t smem_a = (size_t)(Px + 3 * ty * lsx) * sizeof(float2);
     const size_t smem_c = smem_a + 32 * 2 * kEvalTerms * sizeof(double);

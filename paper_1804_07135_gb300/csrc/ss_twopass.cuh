@@ -11,7 +11,7 @@ namespace ss {
 // 17-strided row layout, the z-convolution in place between them.  One shared line per (column, component,
 // layer): 3 NZ KXB lines of t2_line(P) complex elements, read from the spectrum in pass 1 and written back
 // (rows y < ny) in pass B; one shared-memory round trip per pass instead of one per Stockham stage.
-// Pass 2 and pass A take one warp per line (16 columns x 2 parities), or half a warp (odd P/16).
+// Pass 2 and pass A take half a warp per line (16 columns; a warp with two roles per column from P = 448 on).
 //
 // The z-convolution works on sums and differences of mirrored layers.  A component of the tensor is even
 // in z (t) or odd (G), so with n = NZ, e_i = s_i + s_{n-1-i}, o_i = s_i - s_{n-1-i} (i < n/2; the middle layer
@@ -25,8 +25,7 @@ namespace ss {
 // three times; the transforms are linear, so e and o are formed when pass 1 reads the layers and undone
 // when pass B writes them.  Kernel times on one GB300 before and after: 192x192x8 x 128 images 1420 -> 1214 us,
 // 128x128x8 x 192 788 -> 703, 128x128x4 x 384 733 -> 610, 100x100x5 x 32 79 -> 67, 112x112x1 x 60 (xz = yz = 0
-// left out) 40.5 -> 28.6.  What bounds it now (ncu, 192x192x8): no pipe (L1/shared 66%, FMA 45%, issue 54%);
-// 24 warps per SM wait for barriers and shared memory.
+// left out) 40.5 -> 28.6; with roles of whole columns and rows and small CTAs 928, 561, 481, 54 and 22.3.
 template <int NZ, int PAR> struct ZSys {  // PAR 0: (x, y in e; z in o), 1: (x, y in o; z in e)
     static constexpr int ME = (NZ + 1) / 2, MO = NZ / 2;
     static constexpr int NXY = PAR == 0 ? ME : MO, NZC = PAR == 0 ? MO : ME;  // elements of x (and y), and of z
@@ -176,13 +175,13 @@ __device__ __forceinline__ void zconv_t2(float2* A, int kx, int Px, const float*
 }
 
 template <int P, int NZ, int KXB>
-__global__ void __launch_bounds__(yz2p_threads(P, NZ), yz2p_blocks(P, NZ)) yz2p_kernel(GroupArgs<float> g) {
+__global__ void __launch_bounds__(yz2p_threads(P), yz2p_blocks(P)) yz2p_kernel(GroupArgs<float> g) {
     using C = float2;
     constexpr int R2 = P / 16, LS = t2_line(P), L = 3 * NZ * KXB, RC = 16 * T2<P>::NP;  // RC: roles per line
     constexpr int ME = (NZ + 1) / 2, MO = NZ / 2, LP = 3 * ME * KXB;                    // LP: pairs of mirrored layers
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* A = reinterpret_cast<C*>(smem_raw);  // line (b * 3 + c) * NZ + q: e_q for q < ME, o_{q - ME} above
-    const int tid = threadIdx.x, nthr = yz2p_threads(P, NZ);
+    const int tid = threadIdx.x, nthr = yz2p_threads(P);
     const int kx = blockIdx.x * KXB, p = blockIdx.y;
     const int ny = g.ny;
     C* blk = g.spec + ((size_t)p * g.Px + kx) * 3 * NZ * ny;  // KXB consecutive columns are contiguous
@@ -191,11 +190,10 @@ __global__ void __launch_bounds__(yz2p_threads(P, NZ), yz2p_blocks(P, NZ)) yz2p_
     const C* __restrict__ ta = g.t2y + P;                     // pass A
     griddep_wait();
     griddep_launch_dependents();
-    // pass 1, role (n2, mirrored pair of lines, par), n2 fastest: the zero-padded spectrum lines in, rows of
-    // Z of their sum and difference out
-    for (int r = tid; r < 2 * R2 * LP; r += nthr) {
-        const int n2 = r % R2, q = r / R2, lp = q % LP, par = q / LP;
-        const int bc = lp / ME, i = lp % ME;
+    // pass 1, role (n2, mirrored pair of lines), n2 fastest: the zero-padded spectrum lines in, rows of Z of
+    // their sum and difference out
+    for (int r = tid; r < R2 * LP; r += nthr) {
+        const int n2 = r % R2, lp = r / R2, bc = lp / ME, i = lp % ME;
         const C* src = blk + (size_t)(bc * NZ + i) * ny + n2;
         C u[8];
         if (MO == ME || i < MO) {
@@ -213,15 +211,15 @@ __global__ void __launch_bounds__(yz2p_threads(P, NZ), yz2p_blocks(P, NZ)) yz2p_
                 u[j] = cadd(a, v[j]);
                 v[j] = csub(a, v[j]);
             }
-            t2_pass1<P>(v, n2, par, t1, A + (bc * NZ + ME + i) * LS);
+            t2_pass1<P>(v, n2, t1, A + (bc * NZ + ME + i) * LS);
         } else {
 #pragma unroll
             for (int j = 0; j < 8; ++j) u[j] = R2 * j + n2 < ny ? src[R2 * j] : make_float2(0.f, 0.f);
         }
-        t2_pass1<P>(u, n2, par, t1, A + (bc * NZ + i) * LS);
+        t2_pass1<P>(u, n2, t1, A + (bc * NZ + i) * LS);
     }
     __syncthreads();
-    // pass 2: one warp per line (lanes = 16 columns x 2 parities; half a warp for odd P/16)
+    // pass 2: half a warp per line (lanes = 16 columns; a warp where a column takes two roles)
     for (int r = tid; r < RC * L; r += nthr) t2_cols<P, false>(A + r / RC * LS, r & 15, r % RC / 16, tw, ta);
     __syncthreads();
 #pragma unroll 1
@@ -233,20 +231,19 @@ __global__ void __launch_bounds__(yz2p_threads(P, NZ), yz2p_blocks(P, NZ)) yz2p_
     // pass A (the inverse transform of the conjugated field spectra, in place by columns)
     for (int r = tid; r < RC * L; r += nthr) t2_cols<P, true>(A + r / RC * LS, r & 15, r % RC / 16, tw, ta);
     __syncthreads();
-    // pass B, role (y2, mirrored pair of lines, par): rows y < ny of both layers back to the spectrum, conjugated
-    for (int r = tid; r < 2 * R2 * LP; r += nthr) {
-        const int y2 = r % R2, q = r / R2, lp = q % LP, par = q / LP;
-        const int bc = lp / ME, i = lp % ME;
+    // pass B, role (y2, mirrored pair of lines): rows y < ny of both layers back to the spectrum, conjugated
+    for (int r = tid; r < R2 * LP; r += nthr) {
+        const int y2 = r % R2, lp = r / R2, bc = lp / ME, i = lp % ME;
         C v[8];
-        t2_passB(v, A + (bc * NZ + i) * LS, y2, par);
+        t2_passB(v, A + (bc * NZ + i) * LS, y2);
         C* dst = blk + (size_t)(bc * NZ + i) * ny;
         if (MO == ME || i < MO) {
             C w[8];
-            t2_passB(w, A + (bc * NZ + ME + i) * LS, y2, par);
+            t2_passB(w, A + (bc * NZ + ME + i) * LS, y2);
             C* dst2 = blk + (size_t)(bc * NZ + NZ - 1 - i) * ny;
 #pragma unroll
-            for (int m = 0; m < 4; ++m) {
-                const int y = y2 + R2 * (2 * m + par);
+            for (int m = 0; m < 8; ++m) {
+                const int y = y2 + R2 * m;
                 if (y < ny) {
                     dst[y] = cconj(cadd(v[m], w[m]));
                     dst2[y] = cconj(csub(v[m], w[m]));
@@ -254,10 +251,8 @@ __global__ void __launch_bounds__(yz2p_threads(P, NZ), yz2p_blocks(P, NZ)) yz2p_
             }
         } else {
 #pragma unroll
-            for (int m = 0; m < 4; ++m) {
-                const int y = y2 + R2 * (2 * m + par);
-                if (y < ny) dst[y] = cconj(v[m]);
-            }
+            for (int m = 0; m < 8; ++m)
+                if (y2 + R2 * m < ny) dst[y2 + R2 * m] = cconj(v[m]);
         }
     }
 }
@@ -268,18 +263,18 @@ __global__ void __launch_bounds__(yz2p_threads(P, NZ), yz2p_blocks(P, NZ)) yz2p_
 // fastest across a warp: the spectrum's rows of one (kx, c) are contiguous in global memory, and with
 // line strides = 16 / kX2Rows (mod 16) the lanes of a half-warp (kX2Rows rows x 16 / kX2Rows consecutive
 // columns or rows of a line) hit distinct shared-memory banks.
-// xfwd: the gather (Eq. 12) into x-space lines, pass 1 into the transform lines, pass 2 straight to the
-// spectrum spec[p][kx][c][z][y].
-// Resident CTAs the x kernels are compiled for: about 1100 threads per SM, less where their lines take more
-// shared memory (78 KB at P = 512).
-constexpr int x2_blocks(int P) { return P >= 512 ? 2 : 1152 / x2_threads(P); }
+// x sits at row x mod R2, column x / R2 of its line, which is where pass 1 reads its role's inputs and pass B
+// leaves its outputs: both work in place, and the space of separate x-space lines stays with the L1 cache
+// that serves the stencil's neighbours.  Roles of whole columns and rows and lines in place: x-forward and
+// step kernel of 128x128x4 x 384 images 298 -> 253 us and 438 -> 311, of 192x192x8 x 128 437 -> 441 and
+// 662 -> 540, of 64x64x8 x 32 17.0 -> 16.4 and 22.5 -> 18.4 (one GB300).  They are bound by load latency and L1.
+// xfwd: the gather (Eq. 12), pass 1 in place, pass 2 straight to the spectrum spec[p][kx][c][z][y].
 template <int P>
 __global__ void __launch_bounds__(x2_threads(P), x2_blocks(P)) xfwd2p_kernel(GroupArgs<float> g) {
     using C = float2;
-    constexpr int R2 = P / 16, H = T2<P>::H, NP = T2<P>::NP, ROWS = kX2Rows, L = 3 * ROWS, LSX = x2_lsx(P), LB = x2_lb(P);
+    constexpr int R2 = P / 16, H = T2<P>::H, NP = T2<P>::NP, ROWS = kX2Rows, L = 3 * ROWS, LSX = x2_lsx(P);
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* xb = reinterpret_cast<C*>(smem_raw);  // line c * ROWS + yy: the pair at x, fft_pad positions
-    C* A = xb + L * LB;                       // line c * ROWS + yy: rows of Z
+    C* A = reinterpret_cast<C*>(smem_raw);  // line c * ROWS + yy: the pair at x, then rows of Z
     const int tid = threadIdx.x, nthr = blockDim.x;
     const int p = blockIdx.z, z = blockIdx.y, y0 = blockIdx.x * ROWS;
     const int rows = min(ROWS, g.ny - y0), nx = g.nx;
@@ -287,17 +282,17 @@ __global__ void __launch_bounds__(x2_threads(P), x2_blocks(P)) xfwd2p_kernel(Gro
     const C* __restrict__ t1 = g.t2x;  // pass 1
     griddep_wait();
     griddep_launch_dependents();
-    xfwd_gather(g, xb, LB, ROWS, p, z, y0, rows, tid, nthr);
+    xfwd_gather(g, A, LSX, ROWS, p, z, y0, rows, tid, nthr, T2Pos<R2>{});
     __syncthreads();
-    // pass 1, role (yy, n2, c, par)
-    for (int r = tid; r < 2 * R2 * L; r += nthr) {
-        const int yy = r % ROWS, q = r / ROWS, n2 = q % R2, q2 = q / R2, c = q2 % 3, par = q2 / 3;
+    // pass 1, role (yy, n2, c)
+    for (int r = tid; r < R2 * L; r += nthr) {
+        const int yy = r % ROWS, q = r / ROWS, n2 = q % R2, c = q / R2;
         if (yy >= rows) continue;
-        const C* b = xb + (c * ROWS + yy) * LB;
+        C* line = A + (c * ROWS + yy) * LSX;
         C u[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) u[j] = R2 * j + n2 < nx ? b[fft_pad(R2 * j + n2)] : make_float2(0.f, 0.f);
-        t2_pass1<P>(u, n2, par, t1, A + (c * ROWS + yy) * LSX);
+        for (int j = 0; j < 8; ++j) u[j] = R2 * j + n2 < nx ? line[t2_at(n2, j)] : make_float2(0.f, 0.f);
+        t2_pass1<P>(u, n2, t1, line);
     }
     __syncthreads();
     // pass 2, role (yy, k1, par2, c): X[k1 + 16 (NP m + par2)] to the spectrum
@@ -315,19 +310,18 @@ __global__ void __launch_bounds__(x2_threads(P), x2_blocks(P)) xfwd2p_kernel(Gro
     }
 }
 
-// xinv: pass A straight from the spectrum (conjugated) into the transform lines, pass B into x-space
-// lines (fft_pad positions, line c * rows + yy), then the per-site work of xinv_sites in mode MODE.
+// xinv: pass A straight from the spectrum (conjugated), pass B in place, then the per-site work of xinv_sites
+// in mode MODE.
 template <int P, int MODE>
 __global__ void __launch_bounds__(x2_threads(P), x2_blocks(P)) xinv2p_kernel(GroupArgs<float> g, float dt, float* hout) {
     using C = float2;
-    constexpr int R2 = P / 16, H = T2<P>::H, NP = T2<P>::NP, ROWS = kX2Rows, L = 3 * ROWS, LSX = x2_lsx(P), LB = x2_lb(P);
+    constexpr int R2 = P / 16, H = T2<P>::H, NP = T2<P>::NP, ROWS = kX2Rows, L = 3 * ROWS, LSX = x2_lsx(P);
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* A = reinterpret_cast<C*>(smem_raw);  // line c * ROWS + yy: columns of T
-    C* xb = A + L * LSX;                     // line c * rows + yy: the field convolution at x
-    double* red = reinterpret_cast<double*>(xb + L * LB);
+    C* A = reinterpret_cast<C*>(smem_raw);  // line c * ROWS + yy: columns of T, then the field convolution at x
+    double* red = reinterpret_cast<double*>(A + L * LSX);
     const int tid = threadIdx.x, nthr = blockDim.x;
     const int p = blockIdx.z, z = blockIdx.y, y0 = blockIdx.x * ROWS;
-    const int rows = min(ROWS, g.ny - y0), nx = g.nx;
+    const int rows = min(ROWS, g.ny - y0);
     const size_t kstride = (size_t)3 * g.nz * g.ny;
     const C* inp = g.spec + (size_t)p * P * kstride + (size_t)z * g.ny + y0;
     const C* __restrict__ tw = g.twx;
@@ -346,32 +340,31 @@ __global__ void __launch_bounds__(x2_threads(P), x2_blocks(P)) xinv2p_kernel(Gro
         for (int m = 0; m < H; ++m) o[NP * m * kT2Row] = a[m];
     }
     __syncthreads();
-    // pass B, role (yy, y2, c, par): x = y2 + R2 (2m + par) < nx
-    for (int r = tid; r < 2 * R2 * L; r += nthr) {
-        const int yy = r % ROWS, q = r / ROWS, y2 = q % R2, q2 = q / R2, c = q2 % 3, par = q2 / 3;
+    // pass B, role (yy, y2, c): x = y2 + R2 m at (y2, m)
+    for (int r = tid; r < R2 * L; r += nthr) {
+        const int yy = r % ROWS, q = r / ROWS, y2 = q % R2, c = q / R2;
         if (yy >= rows) continue;
+        C* line = A + (c * ROWS + yy) * LSX;
         C v[8];
-        t2_passB(v, A + (c * ROWS + yy) * LSX, y2, par);
-        C* b = xb + (c * rows + yy) * LB;
+        t2_passB(v, line, y2);
 #pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            const int x = y2 + R2 * (2 * m + par);
-            if (x < nx) b[fft_pad(x)] = v[m];
-        }
+        for (int m = 0; m < 8; ++m) line[t2_at(y2, m)] = v[m];
     }
     __syncthreads();
-    xinv_sites<float, true, MODE>(g, dt, hout, xb, LB, red, p, z, y0, rows, tid, nthr);
+    xinv_sites<float, true, MODE>(g, dt, hout, A, LSX, ROWS, red, p, z, y0, rows, tid, nthr, T2Pos<R2>{});
 }
 
 // ---- launchers of one length --------------------------------------------------------------------------
 template <typename T, int P> void t2_xfwd(const GroupArgs<T>& g, cudaStream_t st) {
     const dim3 grid((g.ny + g.ty_a - 1) / g.ty_a, g.nz, g.n_pairs);  // ty_a = kX2Rows (set by the host)
-    launch_pdl(xfwd2p_kernel<P>, grid, dim3(x2_threads(P)), x2_smem(P, false), st, g);
+    const int thr = x2_launch_threads(P, g.nx, (long)grid.x * grid.y * grid.z);
+    launch_pdl(xfwd2p_kernel<P>, grid, dim3(thr), x2_smem(P, false), st, g);
 }
 
 template <typename T, int P>
 void t2_xinv(const GroupArgs<T>& g, int mode, T dt, T* hout, bool pdl, cudaStream_t st) {
-    const dim3 grid((g.ny + g.ty_c - 1) / g.ty_c, g.nz, g.n_pairs), blk(x2_threads(P));
+    const dim3 grid((g.ny + g.ty_c - 1) / g.ty_c, g.nz, g.n_pairs);
+    const dim3 blk(x2_launch_threads(P, g.nx, (long)grid.x * grid.y * grid.z));
     const size_t sm = x2_smem(P, true);
     switch (mode) {
 #define SS_CASE(M) \
@@ -389,17 +382,18 @@ template <typename T, int P> void t2_yz(const GroupArgs<T>& g, cudaStream_t st) 
     const size_t sm = yz2p_smem(P, g.nz, kxb);
     const dim3 grid(g.Px / kxb, g.n_pairs);
 #define SS_CASE(Z, B) \
-    if (g.nz == Z && kxb == B) launch_pdl(yz2p_kernel<P, Z, B>, grid, dim3(yz2p_threads(P, Z)), sm, st, g);
+    if (g.nz == Z && kxb == B) launch_pdl(yz2p_kernel<P, Z, B>, grid, dim3(yz2p_threads(P)), sm, st, g);
     SS_T2_YZ(SS_CASE)
 #undef SS_CASE
 }
 
 template <typename T, int P> void t2_smem_limits(int bytes) {
-    set_dyn_smem(xfwd2p_kernel<P>, bytes);
-#define SS_CASE(M) set_dyn_smem(xinv2p_kernel<P, M>, bytes);
+    constexpr int carve = P <= 384 ? kCarveKb : P <= 448 ? 196 : 228;  // two y/z CTAs
+    set_dyn_smem(xfwd2p_kernel<P>, bytes, carve);
+#define SS_CASE(M) set_dyn_smem(xinv2p_kernel<P, M>, bytes, carve);
     SS_CASE(0) SS_CASE(1) SS_CASE(2) SS_CASE(3) SS_CASE(4) SS_CASE(5)
 #undef SS_CASE
-#define SS_CASE(Z, B) set_dyn_smem(yz2p_kernel<P, Z, B>, bytes);
+#define SS_CASE(Z, B) set_dyn_smem(yz2p_kernel<P, Z, B>, bytes, carve);
     SS_T2_YZ(SS_CASE)
 #undef SS_CASE
 }
