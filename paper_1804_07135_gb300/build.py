@@ -1,7 +1,7 @@
 """Builds libss.so (the C-ABI library) in-tree for sm_103a with nvcc.
 
-The translation units (FP32 kernels, FP64 kernels, host runtime, one unit per length of the two-pass
-transforms) compile in parallel and link into ``paper_1804_07135_gb300/libss.so`` against the shared CUDA runtime.
+The translation units (FP32 kernels, FP64 kernels, host runtime, one unit per length and type of the
+two-pass transforms) compile in parallel and link into ``paper_1804_07135_gb300/libss.so`` against the shared CUDA runtime.
 """
 from __future__ import annotations
 
@@ -72,7 +72,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         return obj
 
     units = [(src, {}) for src in SOURCES]
-    units += [("ss_twopass.cu", {"SS_T2_P": P}) for P in reversed(T2_LENGTHS)]  # the long ones first
+    units += [("ss_twopass.cu", {"SS_T2_P": P, "SS_T2_T": T}) for P in reversed(T2_LENGTHS) for T in ("double", "float")]
     with cf.ThreadPoolExecutor(min(len(units), os.cpu_count() or 8)) as ex:
         objs = list(ex.map(compile_one, units))
     tmp = LIB + f".tmp{os.getpid()}"

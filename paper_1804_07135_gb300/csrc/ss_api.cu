@@ -26,9 +26,9 @@ thread_local std::string g_create_error;
 
 // ---- small helpers --------------------------------------------------------------------------------
 // Padded transform length for n sites, enough for the linear (non-circular) convolution with offsets
-// -(n-1)..(n-1) (Sec. II-A, the zero-padded kernel): padded_smooth(n), except that an FP32 length without
-// two-pass kernels is exchanged for the next one that has them (two_pass: the kernels along this axis have a
-// two-pass form at all).  Lattices of up to 12 sites a side keep the short length: one CTA transforms all of
+// -(n-1)..(n-1) (Sec. II-A, the zero-padded kernel): padded_smooth(n), except that a length without two-pass
+// kernels is exchanged for the next one that has them (two_pass: the kernels along this axis have a two-pass
+// form at all).  Lattices of up to 12 sites a side keep the short length: one CTA transforms all of
 // their lines at once either way.
 int padded_len(int n, bool two_pass) {
     const int m = padded_smooth(n);
@@ -279,8 +279,8 @@ template <typename T> GroupArgs<T> group_args(const ss_ctx* c, const Group& g) {
 // they need.
 void set_rows(Group& g, int ty_a, int ty_c, int thr_a = 256, int thr_c = 256) {
     const size_t cs = 2 * (size_t)g.rbytes;
-    const bool x2 = g.dipole && x2p_ok(g.rbytes, g.Px);  // two-pass x kernels: fixed rows per CTA
-    if (x2) ty_a = ty_c = kX2Rows;
+    const bool x2 = g.dipole && t2_length(g.Px);  // two-pass x kernels: fixed rows per CTA
+    if (x2) ty_a = ty_c = x2_rows(g.rbytes);
     g.ty_a = ty_a;
     g.ty_c = ty_c;
     g.thr_a = thr_a;
@@ -288,9 +288,9 @@ void set_rows(Group& g, int ty_a, int ty_c, int thr_a = 256, int thr_c = 256) {
     g.smem_a = (size_t)(g.Px + 3 * g.ty_a * g.lsx) * cs;
     g.smem_c = (size_t)(g.Px + 3 * g.ty_c * g.lsx) * cs + 32 * 2 * kEvalTerms * sizeof(double);
     if (x2) {
-        g.thr_a = g.thr_c = x2_launch_threads(g.Px, g.nx, (long)((g.ny + kX2Rows - 1) / kX2Rows) * g.nz * g.n_pairs);
-        g.smem_a = x2_smem(g.Px, false);
-        g.smem_c = x2_smem(g.Px, true);
+        g.thr_a = g.thr_c = x2_launch_threads(g.rbytes, g.Px, g.nx, (long)((g.ny + ty_a - 1) / ty_a) * g.nz * g.n_pairs);
+        g.smem_a = x2_smem(g.rbytes, g.Px, false);
+        g.smem_c = x2_smem(g.rbytes, g.Px, true);
     }
     g.smem_c_eval = g.smem_c;
     g.n_eblk = g.nz * ((g.ny + g.ty_c - 1) / g.ty_c);
@@ -319,15 +319,15 @@ void configure_group(Group& g) {
     g.smem_b = (size_t)(g.Py + 3 * g.nz * g.lsy) * cs;
     const size_t slab = (size_t)(g.Py / 2 + 1) * g.nz * 6 * (size_t)g.rbytes;
     if (slab <= 24 * 1024) g.smem_b += slab;
-    if (g.dipole && yz2p_ok(g.rbytes, g.Py, g.nz, g.Px)) {
-        g.thr_b = yz2p_threads(g.Py);
-        g.smem_b = yz2p_smem(g.Py, g.nz, yz2p_kxb_use(g.nz, g.yz_kxb));
+    if (g.dipole && yz2p_ok(g.Py, g.nz, g.Px)) {
+        g.thr_b = yz2p_threads(g.rbytes, g.Py);
+        g.smem_b = yz2p_smem(g.rbytes, g.Py, g.nz, yz2p_kxb_use(g.rbytes, g.nz, g.yz_kxb));
     }
 }
 
 // The two-pass y/z kernel's shared memory for the group's column count (after the autotuner's choice).
 void configure_yz_smem(Group& g) {
-    if (g.dipole && yz2p_ok(g.rbytes, g.Py, g.nz, g.Px)) g.smem_b = yz2p_smem(g.Py, g.nz, yz2p_kxb_use(g.nz, g.yz_kxb));
+    if (g.dipole && yz2p_ok(g.Py, g.nz, g.Px)) g.smem_b = yz2p_smem(g.rbytes, g.Py, g.nz, yz2p_kxb_use(g.rbytes, g.nz, g.yz_kxb));
 }
 
 template <typename T> ss_status build_tensor_spectrum(ss_ctx* c, Group& g) {
@@ -359,7 +359,7 @@ template <typename T> ss_status build_tensor_spectrum(ss_ctx* c, Group& g) {
         // y: columns of length Py, stride Px
         launch_fft_strided_f64(d_data, d_twy, py, 6 * nz * Px, Px, Px, 1, (long)plane, c->cs);
         launch_extract_octant<T>(d_data, (T*)g.dhat, Px, Py, nz,
-                                 dhat_factor(g.rbytes, Py, nz, Px) * 4.0 * M_PI / ((double)Px * Py), c->cs);
+                                 dhat_factor(Py, nz, Px) * 4.0 * M_PI / ((double)Px * Py), c->cs);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->cs);
@@ -506,8 +506,8 @@ template <typename T> ss_status tune_group(ss_ctx* c, Group& g) {
     }
     const size_t cs = 2 * real_size(c);
     std::vector<std::pair<int, int>> cands;  // (threads, rows)
-    if (g.dipole && x2p_ok((int)real_size(c), g.Px)) {
-        cands.push_back({x2_threads(g.Px), kX2Rows});  // one shape: nothing to tune
+    if (g.dipole && t2_length(g.Px)) {
+        cands.push_back({g.thr_a, g.ty_a});  // one shape: nothing to tune
     } else {
         for (int thr : {256, 512})
             for (int ty : {1, 2, 4, 5, 8, 10, 16})
@@ -516,9 +516,10 @@ template <typename T> ss_status tune_group(ss_ctx* c, Group& g) {
                     cands.push_back({thr, ty});
     }
     std::vector<int> kxbs;  // y/z columns per CTA
-    if (g.dipole && yz2p_ok((int)real_size(c), g.Py, g.nz, g.Px) && yz2p_kxb_alt(g.nz) > 0 &&
-        g.Px % yz2p_kxb_alt(g.nz) == 0)
-        kxbs = {yz2p_kxb(g.nz), yz2p_kxb_alt(g.nz)};
+    if (g.dipole && yz2p_ok(g.Py, g.nz, g.Px)) {
+        const YzColumns k = yz2p_columns(g.nz);
+        kxbs.assign(k.v, k.v + k.n);
+    }
     if (cands.size() <= 1 && kxbs.size() <= 1) return SS_OK;
     cudaEvent_t e0, e1;
     CUDA_TRY(c, cudaEventCreate(&e0));
@@ -979,16 +980,16 @@ ss_status ensure_ev64(ss_ctx* c) {
         e.nz = g.nz;
         e.N = g.N;
         e.dipole = g.dipole;
-        e.Px = e.dipole ? padded_len(e.nx, false) : 1;
-        e.Py = e.dipole ? padded_len(e.ny, false) : 1;
+        e.Px = g.Px;
+        e.Py = g.Py;
         e.n_img = g.n_img;
         e.n_pairs = g.n_pairs;
         e.strs = g.strs;
         e.str_img0 = g.str_img0;
         e.str_K = g.str_K;
         e.direct = g.direct;
-        e.planx = make_plan(e.Px);
-        e.plany = make_plan(e.Py);
+        e.planx = g.planx;
+        e.plany = g.plany;
         configure_group(e);
         if (e.smem_a > 227 * 1024 || e.smem_b > 227 * 1024 || e.smem_c > 227 * 1024)
             return fail(c, SS_ERR_INVALID_ARG, "lattice %d x %d x %d: the FP64 evaluation needs more shared memory than a CTA has",
@@ -996,6 +997,8 @@ ss_status ensure_ev64(ss_ctx* c) {
         ev.push_back(e);
     }
     set_smem_limits<double>(227 * 1024);
+    for (Group& e : ev)
+        if (e.dipole) set_t2_smem_limits<double>(e.Px, e.Py, 227 * 1024);
     for (Group& e : ev) TRY(setup_group<double>(c, e));
     CUDA_TRY(c, cudaStreamSynchronize(c->cs));
     c->ev64 = std::move(ev);
@@ -1286,8 +1289,8 @@ ss_status ss_create_batch(int n_strings, const ss_string_desc* descs, const ss_o
     size_t stage = 0;
     for (Group& g : c->groups) {
         g.n_pairs = (g.n_img + 1) / 2;
-        g.Px = g.dipole ? padded_len(g.nx, !use_fp64(c)) : 1;
-        g.Py = g.dipole ? padded_len(g.ny, !use_fp64(c) && g.nz <= kT2MaxNz) : 1;
+        g.Px = g.dipole ? padded_len(g.nx, true) : 1;
+        g.Py = g.dipole ? padded_len(g.ny, g.nz <= kT2MaxNz) : 1;
         g.planx = make_plan(g.Px);
         g.plany = make_plan(g.Py);
         g.rbytes = (int)real_size(c);
@@ -1300,11 +1303,10 @@ ss_status ss_create_batch(int n_strings, const ss_string_desc* descs, const ss_o
     }
     if (use_fp64(c))
         set_smem_limits<double>(227 * 1024);
-    else {
+    else
         set_smem_limits<float>(227 * 1024);
-        for (Group& g : c->groups)
-            if (g.dipole) set_t2_smem_limits(g.Px, g.Py, 227 * 1024);
-    }
+    for (Group& g : c->groups)
+        if (g.dipole) use_fp64(c) ? set_t2_smem_limits<double>(g.Px, g.Py, 227 * 1024) : set_t2_smem_limits<float>(g.Px, g.Py, 227 * 1024);
     {
         ss_status st = dalloc(c, (void**)&c->d_err, sizeof(int));
         if (st != SS_OK) return bail(st);

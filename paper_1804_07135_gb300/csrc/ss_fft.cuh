@@ -163,6 +163,10 @@ template <typename C> __device__ __forceinline__ C caxpy(decltype(C{}.x) a, C x,
 }
 __device__ __forceinline__ float2 caxpy(float a, float2 x, float2 y) { return __ffma2_rn(make_float2(a, a), x, y); }
 
+// element-wise product of two pairs (real and imaginary part each times a real factor)
+template <typename C> __device__ __forceinline__ C emul(C a, C b) { return C{a.x * b.x, a.y * b.y}; }
+__device__ __forceinline__ float2 emul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+
 template <int I> struct ic {
     static constexpr int v = I;
 };

@@ -173,9 +173,9 @@ template <typename T> struct RkArgs {
 
 enum { kErrInvalidSpin = 1, kErrNonFinite = 2, kErrStepCollapse = 4 };
 
-// Lengths P = 16 R2 in two register passes (FP32, ss_fft.cuh, ss_twopass.cuh): a line is R2 = P/16 rows of 16
+// Lengths P = 16 R2 in two register passes (ss_fft.cuh, ss_twopass.cuh): a line is R2 = P/16 rows of 16
 // at row stride kT2Row; the y/z kernel for those Py with 1 to 8 layers, the x kernels for those Px with
-// kX2Rows rows per CTA.  The list covers lattices of up to 256 sites a side; each length is a multiple of 16
+// x2_rows rows per CTA.  The list covers lattices of up to 256 sites a side; each length is a multiple of 16
 // whose passes need DFTs of at most 16 points.
 #define SS_T2_LENGTHS(X) \
     X(32) X(48) X(64) X(80) X(96) X(112) X(128) X(144) X(160) X(192) X(224) X(256) X(288) X(320) X(384) X(448) X(512)
@@ -197,49 +197,74 @@ inline int t2_length_from(int m) {
 constexpr int kT2Row = 17;
 constexpr int kT2MaxNz = 8;
 __host__ __device__ constexpr int t2_line(int P) { return kT2Row * (P / 16); }
-// kx columns per CTA: the default (15 to 24 lines) and the alternative the autotuner also times (12 lines for
-// one or four layers); 0 when nz has no two-pass kernel
-inline int yz2p_kxb(int nz) { return nz == 1 ? 8 : nz == 2 ? 4 : nz <= 4 ? 2 : nz <= kT2MaxNz ? 1 : 0; }
-inline int yz2p_kxb_alt(int nz) { return nz == 1 ? 4 : nz == 4 ? 1 : 0; }
-inline bool yz2p_ok(int real_bytes, int Py, int nz, int Px) {
-    if (real_bytes != 4 || !t2_length(Py)) return false;
-    const int kxb = yz2p_kxb(nz);
-    return kxb > 0 && Px % kxb == 0;
+// kx columns per CTA, the counts with a kernel, largest first (15 to 24 lines, then fewer): the autotuner
+// picks one by time; untuned FP32 launches take the first, FP64 ones the last, whose work spreads most evenly
+// over the SMs (an FP64 launch is bound by each SM's FP64 pipe).  Empty when nz has no two-pass kernel.
+struct YzColumns {
+    int n, v[3];
+};
+inline YzColumns yz2p_columns(int nz) {
+    if (nz == 1) return {3, {8, 4, 2}};
+    if (nz == 2) return {2, {4, 1, 0}};
+    if (nz <= 4) return {2, {2, 1, 0}};
+    return {nz <= kT2MaxNz ? 1 : 0, {1, 0, 0}};
+}
+inline size_t yz2p_smem(int real_bytes, int Py, int nz, int kxb) { return (size_t)3 * nz * kxb * t2_line(Py) * 2 * real_bytes; }
+inline bool yz2p_ok(int Py, int nz, int Px) {
+    if (!t2_length(Py)) return false;
+    const YzColumns k = yz2p_columns(nz);
+    return k.n > 0 && Px % k.v[0] == 0;
 }
 // threads and resident CTAs of the y/z kernel: small CTAs, so that several per SM are in different passes, of
 // 80 registers per thread (64 spill in the z-convolution and the mirrored pass 1); as many as registers and
 // shared memory (24 lines: 26 KB at 128, 78 KB at 384) allow
-__host__ __device__ constexpr int yz2p_threads(int P) { return P <= 128 ? 128 : P <= 256 ? 192 : P <= 320 ? 256 : 384; }
-__host__ __device__ constexpr int yz2p_blocks(int P) {
+// (FP64: the pipe issues two lane-operations per clock and SM, so a few warps with all the registers they want)
+__host__ __device__ constexpr int yz2p_threads(int real_bytes, int P) {
+    if (real_bytes == 8) return P <= 256 ? 128 : 256;
+    return P <= 128 ? 128 : P <= 256 ? 192 : P <= 320 ? 256 : 384;
+}
+__host__ __device__ constexpr int yz2p_blocks(int real_bytes, int P) {
+    if (real_bytes == 8) return P <= 192 ? 3 : P <= 256 ? 2 : 1;
     return P <= 128 ? 6 : P <= 256 ? 4 : P <= 320 ? 3 : 2;
 }
-// columns per CTA a launch uses: the tuned choice when it is one of the two, else the default
-inline int yz2p_kxb_use(int nz, int tuned) { return tuned > 0 && (tuned == yz2p_kxb(nz) || tuned == yz2p_kxb_alt(nz)) ? tuned : yz2p_kxb(nz); }
-inline size_t yz2p_smem(int Py, int nz, int kxb) { return (size_t)3 * nz * kxb * t2_line(Py) * 8; }
+// columns per CTA a launch uses: the tuned count when it is one of them
+inline int yz2p_kxb_use(int real_bytes, int nz, int tuned) {
+    const YzColumns k = yz2p_columns(nz);
+    for (int i = 0; i < k.n; ++i)
+        if (k.v[i] == tuned) return tuned;
+    return k.n == 0 ? 0 : k.v[real_bytes == 8 ? k.n - 1 : 0];
+}
 // Factor of the stored tensor spectrum besides 4 pi / (Px Py): the two-pass y/z kernel convolves sums and
 // differences of mirrored layers, which leaves a factor 2 to be taken out (exact)
-inline double dhat_factor(int real_bytes, int Py, int nz, int Px) {
-    return nz > 1 && yz2p_ok(real_bytes, Py, nz, Px) ? 0.5 : 1.0;
-}
-constexpr int kX2Rows = 4;
+inline double dhat_factor(int Py, int nz, int Px) { return nz > 1 && yz2p_ok(Py, nz, Px) ? 0.5 : 1.0; }
+// rows per CTA of the two-pass x kernels (FP64: more, smaller CTAs, as for the y/z kernel)
+__host__ __device__ constexpr int x2_rows(int real_bytes) { return real_bytes == 8 ? 2 : 4; }
 // x CTAs: pass 2 has 192 roles (up to P = 384), pass 1 has 12 P/16, the sites take 4 nx (even nx) or 8 nx items.
 // The kernels are compiled for up to x2_threads threads in x2_blocks CTAs per SM (64 registers, 80 from P = 288
 // on) and launched with x2_launch_threads of them: on a grid of many waves the smaller block, of which more fit
 // on an SM (128x128x4 x 384 images: step kernel 311 us with 192 threads, 333 with 256); on a small grid the
 // larger one where it takes fewer rounds over the sites (112x112x1 x 60: iteration 56.2 us with 192, 53.7 with
 // 256).
-__host__ __device__ constexpr int x2_threads(int P) { return P <= 64 ? 128 : P <= 128 ? 192 : 256; }
-__host__ __device__ constexpr int x2_blocks(int P) { return P <= 64 ? 8 : P <= 128 ? 5 : P <= 256 ? 4 : 3; }
-inline int x2_launch_threads(int P, int nx, long ctas) {
-    const int hi = x2_threads(P), lo = P > 64 && P <= 256 ? hi - 64 : hi;
+__host__ __device__ constexpr int x2_threads(int real_bytes, int P) {
+    return real_bytes == 8 ? 128 : P <= 64 ? 128 : P <= 128 ? 192 : 256;
+}
+__host__ __device__ constexpr int x2_blocks(int real_bytes, int P) {
+    if (real_bytes == 8) return P <= 256 ? 3 : 2;
+    return P <= 64 ? 8 : P <= 128 ? 5 : P <= 256 ? 4 : 3;
+}
+inline int x2_launch_threads(int real_bytes, int P, int nx, long ctas) {
+    if (real_bytes == 8) return x2_threads(8, P);
+    const int hi = x2_threads(4, P), lo = P > 64 && P <= 256 ? hi - 64 : hi;
     const int items = nx % 2 == 0 ? 4 * nx : 8 * nx;
     return ctas < 10L * 152 && (items + hi - 1) / hi < (items + lo - 1) / lo ? hi : lo;
 }
-__host__ __device__ constexpr int x2_round(int v) { return v + ((16 / kX2Rows - v % 16) + 16) % 16; }
-__host__ __device__ constexpr int x2_lsx(int P) { return x2_round(t2_line(P) - 1); }  // transform lines
-inline bool x2p_ok(int real_bytes, int Px) { return real_bytes == 4 && t2_length(Px); }
-inline size_t x2_smem(int P, bool inverse) {
-    return (size_t)3 * kX2Rows * x2_lsx(P) * 8 + (inverse ? 32 * 2 * kEvalTerms * 8 : 0);
+// line stride of the x kernels: 16 / rows (mod 16)
+__host__ __device__ constexpr int x2_lsx(int real_bytes, int P) {
+    const int v = t2_line(P) - 1;
+    return v + ((16 / x2_rows(real_bytes) - v % 16) + 16) % 16;
+}
+inline size_t x2_smem(int real_bytes, int P, bool inverse) {
+    return (size_t)3 * x2_rows(real_bytes) * x2_lsx(real_bytes, P) * 2 * real_bytes + (inverse ? 32 * 2 * kEvalTerms * 8 : 0);
 }
 // Padded transform length for n sites: the smallest 2^a 3^b >= 2n - 1, or the power of two >= 2n - 1 when that
 // is at most 1/8 longer.
@@ -299,7 +324,7 @@ template <typename T, int P> void t2_xinv(const GroupArgs<T>& g, int mode, T dt,
 template <typename T, int P> void t2_yz(const GroupArgs<T>& g, cudaStream_t st);
 template <typename T, int P> void t2_smem_limits(int bytes);
 // The limits of the two-pass kernels of lengths Px and Py (those that have some).
-void set_t2_smem_limits(int Px, int Py, int bytes);
+template <typename T> void set_t2_smem_limits(int Px, int Py, int bytes);
 void launch_interp_identity(InterpEntry* tab, int img0, int K, cudaStream_t st);
 // the FP32 state [K][3][N] handed to the FP64 energy evaluation: every spin renormalised in FP64
 void launch_widen_unit(const float* src, double* dst, int K, int N, const int* pair_on, cudaStream_t st);

@@ -14,8 +14,10 @@
 #include <math.h>
 
 #include <algorithm>
+#include <mutex>
 #include <type_traits>
 #include <utility>
+#include <vector>
 
 #include "ss_fft.cuh"
 
@@ -23,10 +25,6 @@ namespace ss {
 
 // ------------------------------------------------------------------------------------------------
 // small helpers
-template <typename T> __device__ __forceinline__ T rsqrt_t(T x);
-template <> __device__ __forceinline__ float rsqrt_t<float>(float x) { return rsqrtf(x); }
-template <> __device__ __forceinline__ double rsqrt_t<double>(double x) { return 1.0 / sqrt(x); }
-
 // FP64 square root and reciprocal from FP32 seeds refined by Newton steps of FP64 multiply-adds only
 // (GB300's FP64 division and square root are long instruction sequences); within a few ulp of the
 // correctly rounded results for positive finite arguments in FP32 range.
@@ -45,6 +43,13 @@ __device__ __forceinline__ double rsqrt_nr(double x) {
     y = fma(0.5 * y, fma(-x * y, y, 1.0), y);
     y = fma(0.5 * y, fma(-x * y, y, 1.0), y);
     return y;
+}
+// 1 / sqrt(x): about 10 FP64 operations by rsqrt_nr where its FP32 seed is safe (spins are near unit length),
+// CUDA's square root and division (several times as many) for the rest, zero and infinities among them.
+template <typename T> __device__ __forceinline__ T rsqrt_t(T x);
+template <> __device__ __forceinline__ float rsqrt_t<float>(float x) { return rsqrtf(x); }
+template <> __device__ __forceinline__ double rsqrt_t<double>(double x) {
+    return x > 1e-30 && x < 1e30 ? rsqrt_nr(x) : 1.0 / sqrt(x);
 }
 __device__ __forceinline__ double rcp_nr(double x) {
     double r = (double)(1.0f / (float)x);
@@ -1796,7 +1801,7 @@ __global__ void aos_to_soa_kernel(const Tin* src, T* dst, int K, int N, int* err
         if (!(n2 > 0.0) || !isfinite(n2)) {
             atomicOr(err, kErrInvalidSpin);
         } else {
-            r = 1.0 / sqrt(n2);
+            r = rsqrt_t<double>(n2);
         }
         T* d = dst + k * 3 * N + n;
         d[0] = T(a * r);
@@ -1935,14 +1940,14 @@ static inline void launch_ex(void (*kernel)(KArgs...), dim3 grid, dim3 block, si
     cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
-// The two-pass x-inverse kernel in mode MODE when Px is one of its lengths (rows per CTA kX2Rows, set by
+// The two-pass x-inverse kernel in mode MODE when Px is one of its lengths (rows per CTA x2_rows, set by
 // the host); false otherwise.
-template <int MODE>
-static inline bool launch_xinv2p(const GroupArgs<float>& g, float dt, float* hout, bool pdl, cudaStream_t st) {
-    if (!x2p_ok(4, g.Px)) return false;
+template <int MODE, typename T>
+static inline bool launch_xinv2p(const GroupArgs<T>& g, T dt, T* hout, bool pdl, cudaStream_t st) {
+    if (!t2_length(g.Px)) return false;
     switch (g.Px) {
 #define SS_CASE(P) \
-    case P: t2_xinv<float, P>(g, MODE, dt, hout, pdl, st); break;
+    case P: t2_xinv<T, P>(g, MODE, dt, hout, pdl, st); break;
         SS_T2_LENGTHS(SS_CASE)
 #undef SS_CASE
     }
@@ -1955,8 +1960,8 @@ static inline int grid1d(size_t n, int thr) {
     return (int)(b ? b : 1);
 }
 
-// Layer counts with an unrolled z-convolution in the runtime-plan y/z kernel (FP32; the FP64 path and any
-// other count use the loop over layers).
+// Layer counts with an unrolled z-convolution in the runtime-plan y/z kernel (FP32; FP64 and any other count
+// use the loop over layers).
 #define SS_FOR_NZ(X) X(1) X(4) X(8)
 
 template <typename T> void launch_xfwd(const GroupArgs<T>& g, bool do_fft, int nthr, size_t smem, cudaStream_t st) {
@@ -1965,16 +1970,14 @@ template <typename T> void launch_xfwd(const GroupArgs<T>& g, bool do_fft, int n
         launch_pdl(xfwd_kernel<T, false>, grid, dim3(nthr), 0, st, g);
         return;
     }
-    if constexpr (std::is_same<T, float>::value) {
-        if (x2p_ok(4, g.Px)) {
-            switch (g.Px) {
+    if (t2_length(g.Px)) {
+        switch (g.Px) {
 #define SS_CASE(P) \
-    case P: t2_xfwd<float, P>(g, st); break;
-                SS_T2_LENGTHS(SS_CASE)
+    case P: t2_xfwd<T, P>(g, st); break;
+            SS_T2_LENGTHS(SS_CASE)
 #undef SS_CASE
-            }
-            return;
         }
+        return;
     }
     launch_pdl(xfwd_kernel<T, true>, grid, dim3(nthr), smem, st, g);
 }
@@ -1983,16 +1986,16 @@ template <typename T> void launch_yz(const GroupArgs<T>& g, int nthr, size_t sme
     dim3 grid(g.Px, g.n_pairs);
     const size_t base = (size_t)(g.Py + 3 * g.nz * g.lsy) * sizeof(cplx<T>);
     const int stage = smem >= base + (size_t)(g.Py / 2 + 1) * g.nz * 6 * sizeof(T);
-    if constexpr (std::is_same<T, float>::value) {
-        if (yz2p_ok(4, g.Py, g.nz, g.Px)) {
-            switch (g.Py) {
+    if (yz2p_ok(g.Py, g.nz, g.Px)) {
+        switch (g.Py) {
 #define SS_CASE(P) \
-    case P: t2_yz<float, P>(g, st); break;
-                SS_T2_LENGTHS(SS_CASE)
+    case P: t2_yz<T, P>(g, st); break;
+            SS_T2_LENGTHS(SS_CASE)
 #undef SS_CASE
-            }
-            return;
         }
+        return;
+    }
+    if constexpr (std::is_same<T, float>::value) {
 #define SS_CASE(Z)                                                      \
     if (g.nz == Z) {                                                    \
         launch_pdl(yz_kernel<T, Z>, grid, dim3(nthr), smem, st, g, stage); \
@@ -2011,18 +2014,14 @@ void launch_xinv_step(const GroupArgs<T>& g, bool do_fft, T dt, int nthr, size_t
         launch_pdl(xinv_kernel<T, false, 0>, grid, dim3(nthr), smem, st, g, dt, (T*)nullptr);
         return;
     }
-    if constexpr (std::is_same<T, float>::value) {
-        if (launch_xinv2p<0>(g, dt, nullptr, true, st)) return;
-    }
+    if (launch_xinv2p<0>(g, dt, (T*)nullptr, true, st)) return;
     launch_pdl(xinv_kernel<T, true, 0>, grid, dim3(nthr), smem, st, g, dt, (T*)nullptr);
 }
 
 template <typename T>
 void launch_xinv_eval(const GroupArgs<T>& g, bool do_fft, T* hout, int nthr, size_t smem, cudaStream_t st) {
     dim3 grid((g.ny + g.ty_c - 1) / g.ty_c, g.nz, g.n_pairs);
-    if constexpr (std::is_same<T, float>::value) {
-        if (do_fft && launch_xinv2p<1>(g, T(0), hout, false, st)) return;
-    }
+    if (do_fft && launch_xinv2p<1>(g, T(0), hout, false, st)) return;
     if (do_fft) {
         xinv_kernel<T, true, 1><<<grid, nthr, smem, st>>>(g, T(0), hout);
     } else {
@@ -2034,9 +2033,7 @@ template <typename T, int MODE>
 static void launch_xinv_force_mode(const GroupArgs<T>& g, bool do_fft, T* kout, T flag, int nthr, size_t smem,
                                    cudaStream_t st) {
     dim3 grid((g.ny + g.ty_c - 1) / g.ty_c, g.nz, g.n_pairs);
-    if constexpr (std::is_same<T, float>::value) {
-        if (do_fft && launch_xinv2p<MODE>(g, flag, kout, false, st)) return;
-    }
+    if (do_fft && launch_xinv2p<MODE>(g, flag, kout, false, st)) return;
     if (do_fft)
         xinv_kernel<T, true, MODE><<<grid, nthr, smem, st>>>(g, flag, kout);
     else
@@ -2056,9 +2053,7 @@ void launch_xinv_force(const GroupArgs<T>& g, bool do_fft, T* kout, bool energie
 template <typename T>
 void launch_xinv_step_llg(const GroupArgs<T>& g, bool do_fft, T dt, int nthr, size_t smem, cudaStream_t st) {
     dim3 grid((g.ny + g.ty_c - 1) / g.ty_c, g.nz, g.n_pairs);
-    if constexpr (std::is_same<T, float>::value) {
-        if (do_fft && launch_xinv2p<4>(g, dt, nullptr, true, st)) return;
-    }
+    if (do_fft && launch_xinv2p<4>(g, dt, (T*)nullptr, true, st)) return;
     if (do_fft)
         launch_pdl(xinv_kernel<T, true, 4>, grid, dim3(nthr), smem, st, g, dt, (T*)nullptr);
     else
@@ -2068,9 +2063,7 @@ void launch_xinv_step_llg(const GroupArgs<T>& g, bool do_fft, T dt, int nthr, si
 template <typename T>
 void launch_xinv_step_climb(const GroupArgs<T>& g, bool do_fft, T dt, T* hc, int nthr, size_t smem, cudaStream_t st) {
     dim3 grid((g.ny + g.ty_c - 1) / g.ty_c, g.nz, g.n_pairs);
-    if constexpr (std::is_same<T, float>::value) {
-        if (do_fft && launch_xinv2p<3>(g, dt, hc, true, st)) return;
-    }
+    if (do_fft && launch_xinv2p<3>(g, dt, hc, true, st)) return;
     if (do_fft)
         launch_pdl(xinv_kernel<T, true, 3>, grid, dim3(nthr), smem, st, g, dt, hc);
     else
@@ -2177,31 +2170,46 @@ template <typename F> static inline void set_dyn_smem(F* kernel, int bytes, int 
     if (carve_kb) cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, carve_kb * 100 / 228);
 }
 // One split for every kernel of an iteration (two-pass kernels of up to 384 points, arc, climbing image,
-// spline): an SM changes its split only when it is empty, and with programmatic dependent launch and graph
+// spline, direct sums, Runge-Kutta): an SM changes its split only when it is empty, and with programmatic dependent launch and graph
 // branches it never is, so a kernel that starts on SMs split for another one keeps that split -- the y/z kernel
 // of 384 points ran with one resident CTA behind an x kernel that had asked for less shared memory.  164 KB
 // hold two y/z CTAs of 384 points or three of 256 and leave 92 KB of L1 to the stencil.  The 20-string study on
 // one GB300: 4078 us per iteration with each kernel's own split, 3526 with this one.
-constexpr int kCarveKb = 164;
+// FP64 lines are twice as long (52 KB for 128 points): there every kernel asks for all of it.
+template <typename T> constexpr int carve_kb() { return sizeof(T) == 8 ? 228 : 164; }
+
 template <typename T> void set_smem_limits(int bytes) {
+    constexpr int carve = carve_kb<T>();
     set_dyn_smem(xfwd_kernel<T, true>, bytes);
+    set_dyn_smem(xfwd_kernel<T, false>, bytes, carve);
     set_dyn_smem(yz_kernel<T, 0>, bytes);
     set_dyn_smem(xinv_kernel<T, true, 0>, bytes);
     set_dyn_smem(xinv_kernel<T, true, 1>, bytes);
-    set_dyn_smem(xinv_kernel<T, false, 0>, bytes);
-    set_dyn_smem(xinv_kernel<T, false, 1>, bytes);
+    set_dyn_smem(xinv_kernel<T, false, 0>, bytes, carve);
+    set_dyn_smem(xinv_kernel<T, false, 1>, bytes, carve);
     set_dyn_smem(xinv_kernel<T, true, 2>, bytes);
-    set_dyn_smem(xinv_kernel<T, false, 2>, bytes);
+    set_dyn_smem(xinv_kernel<T, false, 2>, bytes, carve);
     set_dyn_smem(xinv_kernel<T, true, 3>, bytes);
-    set_dyn_smem(xinv_kernel<T, false, 3>, bytes);
+    set_dyn_smem(xinv_kernel<T, false, 3>, bytes, carve);
     set_dyn_smem(xinv_kernel<T, true, 4>, bytes);
-    set_dyn_smem(xinv_kernel<T, false, 4>, bytes);
+    set_dyn_smem(xinv_kernel<T, false, 4>, bytes, carve);
     set_dyn_smem(xinv_kernel<T, true, 5>, bytes);
-    set_dyn_smem(xinv_kernel<T, false, 5>, bytes);
-    set_dyn_smem(spline_apply_kernel<T>, 200 * 1024, kCarveKb);
-    set_dyn_smem(arc_kernel<T>, bytes, kCarveKb);
-    set_dyn_smem(climb_dot_kernel<T>, bytes, kCarveKb);
-    set_dyn_smem(climb_apply_kernel<T>, bytes, kCarveKb);
+    set_dyn_smem(xinv_kernel<T, false, 5>, bytes, carve);
+    set_dyn_smem(spline_apply_kernel<T>, 200 * 1024, carve);
+    set_dyn_smem(arc_kernel<T>, bytes, carve);
+    set_dyn_smem(climb_dot_kernel<T>, bytes, carve);
+#define SS_CASE(M)                                                  \
+    set_dyn_smem(dipole_direct_kernel<T, M, true>, bytes, carve);   \
+    set_dyn_smem(dipole_direct_kernel<T, M, false>, bytes, carve);
+    SS_CASE(1) SS_CASE(2) SS_CASE(4)
+#undef SS_CASE
+#define SS_CASE(S) set_dyn_smem(rk_assemble_kernel<T, S>, bytes, carve);
+    SS_CASE(0) SS_CASE(1) SS_CASE(2) SS_CASE(3) SS_CASE(4) SS_CASE(5) SS_CASE(6)
+#undef SS_CASE
+    set_dyn_smem(rk_finish_kernel<T>, bytes, carve);
+    set_dyn_smem(rk_control_kernel<T>, bytes, carve);
+    set_dyn_smem(rk_commit_kernel<T>, bytes, carve);
+    set_dyn_smem(climb_apply_kernel<T>, bytes, carve);
     if constexpr (std::is_same<T, float>::value) {
 #define SS_CASE(Z) set_dyn_smem(yz_kernel<T, Z>, bytes);
         SS_FOR_NZ(SS_CASE)
@@ -2210,18 +2218,29 @@ template <typename T> void set_smem_limits(int bytes) {
 }
 
 #ifdef SS_COMMON_LAUNCHERS
-void set_t2_smem_limits(int Px, int Py, int bytes) {
+template <typename T> void set_t2_smem_limits(int Px, int Py, int bytes) {
+    // once per device and length: the attributes stay with the kernels, and setting them takes longer than a
+    // small lattice's iteration
+    static std::mutex mu;
+    static std::vector<std::pair<int, int>> done;  // (device, length)
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return;
+    std::lock_guard<std::mutex> lock(mu);
     for (int P : {Px, Py}) {
+        const std::pair<int, int> key(dev, P);
+        if (std::find(done.begin(), done.end(), key) != done.end()) continue;
+        done.push_back(key);
         switch (P) {
 #define SS_CASE(L) \
-    case L: t2_smem_limits<float, L>(bytes); break;
+    case L: t2_smem_limits<T, L>(bytes); break;
             SS_T2_LENGTHS(SS_CASE)
 #undef SS_CASE
             default: break;
         }
-        if (Px == Py) break;
     }
 }
+template void set_t2_smem_limits<float>(int, int, int);
+template void set_t2_smem_limits<double>(int, int, int);
 
 void launch_fft_strided_f64(double2* data, const double2* tw, const FftPlan& plan, int n_lines, long elem_stride,
                             int inner_count, long inner_stride, long outer_stride, cudaStream_t st) {

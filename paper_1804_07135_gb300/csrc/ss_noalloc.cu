@@ -33,7 +33,6 @@ static __device__ __align__(256) unsigned char g_scratch[kNoAllocScratchBytes];
 struct ScratchSlot {
     unsigned char* ptr;
     bool ready;
-    bool limits[513];  // shared-memory limits of the two-pass kernels of a length are raised
 };
 std::mutex g_mu;
 ScratchSlot g_slots[kMaxDevices];
@@ -56,11 +55,7 @@ ss_status scratch_of_current_device(int Px, int Py, unsigned char** out) {
         g_slots[dev].ptr = static_cast<unsigned char*>(p);
         g_slots[dev].ready = true;
     }
-    for (int P : {Px, Py})
-        if (t2_length(P) && !g_slots[dev].limits[P]) {
-            set_t2_smem_limits(P, P, 227 * 1024);
-            g_slots[dev].limits[P] = true;
-        }
+    set_t2_smem_limits<float>(Px, Py, 227 * 1024);
     *out = g_slots[dev].ptr;
     return SS_OK;
 }
@@ -172,7 +167,7 @@ extern "C" ss_status ss_field_noalloc(int nx, int ny, int nz, double J, double D
         }
     }
     if (dip && Px == 128 && ty != 2 && ty != 4) ty = 8;
-    if (dip && (Px == 192 || Px == 256 || Px == 384)) ty = kX2Rows;
+    if (dip && (Px == 192 || Px == 256 || Px == 384)) ty = x2_rows(4);
     const size_t smem_a = (size_t)(Px + 3 * ty * lsx) * sizeof(float2);
     const size_t smem_c = smem_a + 32 * 2 * kEvalTerms * sizeof(double);
     size_t smem_b = (size_t)(Py + 3 * nz * lsy) * sizeof(float2);
@@ -231,7 +226,7 @@ extern "C" ss_status ss_field_noalloc(int nx, int ny, int nz, double J, double D
         na_tensor_fill<<<(int)((cells + 255) / 256 < 4096 ? (cells + 255) / 256 : 4096), 256, 0, st>>>(tens, nx, ny, nz, Px, Py);
         launch_fft_strided_f64(tens, tw64x, px, 6 * nz * Py, 1, 1, 0, Px, st);
         launch_fft_strided_f64(tens, tw64y, py, 6 * nz * Px, Px, Px, 1, (long)Px * Py, st);
-        launch_extract_octant<float>(tens, dhat, Px, Py, nz, dhat_factor(4, Py, nz, Px) * 4.0 * M_PI / ((double)Px * Py), st);
+        launch_extract_octant<float>(tens, dhat, Px, Py, nz, dhat_factor(Py, nz, Px) * 4.0 * M_PI / ((double)Px * Py), st);
     }
     ImgParam<float>* prm = reinterpret_cast<ImgParam<float>*>(base + o_prm);
     InterpEntry* interp = reinterpret_cast<InterpEntry*>(base + o_interp);
@@ -264,7 +259,7 @@ extern "C" ss_status ss_field_noalloc(int nx, int ny, int nz, double J, double D
     g.prm = prm;
     g.interp = interp;
     g.epart = nullptr;  // the field alone
-    g.ty_a = g.ty_c = dip && x2p_ok(4, Px) ? kX2Rows : ty;  // the two-pass x kernels take kX2Rows
+    g.ty_a = g.ty_c = dip && t2_length(Px) ? x2_rows(4) : ty;  // the two-pass x kernels' own count
     g.err = err;
     launch_xfwd<float>(g, dip, thr, smem_a, st);
     if (dip) launch_yz<float>(g, thr_b, smem_b, st);

@@ -6,7 +6,7 @@
 
 namespace ss {
 
-// yz for a two-pass length Py = P (ny <= P/2), FP32, NZ layers, KXB kx columns per CTA: the y-transforms
+// yz for a two-pass length Py = P (ny <= P/2), NZ layers, KXB kx columns per CTA: the y-transforms
 // in two register passes each way (t2_pass1 / t2_cols / t2_passB, ss_fft.cuh) on lines held in the
 // 17-strided row layout, the z-convolution in place between them.  One shared line per (column, component,
 // layer): 3 NZ KXB lines of t2_line(P) complex elements, read from the spectrum in pass 1 and written back
@@ -35,60 +35,59 @@ template <int NZ, int PAR> struct ZSys {  // PAR 0: (x, y in e; z in o), 1: (x, 
 // coefficients (component c, |dz| at d[(|dz| * 6 + c) * DQ]); par the system; fx, fy the parity signs of kx, ky
 // (the tensor's xy, xz, yz are odd in them: flip x and y going in and coming out).  The result replaces the
 // inputs, conjugated (the inverse transform is the conjugate of the forward transform of the conjugate).
-template <int NZ, int PAR, int LS, int DQ>
-__device__ __forceinline__ void zconv_sys(float2* A, const float* __restrict__ d, int par, float fx, float fy) {
+template <int NZ, int PAR, int LS, int DQ, typename T, typename C>
+__device__ __forceinline__ void zconv_sys(C* A, const T* __restrict__ d, int par, T fx, T fy) {
     using S = ZSys<NZ, PAR>;  // the shape; for even NZ both systems share it and par picks one at run time
     constexpr int NA = S::NXY, NB = S::NZC;
     constexpr int NA1 = NA > 0 ? NA : 1, NB1 = NB > 0 ? NB : 1;
-    const float sg = par ? -1.f : 1.f;
-    float2* Ax = A + (par ? S::ME : 0) * LS;
-    float2* Ay = Ax + NZ * LS;
-    float2* Az = A + (2 * NZ + (par ? 0 : S::ME)) * LS;
-    float2 X[NA1], Y[NA1], Z[NB1], HX[NA1], HY[NA1], W[NB1];
-    const float2 fx2 = make_float2(fx, fx), fy2 = make_float2(fy, fy), zero = make_float2(0.f, 0.f);
+    const T sg = par ? T(-1) : T(1);
+    C* Ax = A + (par ? S::ME : 0) * LS;
+    C* Ay = Ax + NZ * LS;
+    C* Az = A + (2 * NZ + (par ? 0 : S::ME)) * LS;
+    C X[NA1], Y[NA1], Z[NB1], HX[NA1], HY[NA1], W[NB1];
+    const C zero = C{T(0), T(0)};
 #pragma unroll
     for (int i = 0; i < NA; ++i) {
-        X[i] = __fmul2_rn(fx2, Ax[i * LS]);
-        Y[i] = __fmul2_rn(fy2, Ay[i * LS]);
+        X[i] = emul(C{fx, fx}, Ax[i * LS]);
+        Y[i] = emul(C{fy, fy}, Ay[i * LS]);
         HX[i] = HY[i] = zero;
     }
 #pragma unroll
     for (int i = 0; i < NB; ++i) {
-        const float2 z = Az[i * LS];
-        Z[i] = make_float2(-z.y, z.x);  // i z
+        const C z = Az[i * LS];
+        Z[i] = C{-z.y, z.x};  // i z
         W[i] = zero;
     }
-    auto load = [&](int c, float (&t)[NZ]) {
+    auto load = [&](int c, T (&t)[NZ]) {
 #pragma unroll
         for (int q = 0; q < NZ; ++q) t[q] = d[(q * 6 + c) * DQ];
     };
-    auto dup = [](float a) { return make_float2(a, a); };
     // t(|i-j|) + s t(n-1-i-j) for an even component
-    auto even = [&](const float (&t)[NZ], float s, int i, int j) {
-        return dup(fmaf(s, t[NZ - 1 - i - j], t[i > j ? i - j : j - i]));
+    auto even = [&](const T (&t)[NZ], T s, int i, int j) {
+        return t[i > j ? i - j : j - i] + s * t[NZ - 1 - i - j];
     };
-    float t[NZ];
+    T t[NZ];
     if constexpr (NA > 0) {
         load(0, t);  // xx
 #pragma unroll
         for (int i = 0; i < NA; ++i)
 #pragma unroll
             for (int j = 0; j <= i; ++j) {
-                const float2 c = even(t, sg, i, j);
-                HX[i] = __ffma2_rn(c, X[j], HX[i]);
-                if (j < i) HX[j] = __ffma2_rn(c, X[i], HX[j]);
+                const T c = even(t, sg, i, j);
+                HX[i] = caxpy(c, X[j], HX[i]);
+                if (j < i) HX[j] = caxpy(c, X[i], HX[j]);
             }
         load(3, t);  // xy
 #pragma unroll
         for (int i = 0; i < NA; ++i)
 #pragma unroll
             for (int j = 0; j <= i; ++j) {
-                const float2 c = even(t, sg, i, j);
-                HX[i] = __ffma2_rn(c, Y[j], HX[i]);
-                HY[i] = __ffma2_rn(c, X[j], HY[i]);
+                const T c = even(t, sg, i, j);
+                HX[i] = caxpy(c, Y[j], HX[i]);
+                HY[i] = caxpy(c, X[j], HY[i]);
                 if (j < i) {
-                    HX[j] = __ffma2_rn(c, Y[i], HX[j]);
-                    HY[j] = __ffma2_rn(c, X[i], HY[j]);
+                    HX[j] = caxpy(c, Y[i], HX[j]);
+                    HY[j] = caxpy(c, X[i], HY[j]);
                 }
             }
         load(1, t);  // yy
@@ -96,42 +95,41 @@ __device__ __forceinline__ void zconv_sys(float2* A, const float* __restrict__ d
         for (int i = 0; i < NA; ++i)
 #pragma unroll
             for (int j = 0; j <= i; ++j) {
-                const float2 c = even(t, sg, i, j);
-                HY[i] = __ffma2_rn(c, Y[j], HY[i]);
-                if (j < i) HY[j] = __ffma2_rn(c, Y[i], HY[j]);
+                const T c = even(t, sg, i, j);
+                HY[i] = caxpy(c, Y[j], HY[i]);
+                if (j < i) HY[j] = caxpy(c, Y[i], HY[j]);
             }
     }
     if constexpr (NA > 0 && NB > 0) {
         // G(i-j) + sg G(n-1-i-j), G(0) = 0: xz, then yz
-        auto odd = [&](const float (&t)[NZ], int i, int j) {
+        auto odd = [&](const T (&t)[NZ], int i, int j) {
             const int p = NZ - 1 - i - j;
-            const float hank = p > 0 ? t[p] : p < 0 ? -t[-p] : 0.f;
-            return dup(i == j ? sg * hank : fmaf(sg, hank, i > j ? t[i - j] : -t[j - i]));
+            const T hank = p > 0 ? t[p] : p < 0 ? -t[-p] : T(0);
+            return i == j ? sg * hank : (i > j ? t[i - j] : -t[j - i]) + sg * hank;
         };
         load(4, t);
 #pragma unroll
         for (int i = 0; i < NA; ++i)
 #pragma unroll
             for (int j = 0; j < NB; ++j) {
-                const float2 c = odd(t, i, j);
-                HX[i] = __ffma2_rn(c, Z[j], HX[i]);
-                W[j] = __ffma2_rn(c, X[i], W[j]);
+                const T c = odd(t, i, j);
+                HX[i] = caxpy(c, Z[j], HX[i]);
+                W[j] = caxpy(c, X[i], W[j]);
             }
         load(5, t);
 #pragma unroll
         for (int i = 0; i < NA; ++i)
 #pragma unroll
             for (int j = 0; j < NB; ++j) {
-                const float2 c = odd(t, i, j);
-                HY[i] = __ffma2_rn(c, Z[j], HY[i]);
-                W[j] = __ffma2_rn(c, Y[i], W[j]);
+                const T c = odd(t, i, j);
+                HY[i] = caxpy(c, Z[j], HY[i]);
+                W[j] = caxpy(c, Y[i], W[j]);
             }
     }
-    const float2 cx = make_float2(fx, -fx), cy = make_float2(fy, -fy);
 #pragma unroll
     for (int i = 0; i < NA; ++i) {
-        Ax[i * LS] = __fmul2_rn(cx, HX[i]);
-        Ay[i * LS] = __fmul2_rn(cy, HY[i]);
+        Ax[i * LS] = emul(C{fx, -fx}, HX[i]);
+        Ay[i * LS] = emul(C{fy, -fy}, HY[i]);
     }
     if constexpr (NB > 0) {
         load(2, t);  // zz
@@ -139,31 +137,31 @@ __device__ __forceinline__ void zconv_sys(float2* A, const float* __restrict__ d
         for (int i = 0; i < NB; ++i)
 #pragma unroll
             for (int j = 0; j <= i; ++j) {
-                const float2 c = even(t, -sg, i, j);
-                W[i] = __ffma2_rn(c, Z[j], W[i]);
-                if (j < i) W[j] = __ffma2_rn(c, Z[i], W[j]);
+                const T c = even(t, -sg, i, j);
+                W[i] = caxpy(c, Z[j], W[i]);
+                if (j < i) W[j] = caxpy(c, Z[i], W[j]);
             }
 #pragma unroll
-        for (int i = 0; i < NB; ++i) Az[i * LS] = make_float2(W[i].y, W[i].x);  // conj(-i W)
+        for (int i = 0; i < NB; ++i) Az[i * LS] = C{W[i].y, W[i].x};  // conj(-i W)
     }
 }
 
 // The z-convolution of one column: one item per (frequency, system), reading and writing its own elements.
-template <int NZ, int P>
-__device__ __forceinline__ void zconv_t2(float2* A, int kx, int Px, const float* dslab, int tid, int nthr) {
+template <int NZ, int P, typename T, typename C>
+__device__ __forceinline__ void zconv_t2(C* A, int kx, int Px, const T* dslab, int tid, int nthr) {
     constexpr int LS = t2_line(P), DQ = P / 2 + 1;
-    const float fx = kx > Px / 2 ? -1.f : 1.f;
+    const T fx = kx > Px / 2 ? T(-1) : T(1);
     for (int it = tid; it < (NZ == 1 ? P : 2 * P); it += nthr) {
         const int par = it >= P ? 1 : 0, ky = it - par * P;
-        const float fy = ky > P / 2 ? -1.f : 1.f;
-        const float* d = dslab + min(ky, P - ky);
-        float2* a = A + t2_pos(ky);
+        const T fy = ky > P / 2 ? T(-1) : T(1);
+        const T* d = dslab + min(ky, P - ky);
+        C* a = A + t2_pos(ky);
         if constexpr (NZ == 1) {  // xz and yz vanish
-            const float2 X = a[0], Y = a[LS], Z = a[2 * LS];
-            const float xx = d[0], yy = d[DQ], zz = d[2 * DQ], xy = fx * fy * d[3 * DQ];
-            a[0] = make_float2(xx * X.x + xy * Y.x, -(xx * X.y + xy * Y.y));
-            a[LS] = make_float2(xy * X.x + yy * Y.x, -(xy * X.y + yy * Y.y));
-            a[2 * LS] = make_float2(zz * Z.x, -zz * Z.y);
+            const C X = a[0], Y = a[LS], Z = a[2 * LS];
+            const T xx = d[0], yy = d[DQ], zz = d[2 * DQ], xy = fx * fy * d[3 * DQ];
+            a[0] = C{xx * X.x + xy * Y.x, -(xx * X.y + xy * Y.y)};
+            a[LS] = C{xy * X.x + yy * Y.x, -(xy * X.y + yy * Y.y)};
+            a[2 * LS] = C{zz * Z.x, -zz * Z.y};
         } else if constexpr (NZ % 2 == 0) {  // the two systems have the same shape
             zconv_sys<NZ, 0, LS, DQ>(a, d, par, fx, fy);
         } else if (par == 0) {
@@ -174,16 +172,17 @@ __device__ __forceinline__ void zconv_t2(float2* A, int kx, int Px, const float*
     }
 }
 
-template <int P, int NZ, int KXB>
-__global__ void __launch_bounds__(yz2p_threads(P), yz2p_blocks(P)) yz2p_kernel(GroupArgs<float> g) {
-    using C = float2;
+template <typename T, int P, int NZ, int KXB>
+__global__ void __launch_bounds__(yz2p_threads(sizeof(T), P), yz2p_blocks(sizeof(T), P)) yz2p_kernel(GroupArgs<T> g) {
+    using C = cplx<T>;
     constexpr int R2 = P / 16, LS = t2_line(P), L = 3 * NZ * KXB, RC = 16 * T2<P>::NP;  // RC: roles per line
     constexpr int ME = (NZ + 1) / 2, MO = NZ / 2, LP = 3 * ME * KXB;                    // LP: pairs of mirrored layers
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* A = reinterpret_cast<C*>(smem_raw);  // line (b * 3 + c) * NZ + q: e_q for q < ME, o_{q - ME} above
-    const int tid = threadIdx.x, nthr = yz2p_threads(P);
+    const int tid = threadIdx.x, nthr = yz2p_threads(sizeof(T), P);
     const int kx = blockIdx.x * KXB, p = blockIdx.y;
     const int ny = g.ny;
+    if (sizeof(T) == 8 && g.pair_on && !g.pair_on[p]) return;  // uniform over the CTA
     C* blk = g.spec + ((size_t)p * g.Px + kx) * 3 * NZ * ny;  // KXB consecutive columns are contiguous
     const C* __restrict__ tw = g.twy;                         // W_P^k
     const C* __restrict__ t1 = g.t2y;                         // pass 1
@@ -202,8 +201,8 @@ __global__ void __launch_bounds__(yz2p_threads(P), yz2p_blocks(P)) yz2p_kernel(G
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 const bool in = R2 * j + n2 < ny;
-                u[j] = in ? src[R2 * j] : make_float2(0.f, 0.f);
-                v[j] = in ? src2[R2 * j] : make_float2(0.f, 0.f);
+                u[j] = in ? src[R2 * j] : C{T(0), T(0)};
+                v[j] = in ? src2[R2 * j] : C{T(0), T(0)};
             }
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
@@ -214,7 +213,7 @@ __global__ void __launch_bounds__(yz2p_threads(P), yz2p_blocks(P)) yz2p_kernel(G
             t2_pass1<P>(v, n2, t1, A + (bc * NZ + ME + i) * LS);
         } else {
 #pragma unroll
-            for (int j = 0; j < 8; ++j) u[j] = R2 * j + n2 < ny ? src[R2 * j] : make_float2(0.f, 0.f);
+            for (int j = 0; j < 8; ++j) u[j] = R2 * j + n2 < ny ? src[R2 * j] : C{T(0), T(0)};
         }
         t2_pass1<P>(u, n2, t1, A + (bc * NZ + i) * LS);
     }
@@ -258,10 +257,10 @@ __global__ void __launch_bounds__(yz2p_threads(P), yz2p_blocks(P)) yz2p_kernel(G
 }
 
 // ------------------------------------------------------------------------------------------------
-// x kernels for a two-pass length Px = P (nx <= P/2), FP32: the x-transforms in two register passes
-// (ss_fft.cuh) on kX2Rows rows of one layer of an image pair per CTA.  Every role order puts the rows
+// x kernels for a two-pass length Px = P (nx <= P/2): the x-transforms in two register passes
+// (ss_fft.cuh) on x2_rows rows of one layer of an image pair per CTA.  Every role order puts the rows
 // fastest across a warp: the spectrum's rows of one (kx, c) are contiguous in global memory, and with
-// line strides = 16 / kX2Rows (mod 16) the lanes of a half-warp (kX2Rows rows x 16 / kX2Rows consecutive
+// line strides = 16 / rows (mod 16) the lanes of a half-warp (rows x 16 / rows consecutive
 // columns or rows of a line) hit distinct shared-memory banks.
 // x sits at row x mod R2, column x / R2 of its line, which is where pass 1 reads its role's inputs and pass B
 // leaves its outputs: both work in place, and the space of separate x-space lines stays with the L1 cache
@@ -269,15 +268,17 @@ __global__ void __launch_bounds__(yz2p_threads(P), yz2p_blocks(P)) yz2p_kernel(G
 // step kernel of 128x128x4 x 384 images 298 -> 253 us and 438 -> 311, of 192x192x8 x 128 437 -> 441 and
 // 662 -> 540, of 64x64x8 x 32 17.0 -> 16.4 and 22.5 -> 18.4 (one GB300).  They are bound by load latency and L1.
 // xfwd: the gather (Eq. 12), pass 1 in place, pass 2 straight to the spectrum spec[p][kx][c][z][y].
-template <int P>
-__global__ void __launch_bounds__(x2_threads(P), x2_blocks(P)) xfwd2p_kernel(GroupArgs<float> g) {
-    using C = float2;
-    constexpr int R2 = P / 16, H = T2<P>::H, NP = T2<P>::NP, ROWS = kX2Rows, L = 3 * ROWS, LSX = x2_lsx(P);
+template <typename T, int P>
+__global__ void __launch_bounds__(x2_threads(sizeof(T), P), x2_blocks(sizeof(T), P)) xfwd2p_kernel(GroupArgs<T> g) {
+    using C = cplx<T>;
+    constexpr int R2 = P / 16, H = T2<P>::H, NP = T2<P>::NP, ROWS = x2_rows(sizeof(T)), L = 3 * ROWS,
+                  LSX = x2_lsx(sizeof(T), P);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* A = reinterpret_cast<C*>(smem_raw);  // line c * ROWS + yy: the pair at x, then rows of Z
     const int tid = threadIdx.x, nthr = blockDim.x;
     const int p = blockIdx.z, z = blockIdx.y, y0 = blockIdx.x * ROWS;
     const int rows = min(ROWS, g.ny - y0), nx = g.nx;
+    if (sizeof(T) == 8 && g.pair_on && !g.pair_on[p]) return;  // uniform over the CTA
     const C* __restrict__ tw = g.twx;  // W_P^k
     const C* __restrict__ t1 = g.t2x;  // pass 1
     griddep_wait();
@@ -291,7 +292,7 @@ __global__ void __launch_bounds__(x2_threads(P), x2_blocks(P)) xfwd2p_kernel(Gro
         C* line = A + (c * ROWS + yy) * LSX;
         C u[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) u[j] = R2 * j + n2 < nx ? line[t2_at(n2, j)] : make_float2(0.f, 0.f);
+        for (int j = 0; j < 8; ++j) u[j] = R2 * j + n2 < nx ? line[t2_at(n2, j)] : C{T(0), T(0)};
         t2_pass1<P>(u, n2, t1, line);
     }
     __syncthreads();
@@ -312,16 +313,19 @@ __global__ void __launch_bounds__(x2_threads(P), x2_blocks(P)) xfwd2p_kernel(Gro
 
 // xinv: pass A straight from the spectrum (conjugated), pass B in place, then the per-site work of xinv_sites
 // in mode MODE.
-template <int P, int MODE>
-__global__ void __launch_bounds__(x2_threads(P), x2_blocks(P)) xinv2p_kernel(GroupArgs<float> g, float dt, float* hout) {
-    using C = float2;
-    constexpr int R2 = P / 16, H = T2<P>::H, NP = T2<P>::NP, ROWS = kX2Rows, L = 3 * ROWS, LSX = x2_lsx(P);
+template <typename T, int P, int MODE>
+__global__ void __launch_bounds__(x2_threads(sizeof(T), P), x2_blocks(sizeof(T), P)) xinv2p_kernel(GroupArgs<T> g, T dt,
+                                                                                                   T* hout) {
+    using C = cplx<T>;
+    constexpr int R2 = P / 16, H = T2<P>::H, NP = T2<P>::NP, ROWS = x2_rows(sizeof(T)), L = 3 * ROWS,
+                  LSX = x2_lsx(sizeof(T), P);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* A = reinterpret_cast<C*>(smem_raw);  // line c * ROWS + yy: columns of T, then the field convolution at x
     double* red = reinterpret_cast<double*>(A + L * LSX);
     const int tid = threadIdx.x, nthr = blockDim.x;
     const int p = blockIdx.z, z = blockIdx.y, y0 = blockIdx.x * ROWS;
     const int rows = min(ROWS, g.ny - y0);
+    if (sizeof(T) == 8 && g.pair_on && !g.pair_on[p]) return;  // uniform over the CTA
     const size_t kstride = (size_t)3 * g.nz * g.ny;
     const C* inp = g.spec + (size_t)p * P * kstride + (size_t)z * g.ny + y0;
     const C* __restrict__ tw = g.twx;
@@ -351,49 +355,53 @@ __global__ void __launch_bounds__(x2_threads(P), x2_blocks(P)) xinv2p_kernel(Gro
         for (int m = 0; m < 8; ++m) line[t2_at(y2, m)] = v[m];
     }
     __syncthreads();
-    xinv_sites<float, true, MODE>(g, dt, hout, A, LSX, ROWS, red, p, z, y0, rows, tid, nthr, T2Pos<R2>{});
+    xinv_sites<T, true, MODE>(g, dt, hout, A, LSX, ROWS, red, p, z, y0, rows, tid, nthr, T2Pos<R2>{});
 }
 
 // ---- launchers of one length --------------------------------------------------------------------------
+// FP64 launches do without programmatic dependent launch: they are bound by each SM's FP64 pipe, and CTAs placed
+// while the previous kernel drains land unevenly (40x50x3 x 16 images, FP64: 223 us per iteration with it, 210
+// without).  FP64 per iteration on one GB300, runtime Stockham plans before and these kernels: 64x64x4 x 16
+// 432 -> 353 us, 72x60x8 x 8 625 -> 415, 70x70x1 x 32 356 -> 223, 128x128x8 x 4 1226 -> 815, 20x20x2 x 16 77 -> 75.
 template <typename T, int P> void t2_xfwd(const GroupArgs<T>& g, cudaStream_t st) {
-    const dim3 grid((g.ny + g.ty_a - 1) / g.ty_a, g.nz, g.n_pairs);  // ty_a = kX2Rows (set by the host)
-    const int thr = x2_launch_threads(P, g.nx, (long)grid.x * grid.y * grid.z);
-    launch_pdl(xfwd2p_kernel<P>, grid, dim3(thr), x2_smem(P, false), st, g);
+    const dim3 grid((g.ny + g.ty_a - 1) / g.ty_a, g.nz, g.n_pairs);  // ty_a = x2_rows (set by the host)
+    const int thr = x2_launch_threads(sizeof(T), P, g.nx, (long)grid.x * grid.y * grid.z);
+    launch_ex(xfwd2p_kernel<T, P>, grid, dim3(thr), x2_smem(sizeof(T), P, false), st, sizeof(T) == 4, g);
 }
 
 template <typename T, int P>
 void t2_xinv(const GroupArgs<T>& g, int mode, T dt, T* hout, bool pdl, cudaStream_t st) {
     const dim3 grid((g.ny + g.ty_c - 1) / g.ty_c, g.nz, g.n_pairs);
-    const dim3 blk(x2_launch_threads(P, g.nx, (long)grid.x * grid.y * grid.z));
-    const size_t sm = x2_smem(P, true);
+    const dim3 blk(x2_launch_threads(sizeof(T), P, g.nx, (long)grid.x * grid.y * grid.z));
+    const size_t sm = x2_smem(sizeof(T), P, true);
     switch (mode) {
 #define SS_CASE(M) \
-    case M: launch_ex(xinv2p_kernel<P, M>, grid, blk, sm, st, pdl, g, dt, hout); break;
+    case M: launch_ex(xinv2p_kernel<T, P, M>, grid, blk, sm, st, pdl && sizeof(T) == 4, g, dt, hout); break;
         SS_CASE(0) SS_CASE(1) SS_CASE(2) SS_CASE(3) SS_CASE(4) SS_CASE(5)
 #undef SS_CASE
     }
 }
 
-// (layers, columns per CTA) of the y/z kernel: yz2p_kxb and yz2p_kxb_alt
-#define SS_T2_YZ(X) X(1, 8) X(1, 4) X(2, 4) X(3, 2) X(4, 2) X(4, 1) X(5, 1) X(6, 1) X(7, 1) X(8, 1)
+// (layers, columns per CTA) of the y/z kernel: yz2p_columns
+#define SS_T2_YZ(X) \
+    X(1, 8) X(1, 4) X(1, 2) X(2, 4) X(2, 1) X(3, 2) X(3, 1) X(4, 2) X(4, 1) X(5, 1) X(6, 1) X(7, 1) X(8, 1)
 template <typename T, int P> void t2_yz(const GroupArgs<T>& g, cudaStream_t st) {
-    int kxb = yz2p_kxb_use(g.nz, g.yz_kxb);
-    if (g.Px % kxb) kxb = yz2p_kxb(g.nz);
-    const size_t sm = yz2p_smem(P, g.nz, kxb);
+    const int kxb = yz2p_kxb_use(sizeof(T), g.nz, g.yz_kxb);  // divides Px: yz2p_ok, and the counts divide the first
+    const size_t sm = yz2p_smem(sizeof(T), P, g.nz, kxb);
     const dim3 grid(g.Px / kxb, g.n_pairs);
 #define SS_CASE(Z, B) \
-    if (g.nz == Z && kxb == B) launch_pdl(yz2p_kernel<P, Z, B>, grid, dim3(yz2p_threads(P)), sm, st, g);
+    if (g.nz == Z && kxb == B) launch_ex(yz2p_kernel<T, P, Z, B>, grid, dim3(yz2p_threads(sizeof(T), P)), sm, st, sizeof(T) == 4, g);
     SS_T2_YZ(SS_CASE)
 #undef SS_CASE
 }
 
 template <typename T, int P> void t2_smem_limits(int bytes) {
-    constexpr int carve = P <= 384 ? kCarveKb : P <= 448 ? 196 : 228;  // two y/z CTAs
-    set_dyn_smem(xfwd2p_kernel<P>, bytes, carve);
-#define SS_CASE(M) set_dyn_smem(xinv2p_kernel<P, M>, bytes, carve);
+    constexpr int carve = sizeof(T) == 8 || P <= 384 ? carve_kb<T>() : P <= 448 ? 196 : 228;  // two FP32 y/z CTAs
+    set_dyn_smem(xfwd2p_kernel<T, P>, bytes, carve);
+#define SS_CASE(M) set_dyn_smem(xinv2p_kernel<T, P, M>, bytes, carve);
     SS_CASE(0) SS_CASE(1) SS_CASE(2) SS_CASE(3) SS_CASE(4) SS_CASE(5)
 #undef SS_CASE
-#define SS_CASE(Z, B) set_dyn_smem(yz2p_kernel<P, Z, B>, bytes, carve);
+#define SS_CASE(Z, B) set_dyn_smem(yz2p_kernel<T, P, Z, B>, bytes, carve);
     SS_T2_YZ(SS_CASE)
 #undef SS_CASE
 }

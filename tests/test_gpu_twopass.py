@@ -42,8 +42,9 @@ def test_x_and_yz_kernels_at_the_edges_of_each_length(i):
     for n in (lo, (lo + hi) // 2 | 1, hi):
         if n > hi:
             continue
-        assert _check((n, 14, nz, 1.0, 0.3, 0.1, 0.03, 3), seed=i)["Px"] == P
-        assert _check((15, n, nz, 1.0, -0.3, 0.1, 0.03, 2), seed=50 + i)["Py"] == P
+        other = 14 if P < 200 else 5
+        assert _check((n, other, nz, 1.0, 0.3, 0.1, 0.03, 3), seed=i)["Px"] == P
+        assert _check((other + 1, n, nz, 1.0, -0.3, 0.1, 0.03, 2), seed=50 + i)["Py"] == P
 
 
 @pytest.mark.parametrize("nz", range(1, 10))
@@ -53,3 +54,21 @@ def test_every_layer_count(nz):
     assert cfg["Px"] == 48 and cfg["Py"] == 64
     cfg = _check((13, 37, nz, 1.0, 0.3, 0.1, 0.03, 2), seed=90 + nz)
     assert cfg["Px"] == 32 and cfg["Py"] == (80 if nz <= 8 else 81)
+
+
+@pytest.mark.parametrize("case", [(13, 30, 1), (24, 40, 2), (50, 17, 3), (33, 20, 4), (75, 6, 5), (4, 100, 6),
+                                  (45, 8, 7), (5, 129, 8), (150, 4, 8)])
+def test_fp64_kernels(case):
+    # the same kernels in FP64: the FP64 field bound of the other parity tests, 1e-12 of max |h|
+    nx, ny, nz = case
+    desc = (nx, ny, nz, 1.0, 0.3, 0.1, 0.03, 3)
+    path = W.random_spins((3, nx * ny * nz, 3), seed=nx)
+    with binding.StringMethod([desc], precision=binding.SS_PREC_FP64) as sm:
+        sm.set_path(0, path)
+        got, e = sm.field(0), sm.energies(0)
+    m = oracle.model(*desc[:7])
+    want = oracle.energies(m, path)
+    assert np.abs(e - want).max() <= 1e-11 * np.abs(want).max()
+    for k in range(3):
+        ref = oracle.field(m, path[k])
+        assert np.abs(got[k] - ref).max() <= 1e-12 * np.abs(ref).max(), k
