@@ -113,6 +113,7 @@ struct Group {
     InterpEntry* interp = nullptr;
     double* epart = nullptr;
     int *d_str_img0 = nullptr, *d_str_K = nullptr;
+    double* d_str_inv = nullptr;
     double *dpart = nullptr, *e_last = nullptr, *eval_terms = nullptr, *eval_E = nullptr, *eval_cn = nullptr;
     int* pair_on = nullptr;  // FP64 evaluation copy: the pairs holding barrier candidates
     // barrier candidates of an FP32 context (ss_barrier): the FP32 energies and round-off bounds select the
@@ -430,14 +431,15 @@ template <typename T> ss_status setup_group(ss_ctx* c, Group& g) {
     a.n_str = nstr;
     a.maxK = maxK;
     // components per tile CTA: 1024 (4 per thread of a 256-thread CTA), more on large lattices so that a
-    // string has at most about 128 tiles -- the finisher sums every tile's partial of every distance
-    a.tile_elems = 1024 * std::max(1, std::min(16, (int)(M / (1024 * 128))));
+    // string has at most 128 tiles -- the finisher sums every tile's partial of every distance
+    a.tile_elems = 1024 * std::max(1, std::min(16, (int)((M + 1024 * 128 - 1) / (1024 * 128))));
     a.n_tiles = (int)((M + a.tile_elems - 1) / a.tile_elems);
     a.kchunk = std::max(1, std::min(8, maxK - 1));
     a.n_kchunks = std::max(1, (maxK - 1 + a.kchunk - 1) / a.kchunk);
     a.reparam = c->opts.reparam_every != 0;
     TRY(dalloc(c, (void**)&g.d_str_img0, nstr * sizeof(int)));
     TRY(dalloc(c, (void**)&g.d_str_K, nstr * sizeof(int)));
+    TRY(dalloc(c, (void**)&g.d_str_inv, nstr * sizeof(double)));
     TRY(dalloc(c, (void**)&g.dpart, (size_t)nstr * maxK * a.n_tiles * sizeof(double)));
     TRY(dalloc(c, (void**)&g.e_last, (size_t)nstr * maxK * sizeof(double)));
     const size_t n_cnt = (size_t)nstr;  // tile CTAs finished per string
@@ -449,12 +451,16 @@ template <typename T> ss_status setup_group(ss_ctx* c, Group& g) {
     TRY(dalloc(c, (void**)&g.pair_on, (size_t)g.n_pairs * sizeof(int)));
     CUDA_TRY(c, cudaMemcpyAsync(g.d_str_img0, g.str_img0.data(), nstr * sizeof(int), cudaMemcpyHostToDevice, c->cs));
     CUDA_TRY(c, cudaMemcpyAsync(g.d_str_K, g.str_K.data(), nstr * sizeof(int), cudaMemcpyHostToDevice, c->cs));
+    std::vector<double> inv(nstr);
+    for (int i = 0; i < nstr; ++i) inv[i] = 1.0 / (double)(g.str_K[i] - 1);
+    CUDA_TRY(c, cudaMemcpyAsync(g.d_str_inv, inv.data(), nstr * sizeof(double), cudaMemcpyHostToDevice, c->cs));
     CUDA_TRY(c, cudaMemsetAsync(g.dpart, 0, (size_t)nstr * maxK * a.n_tiles * sizeof(double), c->cs));
     CUDA_TRY(c, cudaMemsetAsync(g.e_last, 0, (size_t)nstr * maxK * sizeof(double), c->cs));
     CUDA_TRY(c, cudaMemsetAsync(g.s, 0, g.n_img * M * sizeof(T), c->cs));
     CUDA_TRY(c, cudaMemsetAsync(g.sp, 0, g.n_img * M * sizeof(T), c->cs));
     a.str_img0 = g.d_str_img0;
     a.str_K = g.d_str_K;
+    a.str_inv = g.d_str_inv;
     a.dpart = g.dpart;
     a.e_last = g.e_last;
     a.cnt = g.arc_cnt;
@@ -1426,7 +1432,9 @@ ss_status ss_set_reparam(ss_ctx* c, int interp, int climb) {
             CUDA_TRY(c, cudaMemsetAsync(g.climb_img, 0, g.n_img * sizeof(int), c->cs));
         }
         if (interp == SS_INTERP_SPLINE && !a.W) {
-            TRY(dalloc(c, (void**)&a.W, nstr * mk * mk * sizeof(double)));
+            a.w_stride = spline_w_stride(a.maxK);
+            TRY(dalloc(c, (void**)&a.W, nstr * mk * a.w_stride * sizeof(double)));
+            CUDA_TRY(c, cudaMemsetAsync(a.W, 0, nstr * mk * a.w_stride * sizeof(double), c->cs));
             TRY(dalloc(c, (void**)&a.P, nstr * mk * mk * sizeof(double)));
             TRY(dalloc(c, (void**)&a.wcopy, nstr * mk * sizeof(int)));
             CUDA_TRY(c, cudaMemsetAsync(a.wcopy, 0xff, nstr * mk * sizeof(int), c->cs));

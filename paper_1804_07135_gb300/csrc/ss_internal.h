@@ -101,6 +101,7 @@ struct ArcArgs {
     int n_str;             // strings in the group
     const int* str_img0;   // [n_str] first group-local image of each string
     const int* str_K;      // [n_str] images per string
+    const double* str_inv; // [n_str] 1 / (images - 1)
     int maxK;
     int n_tiles;           // spatial tiles of the 3N component vector
     int tile_elems;        // components per tile
@@ -117,7 +118,8 @@ struct ArcArgs {
     double* cpart;         // [n_str][c_tiles][2] (F.tau, tau.tau) partials of the climbing image
     int c_tiles;           // site tiles of kClimbTile per image
     int spline;            // natural cubic spline: the finisher writes W, the apply kernel moves the images
-    double* W;             // [n_str][maxK][maxK] interpolation weights phi_k = sum_q W_kq phi*_q, stored in T
+    double* W;             // [n_str][maxK][w_stride] interpolation weights phi_k = sum_q W_kq phi*_q, [q][k], in T
+    int w_stride;          // spline_w_stride(maxK)
     double* P;             // [n_str][maxK][maxK] scratch: d m_i / d y_q of the spline (in T), column q contiguous
     int* wcopy;            // [n_str][maxK] row k is the identity (image kept as it is)
     int p_dim;             // spline operator columns kept in the finisher's dynamic shared memory (0: none)
@@ -125,6 +127,8 @@ struct ArcArgs {
 
 constexpr int kClimbTile = 256;   // sites per CTA of the climbing-image kernels (one per thread)
 constexpr int kSplineMaxK = 256;  // longest string the spline variant accepts
+constexpr int kSplineRows = 8;    // rows of W a thread of the apply kernel takes at once
+inline int spline_w_stride(int maxK) { return (maxK + kSplineRows - 1) / kSplineRows * kSplineRows + 4; }
 constexpr int kSplineSmemP = 64;  // parts of up to 63 segments keep the spline operator P in shared memory
 
 // Adaptive Runge-Kutta evolution (Sec. III, Dormand-Prince 5(4)): controller state of one ODE system

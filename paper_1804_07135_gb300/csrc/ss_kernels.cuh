@@ -82,10 +82,14 @@ __device__ __forceinline__ void block_reduce_d(double (&v)[NV], double* scratch 
 }
 
 // Block reduction of NV values per thread: summed in T within each warp (fixed shuffle tree), then
-// in FP64 across warps by thread 0 (fixed order).  out valid in thread 0.
+// in FP64 across warps by warp 0 (fixed tree).  out valid in thread 0.  The warp totals wait in T and become FP64
+// once, in warp 0, and the tree has as many levels as there are warps: GB300 issues about two FP64 lane
+// operations per clock and SM, whatever the number of active lanes, so every FP64 warp instruction counts
+// (8 instead of 26 per CTA of the step kernel).
 template <int NV, typename T>
 __device__ __forceinline__ void block_reduce_t2d(T (&v)[NV], double (&out)[NV], double* scratch /* [32*NV] */) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = (blockDim.x + 31) >> 5;
+    T* part = reinterpret_cast<T*>(scratch);
 #pragma unroll
     for (int k = 0; k < NV; ++k)
 #pragma unroll
@@ -93,16 +97,15 @@ __device__ __forceinline__ void block_reduce_t2d(T (&v)[NV], double (&out)[NV], 
     __syncthreads();
     if (lane == 0)
 #pragma unroll
-        for (int k = 0; k < NV; ++k) scratch[warp * NV + k] = double(v[k]);
+        for (int k = 0; k < NV; ++k) part[warp * NV + k] = v[k];
     __syncthreads();
-    // warp totals combined in FP64 by a fixed shuffle tree in warp 0 (dependent FP64 operations are
-    // slow on GB300, so a log-depth tree instead of a sequential loop)
     if (warp == 0) {
+        int top = 1;
+        while (top < nwarp) top <<= 1;  // uniform
 #pragma unroll
         for (int k = 0; k < NV; ++k) {
-            double a = lane < nwarp ? scratch[lane * NV + k] : 0.0;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
+            double a = lane < nwarp ? double(part[lane * NV + k]) : 0.0;
+            for (int o = top >> 1; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
             out[k] = a;
         }
     }
@@ -863,6 +866,22 @@ __device__ __forceinline__ unsigned ticket_acq_rel(unsigned* p) {
     return old;
 }
 
+// Sums of non-negative doubles in fixed point, for the finisher of the FP32 path: 64-bit integers aligned to the
+// largest term's exponent, `up` guard bits below its last place (n terms, up = 10 - ceil(log2 n) >= 0, sum below
+// 2^63 units), each term rounded to nearest.  The error is at most n / 2 units of 2^-(52 + up) of the largest term
+// (n = 128: 2^-49, an FP64 tree's bound is 2^-49 too), exact for terms within a factor 2^up of the largest.
+// Integer additions take a few cycles where a dependent FP64 one takes 65 and every FP64 warp instruction
+// occupies the SM's FP64 pipe for 16.
+__device__ __forceinline__ int fx_exp(unsigned long long bits) { return (int)(bits >> 52); }  // 0x7ff: not finite
+__device__ __forceinline__ unsigned long long fx_term(unsigned long long bits, int e_ref, int up) {
+    const int e = fx_exp(bits), s = e_ref - e;
+    if (e == 0 || s > 63) return 0ull;  // zero (or below 2^-1022)
+    const unsigned long long m = ((bits & 0xfffffffffffffull) | 0x10000000000000ull) << up;
+    return s == 0 ? m : (m + (1ull << (s - 1))) >> s;
+}
+__device__ __forceinline__ int fx_up(int n) { return 10 - (n > 1 ? 32 - __clz(n - 1) : 0); }
+constexpr int kFxTiles = 128;  // tile partials per distance the fixed-point finisher takes
+
 template <typename T>
 __device__ __noinline__ void arc_finish(const GroupArgs<T>& g, const ArcArgs& a, int str, int K, int img0,
                                         double* alpha, double* wsum);
@@ -886,6 +905,8 @@ __device__ __noinline__ void arc_finish_variants(const GroupArgs<T>& g, const Ar
                                                  int kc, const double* s) {
     __shared__ double xs[kArcMaxK];  // knot of image k within its part (kc: 1, the end of part one)
     __shared__ double hh_raw[kSplineMaxK], rh_raw[kSplineMaxK], rden_raw[kSplineMaxK], cp_raw[kSplineMaxK];
+    __shared__ double row_raw[4][kSplineMaxK];  // A, B, C, D of the row's segment
+    __shared__ int row_seg[kSplineMaxK];        // the segment
     // P of a part of up to a.p_dim - 1 segments stays on chip in the launch's dynamic shared memory (the
     // recurrences along a column are dependent, so each step's latency counts); longer parts use the
     // global scratch
@@ -894,7 +915,7 @@ __device__ __noinline__ void arc_finish_variants(const GroupArgs<T>& g, const Ar
     const int tid = threadIdx.x, nthr = blockDim.x;
     const bool split = kc > 0 && kc < K - 1;
     const size_t mk = (size_t)a.maxK;
-    T* W = reinterpret_cast<T*>(a.W) + (size_t)str * mk * mk;
+    T* W = reinterpret_cast<T*>(a.W) + (size_t)str * mk * a.w_stride;
     auto part_lo = [&](int k) { return split && k > kc ? kc : 0; };
     auto part_hi = [&](int k) { return split && k <= kc ? kc : K - 1; };
     for (int k = tid; k < K; k += nthr) {
@@ -934,12 +955,7 @@ __device__ __noinline__ void arc_finish_variants(const GroupArgs<T>& g, const Ar
             e.copy = 0;
         }
         const_cast<InterpEntry*>(g.interp)[img0 + k] = e;
-        if (a.spline) {
-            // identity rows for now; the interior rows of a moving part are rewritten below
-            T* wr = W + (size_t)k * mk;
-            for (int q = 0; q < K; ++q) wr[q] = q == k ? T(1) : T(0);
-            a.wcopy[(size_t)str * mk + k] = keep ? 1 : 0;
-        }
+        if (a.spline) a.wcopy[(size_t)str * mk + k] = keep ? 1 : 0;  // a kept image's row of W is not read
     }
     if (!a.spline) return;
     // the spline operator in the path's precision T (its weights are stored in T; FP64 arithmetic is slow
@@ -948,10 +964,11 @@ __device__ __noinline__ void arc_finish_variants(const GroupArgs<T>& g, const Ar
     T* rh = reinterpret_cast<T*>(rh_raw);
     T* rden = reinterpret_cast<T*>(rden_raw);
     T* cp = reinterpret_cast<T*>(cp_raw);
+    T(*row)[kSplineMaxK] = reinterpret_cast<T(*)[kSplineMaxK]>(row_raw);
     for (int part = 0; part < (split ? 2 : 1); ++part) {
         const int a0 = part == 0 ? 0 : kc, b0 = part == 0 && split ? kc : K - 1, n = b0 - a0;
         const double L = s[b0] - s[a0];
-        __syncthreads();  // identity rows written; the shared factors are free
+        __syncthreads();  // the shared factors are free
         if (!a.reparam || !(L > 0.0) || !isfinite(L) || n < 2) continue;  // uniform: nothing moves here
         bool pos = true;
         for (int i = tid; i < n; i += nthr) {
@@ -963,19 +980,27 @@ __device__ __noinline__ void arc_finish_variants(const GroupArgs<T>& g, const Ar
         const bool ok = __syncthreads_and(pos);
         const bool on_chip = n + 1 <= a.p_dim;
         T* P = on_chip ? reinterpret_cast<T*>(Psm) : reinterpret_cast<T*>(a.P) + (size_t)str * mk * mk;
-        const size_t ps = on_chip ? (size_t)a.p_dim : mk;  // column stride
+        const size_t ps = on_chip ? (size_t)(a.p_dim | 1) : mk;  // column stride (odd on chip: distinct banks)
+        // The recurrences are serial: each keeps its running value in a register and loads ahead of it, so a
+        // step costs the two dependent operations (and thread 0's division), not a trip to shared memory.
         if (ok && tid == 0) {  // elimination factors of the tridiagonal system (m_0 = m_n = 0 known)
+            T c = T(0);
+#pragma unroll 4
             for (int i = 1; i < n; ++i) {
-                const T den = T(2) * (hh[i - 1] + hh[i]) - (i > 1 ? hh[i - 1] * cp[i - 1] : T(0));
-                rden[i] = T(1) / den;
-                cp[i] = (i < n - 1 ? hh[i] : T(0)) * rden[i];
+                const T h0 = hh[i - 1], h1 = hh[i];
+                const T den = T(2) * (h0 + h1) - (i > 1 ? h0 * c : T(0));
+                const T rd = T(1) / den;
+                c = (i < n - 1 ? h1 : T(0)) * rd;
+                rden[i] = rd;
+                cp[i] = c;
             }
         }
         __syncthreads();
         if (ok) {
             for (int q = tid; q <= n; q += nthr) {  // column q of P: d m_i / d y_q, i = 1..n-1
-                T* pc = P + (size_t)q * ps;
+                T* __restrict__ pc = P + (size_t)q * ps;
                 T d = T(0);
+#pragma unroll 4
                 for (int i = 1; i < n; ++i) {
                     T r = T(0);  // d rhs_i / d y_q
                     if (q == i + 1) r = T(6) * rh[i];
@@ -984,7 +1009,11 @@ __device__ __noinline__ void arc_finish_variants(const GroupArgs<T>& g, const Ar
                     d = (r - (i > 1 ? hh[i - 1] * d : T(0))) * rden[i];
                     pc[i] = d;
                 }
-                for (int i = n - 2; i >= 1; --i) pc[i] -= cp[i] * pc[i + 1];
+#pragma unroll 4
+                for (int i = n - 2; i >= 1; --i) {
+                    d = pc[i] - cp[i] * d;
+                    pc[i] = d;
+                }
             }
             __syncthreads();
         }
@@ -998,29 +1027,40 @@ __device__ __noinline__ void arc_finish_variants(const GroupArgs<T>& g, const Ar
                 while (knot(j, a0) > ak);
             }
             const double x0 = knot(j, a0), x1 = knot(j + 1, a0);
-            T* wr = W + (size_t)k * mk;
-            wr[k] = T(0);
-            if (!ok) {
-                const double t = (ak - x0) / (x1 - x0);
-                wr[j] = T(1.0 - t);
-                wr[j + 1] = T(t);
-                continue;
-            }
             const int jr = j - a0;
-            const T h = hh[jr], A = T(x1 - ak) * rh[jr], B = T(ak - x0) * rh[jr];
-            const T C = h * h * (A * A * A - A) * T(1.0 / 6.0), D = h * h * (B * B * B - B) * T(1.0 / 6.0);
-            for (int q = 0; q <= n; ++q) {
-                const T* pc = P + (size_t)q * ps;
-                const T mj = jr > 0 ? pc[jr] : T(0), mj1 = jr + 1 < n ? pc[jr + 1] : T(0);
-                wr[a0 + q] = (q == jr ? A : T(0)) + (q == jr + 1 ? B : T(0)) + C * mj + D * mj1;
+            T A, B, C = T(0), D = T(0);
+            if (ok) {
+                const T h = hh[jr];
+                A = T(x1 - ak) * rh[jr], B = T(ak - x0) * rh[jr];
+                C = h * h * (A * A * A - A) * T(1.0 / 6.0), D = h * h * (B * B * B - B) * T(1.0 / 6.0);
+            } else {  // a zero-length segment: linear rows
+                const double t = (ak - x0) / (x1 - x0);
+                A = T(1.0 - t), B = T(t);
             }
+            row[0][k] = A, row[1][k] = B, row[2][k] = C, row[3][k] = D;
+            row_seg[k] = jr;
+        }
+        __syncthreads();
+        // the rows of W, all threads over (column, row), rows fastest as they are stored
+        for (int e = tid; e < (n - 1) * K; e += nthr) {
+            const int qk = e / (n - 1), k = a0 + 1 + e - qk * (n - 1), q = qk - a0, jr = row_seg[k];
+            T w = T(0);
+            if (q >= 0 && q <= n) {
+                w = (q == jr ? row[0][k] : T(0)) + (q == jr + 1 ? row[1][k] : T(0));
+                if (ok) {
+                    const T* pc = P + (size_t)q * ps;
+                    const T mj = jr > 0 ? pc[jr] : T(0), mj1 = jr + 1 < n ? pc[jr + 1] : T(0);
+                    w = w + row[2][k] * mj + row[3][k] * mj1;
+                }
+            }
+            W[(size_t)qk * a.w_stride + k] = w;
         }
     }
 }
 
 template <typename T>
 __global__ void __launch_bounds__(256, 3) arc_kernel(GroupArgs<T> g, ArcArgs a) {
-    __shared__ double red[32 * kArcMaxChunk];
+    __shared__ T red[32 * kArcMaxChunk];
     __shared__ double alpha[kArcMaxK];  // d_k, then s_k, then alpha*_k
     __shared__ double wsum[32];
     __shared__ int s_flag;
@@ -1035,6 +1075,20 @@ __global__ void __launch_bounds__(256, 3) arc_kernel(GroupArgs<T> g, ArcArgs a) 
     griddep_launch_dependents();
     if (chunk >= n_act) return;  // uniform over the block
     const size_t sb = (size_t)str * a.maxK;
+    // images that stay where they are (no reparametrisation, no climbing image to pick): nothing depends on the
+    // distances but the check for non-finite states, so there is no finisher, and the identity table is written here
+    const bool still = !a.reparam && !a.climb && !a.spline;
+    if (still && blockIdx.x == 0)
+        for (int k = k_lo + tid; k < (chunk == n_act - 1 ? K : k_lo + a.kchunk); k += nthr) {
+            InterpEntry e;
+            e.src0 = e.src1 = img0 + k;
+            e.t = 0.0;
+            e.tf = 0.f;
+            e.omtf = 1.f;
+            e.copy = 1;
+            e.pad = 0;
+            const_cast<InterpEntry*>(g.interp)[img0 + k] = e;
+        }
     if ((int)blockIdx.x == n_tiles) {
         // e_last of the chunk's images from the step kernel's partials
         const int k_hi = chunk == n_act - 1 ? K : k_lo + a.kchunk;
@@ -1104,37 +1158,38 @@ __global__ void __launch_bounds__(256, 3) arc_kernel(GroupArgs<T> g, ArcArgs a) 
         for (int o = 16; o > 0; o >>= 1) part[i] += __shfl_down_sync(0xffffffffu, part[i], o);
     if (lane == 0)
 #pragma unroll
-        for (int i = 0; i < kArcMaxChunk; ++i) red[warp * kArcMaxChunk + i] = double(part[i]);
+        for (int i = 0; i < kArcMaxChunk; ++i) red[warp * kArcMaxChunk + i] = part[i];
     __syncthreads();
     if (warp == 0) {
         static_assert(kArcMaxChunk * 4 == 32, "one lane per (difference, quarter)");
         const int i = lane >> 2, q = lane & 3;
         double v = 0.0;
-        for (int w = q; w < nwarp; w += 4) v += red[w * kArcMaxChunk + i];
+        for (int w = q; w < nwarp; w += 4) v += double(red[w * kArcMaxChunk + i]);
         v += __shfl_down_sync(0xffffffffu, v, 2);
         v += __shfl_down_sync(0xffffffffu, v, 1);
+        if (still) {
+            if (q == 0 && i < nd && !isfinite(v)) atomicOr(g.err, kErrNonFinite);
+            return;
+        }
         if (q == 0 && i < nd) a.dpart[((size_t)str * a.maxK + k_lo + i + 1) * n_tiles + blockIdx.x] = v;
         __syncwarp();
         if (lane == 0)
             s_flag = ticket_acq_rel(&a.cnt[str]) == (unsigned)((n_tiles + (a.climb ? 1 : 0)) * n_act - 1);
     }
+    if (still) return;  // uniform
     __syncthreads();
     if (!s_flag) return;
     arc_finish(g, a, str, K, img0, alpha, wsum);
 }
 
-// The last CTA of a string (every partial it needs is visible after its ticket): distances, arc
-// length, and the reparametrisation of the variant in use.
+// d_k and s_k of a string in FP64 (the FP64 path; more tiles or images than the fixed-point finisher takes): 8 lanes
+// per difference (lane = 8 j + l, four differences per warp), lane l summing tiles l, l + 8, ... in order (loads
+// twelve at a time), then a three-level tree over l.
 template <typename T>
-__device__ __noinline__ void arc_finish(const GroupArgs<T>& g, const ArcArgs& a, int str, int K, int img0,
-                                        double* alpha, double* wsum) {
+__device__ __noinline__ void arc_lengths_f64(const GroupArgs<T>& g, const ArcArgs& a, int str, int K, double* alpha,
+                                             double* wsum) {
     const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5, nwarp = nthr >> 5;
     const int n_tiles = a.n_tiles;
-    // ---- last tile CTA of the string: d_k for k = 1..K-1 ----
-    // 8 lanes per difference (lane = 8 j + l, four differences per warp), lane l summing tiles l, l + 8,
-    // ... in order (loads twelve at a time), then a three-level tree over l: few FP64 instructions, as
-    // GB300 issues FP64 at a low rate
-    if (tid == 0) a.cnt[str] = 0u;  // every tile CTA of the string has counted
     {
         const double* dp = a.dpart + (size_t)str * a.maxK * n_tiles;  // [k][tile]
         const int j = lane >> 3, l = lane & 7;
@@ -1219,52 +1274,125 @@ __device__ __noinline__ void arc_finish(const GroupArgs<T>& g, const ArcArgs& a,
         }
     }
     __syncthreads();
+}
+
+// The last CTA of a string (every partial it needs is visible after its ticket): distances, arc
+// length, and the reparametrisation of the variant in use.
+template <typename T>
+__device__ __noinline__ void arc_finish(const GroupArgs<T>& g, const ArcArgs& a, int str, int K, int img0,
+                                        double* alpha, double* wsum) {
+    const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5, nwarp = nthr >> 5;
+    const int n_tiles = a.n_tiles;
+    // ---- last tile CTA of the string: d_k for k = 1..K-1 and their sums ----
+    if (tid == 0) a.cnt[str] = 0u;  // every tile CTA of the string has counted
+    const bool fx = std::is_same<T, float>::value && n_tiles <= kFxTiles && K <= nthr;  // uniform
+    if (fx) {
+        const unsigned long long* dp = reinterpret_cast<const unsigned long long*>(a.dpart) + (size_t)str * a.maxK * n_tiles;
+        const int j = lane >> 3, l = lane & 7, up = fx_up(n_tiles);
+        for (int k0 = 1 + 4 * warp; k0 < K; k0 += 4 * nwarp) {
+            const int k = k0 + j;
+            unsigned long long x[kFxTiles / 8], s = 0ull;
+            int e = 0;
+#pragma unroll
+            for (int q = 0; q < kFxTiles / 8; ++q) {
+                const int t = l + 8 * q;
+                x[q] = k < K && t < n_tiles ? __ldcg(dp + (size_t)k * n_tiles + t) : 0ull;
+            }
+#pragma unroll
+            for (int q = 0; q < kFxTiles / 8; ++q) e = max(e, fx_exp(x[q]));
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
+#pragma unroll
+            for (int q = 0; q < kFxTiles / 8; ++q) s += fx_term(x[q], e, up);
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (l == 0 && k < K) {
+                double d = 0.0;
+                if (e >= 0x7ff) {  // (a negative NaN's sign bit included)
+                    atomicOr(g.err, kErrNonFinite);
+                    d = NAN;
+                } else if (e > 75) {  // units of 2^(e - 1075 - up)
+                    d = sqrt_nr(__ull2double_rn(s) * __hiloint2double((e - 52 - up) << 20, 0));
+                }
+                alpha[k] = d;  // d_k (Eq. 11)
+            }
+        }
+        if (tid == 0) alpha[0] = 0.0;
+        __syncthreads();
+        // s_k = d_1 + ... + d_k (Eq. 11), one image per thread, in fixed-point units: only ratios of arc lengths
+        // are used from here on
+        __shared__ unsigned long long fsum[32];
+        __shared__ int fmax_e[32];
+        const int nw = (K + 31) >> 5;  // warps holding images
+        const unsigned long long db = tid < K ? (unsigned long long)__double_as_longlong(alpha[tid]) : 0ull;
+        int e = 0;
+        if (warp < nw) {
+            e = (int)__reduce_max_sync(0xffffffffu, (unsigned)fx_exp(db));
+            if (nw > 1 && lane == 0) fmax_e[warp] = e;
+        }
+        if (nw > 1) {  // uniform over the block
+            __syncthreads();
+            for (int w = 0; w < nw; ++w) e = max(e, fmax_e[w]);
+        }
+        unsigned long long v = 0ull;
+        if (warp < nw) {
+            v = fx_term(db, e, fx_up(K));
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned long long u = __shfl_up_sync(0xffffffffu, v, o);
+                if (lane >= o) v += u;
+            }
+            if (nw > 1 && lane == 31) fsum[warp] = v;
+        }
+        if (nw > 1) {
+            __syncthreads();
+            for (int w = 0; w < warp && w < nw; ++w) v += fsum[w];
+        }
+        if (tid < K) alpha[tid] = e >= 0x7ff ? NAN : __ull2double_rn(v);
+        __syncthreads();
+    } else {
+        arc_lengths_f64(g, a, str, K, alpha, wsum);
+    }
     const int kcur = a.climb ? a.kc[str] : -1;  // the image that climbed in this iteration
     if (a.spline || (kcur > 0 && kcur < K - 1)) {
         arc_finish_variants(g, a, str, K, img0, kcur, alpha);
     } else {
         const double sK = alpha[K - 1];
         const bool move = a.reparam && sK > 0.0 && isfinite(sK);
-        if (move && warp < nw) {
-            const double r = rcp_nr(sK);
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (q < per && kb + q < K) alpha[kb + q] *= r;  // alpha*_k = s_k / s_{K-1} (Eq. 12)
-        }
-        __syncthreads();
-        if (warp < nw) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int k = kb + q;
-                if (q >= per || k >= K) continue;
-                InterpEntry e;
-                e.src0 = img0 + k;
-                e.src1 = img0 + k;
-                e.t = 0.0;
-                e.tf = 0.f;
-                e.omtf = 1.f;
-                e.copy = 1;
-                e.pad = 0;
-                if (move && k > 0 && k < K - 1) {
-                    const double ak = (double)k / (double)(K - 1);
-                    // largest j in [0, K-2] with alpha*_j <= ak (alpha* is non-decreasing; alpha*_0 = 0 <= ak),
-                    // walking from j = k: after a few iterations the images are nearly evenly spaced
-                    int j = min(k, K - 2);
-                    if (alpha[j] <= ak) {
-                        while (j < K - 2 && alpha[j + 1] <= ak) ++j;
-                    } else {
-                        do --j;
-                        while (alpha[j] > ak);
-                    }
-                    e.src0 = img0 + j;
-                    e.src1 = img0 + j + 1;
-                    e.t = (ak - alpha[j]) * rcp_nr(alpha[j + 1] - alpha[j]);
-                    e.tf = (float)e.t;
-                    e.omtf = (float)(1.0 - e.t);
-                    e.copy = 0;
+        const double step = move ? sK * a.str_inv[str] : 0.0;  // s_{K-1} / (K-1)
+        for (int k = tid; k < K; k += nthr) {
+            InterpEntry e;
+            e.src0 = img0 + k;
+            e.src1 = img0 + k;
+            e.t = 0.0;
+            e.tf = 0.f;
+            e.omtf = 1.f;
+            e.copy = 1;
+            e.pad = 0;
+            if (move && k > 0 && k < K - 1) {
+                // Eq. 12 scaled by s_{K-1}: alpha*_j <= k / (K-1) is s_j <= k s_{K-1} / (K-1)
+                const double sk = (double)k * step;
+                // largest j in [0, K-2] with s_j <= sk (s is non-decreasing; s_0 = 0 <= sk), walking from j = k:
+                // after a few iterations the images are nearly evenly spaced
+                int j = min(k, K - 2);
+                if (alpha[j] <= sk) {
+                    while (j < K - 2 && alpha[j + 1] <= sk) ++j;
+                } else {
+                    do --j;
+                    while (alpha[j] > sk);
                 }
-                const_cast<InterpEntry*>(g.interp)[img0 + k] = e;
+                // t = num / den: an FP32 reciprocal, then the quotient's residual (~1e-14 relative)
+                const double num = sk - alpha[j], den = alpha[j + 1] - alpha[j];
+                const double r = (double)(1.0f / (float)den);
+                const double t0 = num * r;
+                e.src0 = img0 + j;
+                e.src1 = img0 + j + 1;
+                e.t = std::is_same<T, float>::value ? fma(fma(-t0, den, num), r, t0) : num / den;
+                e.tf = (float)e.t;
+                e.omtf = (float)(1.0 - e.t);
+                e.copy = 0;
             }
+            const_cast<InterpEntry*>(g.interp)[img0 + k] = e;
         }
     }
     if (a.climb) {
@@ -1670,6 +1798,8 @@ __device__ __forceinline__ void climb_site(const GroupArgs<T>& g, const T* hc, i
 template <typename T>
 __global__ void __launch_bounds__(256) climb_dot_kernel(GroupArgs<T> g, ArcArgs a, const T* hc) {
     __shared__ double red[64];
+    griddep_wait();
+    griddep_launch_dependents();
     const int str = blockIdx.y, K = a.str_K[str], kc = a.kc[str];
     if (!(kc > 0 && kc < K - 1)) return;  // uniform over the CTA
     const int img = a.str_img0[str] + kc;
@@ -1693,6 +1823,8 @@ __global__ void __launch_bounds__(256) climb_dot_kernel(GroupArgs<T> g, ArcArgs 
 template <typename T>
 __global__ void __launch_bounds__(256) climb_apply_kernel(GroupArgs<T> g, ArcArgs a, const T* hc, T dt) {
     __shared__ double coef;
+    griddep_wait();
+    griddep_launch_dependents();
     const int str = blockIdx.y, K = a.str_K[str], kc = a.kc[str];
     if (!(kc > 0 && kc < K - 1)) return;  // uniform over the CTA
     const int img = a.str_img0[str] + kc;
@@ -1724,41 +1856,74 @@ __global__ void __launch_bounds__(256) climb_apply_kernel(GroupArgs<T> g, ArcArg
 }
 
 // ---- natural cubic spline: phi_k = normalise(sum_q W_kq phi*_q) in place on sp -----------------------
-// grid (ceil(N / 32), n_str), 256 threads: 32 sites x 8 groups of output rows (row k to group k % 8).
-// Dynamic shared memory: the string's K images at the CTA's 32 sites, [K][3][32], then W [K][K] when
-// w_on_chip (else W is read through L1).  The tile is loaded whole before any row is written back.
+// grid (ceil(N / 32), n_str), 256 threads: 32 sites x 8 groups of output rows, eight consecutive rows per thread
+// and pass (a group's first rows 8 grp, 8 grp + 64, ...), so a spin loaded from shared memory serves eight rows
+// and their weights come as vectors: 24 multiply-adds for 3 + 2 loads instead of 3 for 4.  Dynamic shared
+// memory: the string's K images at the CTA's 32 sites, [K][3][32], then W, [q][row] at row stride a.w_stride (whole
+// vectors, off a multiple of 32 words), when w_on_chip (else W is read through L1).  The tile is loaded whole before any row is written back.  Bound by
+// FP32 issue (2 K^2 N x 3 multiply-adds); 112x112x1 x 60 images: SPLINE_APPLY on one GB300.
 template <typename T>
 __global__ void __launch_bounds__(256) spline_apply_kernel(GroupArgs<T> g, ArcArgs a, int w_on_chip) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T* y = reinterpret_cast<T*>(smem_raw);
     const int str = blockIdx.y, tid = threadIdx.x, lane = tid & 31, grp = tid >> 5;
-    const int K = a.str_K[str], img0 = a.str_img0[str], N = g.N;
+    const int K = a.str_K[str], img0 = a.str_img0[str], N = g.N, ws = a.w_stride;
     const size_t M = (size_t)3 * N, mk = (size_t)a.maxK;
     const int* wc = a.wcopy + (size_t)str * mk;
-    const T* Wg = reinterpret_cast<const T*>(a.W) + (size_t)str * mk * mk;
+    const T* Wg = reinterpret_cast<const T*>(a.W) + (size_t)str * mk * ws;
     T* Ws = y + (size_t)K * 96;
     const int i0 = blockIdx.x * 32, i = i0 + lane;
-    for (int e = tid; e < K * 96; e += 256) {  // (q, c, site): 32 consecutive sites per warp load
-        const int q = e / 96, r = e - 96 * q, c = r >> 5, l = r & 31;
-        y[e] = i0 + l < N ? g.sp[(size_t)(img0 + q) * M + (size_t)c * N + i0 + l] : T(0);
+    griddep_wait();
+    griddep_launch_dependents();
+    // row r of the tile: component r % 3 of image r / 3 at 32 consecutive sites; eight loads in flight per thread
+    const T* src = g.sp + (size_t)img0 * M + i;
+    for (int r0 = grp; r0 < 3 * K; r0 += 64) {
+        T v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = i < N && r0 + 8 * u < 3 * K ? src[(size_t)(r0 + 8 * u) * N] : T(0);
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (r0 + 8 * u < 3 * K) y[(r0 + 8 * u) * 32 + lane] = v[u];
     }
-    if (w_on_chip)
-        for (int e = tid; e < K * K; e += 256) Ws[e] = Wg[(size_t)(e / K) * mk + e % K];
+    if (w_on_chip) {
+        const int nv = (int)((size_t)K * ws * sizeof(T) / 16);
+#pragma unroll 4
+        for (int e = tid; e < nv; e += 256) reinterpret_cast<int4*>(Ws)[e] = reinterpret_cast<const int4*>(Wg)[e];
+    }
     __syncthreads();
     if (i >= N) return;
-    for (int k = 1 + grp; k < K - 1; k += 8) {
-        if (wc[k]) continue;  // kept in place
-        T u[3] = {T(0), T(0), T(0)};
-        const T* wr = w_on_chip ? Ws + (size_t)k * K : Wg + (size_t)k * mk;
+    const T* Wr = w_on_chip ? Ws : Wg;
+    for (int k0 = kSplineRows * grp; k0 < K - 1; k0 += 8 * kSplineRows) {
+        T u[kSplineRows][3];
+#pragma unroll
+        for (int r = 0; r < kSplineRows; ++r) u[r][0] = u[r][1] = u[r][2] = T(0);
+#pragma unroll 2
         for (int q = 0; q < K; ++q) {
-            const T w = wr[q];
+            const T y0 = y[q * 96 + lane], y1 = y[q * 96 + 32 + lane], y2 = y[q * 96 + 64 + lane];
+            constexpr int NV = kSplineRows * sizeof(T) / 16;
+            union {
+                int4 v[NV];
+                T t[kSplineRows];
+            } w;
+            const int4* wv = reinterpret_cast<const int4*>(Wr + (size_t)q * ws + k0);
 #pragma unroll
-            for (int c = 0; c < 3; ++c) u[c] += w * y[q * 96 + c * 32 + lane];
+            for (int v = 0; v < NV; ++v) w.v[v] = wv[v];
+#pragma unroll
+            for (int r = 0; r < kSplineRows; ++r) {
+                u[r][0] += w.t[r] * y0;
+                u[r][1] += w.t[r] * y1;
+                u[r][2] += w.t[r] * y2;
+            }
         }
-        const T r = rsqrt_t<T>(u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
-        T* o = g.sp + (size_t)(img0 + k) * M + i;
 #pragma unroll
-        for (int c = 0; c < 3; ++c) o[(size_t)c * N] = u[c] * r;
+        for (int r = 0; r < kSplineRows; ++r) {
+            const int k = k0 + r;
+            if (k < 1 || k >= K - 1 || wc[k]) continue;  // kept in place
+            const T n = rsqrt_t<T>(u[r][0] * u[r][0] + u[r][1] * u[r][1] + u[r][2] * u[r][2]);
+            T* o = g.sp + (size_t)(img0 + k) * M + i;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) o[(size_t)c * N] = u[r][c] * n;
+        }
     }
 }
 
@@ -2087,22 +2252,22 @@ template <typename T> void launch_dipole_direct(const GroupArgs<T>& g, T* hdir, 
 
 template <typename T> void launch_climb(const GroupArgs<T>& g, const ArcArgs& a, T dt, const T* hc, cudaStream_t st) {
     const dim3 grid(a.c_tiles, a.n_str);
-    climb_dot_kernel<T><<<grid, 256, 0, st>>>(g, a, hc);
-    climb_apply_kernel<T><<<grid, 256, 0, st>>>(g, a, hc, dt);
+    launch_pdl(climb_dot_kernel<T>, grid, dim3(256), 0, st, g, a, hc);
+    launch_pdl(climb_apply_kernel<T>, grid, dim3(256), 0, st, g, a, hc, dt);
 }
 
-// The spline apply kernel's shared memory for strings of up to maxK images: the [maxK][3][32] tile, and
-// W on chip when both fit in 200 KB.
-template <typename T> size_t spline_smem(int maxK, bool* w_on_chip) {
-    const size_t tile = (size_t)maxK * 96 * sizeof(T), w = (size_t)maxK * maxK * sizeof(T);
-    *w_on_chip = tile + w <= 200 * 1024;
+// The spline apply kernel's shared memory for strings of up to maxK images: the [maxK][3][32] tile, and W
+// on chip when both fit in 220 KB.
+template <typename T> size_t spline_smem(int maxK, int w_stride, bool* w_on_chip) {
+    const size_t tile = (size_t)maxK * 96 * sizeof(T), w = (size_t)maxK * w_stride * sizeof(T);
+    *w_on_chip = tile + w <= 220 * 1024;
     return *w_on_chip ? tile + w : tile;
 }
 
 template <typename T> void launch_spline_apply(const GroupArgs<T>& g, const ArcArgs& a, int maxK, cudaStream_t st) {
     bool on_chip = false;
-    const size_t sm = spline_smem<T>(maxK, &on_chip);
-    spline_apply_kernel<T><<<dim3((g.N + 31) / 32, a.n_str), 256, sm, st>>>(g, a, on_chip ? 1 : 0);
+    const size_t sm = spline_smem<T>(maxK, a.w_stride, &on_chip);
+    launch_pdl(spline_apply_kernel<T>, dim3((g.N + 31) / 32, a.n_str), dim3(256), sm, st, g, a, on_chip ? 1 : 0);
 }
 
 template <typename T> void launch_rk_assemble(const GroupArgs<T>& g, const RkArgs<T>& r, int stage, cudaStream_t st) {
@@ -2134,7 +2299,7 @@ template <typename T> void launch_rk_commit(const GroupArgs<T>& g, const RkArgs<
 
 template <typename T> void launch_arc(const GroupArgs<T>& g, const ArcArgs& a, int nthr, cudaStream_t st) {
     dim3 grid(a.n_tiles + 1, a.n_kchunks, a.n_str);  // + one energy CTA per chunk
-    launch_pdl(arc_kernel<T>, grid, dim3(nthr), (size_t)a.p_dim * a.p_dim * sizeof(double), st, g, a);
+    launch_pdl(arc_kernel<T>, grid, dim3(nthr), (size_t)a.p_dim * (a.p_dim | 1) * sizeof(T), st, g, a);
 }
 
 template <typename T>
@@ -2195,7 +2360,7 @@ template <typename T> void set_smem_limits(int bytes) {
     set_dyn_smem(xinv_kernel<T, false, 4>, bytes, carve);
     set_dyn_smem(xinv_kernel<T, true, 5>, bytes);
     set_dyn_smem(xinv_kernel<T, false, 5>, bytes, carve);
-    set_dyn_smem(spline_apply_kernel<T>, 200 * 1024, carve);
+    set_dyn_smem(spline_apply_kernel<T>, bytes, carve);
     set_dyn_smem(arc_kernel<T>, bytes, carve);
     set_dyn_smem(climb_dot_kernel<T>, bytes, carve);
 #define SS_CASE(M)                                                  \
