@@ -654,14 +654,12 @@ def rk_kernel_times(binding, sm, spec, kind, reps=5):
     for n, t in zip(names, ms):
         per[n] = per.get(n, 0.0) + float(t)
     units = spec.n_sites * spec.n_images
-    # algorithmic bytes per site-image (FP32 components, 12 bytes per spin vector): stage s assembles
-    # from y0 and s earlier stages into the stage state, (s + 2) x 12; finish reads y0 and every stage
-    # and writes y5, (stages + 2) x 12
-    b_asm = sum((st + 2) * 12 for st in range(stages)) * units
+    # algorithmic bytes per site-image (FP32 components, 12 bytes per spin vector): finish reads y0 and every
+    # stage and writes y5, (stages + 2) x 12 (the stages' states are formed by the x-inverse kernel: their
+    # entry is empty)
     b_fin = (stages + 2) * 12 * units
     peaks, _ = measured_peaks()
     return {"ms_per_round": {k: round(v, 5) for k, v in per.items()},
-            "assemble_gbs": b_asm / (per["assemble"] * 1e-3) / 1e9,
             "finish_gbs": b_fin / (per["finish"] * 1e-3) / 1e9,
             "hbm_peak_gbs": peaks["hbm_gbs"],
             "note": f"launched one by one; the round's arrays (about {(stages + 4) * 12 * units / 1e9:.2g} GB) "

@@ -148,8 +148,9 @@ ss_status ss_energy_terms(ss_ctx* ctx, int string, double* out);
  * dipole term), the direct dipole sums (with SS_DIPOLE_DIRECT), xinv (in its step, climbing-image or LLG
  * mode), the two climbing-image kernels as one entry (climbing image on), arc (which also
  * reparametrises), the spline apply kernel (spline on).  Runge-Kutta integrators, for each size group an
- * iteration with a single attempt round: the interval's opening (x-forward, copy into y0, control) as
- * one entry, per stage the assembly, xfwd, yz, direct sums and xinv (force mode) as above, then finish,
+ * iteration with a single attempt round: the interval's opening (x-forward, into y0, control) as
+ * one entry, per stage the assembly (an empty entry: the previous stage's xinv forms the state), xfwd (empty
+ * without the FFT dipole term), yz, direct sums and xinv (force mode) as above, then finish,
  * control, commit, arc and spline apply (an interval that needs more attempts is left unfinished; the
  * next ss_step opens a new one).  *n_out receives the number of entries.  The strings advance by
  * reps + 1 iterations.  Synchronises. */

@@ -713,22 +713,45 @@ int rk_sys_count(const ss_ctx* c, const StringRec& r) {
     return rk_per_image(c->integrator) ? r.d.n_images : 1;
 }
 
-// One attempt round of size group g (Sec. III) on stream st: for every stage i, Y_i from y0 and the
-// earlier stages, then k_i = F(Y_i) through the field pipeline (identity table) and the step kernel in
-// force mode; then the fifth-order solution with its scaled error, the step-size control and the commit of
-// accepted attempts.  The first round of an interval also sums the energies of the state the interval
-// starts from (its stage 0 is that state).
+// The arguments of stage s of an attempt: its state Y_s lies in one buffer, which x-forward transforms in place
+// (identity table) and the x-inverse kernel reads; that kernel writes k_s and, from it, y0 and the earlier forces,
+// Y_{s+1} into the next buffer -- y0 itself is Y_0, then sp and s take turns, so no state is copied and none is
+// assembled by a kernel of its own (which read k_s again and took a launch per stage).
+template <typename T> GroupArgs<T> rk_stage_args(const ss_ctx* c, const Group& g, const RkArgs<T>& r, int s) {
+    GroupArgs<T> a = group_args<T>(c, g);
+    a.interp = g.interp_ident;
+    a.s = a.sp = s == 0 ? r.y0 : s % 2 == 1 ? (T*)g.sp : (T*)g.s;
+    if (s + 1 < r.dp.stages) {
+        a.rk.y0 = r.y0;
+        a.rk.k = r.k;
+        a.rk.stride = (size_t)3 * g.N * g.n_img;
+        a.rk.out = (s + 1) % 2 == 1 ? (T*)g.sp : (T*)g.s;
+        a.rk.n = s;
+        for (int q = 0; q < s; ++q) a.rk.a[q] = r.dp.a[s + 1][q];
+        a.rk.a_cur = r.dp.a[s + 1][s];
+        a.rk.st = r.st;
+        a.rk.img_sys = r.img_sys;
+    }
+    return a;
+}
+
+// One attempt round of size group g (Sec. III) on stream st: every stage through the field pipeline, k_i = F(Y_i)
+// and the next stage's state from the x-inverse kernel in force mode; then the fifth-order solution with its
+// scaled error, the step-size control and the commit of accepted attempts.  The first round of an interval also
+// sums the energies of the state the interval starts from (its stage 0 is that state).
 template <typename T> void issue_rk_round(ss_ctx* c, Group& g, bool first, cudaStream_t st) {
     GroupArgs<T> ai = group_args<T>(c, g);
     ai.interp = g.interp_ident;
     RkArgs<T> r = rk_args<T>(c, g);
     const size_t stride = (size_t)3 * g.N * g.n_img;
     for (int s = 0; s < r.dp.stages; ++s) {
-        launch_rk_assemble<T>(ai, r, s, st);
-        launch_xfwd<T>(ai, g.dipole, g.thr_a, g.smem_a, st);
-        if (g.dipole) launch_yz<T>(ai, g.thr_b, g.smem_b, st);
-        if (g.direct) launch_dipole_direct<T>(ai, (T*)g.hdir, (const T*)g.dtab, st);
-        launch_xinv_force<T>(ai, g.dipole, r.k + s * stride, first && s == 0, c->dynamics == SS_DYN_LLG, g.thr_c,
+        const GroupArgs<T> a = rk_stage_args<T>(c, g, r, s);
+        if (g.dipole) {  // without it nothing reads the spectrum, and the state is in place
+            launch_xfwd<T>(a, true, g.thr_a, g.smem_a, st);
+            launch_yz<T>(a, g.thr_b, g.smem_b, st);
+        }
+        if (g.direct) launch_dipole_direct<T>(a, (T*)g.hdir, (const T*)g.dtab, st);
+        launch_xinv_force<T>(a, g.dipole, r.k + s * stride, first && s == 0, c->dynamics == SS_DYN_LLG, g.thr_c,
                              g.smem_c_eval, st);
     }
     launch_rk_finish<T>(ai, r, st);
@@ -746,9 +769,10 @@ template <typename T> cudaError_t capture_rk_group_iteration(ss_ctx* c, Group& g
     GroupArgs<T> ai = a;
     ai.interp = g.interp_ident;
     RkArgs<T> r = rk_args<T>(c, g);
-    launch_xfwd<T>(a, false, g.thr_a, 0, st);  // s = reparametrised state
-    cudaError_t e = cudaMemcpyAsync(r.y0, a.s, (size_t)3 * g.N * g.n_img * sizeof(T), cudaMemcpyDeviceToDevice, st);
-    if (e != cudaSuccess) return e;
+    cudaError_t e = cudaSuccess;
+    GroupArgs<T> a0 = a;
+    a0.s = r.y0;
+    launch_xfwd<T>(a0, false, g.thr_a, 0, st);  // y0 = reparametrised state
     launch_rk_control<T>(ai, r, 1, st);
     issue_rk_round<T>(c, g, true, st);
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -784,8 +808,9 @@ template <typename T> cudaError_t capture_rk_group_iteration(ss_ctx* c, Group& g
 }
 
 // The launches of one Runge-Kutta iteration of group g with a single attempt round, as the timing entries
-// of ss_time_kernels in launch order: the interval's opening (x-forward of the reparametrised state, copy
-// into y0, control in its opening mode), per stage its assembly, x-forward, y/z (FFT dipole term), direct
+// of ss_time_kernels in launch order: the interval's opening (x-forward of the reparametrised state
+// into y0, control in its opening mode), per stage an empty entry (the assembly of its state, which the previous
+// stage's x-inverse kernel does), its x-forward and y/z (FFT dipole term), direct
 // dipole sums (SS_DIPOLE_DIRECT) and x-inverse in force mode, then finish, control, commit, arc and the
 // spline apply kernel (spline on).  An interval that needs more than one attempt is left unfinished (the
 // next ss_step opens a new one).  which_only < 0 launches nothing and returns the number of entries.
@@ -802,17 +827,21 @@ template <typename T> int rk_time_entries(ss_ctx* c, Group& g, int which_only) {
         ++e;
     };
     entry(true, [&] {
-        launch_xfwd<T>(a, false, g.thr_a, 0, c->cs);
-        cudaMemcpyAsync(r.y0, a.s, stride * sizeof(T), cudaMemcpyDeviceToDevice, c->cs);
+        GroupArgs<T> a0 = a;
+        a0.s = r.y0;
+        launch_xfwd<T>(a0, false, g.thr_a, 0, c->cs);
         launch_rk_control<T>(ai, r, 1, c->cs);
     });
     for (int st = 0; st < r.dp.stages; ++st) {
-        entry(true, [&] { launch_rk_assemble<T>(ai, r, st, c->cs); });
-        entry(true, [&] { launch_xfwd<T>(ai, g.dipole, g.thr_a, g.smem_a, c->cs); });
-        entry(g.dipole, [&] { launch_yz<T>(ai, g.thr_b, g.smem_b, c->cs); });
-        entry(g.direct, [&] { launch_dipole_direct<T>(ai, (T*)g.hdir, (const T*)g.dtab, c->cs); });
+        const GroupArgs<T> as = rk_stage_args<T>(c, g, r, st);
+        entry(true, [] {});  // the stage's state: formed by the previous stage's x-inverse kernel
         entry(true, [&] {
-            launch_xinv_force<T>(ai, g.dipole, r.k + st * stride, st == 0, c->dynamics == SS_DYN_LLG, g.thr_c,
+            if (g.dipole) launch_xfwd<T>(as, true, g.thr_a, g.smem_a, c->cs);
+        });
+        entry(g.dipole, [&] { launch_yz<T>(as, g.thr_b, g.smem_b, c->cs); });
+        entry(g.direct, [&] { launch_dipole_direct<T>(as, (T*)g.hdir, (const T*)g.dtab, c->cs); });
+        entry(true, [&] {
+            launch_xinv_force<T>(as, g.dipole, r.k + st * stride, st == 0, c->dynamics == SS_DYN_LLG, g.thr_c,
                                  g.smem_c_eval, c->cs);
         });
     }
@@ -1435,13 +1464,13 @@ ss_status ss_set_reparam(ss_ctx* c, int interp, int climb) {
             a.w_stride = spline_w_stride(a.maxK);
             TRY(dalloc(c, (void**)&a.W, nstr * mk * a.w_stride * sizeof(double)));
             CUDA_TRY(c, cudaMemsetAsync(a.W, 0, nstr * mk * a.w_stride * sizeof(double), c->cs));
-            TRY(dalloc(c, (void**)&a.P, nstr * mk * mk * sizeof(double)));
+            TRY(dalloc(c, (void**)&a.P, nstr * (mk + 1) * mk * sizeof(double)));
             TRY(dalloc(c, (void**)&a.wcopy, nstr * mk * sizeof(int)));
             CUDA_TRY(c, cudaMemsetAsync(a.wcopy, 0xff, nstr * mk * sizeof(int), c->cs));
         }
         a.climb = climb;
         a.spline = interp == SS_INTERP_SPLINE;
-        a.p_dim = a.spline ? std::min(a.maxK, kSplineSmemP) : 0;
+        a.p_dim = a.spline ? spline_p_dim((int)real_size(c), a.maxK) : 0;
     }
     c->interp = interp;
     c->climb = climb;

@@ -163,6 +163,9 @@ template <typename C> __device__ __forceinline__ C caxpy(decltype(C{}.x) a, C x,
 }
 __device__ __forceinline__ float2 caxpy(float a, float2 x, float2 y) { return __ffma2_rn(make_float2(a, a), x, y); }
 
+// y + a x for scalars and pairs alike
+template <typename T> __device__ __forceinline__ T caxpy_v(T a, T x, T y) { return y + a * x; }
+__device__ __forceinline__ float2 caxpy_v(float a, float2 x, float2 y) { return caxpy(a, x, y); }
 // element-wise product of two pairs (real and imaginary part each times a real factor)
 template <typename C> __device__ __forceinline__ C emul(C a, C b) { return C{a.x * b.x, a.y * b.y}; }
 __device__ __forceinline__ float2 emul(float2 a, float2 b) { return __fmul2_rn(a, b); }

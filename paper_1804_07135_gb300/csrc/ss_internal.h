@@ -63,6 +63,20 @@ template <typename T> struct ImgParam {
     T J, D, K, w;
 };
 
+struct RkString;
+// Runge-Kutta stages: where and how the x-inverse kernel in force mode forms the next stage's state
+// (ss_kernels.cuh, rk_next_state); out null: it does not.
+template <typename T> struct RkNext {
+    const T* y0;
+    const T* k;        // earlier stages' forces, `stride` apart
+    size_t stride;
+    T* out;            // [image][3][N]
+    int n;             // earlier stages
+    T a[6], a_cur;     // their weights and this stage's
+    const RkString* st;
+    const int* img_sys;
+};
+
 template <typename T> struct GroupArgs {
     int nx, ny, nz, N;
     int Px, Py;
@@ -90,6 +104,7 @@ template <typename T> struct GroupArgs {
     T llg_a, llg_b;        // precessional dynamics (Eq. 9): 1 / (1 + alpha^2) and alpha / (1 + alpha^2)
     const T* hdir;         // [image][3][N] direct dipole sums (SS_DIPOLE_DIRECT), or null
     const int* pair_on;    // [n_pairs] evaluate only the pairs flagged here (generic kernels), or null: all
+    RkNext<T> rk;          // force modes only
     int yz_kxb;            // kx columns per CTA of the two-pass y/z kernel (autotuned; 0: the default)
 };
 // Energy partials per image of the evaluation mode: the four terms of Eq. 1 (J, D, K, w with the constant
@@ -120,7 +135,7 @@ struct ArcArgs {
     int spline;            // natural cubic spline: the finisher writes W, the apply kernel moves the images
     double* W;             // [n_str][maxK][w_stride] interpolation weights phi_k = sum_q W_kq phi*_q, [q][k], in T
     int w_stride;          // spline_w_stride(maxK)
-    double* P;             // [n_str][maxK][maxK] scratch: d m_i / d y_q of the spline (in T), column q contiguous
+    double* P;             // [n_str][maxK + 1][maxK] scratch: d m_i / d y_q of the spline (in T), column q contiguous
     int* wcopy;            // [n_str][maxK] row k is the identity (image kept as it is)
     int p_dim;             // spline operator columns kept in the finisher's dynamic shared memory (0: none)
 };
@@ -129,7 +144,8 @@ constexpr int kClimbTile = 256;   // sites per CTA of the climbing-image kernels
 constexpr int kSplineMaxK = 256;  // longest string the spline variant accepts
 constexpr int kSplineRows = 8;    // rows of W a thread of the apply kernel takes at once
 inline int spline_w_stride(int maxK) { return (maxK + kSplineRows - 1) / kSplineRows * kSplineRows + 4; }
-constexpr int kSplineSmemP = 64;  // parts of up to 63 segments keep the spline operator P in shared memory
+// columns of the spline operator P the arc kernel keeps on chip (66 KB of FP32 or 33 KB of FP64)
+inline int spline_p_dim(int real_bytes, int maxK) { const int cap = real_bytes == 4 ? 128 : 64; return maxK + 1 < cap ? maxK + 1 : cap; }
 
 // Adaptive Runge-Kutta evolution (Sec. III, Dormand-Prince 5(4)): controller state of one ODE system
 // (a whole string, or one image under per-image step control).
@@ -306,7 +322,6 @@ template <typename T> void launch_xinv_step_llg(const GroupArgs<T>& g, bool do_f
 template <typename T> void launch_dipole_direct(const GroupArgs<T>& g, T* hdir, const T* dtab, cudaStream_t st);
 template <typename T> void launch_climb(const GroupArgs<T>& g, const ArcArgs& a, T dt, const T* hc, cudaStream_t st);
 template <typename T> void launch_spline_apply(const GroupArgs<T>& g, const ArcArgs& a, int maxK, cudaStream_t st);
-template <typename T> void launch_rk_assemble(const GroupArgs<T>& g, const RkArgs<T>& r, int stage, cudaStream_t st);
 template <typename T> void launch_rk_finish(const GroupArgs<T>& g, const RkArgs<T>& r, cudaStream_t st);
 template <typename T>
 void launch_rk_control(const GroupArgs<T>& g, const RkArgs<T>& r, int begin, cudaStream_t st);

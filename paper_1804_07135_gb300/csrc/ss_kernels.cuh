@@ -51,12 +51,9 @@ template <> __device__ __forceinline__ float rsqrt_t<float>(float x) { return rs
 template <> __device__ __forceinline__ double rsqrt_t<double>(double x) {
     return x > 1e-30 && x < 1e30 ? rsqrt_nr(x) : 1.0 / sqrt(x);
 }
-__device__ __forceinline__ double rcp_nr(double x) {
-    double r = (double)(1.0f / (float)x);
-    r = fma(r, fma(-x, r, 1.0), r);
-    r = fma(r, fma(-x, r, 1.0), r);
-    return r;
-}
+// correctly rounded reciprocals
+__device__ __forceinline__ float rcp_t(float x) { return __frcp_rn(x); }
+__device__ __forceinline__ double rcp_t(double x) { return 1.0 / x; }
 
 // Fixed-order block reduction of NV doubles per thread; result valid in thread 0.
 template <int NV>
@@ -137,6 +134,7 @@ __device__ __forceinline__ void xfwd_gather(const GroupArgs<T>& g, cplx<T>* buf,
     using C = cplx<T>;
     const int nx = g.nx, N = g.N;
     const int ia = 2 * p;
+    const bool in_place = g.s == g.sp;  // identity table on one buffer (Runge-Kutta stages): nothing to store
     // the pair's two table entries, loaded once (the stores below could alias them for the compiler)
     InterpEntry ent[2];
 #pragma unroll
@@ -177,7 +175,7 @@ __device__ __forceinline__ void xfwd_gather(const GroupArgs<T>& g, cplx<T>* buf,
                     float* d = g.s + (size_t)im * 3 * N + site;
 #pragma unroll
                     for (int c = 0; c < 3; ++c) {
-                        *reinterpret_cast<float2*>(d + (size_t)c * N) = u[c];
+                        if (!in_place) *reinterpret_cast<float2*>(d + (size_t)c * N) = u[c];
                         out[h][0][c] = u[c].x;
                         out[h][1][c] = u[c].y;
                     }
@@ -217,10 +215,12 @@ __device__ __forceinline__ void xfwd_gather(const GroupArgs<T>& g, cplx<T>* buf,
                     u1 *= r;
                     u2 *= r;
                 }
-                T* d = g.s + (size_t)im * 3 * N + site;
-                d[0] = u0;
-                d[N] = u1;
-                d[2 * N] = u2;
+                if (!in_place) {
+                    T* d = g.s + (size_t)im * 3 * N + site;
+                    d[0] = u0;
+                    d[N] = u1;
+                    d[2 * N] = u2;
+                }
                 out[h][0] = u0;
                 out[h][1] = u1;
                 out[h][2] = u2;
@@ -531,7 +531,19 @@ __device__ __forceinline__ T step_site(const T* s0, const T* hf, T dt, T* un) {
     return T(-0.5) * sh;
 }
 
-// Step modes (0, 3, 4 of xinv_sites), FP32, even nx: two adjacent sites (x even, x + 1) per thread and
+// Runge-Kutta stage (force modes): the next stage's state at component offset o (image im), given this stage's
+// force f there, y0 + hs (sum_{q < n} a_q k_q + a_n f); V is T or the vector type of adjacent sites.
+template <typename T, typename V>
+__device__ __forceinline__ void rk_next_state(const RkNext<T>& r, T hs, size_t o, V f) {
+    V acc{};
+#pragma unroll
+    for (int q = 0; q < 6; ++q)
+        if (q < r.n) acc = caxpy_v(r.a[q], *reinterpret_cast<const V*>(r.k + q * r.stride + o), acc);
+    acc = caxpy_v(r.a_cur, f, acc);
+    *reinterpret_cast<V*>(r.out + o) = caxpy_v(hs, acc, *reinterpret_cast<const V*>(r.y0 + o));
+}
+
+// Step and force modes (all but 1 of xinv_sites), FP32, even nx: two adjacent sites (x even, x + 1) per thread and
 // pass, so the spin planes move as float2 (one load serves both sites' y and z neighbours, and the inner
 // x neighbours come from the pair itself).  eacc[h] accumulates the energy terms of image 2p + h.
 template <int MODE, typename Pos>
@@ -541,6 +553,7 @@ __device__ __forceinline__ void xinv_sites_step2(const GroupArgs<float>& g, floa
     const int nx = g.nx, ny = g.ny, nz = g.nz, N = g.N, hx = nx >> 1;
     const int ia = 2 * p;
     const float2 zero = make_float2(0.f, 0.f);
+    constexpr bool FORCE = MODE == 2 || MODE == 5;
 #pragma unroll 1
     for (int it = tid; it < 2 * rows * hx; it += nthr) {
         const int h = it / (rows * hx);
@@ -588,7 +601,7 @@ __device__ __forceinline__ void xinv_sites_step2(const GroupArgs<float>& g, floa
             } else {
                 const float sh = s0[0] * hf[0] + s0[1] * hf[1] + s0[2] * hf[2];
                 eacc[h] += -0.5f * sh;
-                if (MODE == 3) {  // the climbing image: its force, stepped by the climbing-image kernels
+                if (MODE == 2 || MODE == 3) {  // the force (climbing image: stepped by the climbing-image kernels)
 #pragma unroll
                     for (int c = 0; c < 3; ++c) un[k][c] = hf[c] - sh * s0[c];
                 } else {  // Eq. 9
@@ -596,14 +609,30 @@ __device__ __forceinline__ void xinv_sites_step2(const GroupArgs<float>& g, floa
                                           s0[0] * hf[1] - s0[1] * hf[0]};
                     float u[3];
 #pragma unroll
-                    for (int c = 0; c < 3; ++c) u[c] = s0[c] + dt * (-g.llg_a * sxh[c] + g.llg_b * (hf[c] - sh * s0[c]));
-                    const float r = rsqrtf(u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
+                    for (int c = 0; c < 3; ++c) u[c] = -g.llg_a * sxh[c] + g.llg_b * (hf[c] - sh * s0[c]);
+                    if (MODE == 5) {
 #pragma unroll
-                    for (int c = 0; c < 3; ++c) un[k][c] = u[c] * r;
+                        for (int c = 0; c < 3; ++c) un[k][c] = u[c];
+                    } else {
+#pragma unroll
+                        for (int c = 0; c < 3; ++c) u[c] = s0[c] + dt * u[c];
+                        const float r = rsqrtf(u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
+#pragma unroll
+                        for (int c = 0; c < 3; ++c) un[k][c] = u[c] * r;
+                    }
                 }
             }
         }
-        float* __restrict__ o = (MODE == 3 && climbs[h] ? hout : g.sp) + (size_t)im * 3 * N + site;
+        if constexpr (FORCE) {
+            if (g.rk.out) {  // uniform over the grid
+                const RkString& S = g.rk.st[g.rk.img_sys[im]];
+                const float hs = S.done ? 0.f : (float)S.hs;
+#pragma unroll
+                for (int c = 0; c < 3; ++c)
+                    rk_next_state(g.rk, hs, (size_t)im * 3 * N + (size_t)c * N + site, make_float2(un[0][c], un[1][c]));
+            }
+        }
+        float* __restrict__ o = (FORCE || (MODE == 3 && climbs[h]) ? hout : g.sp) + (size_t)im * 3 * N + site;
 #pragma unroll
         for (int c = 0; c < 3; ++c) *reinterpret_cast<float2*>(o + (size_t)c * N) = make_float2(un[0][c], un[1][c]);
     }
@@ -637,7 +666,7 @@ __device__ __forceinline__ void xinv_sites(const GroupArgs<T>& g, T dt, T* hout,
         for (int h = 0; h < 2; ++h)
             if (ia + h < g.n_img) climbs[h] = g.climb_img[ia + h];
     }
-    if constexpr ((MODE == 0 || MODE == 3 || MODE == 4) && HAS_CONV && std::is_same<T, float>::value) {
+    if constexpr (MODE != 1 && HAS_CONV && std::is_same<T, float>::value) {
         if ((nx & 1) == 0) {  // uniform over the grid
             xinv_sites_step2<MODE>(g, dt, hout, buf, ls, lrows, p, z, y0, rows, tid, nthr, climbs, eacc, pos);
             done = true;
@@ -692,6 +721,15 @@ __device__ __forceinline__ void xinv_sites(const GroupArgs<T>& g, T dt, T* hout,
             const T sh = s0[0] * hf[0] + s0[1] * hf[1] + s0[2] * hf[2];
             eacc[h] += T(-0.5) * sh;
             T* __restrict__ o = hout + (size_t)im * 3 * N + site;
+            if constexpr (MODE == 2) {
+                if (g.rk.out) {  // uniform over the grid
+                    const RkString& S = g.rk.st[g.rk.img_sys[im]];
+                    const T hs = S.done ? T(0) : T(S.hs);
+#pragma unroll
+                    for (int c = 0; c < 3; ++c)
+                        rk_next_state(g.rk, hs, (size_t)im * 3 * N + (size_t)c * N + site, hf[c] - sh * s0[c]);
+                }
+            }
 #pragma unroll
             for (int c = 0; c < 3; ++c) o[(size_t)c * N] = hf[c] - sh * s0[c];
         } else if (MODE == 4 || MODE == 5) {
@@ -711,6 +749,13 @@ __device__ __forceinline__ void xinv_sites(const GroupArgs<T>& g, T dt, T* hout,
 #pragma unroll
                 for (int c = 0; c < 3; ++c) o[(size_t)c * N] = u[c] * r;
             } else {
+                if (g.rk.out) {  // uniform over the grid
+                    const RkString& S = g.rk.st[g.rk.img_sys[im]];
+                    const T hs = S.done ? T(0) : T(S.hs);
+#pragma unroll
+                    for (int c = 0; c < 3; ++c)
+                        rk_next_state(g.rk, hs, (size_t)im * 3 * N + (size_t)c * N + site, f[c]);
+                }
                 T* __restrict__ o = hout + (size_t)im * 3 * N + site;
 #pragma unroll
                 for (int c = 0; c < 3; ++c) o[(size_t)c * N] = f[c];
@@ -898,7 +943,7 @@ __device__ __noinline__ void arc_finish(const GroupArgs<T>& g, const ArcArgs& a,
 // the shared elimination factors), and on segment [x_j, x_{j+1}] the spline is
 // A y_j + B y_{j+1} + C m_j + D m_{j+1} with A = (x_{j+1} - x) / h_j, B = (x - x_j) / h_j,
 // C = h_j^2 (A^3 - A) / 6, D = h_j^2 (B^3 - B) / 6.  A part with a zero-length segment takes the linear
-// rows instead; images that keep their place get identity rows.  Each knot, segment reciprocal and
+// rows instead; the rows of images that keep their place are not used.  Each knot, segment reciprocal and
 // elimination factor is formed once (GB300 issues FP64 division slowly).
 template <typename T>
 __device__ __noinline__ void arc_finish_variants(const GroupArgs<T>& g, const ArcArgs& a, int str, int K, int img0,
@@ -907,11 +952,9 @@ __device__ __noinline__ void arc_finish_variants(const GroupArgs<T>& g, const Ar
     __shared__ double hh_raw[kSplineMaxK], rh_raw[kSplineMaxK], rden_raw[kSplineMaxK], cp_raw[kSplineMaxK];
     __shared__ double row_raw[4][kSplineMaxK];  // A, B, C, D of the row's segment
     __shared__ int row_seg[kSplineMaxK];        // the segment
-    // P of a part of up to a.p_dim - 1 segments stays on chip in the launch's dynamic shared memory (the
-    // recurrences along a column are dependent, so each step's latency counts); longer parts use the
-    // global scratch
+    // P of up to a.p_dim columns stays on chip in the launch's dynamic shared memory (the recurrences along a
+    // column are dependent, so each step's latency counts); longer strings use the global scratch
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    double* Psm = reinterpret_cast<double*>(smem_raw);
     const int tid = threadIdx.x, nthr = blockDim.x;
     const bool split = kc > 0 && kc < K - 1;
     const size_t mk = (size_t)a.maxK;
@@ -959,102 +1002,121 @@ __device__ __noinline__ void arc_finish_variants(const GroupArgs<T>& g, const Ar
     }
     if (!a.spline) return;
     // the spline operator in the path's precision T (its weights are stored in T; FP64 arithmetic is slow
-    // on GB300 and buys the FP32 path nothing); knots and targets as computed above
-    T* hh = reinterpret_cast<T*>(hh_raw);
-    T* rh = reinterpret_cast<T*>(rh_raw);
-    T* rden = reinterpret_cast<T*>(rden_raw);
-    T* cp = reinterpret_cast<T*>(cp_raw);
+    // on GB300 and buys the FP32 path nothing); knots and targets as computed above.  Both parts of a split
+    // string go through each phase together.  Segment j lies between images j and j + 1.
+    T* __restrict__ hh = reinterpret_cast<T*>(hh_raw);
+    T* __restrict__ rh = reinterpret_cast<T*>(rh_raw);
+    T* __restrict__ rden = reinterpret_cast<T*>(rden_raw);
+    T* __restrict__ cp = reinterpret_cast<T*>(cp_raw);
     T(*row)[kSplineMaxK] = reinterpret_cast<T(*)[kSplineMaxK]>(row_raw);
-    for (int part = 0; part < (split ? 2 : 1); ++part) {
-        const int a0 = part == 0 ? 0 : kc, b0 = part == 0 && split ? kc : K - 1, n = b0 - a0;
-        const double L = s[b0] - s[a0];
-        __syncthreads();  // the shared factors are free
-        if (!a.reparam || !(L > 0.0) || !isfinite(L) || n < 2) continue;  // uniform: nothing moves here
-        bool pos = true;
-        for (int i = tid; i < n; i += nthr) {
-            const double hd = knot(a0 + i + 1, a0) - knot(a0 + i, a0);
-            hh[i] = T(hd);
-            pos = pos && hd > 0.0 && hh[i] > T(0);
-            if (pos) rh[i] = T(1) / hh[i];
-        }
-        const bool ok = __syncthreads_and(pos);
-        const bool on_chip = n + 1 <= a.p_dim;
-        T* P = on_chip ? reinterpret_cast<T*>(Psm) : reinterpret_cast<T*>(a.P) + (size_t)str * mk * mk;
-        const size_t ps = on_chip ? (size_t)(a.p_dim | 1) : mk;  // column stride (odd on chip: distinct banks)
-        // The recurrences are serial: each keeps its running value in a register and loads ahead of it, so a
-        // step costs the two dependent operations (and thread 0's division), not a trip to shared memory.
-        if (ok && tid == 0) {  // elimination factors of the tridiagonal system (m_0 = m_n = 0 known)
-            T c = T(0);
-#pragma unroll 4
-            for (int i = 1; i < n; ++i) {
-                const T h0 = hh[i - 1], h1 = hh[i];
-                const T den = T(2) * (h0 + h1) - (i > 1 ? h0 * c : T(0));
-                const T rd = T(1) / den;
-                c = (i < n - 1 ? h1 : T(0)) * rd;
-                rden[i] = rd;
-                cp[i] = c;
+    bool pos[2] = {true, true};
+    for (int j = tid; j < K - 1; j += nthr) {
+        const int part = split && j >= kc, a0 = part ? kc : 0;
+        const double hd = knot(j + 1, a0) - knot(j, a0);
+        const T h = T(hd);
+        hh[j] = h;
+        const bool p = hd > 0.0 && h > T(0);
+        rh[j] = p ? rcp_t(h) : T(0);
+        if (!p) pos[part] = false;
+    }
+    bool ok[2], moves[2];  // (uniform) a part without zero-length segments; a part some image of which moves
+    ok[0] = __syncthreads_and(pos[0]);
+    ok[1] = __syncthreads_and(pos[1]);
+#pragma unroll
+    for (int part = 0; part < 2; ++part) {
+        const int a0 = part ? kc : 0, b0 = part == 0 && split ? kc : K - 1;
+        const double L = part == 0 || split ? s[b0] - s[a0] : 0.0;
+        moves[part] = a.reparam && L > 0.0 && isfinite(L) && b0 - a0 >= 2;
+    }
+    const int ncol = split ? K + 1 : K;  // columns: the images of part one, then those of part two (kc in both)
+    const bool on_chip = ncol <= a.p_dim;
+    T* __restrict__ P = on_chip ? reinterpret_cast<T*>(smem_raw) : reinterpret_cast<T*>(a.P) + (size_t)str * (mk + 1) * mk;
+    const size_t ps = on_chip ? (size_t)(a.p_dim | 1) : mk;  // column stride (odd on chip: distinct banks)
+    // The recurrences are serial: each keeps its running value in a register and loads one step ahead, so a step
+    // costs its dependent operations and not a trip to shared memory.
+    if (tid == 0 || (split && tid == 32)) {  // elimination factors of the tridiagonal systems (m = 0 at the ends)
+        const int part = tid != 0, a0 = part ? kc : 0, b0 = part == 0 && split ? kc : K - 1;
+        if (moves[part] && ok[part]) {
+            T c = T(0), h0 = hh[a0], h1 = hh[a0 + 1];
+            for (int k = a0 + 1; k < b0; ++k) {
+                const T hn = k + 1 < b0 ? hh[k + 1] : T(0);
+                const T rd = rcp_t(T(2) * (h0 + h1) - h0 * c);
+                c = (k < b0 - 1 ? h1 : T(0)) * rd;
+                rden[k] = rd;
+                cp[k] = c;
+                h0 = h1;
+                h1 = hn;
             }
         }
-        __syncthreads();
-        if (ok) {
-            for (int q = tid; q <= n; q += nthr) {  // column q of P: d m_i / d y_q, i = 1..n-1
-                T* __restrict__ pc = P + (size_t)q * ps;
-                T d = T(0);
-#pragma unroll 4
-                for (int i = 1; i < n; ++i) {
-                    T r = T(0);  // d rhs_i / d y_q
-                    if (q == i + 1) r = T(6) * rh[i];
-                    if (q == i) r = T(-6) * (rh[i] + rh[i - 1]);
-                    if (q == i - 1) r = T(6) * rh[i - 1];
-                    d = (r - (i > 1 ? hh[i - 1] * d : T(0))) * rden[i];
-                    pc[i] = d;
-                }
-#pragma unroll 4
-                for (int i = n - 2; i >= 1; --i) {
-                    d = pc[i] - cp[i] * d;
-                    pc[i] = d;
-                }
-            }
-            __syncthreads();
+    }
+    __syncthreads();
+    for (int c = tid; c < ncol; c += nthr) {  // column c: d m_k / d y_q for the interior images k of its part
+        const int part = split && c > kc, q = c - part;
+        const int a0 = part ? kc : 0, b0 = part == 0 && split ? kc : K - 1;
+        if (!(moves[part] && ok[part])) continue;
+        T* __restrict__ pc = P + (size_t)c * ps;
+        // d rhs_k / d y_q, nonzero for k = q - 1, q, q + 1
+        const T rl = q > a0 ? rh[q - 1] : T(0), rr = q < b0 ? rh[q] : T(0);
+        const T r0 = T(6) * rl, r1 = T(-6) * (rr + rl), r2 = T(6) * rr;
+        T d = T(0), h = hh[a0], rd = rden[a0 + 1];
+        for (int k = a0 + 1; k < b0; ++k) {
+            const T hn = hh[k], rn = k + 1 < b0 ? rden[k + 1] : T(0);
+            const T r = k == q - 1 ? r0 : k == q ? r1 : k == q + 1 ? r2 : T(0);
+            d = (r - h * d) * rd;
+            pc[k] = d;
+            h = hn;
+            rd = rn;
         }
-        for (int k = a0 + 1 + tid; k < b0; k += nthr) {
-            const double ak = (double)(k - a0) / (double)n;
-            int j = min(k, b0 - 1);
-            if (knot(j, a0) <= ak) {
-                while (j < b0 - 1 && knot(j + 1, a0) <= ak) ++j;
-            } else {
-                do --j;
-                while (knot(j, a0) > ak);
-            }
-            const double x0 = knot(j, a0), x1 = knot(j + 1, a0);
-            const int jr = j - a0;
-            T A, B, C = T(0), D = T(0);
-            if (ok) {
-                const T h = hh[jr];
-                A = T(x1 - ak) * rh[jr], B = T(ak - x0) * rh[jr];
-                C = h * h * (A * A * A - A) * T(1.0 / 6.0), D = h * h * (B * B * B - B) * T(1.0 / 6.0);
-            } else {  // a zero-length segment: linear rows
-                const double t = (ak - x0) / (x1 - x0);
-                A = T(1.0 - t), B = T(t);
-            }
-            row[0][k] = A, row[1][k] = B, row[2][k] = C, row[3][k] = D;
-            row_seg[k] = jr;
+        T pk = b0 - 2 > a0 ? pc[b0 - 2] : T(0), ck = b0 - 2 > a0 ? cp[b0 - 2] : T(0);
+        for (int k = b0 - 2; k > a0; --k) {
+            const T pn = k - 1 > a0 ? pc[k - 1] : T(0), cn = k - 1 > a0 ? cp[k - 1] : T(0);
+            d = pk - ck * d;
+            pc[k] = d;
+            pk = pn;
+            ck = cn;
         }
-        __syncthreads();
-        // the rows of W, all threads over (column, row), rows fastest as they are stored
-        for (int e = tid; e < (n - 1) * K; e += nthr) {
-            const int qk = e / (n - 1), k = a0 + 1 + e - qk * (n - 1), q = qk - a0, jr = row_seg[k];
-            T w = T(0);
-            if (q >= 0 && q <= n) {
-                w = (q == jr ? row[0][k] : T(0)) + (q == jr + 1 ? row[1][k] : T(0));
-                if (ok) {
-                    const T* pc = P + (size_t)q * ps;
-                    const T mj = jr > 0 ? pc[jr] : T(0), mj1 = jr + 1 < n ? pc[jr + 1] : T(0);
-                    w = w + row[2][k] * mj + row[3][k] * mj1;
-                }
-            }
-            W[(size_t)qk * a.w_stride + k] = w;
+    }
+    for (int k = 1 + tid; k < K - 1; k += nthr) {
+        const int part = split && k > kc, a0 = part_lo(k), b0 = part_hi(k), n = b0 - a0;
+        if (!moves[part] || k == b0) continue;
+        const double ak = (double)(k - a0) / (double)n;
+        int j = min(k, b0 - 1);
+        if (knot(j, a0) <= ak) {
+            while (j < b0 - 1 && knot(j + 1, a0) <= ak) ++j;
+        } else {
+            do --j;
+            while (knot(j, a0) > ak);
         }
+        const double x0 = knot(j, a0), x1 = knot(j + 1, a0);
+        T A, B, C = T(0), D = T(0);
+        if (ok[part]) {
+            const T h = hh[j];
+            A = T(x1 - ak) * rh[j], B = T(ak - x0) * rh[j];
+            C = h * h * (A * A * A - A) * T(1.0 / 6.0), D = h * h * (B * B * B - B) * T(1.0 / 6.0);
+        } else {  // a zero-length segment: linear rows
+            const double t = (ak - x0) / (x1 - x0);
+            A = T(1.0 - t), B = T(t);
+        }
+        row[0][k] = A, row[1][k] = B, row[2][k] = C, row[3][k] = D;
+        row_seg[k] = j;
+    }
+    __syncthreads();
+    // the rows of W, all threads over (column, row), rows fastest as they are stored
+    for (int e = tid; e < (K - 2) * K; e += nthr) {
+        const int q = e / (K - 2), k = 1 + e - q * (K - 2);
+        const int part = split && k > kc, a0 = part_lo(k), b0 = part_hi(k);
+        if (!moves[part] || k == b0) continue;  // a kept image
+        const int j = row_seg[k];
+        T w = T(0);
+        if (q >= a0 && q <= b0) {
+            w = (q == j ? row[0][k] : T(0)) + (q == j + 1 ? row[1][k] : T(0));
+            if (ok[part]) {
+                const T* pc = P + (size_t)(q + part) * ps;
+                const T mj = j > a0 ? pc[j] : T(0), mj1 = j + 1 < b0 ? pc[j + 1] : T(0);
+                w = w + row[2][k] * mj + row[3][k] * mj1;
+            }
+        }
+        W[(size_t)q * a.w_stride + k] = w;
     }
 }
 
@@ -1429,9 +1491,9 @@ __device__ __noinline__ void arc_finish(const GroupArgs<T>& g, const ArcArgs& a,
 
 // ------------------------------------------------------------------------------------------------
 // Adaptive Runge-Kutta evolution of the images (Sec. III: explicit Runge-Kutta with step-size control,
-// the Dormand-Prince 5(4) pair).  Per attempt, for each stage i: Y_i = y0 + hs sum_{q<i} a_iq k_q
-// (rk_assemble into sp), then the field pipeline with an identity table and the step kernel in force
-// mode gives k_i = F(Y_i) (Eq. 13); rk_finish forms y5 = y0 + hs sum b_q k_q and the squared scaled
+// the Dormand-Prince 5(4) pair).  Per attempt, for each stage i, the field pipeline on the state
+// Y_i = y0 + hs sum_{q<i} a_iq k_q (x-forward in place) and the x-inverse kernel in force mode, which writes
+// k_i = F(Y_i) (Eq. 13) and forms Y_{i+1} (rk_next_state); rk_finish forms y5 = y0 + hs sum b_q k_q and the squared scaled
 // error (hs sum (b_q - bhat_q) k_q / (atol + rtol max(|y0|, |y5|)))^2 per tile; rk_control (one CTA per
 // ODE system) sums it in a fixed order, accepts when sqrt(mean) <= 1 and picks the next step; rk_commit
 // renormalises the accepted y5 into y0 (and into sp once the string's interval is complete).
@@ -1483,7 +1545,6 @@ template <typename T> DpCoef<T> dp_coefficients(int method) {
 }
 constexpr int kRkTile = 1024;  // components per CTA of the element-wise Runge-Kutta kernels
 
-// grid (tiles, images), 256 threads
 // FP32 with N a multiple of 4: the element-wise Runge-Kutta kernels move float4s, one per thread and
 // tile (kRkTile = 4 x 256), so every thread has all of its loads in flight at once
 template <typename T> __device__ __forceinline__ bool rk_vec4(const GroupArgs<T>& g) {
@@ -1493,36 +1554,11 @@ __device__ __forceinline__ float4 f4_fma(float a, float4 x, float4 y) {
     return make_float4(fmaf(a, x.x, y.x), fmaf(a, x.y, y.y), fmaf(a, x.z, y.z), fmaf(a, x.w, y.w));
 }
 
-template <typename T, int STAGE>
-__global__ void __launch_bounds__(256) rk_assemble_kernel(GroupArgs<T> g, RkArgs<T> r) {
-    const int im = blockIdx.y;
-    const size_t M = (size_t)3 * g.N, base = (size_t)im * M, stride = (size_t)g.n_img * M;
-    const RkString& S = r.st[r.img_sys[im]];
-    const T hs = S.done ? T(0) : T(S.hs);
-    if constexpr (std::is_same<T, float>::value) {
-        if (rk_vec4(g)) {
-            const size_t e4 = (size_t)blockIdx.x * (kRkTile / 4) + threadIdx.x;
-            if (4 * e4 >= M) return;
-            float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-            for (int q = 0; q < STAGE; ++q)
-                a = f4_fma(r.dp.a[STAGE][q], reinterpret_cast<const float4*>(r.k + q * stride + base)[e4], a);
-            reinterpret_cast<float4*>(g.sp + base)[e4] = f4_fma(hs, a, reinterpret_cast<const float4*>(r.y0 + base)[e4]);
-            return;
-        }
-    }
-    const size_t e1 = min(M, (size_t)(blockIdx.x + 1) * kRkTile);
-    for (size_t e = (size_t)blockIdx.x * kRkTile + threadIdx.x; e < e1; e += blockDim.x) {
-        T a = T(0);
-#pragma unroll
-        for (int q = 0; q < STAGE; ++q) a += r.dp.a[STAGE][q] * r.k[q * stride + base + e];
-        g.sp[base + e] = r.y0[base + e] + hs * a;
-    }
-}
-
 // grid (tiles, images), 256 threads
 template <typename T>
 __global__ void __launch_bounds__(256) rk_finish_kernel(GroupArgs<T> g, RkArgs<T> r) {
+    griddep_wait();
+    griddep_launch_dependents();
     __shared__ double red[32];
     const int im = blockIdx.y;
     const size_t M = (size_t)3 * g.N, base = (size_t)im * M, stride = (size_t)g.n_img * M;
@@ -1582,6 +1618,8 @@ __global__ void __launch_bounds__(256) rk_finish_kernel(GroupArgs<T> g, RkArgs<T
 // first step cut to T) and marks every system active.
 template <typename T>
 __global__ void __launch_bounds__(256) rk_control_kernel(GroupArgs<T> g, RkArgs<T> r, int begin) {
+    griddep_wait();
+    griddep_launch_dependents();
     __shared__ double red[32];
     const int s = blockIdx.x;
     const double T_int = r.T_int;
@@ -1647,6 +1685,8 @@ __global__ void __launch_bounds__(256) rk_control_kernel(GroupArgs<T> g, RkArgs<
 // accepted; also into sp once the string's interval is complete
 template <typename T>
 __global__ void __launch_bounds__(256) rk_commit_kernel(GroupArgs<T> g, RkArgs<T> r) {
+    griddep_wait();
+    griddep_launch_dependents();
     const int im = blockIdx.y;
     const RkString& S = r.st[r.img_sys[im]];
     if (!S.accepted) return;  // uniform over the CTA
@@ -2198,11 +2238,11 @@ template <typename T, int MODE>
 static void launch_xinv_force_mode(const GroupArgs<T>& g, bool do_fft, T* kout, T flag, int nthr, size_t smem,
                                    cudaStream_t st) {
     dim3 grid((g.ny + g.ty_c - 1) / g.ty_c, g.nz, g.n_pairs);
-    if (do_fft && launch_xinv2p<MODE>(g, flag, kout, false, st)) return;
+    if (do_fft && launch_xinv2p<MODE>(g, flag, kout, true, st)) return;
     if (do_fft)
-        xinv_kernel<T, true, MODE><<<grid, nthr, smem, st>>>(g, flag, kout);
+        launch_pdl(xinv_kernel<T, true, MODE>, grid, dim3(nthr), smem, st, g, flag, kout);
     else
-        xinv_kernel<T, false, MODE><<<grid, nthr, smem, st>>>(g, flag, kout);
+        launch_pdl(xinv_kernel<T, false, MODE>, grid, dim3(nthr), smem, st, g, flag, kout);
 }
 
 template <typename T>
@@ -2270,31 +2310,18 @@ template <typename T> void launch_spline_apply(const GroupArgs<T>& g, const ArcA
     launch_pdl(spline_apply_kernel<T>, dim3((g.N + 31) / 32, a.n_str), dim3(256), sm, st, g, a, on_chip ? 1 : 0);
 }
 
-template <typename T> void launch_rk_assemble(const GroupArgs<T>& g, const RkArgs<T>& r, int stage, cudaStream_t st) {
-    const dim3 grid(r.n_tiles, g.n_img);
-    switch (stage) {
-        case 0: rk_assemble_kernel<T, 0><<<grid, 256, 0, st>>>(g, r); break;
-        case 1: rk_assemble_kernel<T, 1><<<grid, 256, 0, st>>>(g, r); break;
-        case 2: rk_assemble_kernel<T, 2><<<grid, 256, 0, st>>>(g, r); break;
-        case 3: rk_assemble_kernel<T, 3><<<grid, 256, 0, st>>>(g, r); break;
-        case 4: rk_assemble_kernel<T, 4><<<grid, 256, 0, st>>>(g, r); break;
-        case 5: rk_assemble_kernel<T, 5><<<grid, 256, 0, st>>>(g, r); break;
-        default: rk_assemble_kernel<T, 6><<<grid, 256, 0, st>>>(g, r); break;
-    }
-}
-
 template <typename T> void launch_rk_finish(const GroupArgs<T>& g, const RkArgs<T>& r, cudaStream_t st) {
-    rk_finish_kernel<T><<<dim3(r.n_tiles, g.n_img), 256, 0, st>>>(g, r);
+    launch_pdl(rk_finish_kernel<T>, dim3(r.n_tiles, g.n_img), dim3(256), 0, st, g, r);
 }
 
 template <typename T>
 void launch_rk_control(const GroupArgs<T>& g, const RkArgs<T>& r, int begin, cudaStream_t st) {
-    rk_control_kernel<T><<<r.n_sys, 256, 0, st>>>(g, r, begin);
+    launch_pdl(rk_control_kernel<T>, dim3(r.n_sys), dim3(256), 0, st, g, r, begin);
 }
 
 template <typename T> void launch_rk_commit(const GroupArgs<T>& g, const RkArgs<T>& r, cudaStream_t st) {
     const int per = std::is_same<T, float>::value && (g.N & 3) == 0 ? 4 : 1;  // sites per thread
-    rk_commit_kernel<T><<<dim3((g.N / per + 255) / 256, g.n_img), 256, 0, st>>>(g, r);
+    launch_pdl(rk_commit_kernel<T>, dim3((g.N / per + 255) / 256, g.n_img), dim3(256), 0, st, g, r);
 }
 
 template <typename T> void launch_arc(const GroupArgs<T>& g, const ArcArgs& a, int nthr, cudaStream_t st) {
@@ -2368,9 +2395,6 @@ template <typename T> void set_smem_limits(int bytes) {
     set_dyn_smem(dipole_direct_kernel<T, M, false>, bytes, carve);
     SS_CASE(1) SS_CASE(2) SS_CASE(4)
 #undef SS_CASE
-#define SS_CASE(S) set_dyn_smem(rk_assemble_kernel<T, S>, bytes, carve);
-    SS_CASE(0) SS_CASE(1) SS_CASE(2) SS_CASE(3) SS_CASE(4) SS_CASE(5) SS_CASE(6)
-#undef SS_CASE
     set_dyn_smem(rk_finish_kernel<T>, bytes, carve);
     set_dyn_smem(rk_control_kernel<T>, bytes, carve);
     set_dyn_smem(rk_commit_kernel<T>, bytes, carve);
@@ -2442,7 +2466,6 @@ void launch_widen_unit(const float* src, double* dst, int K, int N, const int* p
     template void launch_dipole_direct<T>(const GroupArgs<T>&, T*, const T*, cudaStream_t);                    \
     template void launch_spline_apply<T>(const GroupArgs<T>&, const ArcArgs&, int, cudaStream_t);              \
     template DpCoef<T> dp_coefficients<T>(int);                                                               \
-    template void launch_rk_assemble<T>(const GroupArgs<T>&, const RkArgs<T>&, int, cudaStream_t);             \
     template void launch_rk_finish<T>(const GroupArgs<T>&, const RkArgs<T>&, cudaStream_t);                    \
     template void launch_rk_control<T>(const GroupArgs<T>&, const RkArgs<T>&, int, cudaStream_t);                \
     template void launch_rk_commit<T>(const GroupArgs<T>&, const RkArgs<T>&, cudaStream_t);                    \
