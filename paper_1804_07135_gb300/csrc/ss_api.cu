@@ -249,6 +249,8 @@ template <typename T> GroupArgs<T> group_args(const ss_ctx* c, const Group& g) {
     a.Py = g.Py;
     a.n_img = g.n_img;
     a.n_pairs = g.n_pairs;
+    a.m_nx = fast_div_m(g.nx);
+    a.m_hx = fast_div_m(g.nx / 2);
     a.lsx = g.lsx;
     a.lsy = g.lsy;
     a.s = (T*)g.s;
@@ -281,7 +283,7 @@ template <typename T> GroupArgs<T> group_args(const ss_ctx* c, const Group& g) {
 void set_rows(Group& g, int ty_a, int ty_c, int thr_a = 256, int thr_c = 256) {
     const size_t cs = 2 * (size_t)g.rbytes;
     const bool x2 = g.dipole && t2_length(g.Px);  // two-pass x kernels: fixed rows per CTA
-    if (x2) ty_a = ty_c = x2_rows(g.rbytes);
+    if (x2) ty_a = ty_c = x2_rows(g.rbytes, g.Px);
     g.ty_a = ty_a;
     g.ty_c = ty_c;
     g.thr_a = thr_a;

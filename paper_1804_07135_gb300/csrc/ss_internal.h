@@ -58,6 +58,13 @@ struct InterpEntry {
     int pad;
 };
 
+// n / d by a multiplication, m = fast_div_m(d), exact for n d < 2^32 (m = ceil(2^32 / d), 0 stands for d = 1: the
+// product n m exceeds n 2^32 / d by less than n d / d)
+inline unsigned fast_div_m(unsigned d) { return d <= 1 ? 0u : (unsigned)(((1ull << 32) + d - 1) / d); }
+#ifdef __CUDACC__
+__device__ __forceinline__ int fast_div(int n, unsigned m) { return m ? (int)__umulhi((unsigned)n, m) : n; }
+#endif
+
 // Constants of the string an image belongs to.
 template <typename T> struct ImgParam {
     T J, D, K, w;
@@ -81,6 +88,7 @@ template <typename T> struct GroupArgs {
     int nx, ny, nz, N;
     int Px, Py;
     int n_img, n_pairs;
+    unsigned m_nx, m_hx;  // fast_div multipliers of nx and nx / 2
     int lsx, lsy;  // shared-memory line strides (complex elements) of the x and y transforms
     T* s;
     T* sp;
@@ -257,20 +265,23 @@ inline int yz2p_kxb_use(int real_bytes, int nz, int tuned) {
 // Factor of the stored tensor spectrum besides 4 pi / (Px Py): the two-pass y/z kernel convolves sums and
 // differences of mirrored layers, which leaves a factor 2 to be taken out (exact)
 inline double dhat_factor(int Py, int nz, int Px) { return nz > 1 && yz2p_ok(Py, nz, Px) ? 0.5 : 1.0; }
-// rows per CTA of the two-pass x kernels (FP64: more, smaller CTAs, as for the y/z kernel)
-__host__ __device__ constexpr int x2_rows(int real_bytes) { return real_bytes == 8 ? 2 : 4; }
-// x CTAs: pass 2 has 192 roles (up to P = 384), pass 1 has 12 P/16, the sites take 4 nx (even nx) or 8 nx items.
+// rows per CTA of the two-pass x kernels: 4, from 384 points on 8 (64-byte instead of 32-byte pieces of the spectrum,
+// fewer rows shared with neighbouring CTAs: 192x192x8 x 128 images x-forward 425 -> 382 us, step kernel 527 -> 480;
+// at 256 points the step kernel loses, 310 -> 322 on 128x128x4 x 384).  FP64: more, smaller CTAs, as for the y/z kernel
+__host__ __device__ constexpr int x2_rows(int real_bytes, int P) { return real_bytes == 8 ? 2 : P >= 384 ? 8 : 4; }
+// x CTAs: pass 2 has 48 roles per row (up to P = 384), pass 1 has 3 P/16 per row, the sites of four rows take 4 nx
+// (even nx) or 8 nx items.
 // The kernels are compiled for up to x2_threads threads in x2_blocks CTAs per SM (64 registers, 80 from P = 288
 // on) and launched with x2_launch_threads of them: on a grid of many waves the smaller block, of which more fit
 // on an SM (128x128x4 x 384 images: step kernel 311 us with 192 threads, 333 with 256); on a small grid the
 // larger one where it takes fewer rounds over the sites (112x112x1 x 60: iteration 56.2 us with 192, 53.7 with
 // 256).
 __host__ __device__ constexpr int x2_threads(int real_bytes, int P) {
-    return real_bytes == 8 ? 128 : P <= 64 ? 128 : P <= 128 ? 192 : 256;
+    return real_bytes == 8 ? 128 : P <= 64 ? 128 : P <= 128 ? 192 : P <= 320 ? 256 : 384;
 }
 __host__ __device__ constexpr int x2_blocks(int real_bytes, int P) {
     if (real_bytes == 8) return P <= 256 ? 3 : 2;
-    return P <= 64 ? 8 : P <= 128 ? 5 : P <= 256 ? 4 : 3;
+    return P <= 64 ? 8 : P <= 128 ? 5 : P <= 256 ? 4 : P <= 320 ? 3 : 2;
 }
 inline int x2_launch_threads(int real_bytes, int P, int nx, long ctas) {
     if (real_bytes == 8) return x2_threads(8, P);
@@ -281,10 +292,10 @@ inline int x2_launch_threads(int real_bytes, int P, int nx, long ctas) {
 // line stride of the x kernels: 16 / rows (mod 16)
 __host__ __device__ constexpr int x2_lsx(int real_bytes, int P) {
     const int v = t2_line(P) - 1;
-    return v + ((16 / x2_rows(real_bytes) - v % 16) + 16) % 16;
+    return v + ((16 / x2_rows(real_bytes, P) - v % 16) + 16) % 16;
 }
 inline size_t x2_smem(int real_bytes, int P, bool inverse) {
-    return (size_t)3 * x2_rows(real_bytes) * x2_lsx(real_bytes, P) * 2 * real_bytes + (inverse ? 32 * 2 * kEvalTerms * 8 : 0);
+    return (size_t)3 * x2_rows(real_bytes, P) * x2_lsx(real_bytes, P) * 2 * real_bytes + (inverse ? 32 * 2 * kEvalTerms * 8 : 0);
 }
 // Padded transform length for n sites: the smallest 2^a 3^b >= 2n - 1, or the power of two >= 2n - 1 when that
 // is at most 1/8 longer.

@@ -145,7 +145,7 @@ __device__ __forceinline__ void xfwd_gather(const GroupArgs<T>& g, cplx<T>* buf,
             // two adjacent sites (x even, x + 1) per thread: the spin planes move as float2
             const int hx = nx >> 1;
             for (int it = tid; it < rows * hx; it += nthr) {
-                const int yy = it / hx, x = 2 * (it - yy * hx);
+                const int yy = fast_div(it, g.m_hx), x = 2 * (it - yy * hx);
                 const int site = (z * g.ny + y0 + yy) * nx + x;
                 float out[2][2][3];  // [image][site][component]
 #pragma unroll
@@ -192,7 +192,7 @@ __device__ __forceinline__ void xfwd_gather(const GroupArgs<T>& g, cplx<T>* buf,
         }
     }
     for (int it = tid; it < rows * nx; it += nthr) {
-        const int yy = it / nx, x = it - yy * nx;
+        const int yy = fast_div(it, g.m_nx), x = it - yy * nx;
         const int site = (z * g.ny + y0 + yy) * nx + x;
         T out[2][3];
 #pragma unroll
@@ -556,9 +556,9 @@ __device__ __forceinline__ void xinv_sites_step2(const GroupArgs<float>& g, floa
     constexpr bool FORCE = MODE == 2 || MODE == 5;
 #pragma unroll 1
     for (int it = tid; it < 2 * rows * hx; it += nthr) {
-        const int h = it / (rows * hx);
+        const int h = it >= rows * hx;
         const int rem = it - h * rows * hx;
-        const int yy = rem / hx, x = 2 * (rem - yy * hx);
+        const int yy = fast_div(rem, g.m_hx), x = 2 * (rem - yy * hx);
         const int im = ia + h;
         if (im >= g.n_img) continue;
         const int y = y0 + yy;
@@ -676,9 +676,9 @@ __device__ __forceinline__ void xinv_sites(const GroupArgs<T>& g, T dt, T* hout,
     // before either is stored
 #pragma unroll 2
     for (int it = done ? 2 * rows * nx : tid; it < 2 * rows * nx; it += nthr) {
-        const int h = it / (rows * nx);
+        const int h = it >= rows * nx;
         const int rem = it - h * rows * nx;
-        const int yy = rem / nx, x = rem - yy * nx;
+        const int yy = fast_div(rem, g.m_nx), x = rem - yy * nx;
         const int im = ia + h;
         if (im >= g.n_img) continue;
         const int y = y0 + yy;

@@ -167,7 +167,7 @@ extern "C" ss_status ss_field_noalloc(int nx, int ny, int nz, double J, double D
         }
     }
     if (dip && Px == 128 && ty != 2 && ty != 4) ty = 8;
-    if (dip && (Px == 192 || Px == 256 || Px == 384)) ty = x2_rows(4);
+    if (dip && (Px == 192 || Px == 256 || Px == 384)) ty = 4;
     const size_t smem_a = (size_t)(Px + 3 * ty * lsx) * sizeof(float2);
     const size_t smem_c = smem_a + 32 * 2 * kEvalTerms * sizeof(double);
     size_t smem_b = (size_t)(Py + 3 * nz * lsy) * sizeof(float2);
@@ -244,6 +244,8 @@ extern "C" ss_status ss_field_noalloc(int nx, int ny, int nz, double J, double D
     g.Py = Py;
     g.n_img = n_images;
     g.n_pairs = pairs;
+    g.m_nx = fast_div_m(nx);
+    g.m_hx = fast_div_m(nx / 2);
     g.lsx = lsx;
     g.lsy = lsy;
     g.s = s;
@@ -259,7 +261,7 @@ extern "C" ss_status ss_field_noalloc(int nx, int ny, int nz, double J, double D
     g.prm = prm;
     g.interp = interp;
     g.epart = nullptr;  // the field alone
-    g.ty_a = g.ty_c = dip && t2_length(Px) ? x2_rows(4) : ty;  // the two-pass x kernels' own count
+    g.ty_a = g.ty_c = dip && t2_length(Px) ? x2_rows(4, Px) : ty;  // the two-pass x kernels' own count
     g.err = err;
     launch_xfwd<float>(g, dip, thr, smem_a, st);
     if (dip) launch_yz<float>(g, thr_b, smem_b, st);

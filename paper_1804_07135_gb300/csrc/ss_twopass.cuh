@@ -271,7 +271,7 @@ __global__ void __launch_bounds__(yz2p_threads(sizeof(T), P), yz2p_blocks(sizeof
 template <typename T, int P>
 __global__ void __launch_bounds__(x2_threads(sizeof(T), P), x2_blocks(sizeof(T), P)) xfwd2p_kernel(GroupArgs<T> g) {
     using C = cplx<T>;
-    constexpr int R2 = P / 16, H = T2<P>::H, NP = T2<P>::NP, ROWS = x2_rows(sizeof(T)), L = 3 * ROWS,
+    constexpr int R2 = P / 16, H = T2<P>::H, NP = T2<P>::NP, ROWS = x2_rows(sizeof(T), P), L = 3 * ROWS,
                   LSX = x2_lsx(sizeof(T), P);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* A = reinterpret_cast<C*>(smem_raw);  // line c * ROWS + yy: the pair at x, then rows of Z
@@ -317,7 +317,7 @@ template <typename T, int P, int MODE>
 __global__ void __launch_bounds__(x2_threads(sizeof(T), P), x2_blocks(sizeof(T), P)) xinv2p_kernel(GroupArgs<T> g, T dt,
                                                                                                    T* hout) {
     using C = cplx<T>;
-    constexpr int R2 = P / 16, H = T2<P>::H, NP = T2<P>::NP, ROWS = x2_rows(sizeof(T)), L = 3 * ROWS,
+    constexpr int R2 = P / 16, H = T2<P>::H, NP = T2<P>::NP, ROWS = x2_rows(sizeof(T), P), L = 3 * ROWS,
                   LSX = x2_lsx(sizeof(T), P);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* A = reinterpret_cast<C*>(smem_raw);  // line c * ROWS + yy: columns of T, then the field convolution at x
