@@ -166,9 +166,20 @@ __device__ __forceinline__ float2 caxpy(float a, float2 x, float2 y) { return __
 // y + a x for scalars and pairs alike
 template <typename T> __device__ __forceinline__ T caxpy_v(T a, T x, T y) { return y + a * x; }
 __device__ __forceinline__ float2 caxpy_v(float a, float2 x, float2 y) { return caxpy(a, x, y); }
-// element-wise product of two pairs (real and imaginary part each times a real factor)
-template <typename C> __device__ __forceinline__ C emul(C a, C b) { return C{a.x * b.x, a.y * b.y}; }
-__device__ __forceinline__ float2 emul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+// v with its sign flipped where the top bit of s is set
+__device__ __forceinline__ float flip_sign(float v, unsigned s) { return __uint_as_float(__float_as_uint(v) ^ s); }
+__device__ __forceinline__ double flip_sign(double v, unsigned s) {
+    return __hiloint2double(__double2hiint(v) ^ (int)s, __double2loint(v));
+}
+// f v, or conj(f v), for a real f = +-1 given as its sign bit: one paired multiplication in FP32, bit operations in
+// FP64, whose pipe is the narrow one
+__device__ __forceinline__ float2 sign_mul(float2 v, unsigned f, bool conj) {
+    const float a = flip_sign(1.f, f);
+    return __fmul2_rn(make_float2(a, conj ? -a : a), v);
+}
+__device__ __forceinline__ double2 sign_mul(double2 v, unsigned f, bool conj) {
+    return make_double2(flip_sign(v.x, f), flip_sign(v.y, conj ? f ^ 0x80000000u : f));
+}
 
 template <int I> struct ic {
     static constexpr int v = I;

@@ -55,24 +55,40 @@ template <> __device__ __forceinline__ double rsqrt_t<double>(double x) {
 __device__ __forceinline__ float rcp_t(float x) { return __frcp_rn(x); }
 __device__ __forceinline__ double rcp_t(double x) { return 1.0 / x; }
 
-// Fixed-order block reduction of NV doubles per thread; result valid in thread 0.
+// Fixed-order block reduction of NV doubles per thread; result valid in thread 0.  Within a warp the values are
+// halved while the lanes are (lanes exchange the halves they give up), so NV = 8 values take 4 + 2 + 1 + 1 + 1
+// additions instead of 5 each.
 template <int NV>
 __device__ __forceinline__ void block_reduce_d(double (&v)[NV], double* scratch /* [32*NV] */) {
+    constexpr int W = NV <= 1 ? 1 : NV <= 2 ? 2 : NV <= 4 ? 4 : 8;  // values carried, a power of two
+    static_assert(NV <= 8, "at most eight values");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = (blockDim.x + 31) >> 5;
+    double w[W];
 #pragma unroll
-    for (int k = 0; k < NV; ++k)
+    for (int k = 0; k < W; ++k) w[k] = k < NV ? v[k] : 0.0;
+    int o = 16;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
+    for (int n = W; n > 1; n >>= 1, o >>= 1) {
+        const bool up = lane & o;  // this lane keeps the upper half of the values
+#pragma unroll
+        for (int k = 0; k < n / 2; ++k) {
+            const double give = up ? w[k] : w[k + n / 2], keep = up ? w[k + n / 2] : w[k];
+            w[k] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+    }
+#pragma unroll
+    for (; o > 0; o >>= 1) w[0] += __shfl_xor_sync(0xffffffffu, w[0], o);
+    // lane's value index: its top log2 W lane bits, highest bit first
+    constexpr int S = W == 8 ? 2 : W == 4 ? 3 : W == 2 ? 4 : 5;
+    const int idx = lane >> S;
     __syncthreads();
-    if (lane == 0)
-#pragma unroll
-        for (int k = 0; k < NV; ++k) scratch[warp * NV + k] = v[k];
+    if ((lane & ((1 << S) - 1)) == 0 && idx < NV) scratch[warp * NV + idx] = w[0];
     __syncthreads();
     if (threadIdx.x == 0) {
 #pragma unroll
         for (int k = 0; k < NV; ++k) {
             double a = 0.0;
-            for (int w = 0; w < nwarp; ++w) a += scratch[w * NV + k];
+            for (int w2 = 0; w2 < nwarp; ++w2) a += scratch[w2 * NV + k];
             v[k] = a;
         }
     }
@@ -653,7 +669,9 @@ __device__ __forceinline__ void xinv_sites(const GroupArgs<T>& g, T dt, T* hout,
     using C = cplx<T>;
     const int nx = g.nx, ny = g.ny, nz = g.nz, N = g.N;
     const int ia = 2 * p;
-    constexpr int NV = MODE == 1 ? 2 * kEvalTerms : 2;
+    // evaluation terms per image: in FP64 the four of Eq. 1, in FP32 also the convolution's squared norm
+    constexpr int NT = MODE != 1 ? 1 : std::is_same<T, float>::value ? kEvalTerms : 4;
+    constexpr int NV = 2 * NT;
     double acc[NV];
 #pragma unroll
     for (int k = 0; k < NV; ++k) acc[k] = 0.0;
@@ -709,7 +727,7 @@ __device__ __forceinline__ void xinv_sites(const GroupArgs<T>& g, T dt, T* hout,
             for (int c = 0; c < 3; ++c) conv[c] = g.hdir[(size_t)im * 3 * N + (size_t)c * N + site];
         }
         T hf[3];
-        local_field(pr, s0, xp, xm, yp, ym, zp, zm, conv, hf);
+        if (MODE != 1 || hout) local_field(pr, s0, xp, xm, yp, ym, zp, zm, conv, hf);
         if (MODE == 0 || (MODE == 3 && !climbs[h])) {
             T un[3];
             eacc[h] += step_site(s0, hf, dt, un);
@@ -761,23 +779,25 @@ __device__ __forceinline__ void xinv_sites(const GroupArgs<T>& g, T dt, T* hout,
                 for (int c = 0; c < 3; ++c) o[(size_t)c * N] = f[c];
             }
         } else {
-            // Eq. 1's terms with their constants set to 1, of the spins renormalised per site, bonds to +x,
-            // +y, +z counted once, and the squared norm of the dipole convolution.  In the path's
-            // precision R: the FP64 path sums FP64 terms; the FP32 path's evaluation (its energies only
-            // select the images the FP64 evaluation computes, and bound their own round-off) keeps the
-            // terms in FP32 and sums them per thread in FP32 and across warps in FP64
+            // Eq. 1's terms with their constants set to 1, bonds to +x, +y, +z counted once, and (FP32) the squared
+            // norm of the dipole convolution.  In the path's precision R: the FP64 path sums FP64 terms of its
+            // states, which are unit vectors to rounding (normalised by the step, the gather or widen_unit); the
+            // FP32 path's evaluation (its energies only select the images the FP64 evaluation computes, and bound
+            // their own round-off) renormalises per site, keeps the terms in FP32 and sums them per thread in
+            // FP32 and across warps in FP64
             using R = T;
             auto nrm = [](const T* v, R* o) {
-                const R a = v[0], b = v[1], c = v[2];
-                const R n2 = a * a + b * b + c * c;
-                R r = R(0);
-                if constexpr (std::is_same<T, float>::value)
-                    r = n2 > 0.f ? rsqrtf(n2) : 0.f;
-                else
-                    r = n2 > 0.0 ? rsqrt_nr(n2) : 0.0;
-                o[0] = a * r;
-                o[1] = b * r;
-                o[2] = c * r;
+                if constexpr (std::is_same<T, float>::value) {
+                    const R n2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
+                    const R r = n2 > 0.f ? rsqrtf(n2) : 0.f;
+                    o[0] = v[0] * r;
+                    o[1] = v[1] * r;
+                    o[2] = v[2] * r;
+                } else {
+                    o[0] = v[0];
+                    o[1] = v[1];
+                    o[2] = v[2];
+                }
             };
             R si[3], sx[3], sy[3], sz[3];
             nrm(s0, si);
@@ -798,19 +818,22 @@ __device__ __forceinline__ void xinv_sites(const GroupArgs<T>& g, T dt, T* hout,
             }
             const R tK = -si[2] * si[2];
             const R tw_ = R(-0.5) * (conv[0] * si[0] + conv[1] * si[1] + conv[2] * si[2]);
-            const R cn = conv[0] * conv[0] + conv[1] * conv[1] + conv[2] * conv[2];
             if constexpr (std::is_same<T, float>::value) {
+                const R cn = conv[0] * conv[0] + conv[1] * conv[1] + conv[2] * conv[2];
                 facc[kEvalTerms * h + 0] += tJ;
                 facc[kEvalTerms * h + 1] += tD;
                 facc[kEvalTerms * h + 2] += tK;
                 facc[kEvalTerms * h + 3] += tw_;
                 facc[kEvalTerms * h + 4] += cn;
             } else {
-                acc[kEvalTerms * h + 0] += tJ;
-                acc[kEvalTerms * h + 1] += tD;
-                acc[kEvalTerms * h + 2] += tK;
-                acc[kEvalTerms * h + 3] += tw_;
-                acc[kEvalTerms * h + 4] += cn;
+#pragma unroll
+                for (int i = 0; i < 2; ++i)  // (constant indices: the sums stay in registers)
+                    if (i == h) {
+                        acc[NT * i + 0] += tJ;
+                        acc[NT * i + 1] += tD;
+                        acc[NT * i + 2] += tK;
+                        acc[NT * i + 3] += tw_;
+                    }
             }
             if (hout) {
                 T* o = hout + (size_t)im * 3 * N + site;
@@ -839,7 +862,7 @@ __device__ __forceinline__ void xinv_sites(const GroupArgs<T>& g, T dt, T* hout,
                 g.epart[(size_t)blk * g.n_img + im] = acc[h];  // [block][image]
             } else {
                 for (int k = 0; k < kEvalTerms; ++k)
-                    g.epart[((size_t)blk * g.n_img + im) * kEvalTerms + k] = acc[kEvalTerms * h + k];
+                    g.epart[((size_t)blk * g.n_img + im) * kEvalTerms + k] = k < NT ? acc[NT * h + k] : 0.0;
             }
         }
     }
@@ -852,7 +875,7 @@ __device__ __forceinline__ void xinv_sites(const GroupArgs<T>& g, T dt, T* hout,
 //     + 2 K s_z z                                                        (Eq. 5)
 //     + w * dipole convolution                                           (Eq. 6)
 // MODE 0 (step): e += -(1/2) h.s (Eq. 8), s' = normalise(s + dt (h - (s.h) s)) (Eqs. 10, 13).
-// MODE 1 (eval): FP64 energy terms of the FP64-renormalised spins, bonds to +x, +y, +z counted once
+// MODE 1 (eval): energy terms of the unit spins in the path's precision, bonds to +x, +y, +z counted once
 //                (Eq. 1): tJ = -sum s_i.s_j, tD = sum (r_ij x z).(s_i x s_j), tK = -sum s_z^2,
 //                tw = -(1/2) sum conv.s; optionally the field h.
 template <typename T, bool DO_FFT, int MODE>
@@ -1739,10 +1762,6 @@ __global__ void __launch_bounds__(256) rk_commit_kernel(GroupArgs<T> g, RkArgs<T
 // M (images that share a table load) is 4 while the grid still fills the chip twice, fewer on small
 // lattices, where CTAs are what is missing.
 constexpr int kDirTile = 256, kDirWarps = 8;
-__device__ __forceinline__ float flip_sign(float v, unsigned s) { return __uint_as_float(__float_as_uint(v) ^ s); }
-__device__ __forceinline__ double flip_sign(double v, unsigned s) {
-    return __hiloint2double(__double2hiint(v) ^ (int)s, __double2loint(v));
-}
 template <typename T, int M, bool FILM>
 __global__ void __launch_bounds__(32 * kDirWarps) dipole_direct_kernel(GroupArgs<T> g, T* hdir, const T* __restrict__ dtab) {
     constexpr int Q = 3 * M;
@@ -1901,7 +1920,7 @@ __global__ void __launch_bounds__(256) climb_apply_kernel(GroupArgs<T> g, ArcArg
 // and their weights come as vectors: 24 multiply-adds for 3 + 2 loads instead of 3 for 4.  Dynamic shared
 // memory: the string's K images at the CTA's 32 sites, [K][3][32], then W, [q][row] at row stride a.w_stride (whole
 // vectors, off a multiple of 32 words), when w_on_chip (else W is read through L1).  The tile is loaded whole before any row is written back.  Bound by
-// FP32 issue (2 K^2 N x 3 multiply-adds); 112x112x1 x 60 images: SPLINE_APPLY on one GB300.
+// FP32 issue (2 K^2 N x 3 multiply-adds); 112x112x1 x 60 images: 32.7 -> 18.3 us on one GB300.
 template <typename T>
 __global__ void __launch_bounds__(256) spline_apply_kernel(GroupArgs<T> g, ArcArgs a, int w_on_chip) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1967,30 +1986,35 @@ __global__ void __launch_bounds__(256) spline_apply_kernel(GroupArgs<T> g, ArcAr
     }
 }
 
-// eval reduce: grid (n_str), thread per image: terms[str][k][4], energies[str][k] and (when cnorm2 is
-// given) the squared norm of the dipole convolution cnorm2[str][k], in FP64.  Images of pairs that
-// g.pair_on leaves out are skipped (their partials were not written).
+// eval reduce: grid (n_str, maxK), one warp per term (kEvalTerms warps): terms[str][k][4], energies[str][k] and (when
+// cnorm2 is given) the squared norm of the dipole convolution cnorm2[str][k], in FP64.  Images of pairs that
+// g.pair_on leaves out are skipped (their partials were not written).  A lane sums every 32nd block's partial, eight
+// loads at a time: one thread per image took a chain of n_eblk dependent FP64 additions per term (65 cycles each:
+// 64x64x8 x 32 images, FP64, 79.9 -> 5.0 us on one GB300, FP32 36.0 -> 4.1 us).
 template <typename T>
-__global__ void eval_reduce_kernel(GroupArgs<T> g, ArcArgs a, double* terms, double* energies, double* cnorm2) {
-    const int str = blockIdx.x;
-    const int K = a.str_K[str], img0 = a.str_img0[str];
-    for (int k = threadIdx.x; k < K; k += blockDim.x) {
-        const int im = img0 + k;
-        if (g.pair_on && !g.pair_on[im >> 1]) continue;
-        double t[kEvalTerms];
-        for (int q = 0; q < kEvalTerms; ++q) {
-            double v = 0.0;
-            const double* ep = g.epart + (size_t)im * kEvalTerms + q;
-            for (int b = 0; b < g.n_eblk; ++b) v += ep[(size_t)b * g.n_img * kEvalTerms];
-            t[q] = v;
-            if (q < 4) terms[((size_t)str * a.maxK + k) * 4 + q] = v;
-        }
-        if (cnorm2) cnorm2[(size_t)str * a.maxK + k] = t[4];
-        const ImgParam<T> pr = g.prm[im];
-        const double e = (double)pr.J * t[0] + (double)pr.D * t[1] + (double)pr.K * t[2] + (double)pr.w * t[3];
-        energies[(size_t)str * a.maxK + k] = e;
-        if (!isfinite(e)) atomicOr(g.err, kErrNonFinite);
-    }
+__global__ void __launch_bounds__(32 * kEvalTerms) eval_reduce_kernel(GroupArgs<T> g, ArcArgs a, double* terms,
+                                                                      double* energies, double* cnorm2) {
+    __shared__ double t[kEvalTerms];
+    const int str = blockIdx.x, k = blockIdx.y, lane = threadIdx.x & 31, q = threadIdx.x >> 5;
+    if (k >= a.str_K[str]) return;  // uniform over the CTA
+    const int im = a.str_img0[str] + k;
+    if (g.pair_on && !g.pair_on[im >> 1]) return;
+    const double* ep = g.epart + (size_t)im * kEvalTerms + q;
+    const size_t stride = (size_t)g.n_img * kEvalTerms;
+    double v = 0.0;
+#pragma unroll 8
+    for (int b = lane; b < g.n_eblk; b += 32) v += ep[b * stride];
+    v = warp_sum_d(v);
+    if (lane == 0) t[q] = v;
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    const size_t o = (size_t)str * a.maxK + k;
+    for (int i = 0; i < 4; ++i) terms[o * 4 + i] = t[i];
+    if (cnorm2) cnorm2[o] = t[4];
+    const ImgParam<T> pr = g.prm[im];
+    const double e = (double)pr.J * t[0] + (double)pr.D * t[1] + (double)pr.K * t[2] + (double)pr.w * t[3];
+    energies[o] = e;
+    if (!isfinite(e)) atomicOr(g.err, kErrNonFinite);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -2332,7 +2356,7 @@ template <typename T> void launch_arc(const GroupArgs<T>& g, const ArcArgs& a, i
 template <typename T>
 void launch_eval_reduce(const GroupArgs<T>& g, const ArcArgs& a, double* terms, double* energies, double* cnorm2,
                         cudaStream_t st) {
-    eval_reduce_kernel<T><<<a.n_str, 128, 0, st>>>(g, a, terms, energies, cnorm2);
+    eval_reduce_kernel<T><<<dim3(a.n_str, a.maxK), 32 * kEvalTerms, 0, st>>>(g, a, terms, energies, cnorm2);
 }
 
 template <typename T, typename Tin>

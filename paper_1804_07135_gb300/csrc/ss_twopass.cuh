@@ -33,10 +33,10 @@ template <int NZ, int PAR> struct ZSys {  // PAR 0: (x, y in e; z in o), 1: (x, 
 
 // One system at one frequency: A points at the frequency's element of line 0 (line stride LS), d at its
 // coefficients (component c, |dz| at d[(|dz| * 6 + c) * DQ]); par the system; fx, fy the parity signs of kx, ky
-// (the tensor's xy, xz, yz are odd in them: flip x and y going in and coming out).  The result replaces the
-// inputs, conjugated (the inverse transform is the conjugate of the forward transform of the conjugate).
+// as sign bits (the tensor's xy, xz, yz are odd in them: flip x and y going in and coming out).  The result
+// replaces the inputs, conjugated (the inverse transform is the conjugate of the forward transform of the conjugate).
 template <int NZ, int PAR, int LS, int DQ, typename T, typename C>
-__device__ __forceinline__ void zconv_sys(C* A, const T* __restrict__ d, int par, T fx, T fy) {
+__device__ __forceinline__ void zconv_sys(C* A, const T* __restrict__ d, int par, unsigned fx, unsigned fy) {
     using S = ZSys<NZ, PAR>;  // the shape; for even NZ both systems share it and par picks one at run time
     constexpr int NA = S::NXY, NB = S::NZC;
     constexpr int NA1 = NA > 0 ? NA : 1, NB1 = NB > 0 ? NB : 1;
@@ -48,8 +48,8 @@ __device__ __forceinline__ void zconv_sys(C* A, const T* __restrict__ d, int par
     const C zero = C{T(0), T(0)};
 #pragma unroll
     for (int i = 0; i < NA; ++i) {
-        X[i] = emul(C{fx, fx}, Ax[i * LS]);
-        Y[i] = emul(C{fy, fy}, Ay[i * LS]);
+        X[i] = sign_mul(Ax[i * LS], fx, false);
+        Y[i] = sign_mul(Ay[i * LS], fy, false);
         HX[i] = HY[i] = zero;
     }
 #pragma unroll
@@ -128,8 +128,8 @@ __device__ __forceinline__ void zconv_sys(C* A, const T* __restrict__ d, int par
     }
 #pragma unroll
     for (int i = 0; i < NA; ++i) {
-        Ax[i * LS] = emul(C{fx, -fx}, HX[i]);
-        Ay[i * LS] = emul(C{fy, -fy}, HY[i]);
+        Ax[i * LS] = sign_mul(HX[i], fx, true);
+        Ay[i * LS] = sign_mul(HY[i], fy, true);
     }
     if constexpr (NB > 0) {
         load(2, t);  // zz
@@ -150,15 +150,15 @@ __device__ __forceinline__ void zconv_sys(C* A, const T* __restrict__ d, int par
 template <int NZ, int P, typename T, typename C>
 __device__ __forceinline__ void zconv_t2(C* A, int kx, int Px, const T* dslab, int tid, int nthr) {
     constexpr int LS = t2_line(P), DQ = P / 2 + 1;
-    const T fx = kx > Px / 2 ? T(-1) : T(1);
+    const unsigned fx = kx > Px / 2 ? 0x80000000u : 0u;  // the parity signs of kx, ky, as sign bits
     for (int it = tid; it < (NZ == 1 ? P : 2 * P); it += nthr) {
         const int par = it >= P ? 1 : 0, ky = it - par * P;
-        const T fy = ky > P / 2 ? T(-1) : T(1);
+        const unsigned fy = ky > P / 2 ? 0x80000000u : 0u;
         const T* d = dslab + min(ky, P - ky);
         C* a = A + t2_pos(ky);
         if constexpr (NZ == 1) {  // xz and yz vanish
             const C X = a[0], Y = a[LS], Z = a[2 * LS];
-            const T xx = d[0], yy = d[DQ], zz = d[2 * DQ], xy = fx * fy * d[3 * DQ];
+            const T xx = d[0], yy = d[DQ], zz = d[2 * DQ], xy = flip_sign(d[3 * DQ], fx ^ fy);
             a[0] = C{xx * X.x + xy * Y.x, -(xx * X.y + xy * Y.y)};
             a[LS] = C{xy * X.x + yy * Y.x, -(xy * X.y + yy * Y.y)};
             a[2 * LS] = C{zz * Z.x, -zz * Z.y};
