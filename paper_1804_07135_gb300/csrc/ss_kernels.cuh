@@ -2018,12 +2018,50 @@ __global__ void __launch_bounds__(32 * kEvalTerms) eval_reduce_kernel(GroupArgs<
 }
 
 // ------------------------------------------------------------------------------------------------
-// layout conversion: caller [K][N][3] <-> internal [K][3][N]; input spins normalised in FP64.
+// (a, b, c) / |(a, b, c)| in pairs of FP32 numbers, without the FP64 pipe (16 times slower than the FP32 one): the
+// squared norm h + l by error-free products, y = rsqrt(h) with its residual e = 1 - (h + l) y^2, and the components
+// x (y + y e / 2 + 3 y e^2 / 8) with the products' rounding errors added, each rounded once.  Error before that last
+// rounding below 1e-13 of the component (e ~ 3e-7; of components above 1e-30): FP64 arithmetic rounded to FP32
+// differs in one of 10^7 roundings.  False where a term might leave
+// the FP32 range (or a component is not finite): the caller then takes the FP64 path.
+__device__ __forceinline__ bool unit_f32(float a, float b, float c, float (&o)[3]) {
+    const float aa = __fmul_rn(a, a), bb = __fmul_rn(b, b), cc = __fmul_rn(c, c);  // (_rn: never fused into the sums)
+    const float t = __fadd_rn(aa, bb), h = __fadd_rn(t, cc);
+    if (!(h > 1e-6f && h < 1e6f)) return false;
+    float l = fmaf(a, a, -aa) + fmaf(b, b, -bb) + fmaf(c, c, -cc);
+    const float bv = __fsub_rn(t, aa), cv = __fsub_rn(h, t);  // and the rounding errors of the two sums
+    l += __fsub_rn(aa, __fsub_rn(t, bv)) + __fsub_rn(bb, bv) + __fsub_rn(t, __fsub_rn(h, cv)) + __fsub_rn(cc, cv);
+    const float y = rsqrtf(h), p = __fmul_rn(h, y), pe = fmaf(h, y, -p);
+    const float e = fmaf(-p, y, 1.f) - (pe + l * y) * y;
+    const float d = fmaf(0.375f * e, e, 0.5f * e) * y;
+    const float v[3] = {a, b, c};
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const float q = __fmul_rn(v[i], y);
+        o[i] = __fadd_rn(q, fmaf(v[i], d, fmaf(v[i], y, -q)));
+    }
+    return true;
+}
+
+// layout conversion: caller [K][N][3] <-> internal [K][3][N]; grid (site tiles of 256, images).  Input spins are
+// normalised in FP64, or in pairs of FP32 numbers where input and state are FP32 (64x64x8 x 32 images: in FP64
+// 48.4 us on one GB300, bound by that pipe; 6.2 us now).
 template <typename T, typename Tin>
-__global__ void aos_to_soa_kernel(const Tin* src, T* dst, int K, int N, int* err) {
-    const size_t total = (size_t)K * N;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const size_t k = i / N, n = i - k * N;
+__global__ void __launch_bounds__(256) aos_to_soa_kernel(const Tin* src, T* dst, int K, int N, int* err) {
+    const int n = blockIdx.x * blockDim.x + threadIdx.x;
+    if (n >= N) return;
+    for (int k = blockIdx.y; k < K; k += gridDim.y) {
+        const size_t i = (size_t)k * N + n;
+        T* d = dst + (size_t)k * 3 * N + n;
+        if constexpr (std::is_same<T, float>::value && std::is_same<Tin, float>::value) {
+            float o[3];
+            if (unit_f32(src[3 * i], src[3 * i + 1], src[3 * i + 2], o)) {
+                d[0] = o[0];
+                d[N] = o[1];
+                d[2 * (size_t)N] = o[2];
+                continue;
+            }
+        }
         const double a = src[3 * i], b = src[3 * i + 1], c = src[3 * i + 2];
         const double n2 = a * a + b * b + c * c;
         double r = 0.0;
@@ -2032,22 +2070,22 @@ __global__ void aos_to_soa_kernel(const Tin* src, T* dst, int K, int N, int* err
         } else {
             r = rsqrt_t<double>(n2);
         }
-        T* d = dst + k * 3 * N + n;
         d[0] = T(a * r);
         d[N] = T(b * r);
-        d[2 * N] = T(c * r);
+        d[2 * (size_t)N] = T(c * r);
     }
 }
 
 template <typename T, typename Tout>
-__global__ void soa_to_aos_kernel(const T* src, Tout* dst, int K, int N, Tout scale) {
-    const size_t total = (size_t)K * N;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const size_t k = i / N, n = i - k * N;
-        const T* s = src + k * 3 * N + n;
+__global__ void __launch_bounds__(256) soa_to_aos_kernel(const T* src, Tout* dst, int K, int N, Tout scale) {
+    const int n = blockIdx.x * blockDim.x + threadIdx.x;
+    if (n >= N) return;
+    for (int k = blockIdx.y; k < K; k += gridDim.y) {
+        const size_t i = (size_t)k * N + n;
+        const T* s = src + (size_t)k * 3 * N + n;
         dst[3 * i] = scale * Tout(s[0]);
         dst[3 * i + 1] = scale * Tout(s[N]);
-        dst[3 * i + 2] = scale * Tout(s[2 * N]);
+        dst[3 * i + 2] = scale * Tout(s[2 * (size_t)N]);
     }
 }
 
@@ -2111,11 +2149,17 @@ __global__ void widen_unit_kernel(const float* __restrict__ src, double* __restr
         if (pair_on && !pair_on[k >> 1]) continue;  // uniform over the CTA
         const size_t b = (size_t)k * 3 * N + n;
         const double a0 = src[b], a1 = src[b + N], a2 = src[b + 2 * (size_t)N];
-        const double n2 = a0 * a0 + a1 * a1 + a2 * a2;
-        const double r = n2 > 0.0 ? rsqrt_nr(n2) : 0.0;
-        dst[b] = a0 * r;
-        dst[b + N] = a1 * r;
-        dst[b + 2 * (size_t)N] = a2 * r;
+        const double e = -fma(a2, a2, fma(a1, a1, fma(a0, a0, -1.0)));
+        double q;  // 1 / sqrt(1 - e) - 1
+        if (fabsf((float)e) < 1e-4f) {  // spins normalised in FP32 (e ~ 1e-7): the series up to e^3, < 3e-17 off
+            q = e * fma(e, fma(e, 0.3125, 0.375), 0.5);
+        } else {
+            const double n2 = a0 * a0 + a1 * a1 + a2 * a2;
+            q = (n2 > 0.0 ? rsqrt_nr(n2) : 0.0) - 1.0;
+        }
+        dst[b] = fma(a0, q, a0);
+        dst[b + N] = fma(a1, q, a1);
+        dst[b + 2 * (size_t)N] = fma(a2, q, a2);
     }
 }
 
@@ -2361,12 +2405,12 @@ void launch_eval_reduce(const GroupArgs<T>& g, const ArcArgs& a, double* terms, 
 
 template <typename T, typename Tin>
 void launch_aos_to_soa(const Tin* src, T* dst, int K, int N, int* err, cudaStream_t st) {
-    aos_to_soa_kernel<T, Tin><<<grid1d((size_t)K * N, 256), 256, 0, st>>>(src, dst, K, N, err);
+    aos_to_soa_kernel<T, Tin><<<dim3((N + 255) / 256, std::min(K, 65535)), 256, 0, st>>>(src, dst, K, N, err);
 }
 
 template <typename T, typename Tout>
 void launch_soa_to_aos(const T* src, Tout* dst, int K, int N, Tout scale, cudaStream_t st) {
-    soa_to_aos_kernel<T, Tout><<<grid1d((size_t)K * N, 256), 256, 0, st>>>(src, dst, K, N, scale);
+    soa_to_aos_kernel<T, Tout><<<dim3((N + 255) / 256, std::min(K, 65535)), 256, 0, st>>>(src, dst, K, N, scale);
 }
 
 template <typename T>

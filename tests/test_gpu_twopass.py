@@ -72,3 +72,32 @@ def test_fp64_kernels(case):
     for k in range(3):
         ref = oracle.field(m, path[k])
         assert np.abs(got[k] - ref).max() <= 1e-12 * np.abs(ref).max(), k
+
+
+def test_fp32_input_spins_normalised_to_the_last_bit():
+    # FP32 spins of any norm, in and beyond the range the FP32-pair arithmetic takes (squared norms 1e-6 to 1e6),
+    # with components that vanish or underflow.  Tolerance: one rounding to FP32 (0.5 units in the last place), and
+    # 1e-6 for what the arithmetic before it may leave.
+    rng = np.random.default_rng(5)
+    nx, ny, K = 23, 13, 5
+    v = W.random_spins((K, nx * ny, 3), seed=3)
+    scale = 10.0 ** rng.choice([0, 0, -1, 1, -2.9, 2.9, -3.1, 3.1, -15, 15], (K, nx * ny, 1))
+    v = (v * scale).astype(np.float32)
+    v[0, ::3, 0] = 0.0
+    v[1, ::4, 1:] = 0.0
+    v[2, ::5, 2] *= np.float32(1e-20)
+    v[3, :, 0] = np.float32(2.0 ** -63)
+    with binding.StringMethod([(nx, ny, 1, 1.0, 0.3, 0.1, 0.0, K)]) as sm:
+        sm.set_path(0, v)
+        got = sm.get_path(0)
+        w = v.astype(np.longdouble)
+        ref = w / np.sqrt((w * w).sum(-1, keepdims=True))
+        ulp = np.maximum(np.spacing(np.abs(ref).astype(np.float32)), np.float32(1e-45)).astype(np.longdouble)
+        assert (np.abs(got.astype(np.float32) - ref) / ulp).max() <= 0.5 + 1e-6
+        for bad in ([0, 0, 0], [np.inf, 0, 1], [np.nan, 1, 0]):
+            w = v.copy()
+            w[4, -1] = bad
+            with pytest.raises(binding.SsError):
+                sm.set_path(0, w)
+                sm.get_path(0)
+            sm.set_path(0, v)
