@@ -913,9 +913,13 @@ template <typename T> void issue_eval(ss_ctx* c, Group& g, T* hout, cudaStream_t
     GroupArgs<T> a = group_args<T>(c, g);
     a.pair_on = pair_on;
     launch_xfwd<T>(a, g.dipole, g.thr_a, g.smem_a, st);
-    if (g.dipole) launch_yz<T>(a, g.thr_b, g.smem_b, st);
+    if constexpr (std::is_same<T, double>::value)  // energies alone: their dipole term from the spectrum
+        a.w_spec = g.dipole && !hout && yzq2p_ok(g.Py, g.nz, g.Px);
+    if constexpr (std::is_same<T, double>::value)
+        if (a.w_spec) launch_yzq(a, st);
+    if (g.dipole && !a.w_spec) launch_yz<T>(a, g.thr_b, g.smem_b, st);
     if (g.direct) launch_dipole_direct<T>(a, (T*)g.hdir, (const T*)g.dtab, st);
-    launch_xinv_eval<T>(a, g.dipole, hout, g.thr_c, g.smem_c_eval, st);
+    launch_xinv_eval<T>(a, g.dipole && !a.w_spec, hout, g.thr_c, g.smem_c_eval, st);
     launch_eval_reduce<T>(a, g.arc, g.eval_terms, g.eval_E, g.eval_cn, st);
 }
 

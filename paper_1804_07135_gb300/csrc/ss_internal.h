@@ -113,6 +113,7 @@ template <typename T> struct GroupArgs {
     const T* hdir;         // [image][3][N] direct dipole sums (SS_DIPOLE_DIRECT), or null
     const int* pair_on;    // [n_pairs] evaluate only the pairs flagged here (generic kernels), or null: all
     RkNext<T> rk;          // force modes only
+    int w_spec;            // evaluation: the dipole term per (column <= Px / 2, pair) is in the spectrum (FP64)
     int yz_kxb;            // kx columns per CTA of the two-pass y/z kernel (autotuned; 0: the default)
 };
 // Energy partials per image of the evaluation mode: the four terms of Eq. 1 (J, D, K, w with the constant
@@ -237,7 +238,7 @@ inline YzColumns yz2p_columns(int nz) {
     if (nz <= 4) return {2, {2, 1, 0}};
     return {nz <= kT2MaxNz ? 1 : 0, {1, 0, 0}};
 }
-inline size_t yz2p_smem(int real_bytes, int Py, int nz, int kxb) { return (size_t)3 * nz * kxb * t2_line(Py) * 2 * real_bytes; }
+__host__ __device__ constexpr size_t yz2p_smem(int real_bytes, int Py, int nz, int kxb) { return (size_t)3 * nz * kxb * t2_line(Py) * 2 * real_bytes; }
 inline bool yz2p_ok(int Py, int nz, int Px) {
     if (!t2_length(Py)) return false;
     const YzColumns k = yz2p_columns(nz);
@@ -255,6 +256,10 @@ __host__ __device__ constexpr int yz2p_blocks(int real_bytes, int P) {
     if (real_bytes == 8) return P <= 192 ? 3 : P <= 256 ? 2 : 1;
     return P <= 128 ? 6 : P <= 256 ? 4 : P <= 320 ? 3 : 2;
 }
+// The FP64 energy kernel keeps two columns in shared memory (227 KB, less its reduction's): 8 layers up to 256 points
+constexpr int kYzqThreads = 128;
+__host__ __device__ constexpr bool yzq2p_fits(int P, int nz) { return yz2p_smem(8, P, nz, 2) <= 226 * 1024; }
+inline bool yzq2p_ok(int Py, int nz, int Px) { return yz2p_ok(Py, nz, Px) && yzq2p_fits(Py, nz); }
 // columns per CTA a launch uses: the tuned count when it is one of them
 inline int yz2p_kxb_use(int real_bytes, int nz, int tuned) {
     const YzColumns k = yz2p_columns(nz);
@@ -318,6 +323,7 @@ template <typename T> void launch_xfwd(const GroupArgs<T>& g, bool do_fft, int n
 template <typename T> void launch_yz(const GroupArgs<T>& g, int nthr, size_t smem, cudaStream_t st);
 template <typename T>
 void launch_xinv_step(const GroupArgs<T>& g, bool do_fft, T dt, int nthr, size_t smem, cudaStream_t st);
+void launch_yzq(const GroupArgs<double>& g, cudaStream_t st);  // where yzq2p_ok
 template <typename T>
 void launch_xinv_eval(const GroupArgs<T>& g, bool do_fft, T* hout, int nthr, size_t smem, cudaStream_t st);
 // Runge-Kutta stage: the force of Eq. 13 (or with llg the right-hand side of Eq. 9) at the state in s
@@ -352,6 +358,7 @@ void launch_soa_to_aos(const T* src, Tout* dst, int K, int N, Tout scale, cudaSt
 template <typename T, int P> void t2_xfwd(const GroupArgs<T>& g, cudaStream_t st);
 template <typename T, int P> void t2_xinv(const GroupArgs<T>& g, int mode, T dt, T* hout, bool pdl, cudaStream_t st);
 template <typename T, int P> void t2_yz(const GroupArgs<T>& g, cudaStream_t st);
+template <typename T, int P> void t2_yzq(const GroupArgs<T>& g, cudaStream_t st);  // double only
 template <typename T, int P> void t2_smem_limits(int bytes);
 // The limits of the two-pass kernels of lengths Px and Py (those that have some).
 template <typename T> void set_t2_smem_limits(int Px, int Py, int bytes);

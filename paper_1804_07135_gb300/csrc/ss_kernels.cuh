@@ -2004,6 +2004,13 @@ __global__ void __launch_bounds__(32 * kEvalTerms) eval_reduce_kernel(GroupArgs<
     double v = 0.0;
 #pragma unroll 8
     for (int b = lane; b < g.n_eblk; b += 32) v += ep[b * stride];
+    if constexpr (std::is_same<T, double>::value)
+        if (g.w_spec && q == 3) {  // left by yzq2p_kernel
+            const size_t col = (size_t)3 * g.nz * g.ny;
+            const double* sp = reinterpret_cast<const double*>(g.spec + (size_t)(im >> 1) * g.Px * col) + (im & 1);
+#pragma unroll 4
+            for (int kx = lane; kx <= g.Px / 2; kx += 32) v += sp[2 * kx * col];
+        }
     v = warp_sum_d(v);
     if (lane == 0) t[q] = v;
     __syncthreads();
@@ -2301,6 +2308,17 @@ void launch_xinv_eval(const GroupArgs<T>& g, bool do_fft, T* hout, int nthr, siz
         xinv_kernel<T, false, 1><<<grid, nthr, smem, st>>>(g, T(0), hout);
     }
 }
+
+#ifdef SS_COMMON_LAUNCHERS
+void launch_yzq(const GroupArgs<double>& g, cudaStream_t st) {
+    switch (g.Py) {
+#define SS_CASE(P) \
+    case P: t2_yzq<double, P>(g, st); break;
+        SS_T2_LENGTHS(SS_CASE)
+#undef SS_CASE
+    }
+}
+#endif
 
 template <typename T, int MODE>
 static void launch_xinv_force_mode(const GroupArgs<T>& g, bool do_fft, T* kout, T flag, int nthr, size_t smem,

@@ -257,6 +257,193 @@ __global__ void __launch_bounds__(yz2p_threads(sizeof(T), P), yz2p_blocks(sizeof
 }
 
 // ------------------------------------------------------------------------------------------------
+// Dipole energies without the field (FP64): by Parseval's theorem sum_sites conv.s is the sum over frequencies of
+// conj(S).(T S), so an evaluation that wants no field stops at the spectrum: no inverse transforms, and the step
+// kernel in evaluation mode has no spectrum to read.  The spectrum of an image pair is Z = A + i B with A and B those
+// of real functions: A(k) = (Z(k) + conj Z(-k)) / 2, i B(k) = (Z(k) - conj Z(-k)) / 2, which needs the columns kx and
+// Px - kx side by side: both live in the CTA's shared memory, and it does both images at kx (weight 2 where the
+// columns differ).  Every real vector v (real and imaginary part of A and of B) takes v^T M v of the real symmetric
+// matrix M of its system (ZSys above) by its lower triangle: 90 multiply-adds at 8 layers where T v takes 144.
+// Bound by the FP64 pipe.  On one GB300, y/z and step kernel in evaluation mode before and now: 64x64x8 x 32 images
+// 815 + 220 -> 483 + 80 us, 64x64x4 x 16 194 + 60 -> 116 + 25, one image pair of 64x64x8 183 + 36 -> 139 + 26.
+// Errors against the oracle are unchanged (8e-15 of the largest energy at most; the w terms move by 4e-16).
+
+// Half of v^T M v summed over real and imaginary part of image A (qa) and image B (qb), each twice the spectrum, for
+// one system at one frequency: A0 and A1 point at the elements of line 0 at k and -k; d, par, fx, fy as for zconv_sys.
+template <int NZ, int PAR, int LS, int DQ>
+__device__ __forceinline__ void zquad_sys(const double2* A0, const double2* A1, const double* __restrict__ d, int par,
+                                          unsigned fx, unsigned fy, double& qa, double& qb) {
+    using S = ZSys<NZ, PAR>;
+    constexpr int NA = S::NXY, NB = S::NZC;
+    constexpr int NA1 = NA > 0 ? NA : 1, NB1 = NB > 0 ? NB : 1;
+    const double sg = par ? -1.0 : 1.0;
+    const int lx = (par ? S::ME : 0) * LS, lz = (2 * NZ + (par ? 0 : S::ME)) * LS;
+    struct V {  // the four real vectors' components
+        double v[4];
+    };
+    auto load2 = [&](int at, unsigned f) {  // f: sign of the component's real couplings
+        const double2 a = A0[at], b = A1[at];
+        return V{{flip_sign(a.x + b.x, f), flip_sign(a.y - b.y, f), flip_sign(a.x - b.x, f), flip_sign(a.y + b.y, f)}};
+    };
+    V X[NA1], Y[NA1], Z[NB1], h;  // h: a row of M's lower triangle times the vectors
+#pragma unroll
+    for (int i = 0; i < NA; ++i) {
+        X[i] = load2(lx + i * LS, fx);
+        Y[i] = load2(lx + (NZ + i) * LS, fy);
+    }
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {  // i z
+        const V z = load2(lz + i * LS, 0u);
+        Z[i] = V{{-z.v[1], z.v[0], -z.v[3], z.v[2]}};
+    }
+    auto load = [&](int c, double (&t)[NZ]) {
+#pragma unroll
+        for (int q = 0; q < NZ; ++q) t[q] = d[(q * 6 + c) * DQ];
+    };
+    auto even = [&](const double (&t)[NZ], double s, int i, int j) {
+        return t[i > j ? i - j : j - i] + s * t[NZ - 1 - i - j];
+    };
+    auto odd = [&](const double (&t)[NZ], int i, int j) {
+        const int p = NZ - 1 - i - j;
+        const double hank = p > 0 ? t[p] : p < 0 ? -t[-p] : 0.0;
+        return i == j ? sg * hank : (i > j ? t[i - j] : -t[j - i]) + sg * hank;
+    };
+    auto axpy = [&](double c, const V& x) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) h.v[k] = fma(c, x.v[k], h.v[k]);
+    };
+    auto zero = [&] {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) h.v[k] = 0.0;
+    };
+    auto dot = [&](const V& x) {
+        qa = fma(x.v[0], h.v[0], fma(x.v[1], h.v[1], qa));
+        qb = fma(x.v[2], h.v[2], fma(x.v[3], h.v[3], qb));
+    };
+    // rows i of a diagonal block t (sign s), lower triangle with half its diagonal
+    auto block = [&](const double (&t)[NZ], double s, const auto& x, int i) {
+#pragma unroll
+        for (int j = 0; j <= i; ++j) axpy(j < i ? even(t, s, i, j) : 0.5 * even(t, s, i, j), x[j]);
+    };
+    double t[NZ], u[NZ];
+    if constexpr (NA > 0) {
+        load(0, t);  // xx
+#pragma unroll
+        for (int i = 0; i < NA; ++i) {
+            zero();
+            block(t, sg, X, i);
+            dot(X[i]);
+        }
+        load(1, t);  // yy, and xy with every x
+        load(3, u);
+#pragma unroll
+        for (int i = 0; i < NA; ++i) {
+            zero();
+            block(t, sg, Y, i);
+#pragma unroll
+            for (int j = 0; j < NA; ++j) axpy(even(u, sg, i, j), X[j]);
+            dot(Y[i]);
+        }
+    }
+    if constexpr (NB > 0) {
+        load(2, t);  // zz
+#pragma unroll
+        for (int i = 0; i < NB; ++i) {
+            zero();
+            block(t, -sg, Z, i);
+            dot(Z[i]);
+        }
+    }
+    if constexpr (NA > 0 && NB > 0) {
+        load(4, t);  // xz, yz
+        load(5, u);
+#pragma unroll
+        for (int j = 0; j < NB; ++j) {
+            zero();
+#pragma unroll
+            for (int i = 0; i < NA; ++i) {
+                axpy(odd(t, i, j), X[i]);
+                axpy(odd(u, i, j), Y[i]);
+            }
+            dot(Z[j]);
+        }
+    }
+}
+
+// grid (Px / 2 + 1, pairs): columns kx and Px - kx of a pair; -(1/2) sum conv.s over them, per image, replaces the
+// first spectrum element of column kx (its two parts), where the evaluation's reduction finds it.
+template <int P, int NZ>
+__global__ void __launch_bounds__(kYzqThreads, 2) yzq2p_kernel(GroupArgs<double> g) {
+    using C = double2;
+    constexpr int R2 = P / 16, LS = t2_line(P), L = 6 * NZ, RC = 16 * T2<P>::NP;
+    constexpr int ME = (NZ + 1) / 2, MO = NZ / 2, LP = 6 * ME, DQ = P / 2 + 1;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ double red[kYzqThreads / 32 * 2];
+    C* A = reinterpret_cast<C*>(smem_raw);  // line (b * 3 + c) * NZ + q of column b: e_q for q < ME, o_{q - ME} above
+    const int tid = threadIdx.x, nthr = kYzqThreads;
+    const int kx = blockIdx.x, p = blockIdx.y, kx1 = kx ? g.Px - kx : 0;
+    const int ny = g.ny;
+    if (g.pair_on && !g.pair_on[p]) return;  // uniform over the CTA
+    const size_t col = (size_t)3 * NZ * ny;
+    C* blk0 = g.spec + ((size_t)p * g.Px + kx) * col;
+    const C* blk1 = g.spec + ((size_t)p * g.Px + kx1) * col;
+    const C* __restrict__ tw = g.twy;
+    const C* __restrict__ t1 = g.t2y;
+    const C* __restrict__ ta = g.t2y + P;
+    griddep_wait();
+    griddep_launch_dependents();
+    // pass 1 and pass 2 as in yz2p_kernel
+    for (int r = tid; r < R2 * LP; r += nthr) {
+        const int n2 = r % R2, lp = r / R2, bc = lp / ME, i = lp % ME;
+        const C* src = (bc < 3 ? blk0 + bc * NZ * ny : blk1 + (bc - 3) * NZ * ny) + n2;
+        const bool two = MO == ME || i < MO;
+        const C* s0 = src + i * ny;
+        const C* s1 = src + (NZ - 1 - i) * ny;
+        C u[8], v[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const bool in = R2 * j + n2 < ny;
+            u[j] = in ? s0[R2 * j] : C{0.0, 0.0};
+            v[j] = in && two ? s1[R2 * j] : C{0.0, 0.0};
+        }
+        if (two) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const C a = u[j];
+                u[j] = cadd(a, v[j]);
+                v[j] = csub(a, v[j]);
+            }
+            t2_pass1<P>(v, n2, t1, A + (bc * NZ + ME + i) * LS);
+        }
+        t2_pass1<P>(u, n2, t1, A + (bc * NZ + i) * LS);
+    }
+    __syncthreads();
+    for (int r = tid; r < RC * L; r += nthr) t2_cols<P, false>(A + r / RC * LS, r & 15, r % RC / 16, tw, ta);
+    __syncthreads();
+    const double* dslab = g.dhat + (size_t)kx * DQ * NZ * 6;
+    double q[2] = {0.0, 0.0};
+    for (int it = tid; it < 2 * P; it += nthr) {
+        const int par = it >= P ? 1 : 0, ky = it - par * P;
+        const unsigned fy = ky > P / 2 ? 0x80000000u : 0u;  // (kx <= Px / 2: no sign of its own)
+        const double* d = dslab + min(ky, P - ky);
+        const C* a = A + t2_pos(ky);
+        const C* b = A + 3 * NZ * LS + t2_pos(ky ? P - ky : 0);
+        if constexpr (NZ % 2 == 0) {
+            zquad_sys<NZ, 0, LS, DQ>(a, b, d, par, 0u, fy, q[0], q[1]);
+        } else if (par == 0) {
+            zquad_sys<NZ, 0, LS, DQ>(a, b, d, 0, 0u, fy, q[0], q[1]);
+        } else {
+            zquad_sys<NZ, 1, LS, DQ>(a, b, d, 1, 0u, fy, q[0], q[1]);
+        }
+    }
+    block_reduce_d<2>(q, red);
+    // -(1/2) times 1/4 (A and B doubled) times 2 (half of the form), once more for the column Px - kx; one layer's
+    // tensor comes without the factor of mirrored layers (dhat_factor)
+    const double f = (kx1 == kx ? -0.25 : -0.5) * (NZ == 1 ? 0.5 : 1.0);
+    if (tid == 0) blk0[0] = C{f * q[0], f * q[1]};
+}
+
+// ------------------------------------------------------------------------------------------------
 // x kernels for a two-pass length Px = P (nx <= P/2): the x-transforms in two register passes
 // (ss_fft.cuh) on x2_rows rows of one layer of an image pair per CTA.  Every role order puts the rows
 // fastest across a warp: the spectrum's rows of one (kx, c) are contiguous in global memory, and with
@@ -395,6 +582,20 @@ template <typename T, int P> void t2_yz(const GroupArgs<T>& g, cudaStream_t st) 
 #undef SS_CASE
 }
 
+// (layer counts whose two columns fit: yzq2p_ok)
+template <typename T, int P> void t2_yzq(const GroupArgs<T>& g, cudaStream_t st) {
+    if constexpr (sizeof(T) == 8) {
+        const dim3 grid(g.Px / 2 + 1, g.n_pairs);
+        const size_t sm = yz2p_smem(8, P, g.nz, 2);
+#define SS_CASE(Z)                    \
+    if constexpr (yzq2p_fits(P, Z)) { \
+        if (g.nz == Z) launch_ex(yzq2p_kernel<P, Z>, grid, dim3(kYzqThreads), sm, st, false, g); \
+    }
+        SS_CASE(1) SS_CASE(2) SS_CASE(3) SS_CASE(4) SS_CASE(5) SS_CASE(6) SS_CASE(7) SS_CASE(8)
+#undef SS_CASE
+    }
+}
+
 template <typename T, int P> void t2_smem_limits(int bytes) {
     constexpr int carve = sizeof(T) == 8 || P <= 384 ? carve_kb<T>() : P <= 448 ? 196 : 228;  // two FP32 y/z CTAs
     set_dyn_smem(xfwd2p_kernel<T, P>, bytes, carve);
@@ -404,12 +605,19 @@ template <typename T, int P> void t2_smem_limits(int bytes) {
 #define SS_CASE(Z, B) set_dyn_smem(yz2p_kernel<T, P, Z, B>, bytes, carve);
     SS_T2_YZ(SS_CASE)
 #undef SS_CASE
+    if constexpr (sizeof(T) == 8) {
+#define SS_CASE(Z) \
+    if constexpr (yzq2p_fits(P, Z)) set_dyn_smem(yzq2p_kernel<P, Z>, bytes, carve);
+        SS_CASE(1) SS_CASE(2) SS_CASE(3) SS_CASE(4) SS_CASE(5) SS_CASE(6) SS_CASE(7) SS_CASE(8)
+#undef SS_CASE
+    }
 }
 
 #define SS_T2_INSTANTIATE(T, P)                                                                  \
     template void t2_xfwd<T, P>(const GroupArgs<T>&, cudaStream_t);                               \
     template void t2_xinv<T, P>(const GroupArgs<T>&, int, T, T*, bool, cudaStream_t);             \
     template void t2_yz<T, P>(const GroupArgs<T>&, cudaStream_t);                                 \
+    template void t2_yzq<T, P>(const GroupArgs<T>&, cudaStream_t);                                \
     template void t2_smem_limits<T, P>(int);
 
 }  // namespace ss

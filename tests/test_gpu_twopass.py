@@ -74,6 +74,29 @@ def test_fp64_kernels(case):
         assert np.abs(got[k] - ref).max() <= 1e-12 * np.abs(ref).max(), k
 
 
+# Energies alone stop at the spectrum (two columns of it in shared memory): every layer count, even and odd image
+# counts, x lengths with and without a middle column, the largest y length that fits and the first that does not
+@pytest.mark.parametrize("case", [(20, 33, 1, 3), (40, 30, 2, 2), (17, 24, 3, 4), (30, 64, 4, 5), (5, 30, 5, 2),
+                                  (21, 50, 6, 3), (7, 16, 7, 2), (33, 20, 8, 3), (5, 128, 8, 3), (4, 129, 8, 2),
+                                  (6, 256, 1, 3), (3, 14, 2, 2), (150, 9, 5, 3), (4, 222, 4, 2), (2, 130, 5, 2)])
+def test_energies_without_the_field(case):
+    # bounds of the other energy tests: FP64 context 1e-11 of the largest energy's terms, an FP32 context's FP64
+    # energies the same against the oracle at its own stored (FP32) spins
+    nx, ny, nz, n = case
+    desc = (nx, ny, nz, 1.0, 0.3, 0.1, 0.4, n)
+    m = oracle.model(*desc[:7])
+    path = W.random_spins((n, nx * ny * nz, 3), seed=nx)
+    for prec in (binding.SS_PREC_FP64, binding.SS_PREC_FP32):
+        with binding.StringMethod([desc], precision=prec) as sm:
+            sm.set_path(0, path)
+            s = sm.get_path(0)
+            s = s / np.linalg.norm(s, axis=-1, keepdims=True)
+            want = oracle.energies(m, s)
+            e = sm.energies(0)
+        scale = np.abs(want).max() + nx * ny * nz
+        assert np.abs(e - want).max() <= 1e-11 * scale
+
+
 def test_fp32_input_spins_normalised_to_the_last_bit():
     # FP32 spins of any norm, in and beyond the range the FP32-pair arithmetic takes (squared norms 1e-6 to 1e6),
     # with components that vanish or underflow.  Tolerance: one rounding to FP32 (0.5 units in the last place), and
