@@ -31,12 +31,12 @@ template <int NZ, int PAR> struct ZSys {  // PAR 0: (x, y in e; z in o), 1: (x, 
     static constexpr int NXY = PAR == 0 ? ME : MO, NZC = PAR == 0 ? MO : ME;  // elements of x (and y), and of z
 };
 
-// One system at one frequency: A points at the frequency's element of line 0 (line stride LS), d at its
-// coefficients (component c, |dz| at d[(|dz| * 6 + c) * DQ]); par the system; fx, fy the parity signs of kx, ky
+// One system at one frequency: A points at the frequency's element of line 0 (line stride LS), load(c, t) gets
+// its coefficients of component c, |dz| = 0 .. NZ - 1; par the system; fx, fy the parity signs of kx, ky
 // as sign bits (the tensor's xy, xz, yz are odd in them: flip x and y going in and coming out).  The result
 // replaces the inputs, conjugated (the inverse transform is the conjugate of the forward transform of the conjugate).
-template <int NZ, int PAR, int LS, int DQ, typename T, typename C>
-__device__ __forceinline__ void zconv_sys(C* A, const T* __restrict__ d, int par, unsigned fx, unsigned fy) {
+template <int NZ, int PAR, int LS, typename T, typename C, typename LOAD>
+__device__ __forceinline__ void zconv_sys(C* A, const LOAD& load, int par, unsigned fx, unsigned fy) {
     using S = ZSys<NZ, PAR>;  // the shape; for even NZ both systems share it and par picks one at run time
     constexpr int NA = S::NXY, NB = S::NZC;
     constexpr int NA1 = NA > 0 ? NA : 1, NB1 = NB > 0 ? NB : 1;
@@ -58,10 +58,6 @@ __device__ __forceinline__ void zconv_sys(C* A, const T* __restrict__ d, int par
         Z[i] = C{-z.y, z.x};  // i z
         W[i] = zero;
     }
-    auto load = [&](int c, T (&t)[NZ]) {
-#pragma unroll
-        for (int q = 0; q < NZ; ++q) t[q] = d[(q * 6 + c) * DQ];
-    };
     // t(|i-j|) + s t(n-1-i-j) for an even component
     auto even = [&](const T (&t)[NZ], T s, int i, int j) {
         return t[i > j ? i - j : j - i] + s * t[NZ - 1 - i - j];
@@ -146,28 +142,69 @@ __device__ __forceinline__ void zconv_sys(C* A, const T* __restrict__ d, int par
     }
 }
 
-// The z-convolution of one column: one item per (frequency, system), reading and writing its own elements.
+// The z-convolution at one frequency of one column, in place.  par: the system, for the layer counts that take
+// one item each (kZBoth: one item for both).
+template <int NZ, typename T> constexpr bool kZBoth = sizeof(T) == 4 && NZ >= 2 && NZ <= 4;
 template <int NZ, int P, typename T, typename C>
-__device__ __forceinline__ void zconv_t2(C* A, int kx, int Px, const T* dslab, int tid, int nthr) {
+__device__ __forceinline__ void zconv_item(C* A, int kx, int ky, int par, int Px, const T* dslab) {
     constexpr int LS = t2_line(P), DQ = P / 2 + 1;
     const unsigned fx = kx > Px / 2 ? 0x80000000u : 0u;  // the parity signs of kx, ky, as sign bits
-    for (int it = tid; it < (NZ == 1 ? P : 2 * P); it += nthr) {
-        const int par = it >= P ? 1 : 0, ky = it - par * P;
-        const unsigned fy = ky > P / 2 ? 0x80000000u : 0u;
-        const T* d = dslab + min(ky, P - ky);
-        C* a = A + t2_pos(ky);
-        if constexpr (NZ == 1) {  // xz and yz vanish
-            const C X = a[0], Y = a[LS], Z = a[2 * LS];
-            const T xx = d[0], yy = d[DQ], zz = d[2 * DQ], xy = flip_sign(d[3 * DQ], fx ^ fy);
-            a[0] = C{xx * X.x + xy * Y.x, -(xx * X.y + xy * Y.y)};
-            a[LS] = C{xy * X.x + yy * Y.x, -(xy * X.y + yy * Y.y)};
-            a[2 * LS] = C{zz * Z.x, -zz * Z.y};
+    const unsigned fy = ky > P / 2 ? 0x80000000u : 0u;
+    const T* d = dslab + min(ky, P - ky);
+    C* a = A + t2_pos(ky);
+    if constexpr (NZ == 1) {  // xz and yz vanish
+        const C X = a[0], Y = a[LS], Z = a[2 * LS];
+        const T xx = d[0], yy = d[DQ], zz = d[2 * DQ], xy = flip_sign(d[3 * DQ], fx ^ fy);
+        a[0] = C{xx * X.x + xy * Y.x, -(xx * X.y + xy * Y.y)};
+        a[LS] = C{xy * X.x + yy * Y.x, -(xy * X.y + yy * Y.y)};
+        a[2 * LS] = C{zz * Z.x, -zz * Z.y};
+    } else {
+        auto load = [&](int c, T (&t)[NZ]) {
+#pragma unroll
+            for (int q = 0; q < NZ; ++q) t[q] = d[(q * 6 + c) * DQ];
+        };
+        if constexpr (kZBoth<NZ, T>) {
+            T all[6][NZ];
+#pragma unroll
+            for (int c = 0; c < 6; ++c) load(c, all[c]);
+            auto kept = [&](int c, T (&t)[NZ]) {
+#pragma unroll
+                for (int q = 0; q < NZ; ++q) t[q] = all[c][q];
+            };
+            zconv_sys<NZ, 0, LS, T>(a, kept, 0, fx, fy);
+            zconv_sys<NZ, 1, LS, T>(a, kept, 1, fx, fy);
         } else if constexpr (NZ % 2 == 0) {  // the two systems have the same shape
-            zconv_sys<NZ, 0, LS, DQ>(a, d, par, fx, fy);
+            zconv_sys<NZ, 0, LS, T>(a, load, par, fx, fy);
         } else if (par == 0) {
-            zconv_sys<NZ, 0, LS, DQ>(a, d, 0, fx, fy);
+            zconv_sys<NZ, 0, LS, T>(a, load, 0, fx, fy);
         } else {
-            zconv_sys<NZ, 1, LS, DQ>(a, d, 1, fx, fy);
+            zconv_sys<NZ, 1, LS, T>(a, load, 1, fx, fy);
+        }
+    }
+}
+// The z-convolution of the columns kx0 .. kx0 + KXB - 1.  FP32, two to four layers: an item takes both systems, so
+// that the tensor's coefficients, as many bytes as the spectrum elements, are read once, and the columns' items
+// run on in one loop.  Before and after on one GB300: 128x128x4 x 384 images 482 -> 462 us, 96x96x4 x 192 148 ->
+// 141.  With more layers the coefficients do not fit in the registers, and one loop over the columns changed nothing
+// at one layer and cost 9% at eight (28.2 -> 30.9 us, 64x64x8 x 32).
+template <int NZ, int KXB, int P, typename T, typename C>
+__device__ __forceinline__ void zconv_t2(C* A, int kx0, int Px, const T* dhat, int tid, int nthr) {
+    constexpr int LS = t2_line(P), SLAB = (P / 2 + 1) * NZ * 6;
+    if constexpr (kZBoth<NZ, T>) {
+#pragma unroll 1
+        for (int it = tid; it < KXB * P; it += nthr) {
+            const int b = it / P, kx = kx0 + b;
+            zconv_item<NZ, P>(A + b * 3 * NZ * LS, kx, it % P, 0, Px, dhat + (size_t)min(kx, Px - kx) * SLAB);
+        }
+    } else {
+#pragma unroll 1
+        for (int b = 0; b < KXB; ++b) {
+            const int kx = kx0 + b;
+            const T* dslab = dhat + (size_t)min(kx, Px - kx) * SLAB;
+            for (int it = tid; it < (NZ == 1 ? P : 2 * P); it += nthr) {
+                const int par = it >= P ? 1 : 0;
+                zconv_item<NZ, P>(A + b * 3 * NZ * LS, kx, it - par * P, par, Px, dslab);
+            }
         }
     }
 }
@@ -221,11 +258,7 @@ __global__ void __launch_bounds__(yz2p_threads(sizeof(T), P), yz2p_blocks(sizeof
     // pass 2: half a warp per line (lanes = 16 columns; a warp where a column takes two roles)
     for (int r = tid; r < RC * L; r += nthr) t2_cols<P, false>(A + r / RC * LS, r & 15, r % RC / 16, tw, ta);
     __syncthreads();
-#pragma unroll 1
-    for (int b = 0; b < KXB; ++b) {
-        const int kxb = kx + b, kxo = min(kxb, g.Px - kxb);
-        zconv_t2<NZ, P>(A + b * 3 * NZ * LS, kxb, g.Px, g.dhat + (size_t)kxo * (P / 2 + 1) * NZ * 6, tid, nthr);
-    }
+    zconv_t2<NZ, KXB, P>(A, kx, g.Px, g.dhat, tid, nthr);
     __syncthreads();
     // pass A (the inverse transform of the conjugated field spectra, in place by columns)
     for (int r = tid; r < RC * L; r += nthr) t2_cols<P, true>(A + r / RC * LS, r & 15, r % RC / 16, tw, ta);
