@@ -249,11 +249,11 @@ inline bool yz2p_ok(int Py, int nz, int Px) {
 // shared memory (24 lines: 26 KB at 128, 78 KB at 384) allow
 // (FP64: the pipe issues two lane-operations per clock and SM, so a few warps with all the registers they want)
 __host__ __device__ constexpr int yz2p_threads(int real_bytes, int P) {
-    if (real_bytes == 8) return P <= 256 ? 128 : 256;
+    if (real_bytes == 8) return P <= 32 ? 64 : P <= 256 ? 128 : 256;
     return P <= 128 ? 128 : P <= 256 ? 192 : P <= 320 ? 256 : 384;
 }
 __host__ __device__ constexpr int yz2p_blocks(int real_bytes, int P) {
-    if (real_bytes == 8) return P <= 192 ? 3 : P <= 256 ? 2 : 1;
+    if (real_bytes == 8) return P <= 32 ? 6 : P <= 192 ? 3 : P <= 256 ? 2 : 1;
     return P <= 128 ? 6 : P <= 256 ? 4 : P <= 320 ? 3 : 2;
 }
 // The FP64 energy kernel keeps two columns in shared memory (227 KB, less its reduction's): 8 layers up to 256 points

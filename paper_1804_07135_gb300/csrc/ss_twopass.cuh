@@ -579,14 +579,12 @@ __global__ void __launch_bounds__(x2_threads(sizeof(T), P), x2_blocks(sizeof(T),
 }
 
 // ---- launchers of one length --------------------------------------------------------------------------
-// FP64 launches do without programmatic dependent launch: they are bound by each SM's FP64 pipe, and CTAs placed
-// while the previous kernel drains land unevenly (40x50x3 x 16 images, FP64: 223 us per iteration with it, 210
-// without).  FP64 per iteration on one GB300, runtime Stockham plans before and these kernels: 64x64x4 x 16
+// FP64 per iteration on one GB300, runtime Stockham plans before and these kernels: 64x64x4 x 16
 // 432 -> 353 us, 72x60x8 x 8 625 -> 415, 70x70x1 x 32 356 -> 223, 128x128x8 x 4 1226 -> 815, 20x20x2 x 16 77 -> 75.
 template <typename T, int P> void t2_xfwd(const GroupArgs<T>& g, cudaStream_t st) {
     const dim3 grid((g.ny + g.ty_a - 1) / g.ty_a, g.nz, g.n_pairs);  // ty_a = x2_rows (set by the host)
     const int thr = x2_launch_threads(sizeof(T), P, g.nx, (long)grid.x * grid.y * grid.z);
-    launch_ex(xfwd2p_kernel<T, P>, grid, dim3(thr), x2_smem(sizeof(T), P, false), st, sizeof(T) == 4, g);
+    launch_ex(xfwd2p_kernel<T, P>, grid, dim3(thr), x2_smem(sizeof(T), P, false), st, pdl_fft(g), g);
 }
 
 template <typename T, int P>
@@ -596,7 +594,7 @@ void t2_xinv(const GroupArgs<T>& g, int mode, T dt, T* hout, bool pdl, cudaStrea
     const size_t sm = x2_smem(sizeof(T), P, true);
     switch (mode) {
 #define SS_CASE(M) \
-    case M: launch_ex(xinv2p_kernel<T, P, M>, grid, blk, sm, st, pdl && sizeof(T) == 4, g, dt, hout); break;
+    case M: launch_ex(xinv2p_kernel<T, P, M>, grid, blk, sm, st, pdl && pdl_fft(g), g, dt, hout); break;
         SS_CASE(0) SS_CASE(1) SS_CASE(2) SS_CASE(3) SS_CASE(4) SS_CASE(5)
 #undef SS_CASE
     }
@@ -610,7 +608,7 @@ template <typename T, int P> void t2_yz(const GroupArgs<T>& g, cudaStream_t st) 
     const size_t sm = yz2p_smem(sizeof(T), P, g.nz, kxb);
     const dim3 grid(g.Px / kxb, g.n_pairs);
 #define SS_CASE(Z, B) \
-    if (g.nz == Z && kxb == B) launch_ex(yz2p_kernel<T, P, Z, B>, grid, dim3(yz2p_threads(sizeof(T), P)), sm, st, sizeof(T) == 4, g);
+    if (g.nz == Z && kxb == B) launch_ex(yz2p_kernel<T, P, Z, B>, grid, dim3(yz2p_threads(sizeof(T), P)), sm, st, pdl_fft(g), g);
     SS_T2_YZ(SS_CASE)
 #undef SS_CASE
 }

@@ -124,3 +124,22 @@ def test_fp32_input_spins_normalised_to_the_last_bit():
                 sm.set_path(0, w)
                 sm.get_path(0)
             sm.set_path(0, v)
+
+
+# FP64 lengths at the lines of their rule: few y/z CTAs (short lengths), a two-pass x length too much longer (short x
+# beside a two-pass y), about as long, and one whose short x the y/z kernel does not take
+@pytest.mark.parametrize("case,Px,Py", [((13, 17, 2, 11), 27, 36), ((13, 17, 2, 13), 32, 48), ((25, 32, 8, 8), 54, 64),
+                                        ((19, 14, 5, 10), 48, 32), ((14, 20, 4, 14), 32, 48), ((5, 14, 3, 6), 9, 27)])
+def test_fp64_padded_lengths(case, Px, Py):
+    nx, ny, nz, n = case
+    desc = (nx, ny, nz, 1.0, 0.3, 0.1, 0.03, n)
+    path = W.random_spins((n, nx * ny * nz, 3), seed=ny)
+    with binding.StringMethod([desc], precision=binding.SS_PREC_FP64) as sm:
+        cfg = sm.launch_config(0)
+        sm.set_path(0, path)
+        got = sm.field(0)
+    assert (cfg["Px"], cfg["Py"]) == (Px, Py)
+    m = oracle.model(*desc[:7])
+    for k in (0, n - 1):  # the FP64 field bound
+        ref = oracle.field(m, path[k])
+        assert np.abs(got[k] - ref).max() <= 1e-12 * np.abs(ref).max(), k
