@@ -25,38 +25,6 @@ namespace {
 thread_local std::string g_create_error;
 
 // ---- small helpers --------------------------------------------------------------------------------
-// Padded transform length for n sites, enough for the linear (non-circular) convolution with offsets
-// -(n-1)..(n-1) (Sec. II-A, the zero-padded kernel): padded_smooth(n), except that a length without two-pass
-// kernels is exchanged for the next one that has them (two_pass: the kernels along this axis have a two-pass
-// form at all).  Lattices of up to 12 sites a side keep the short length: one CTA transforms all of
-// their lines at once either way.
-int padded_len(int n, bool two_pass) {
-    const int m = padded_smooth(n);
-    if (!two_pass || n <= 12 || t2_length(m)) return m;
-    const int t = t2_length_from(2 * n - 1);
-    return t ? t : m;
-}
-
-// The padded lengths of an FP64 group, whose kernels' time goes with the work they issue to the FP64 pipe.  The
-// two-pass y/z kernel leaves lanes idle at short lengths, which a grid of one or two CTAs per SM does not hide: up to
-// kYz64Few of them the short lengths.  And its time goes with Px: a two-pass Px more than a tenth above the short one
-// does not pay where the y/z kernel is the same with either.  Per iteration on one GB300, two-pass and short
-// lengths: 13x17x2 x 11 images (192 CTAs) 68 and 54 us, 14x22x3 x 10 (160) 74 and 60, 17x17x1 x 11 (144) 56 and 52,
-// 50x26x1 x 8 (224) 64 and 77, 13x17x1 x 30 (240) 56 and 64; short Px alone: 25x32x8 x 44 (64 or 54) 510 and 446,
-// 25x25x8 x 40 430 and 399.
-constexpr long kYz64Few = 200;
-void padded_lens_f64(int nx, int ny, int nz, int n_pairs, int* Px, int* Py) {
-    const int sx = padded_smooth(nx), tx = padded_len(nx, true);
-    *Py = padded_len(ny, nz <= kT2MaxNz);
-    const int kxb = yz2p_kxb_use(8, nz, 0);
-    if (kxb > 0 && (long)(tx / kxb) * n_pairs <= kYz64Few) {
-        *Px = sx;
-        *Py = padded_smooth(ny);
-    } else {
-        *Px = 10 * tx > 11 * sx && yz2p_ok(*Py, nz, sx) == yz2p_ok(*Py, nz, tx) ? sx : tx;
-    }
-}
-
 FftPlan make_plan(int P) { return fft_make_plan(P); }
 
 // Eq. 7 at an integer lattice offset (entries xx, yy, zz, xy, xz, yz), with its 1/(4 pi).
@@ -1352,14 +1320,13 @@ ss_status ss_create_batch(int n_strings, const ss_string_desc* descs, const ss_o
         g.n_pairs = (g.n_img + 1) / 2;
         g.rbytes = (int)real_size(c);
         g.Px = g.Py = 1;
-        if (g.dipole && g.rbytes == 8) {
-            padded_lens_f64(g.nx, g.ny, g.nz, g.n_pairs, &g.Px, &g.Py);
-        } else if (g.dipole) {
-            g.Px = padded_len(g.nx, true);
-            g.Py = padded_len(g.ny, g.nz <= kT2MaxNz);
-        }
+        if (g.dipole) padded_lengths(g.rbytes, g.nx, g.ny, g.nz, g.n_pairs, &g.Px, &g.Py);
         g.planx = make_plan(g.Px);
         g.plany = make_plan(g.Py);
+        if (g.dipole && ((!t2_length(g.Px) && !fft_plan_2348(g.planx)) ||
+                         (!yz2p_ok(g.Py, g.nz, g.Px) && !fft_plan_2348(g.plany))))  // padded_lengths never asks for it
+            return bail(fail(c, SS_ERR_INVALID_ARG, "lattice %d x %d x %d: no kernel for the padded lengths %d x %d", g.nx,
+                             g.ny, g.nz, g.Px, g.Py));
         configure_group(g);
         const size_t smem_max = 227 * 1024;
         if (g.smem_a > smem_max || g.smem_b > smem_max || g.smem_c > smem_max)

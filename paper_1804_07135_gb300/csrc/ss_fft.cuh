@@ -281,7 +281,7 @@ template <typename C> struct Dft<20, C> : DftCt<5, 4, C> {};
 template <typename C> struct Dft<24, C> : DftCt<3, 8, C> {};
 
 // Host-side plan: radices 8, 4, 2 first (largest first), then 3s, 5s and 7s (the last two only in the setup
-// transforms of the tensor spectrum: a length with those factors has two-pass kernels).
+// transforms of the tensor spectrum: padded_lengths gives a length with those factors to two-pass kernels alone).
 inline FftPlan fft_make_plan(int P) {
     FftPlan p{};
     p.P = P;
@@ -317,6 +317,13 @@ inline FftPlan fft_make_plan(int P) {
         ns *= R;
     }
     return p;
+}
+
+// The kernels of the runtime plans have stages for the plan's radices: fft_lines without R57.
+inline bool fft_plan_2348(const FftPlan& p) {
+    for (int s = 0; s < p.nstages; ++s)
+        if (p.radix[s] == 5 || p.radix[s] == 7) return false;
+    return true;
 }
 
 // Elements each thread holds in registers per stage: 8 (9 for radix 3).  Lines are transformed in

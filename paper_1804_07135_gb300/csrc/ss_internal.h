@@ -27,8 +27,8 @@ constexpr int kMinBlocksYz = 2;
 constexpr int kArcMaxChunk = 8;     // image differences one arc CTA accumulates
 constexpr int kArcMaxK = 1024;      // images per string
 
-// Mixed-radix (2, 3, 4, 8) plan of a length-P complex FFT, stages in Stockham order (powers of two
-// first, so the stride Ns of every power-of-two stage and of the first radix-3 stage is a power of two).
+// Mixed-radix (2, 3, 4, 8; 5 and 7 in the setup transforms) plan of a length-P complex FFT, stages in Stockham order
+// (powers of two first, so the stride Ns of every power-of-two stage and of the first radix-3 stage is a power of two).
 // Per stage: q = P/R butterflies per line, ns = product of the earlier radices, tw = P/(ns*R) (twiddle
 // index step); ns_mask = ns - 1 when ns is a power of two, else -1.
 struct FftPlan {
@@ -315,6 +315,45 @@ inline int padded_smooth(int n) {
     int p2 = 1;
     while (p2 < 2 * n - 1) p2 <<= 1;
     return 8 * p2 <= 9 * m ? p2 : m;
+}
+// Padded transform length for n sites, enough for the linear (non-circular) convolution with offsets
+// -(n-1)..(n-1) (Sec. II-A, the zero-padded kernel), where the kernels along the axis have a two-pass form:
+// padded_smooth(n), except that a length without two-pass kernels is exchanged for the next one that has them.
+// Lattices of up to 12 sites a side keep the short length: one CTA transforms all of their lines at once either way.
+inline int padded_len(int n) {
+    const int m = padded_smooth(n);
+    if (n <= 12 || t2_length(m)) return m;
+    const int t = t2_length_from(2 * n - 1);
+    return t ? t : m;
+}
+
+// The padded lengths of a lattice, Px first: the two-pass x kernels take every t2_length, but the two-pass y/z kernel
+// takes Py only together with a Px that its columns per CTA divide (yz2p_ok).  Where it does not (Px = 18 at one
+// layer, say), the runtime-plan kernel transforms y, and that one has stages of radix 2, 3, 4 and 8 alone: Py is then
+// padded_smooth(ny), never a two-pass length with a factor 5 or 7.
+//
+// FP64 kernels' time goes with the work they issue to the FP64 pipe.  The two-pass y/z kernel leaves lanes idle at
+// short lengths, which a grid of one or two CTAs per SM does not hide: up to kYz64Few of them the short lengths.  And
+// its time goes with Px: a two-pass Px more than a tenth above the short one does not pay where the y/z kernel is the
+// same with either.  Per iteration on one GB300, two-pass and short lengths: 13x17x2 x 11 images (192 CTAs) 68 and
+// 54 us, 14x22x3 x 10 (160) 74 and 60, 17x17x1 x 11 (144) 56 and 52, 50x26x1 x 8 (224) 64 and 77, 13x17x1 x 30 (240)
+// 56 and 64; short Px alone: 25x32x8 x 44 (64 or 54) 510 and 446, 25x25x8 x 40 430 and 399.
+constexpr long kYz64Few = 200;
+inline void padded_lengths(int real_bytes, int nx, int ny, int nz, int n_pairs, int* Px, int* Py) {
+    const int sx = padded_smooth(nx), sy = padded_smooth(ny);
+    const int tx = padded_len(nx), ty = nz <= kT2MaxNz ? padded_len(ny) : sy;
+    *Px = tx;
+    *Py = ty;
+    if (real_bytes == 8) {
+        const int kxb = yz2p_kxb_use(8, nz, 0);
+        if (kxb > 0 && (long)(tx / kxb) * n_pairs <= kYz64Few) {
+            *Px = sx;
+            *Py = sy;
+        } else if (10 * tx > 11 * sx && yz2p_ok(ty, nz, sx) == yz2p_ok(ty, nz, tx)) {
+            *Px = sx;
+        }
+    }
+    if (!yz2p_ok(*Py, nz, *Px)) *Py = sy;
 }
 
 

@@ -1,0 +1,38 @@
+"""Fields and energies where the x length keeps the two-pass y/z kernel away: narrow strips and wide films whose Px its
+columns per CTA do not divide, with a ny whose two-pass length has a factor 5 or 7, in both precisions, against the
+FP64 oracle.  Bounds of the other parity tests: FP32 field 1e-5 of max |h|, FP64 field 1e-12, energies 1e-11 of the
+largest energy's terms.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1804_07135_gb300 import binding
+from paper_1804_07135_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+# (nx, ny, nz, images); the last three have the image pairs that take FP64 past its rule for small grids
+CASES = [(9, 35, 1, 2), (9, 100, 1, 3), (6, 50, 1, 2), (5, 76, 3, 3), (2, 100, 4, 2), (3, 150, 2, 2), (350, 35, 1, 2),
+         (326, 33, 2, 2), (9, 33, 1, 240), (2, 40, 4, 140), (9, 50, 1, 240)]
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("case", CASES)
+def test_field_and_energies(case, precision):
+    nx, ny, nz, n = case
+    desc = (nx, ny, nz, 1.0, 0.3, 0.1, 0.4, n)
+    path = W.random_spins((n, nx * ny * nz, 3), seed=nx + ny)
+    prec = binding.SS_PREC_FP64 if precision == "fp64" else binding.SS_PREC_FP32
+    with binding.StringMethod([desc], precision=prec) as sm:
+        sm.set_path(0, path)
+        s = sm.get_path(0)
+        field, energies = sm.field(0), sm.energies(0)
+    s = s / np.linalg.norm(s, axis=-1, keepdims=True)
+    m = oracle.model(*desc[:7])
+    some = sorted({0, 1, n - 1})
+    want = oracle.energies(m, s[some])
+    assert np.abs(energies[some] - want).max() <= 1e-11 * (np.abs(want).max() + nx * ny * nz)
+    for k in some:
+        ref = oracle.field(m, s[k])
+        assert np.abs(field[k] - ref).max() <= (1e-12 if precision == "fp64" else 1e-5) * np.abs(ref).max(), k
