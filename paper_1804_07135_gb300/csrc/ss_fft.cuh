@@ -383,7 +383,9 @@ __device__ __forceinline__ void fft_stage(C* buf, const C* tw, int LS, int L, in
 
 // Forward FFT of L lines (stride LS, elements at fft_pad positions) in shared memory.  Must be called
 // by every thread of the block, with blockDim.x >= fft_min_threads(P).  Ends synchronised.  R57: the plan
-// may hold radices 5 and 7.
+// may hold radices 5 and 7 (setup).  Kernels without them are compiled without their cases: empty ones in the switch cost
+// the runtime-plan y/z kernel 2 to 3% (481x450x1 x 9 images, 1024 points: 306.4 us with, 301.0 without on one GB300;
+// 168x9x4 x 40: 187.9 and 181.5).
 template <bool R57 = false, typename C>
 __device__ __forceinline__ void fft_lines(C* buf, const C* tw, const FftPlan& plan, int LS, int L, int tid, int nthr) {
     const int lpp = max(1, fft_lines_per_pass(nthr, plan.P));  // the host guarantees >= 1; never loop forever
@@ -392,16 +394,20 @@ __device__ __forceinline__ void fft_lines(C* buf, const C* tw, const FftPlan& pl
         C* b = buf + l0 * LS;
         for (int st = 0; st < plan.nstages; ++st) {
             const int Q = plan.q[st], Ns = plan.ns[st], tws = plan.tw[st], msk = plan.ns_mask[st];
+            if constexpr (R57) {
+                if (plan.radix[st] == 5) {
+                    fft_stage<5>(b, tw, LS, nl, Q, Ns, tws, msk, tid, nthr);
+                    continue;
+                }
+                if (plan.radix[st] == 7) {
+                    fft_stage<7>(b, tw, LS, nl, Q, Ns, tws, msk, tid, nthr);
+                    continue;
+                }
+            }
             switch (plan.radix[st]) {
                 case 8: fft_stage<8>(b, tw, LS, nl, Q, Ns, tws, msk, tid, nthr); break;
                 case 4: fft_stage<4>(b, tw, LS, nl, Q, Ns, tws, msk, tid, nthr); break;
                 case 3: fft_stage<3>(b, tw, LS, nl, Q, Ns, tws, msk, tid, nthr); break;
-                case 5:
-                    if constexpr (R57) fft_stage<5>(b, tw, LS, nl, Q, Ns, tws, msk, tid, nthr);
-                    break;
-                case 7:
-                    if constexpr (R57) fft_stage<7>(b, tw, LS, nl, Q, Ns, tws, msk, tid, nthr);
-                    break;
                 default: fft_stage<2>(b, tw, LS, nl, Q, Ns, tws, msk, tid, nthr); break;
             }
         }
