@@ -151,7 +151,7 @@ struct ArcArgs {
 
 constexpr int kClimbTile = 256;   // sites per CTA of the climbing-image kernels (one per thread)
 constexpr int kSplineMaxK = 256;  // longest string the spline variant accepts
-constexpr int kSplineRows = 8;    // rows of W a thread of the apply kernel takes at once
+constexpr int kSplineRows = 8;    // rows of W a thread of the FP32 apply kernel takes at once
 inline int spline_w_stride(int maxK) { return (maxK + kSplineRows - 1) / kSplineRows * kSplineRows + 4; }
 // columns of the spline operator P the arc kernel keeps on chip (66 KB of FP32 or 33 KB of FP64)
 inline int spline_p_dim(int real_bytes, int maxK) { const int cap = real_bytes == 4 ? 128 : 64; return maxK + 1 < cap ? maxK + 1 : cap; }

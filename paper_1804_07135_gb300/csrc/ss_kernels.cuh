@@ -1915,12 +1915,16 @@ __global__ void __launch_bounds__(256) climb_apply_kernel(GroupArgs<T> g, ArcArg
 }
 
 // ---- natural cubic spline: phi_k = normalise(sum_q W_kq phi*_q) in place on sp -----------------------
-// grid (ceil(N / 32), n_str), 256 threads: 32 sites x 8 groups of output rows, eight consecutive rows per thread
+// grid (ceil(N / 32), n_str), 256 threads: 32 sites x 8 groups of output rows.  FP32: eight consecutive rows per thread
 // and pass (a group's first rows 8 grp, 8 grp + 64, ...), so a spin loaded from shared memory serves eight rows
-// and their weights come as vectors: 24 multiply-adds for 3 + 2 loads instead of 3 for 4.  Dynamic shared
+// and their weights come as vectors: 24 multiply-adds for 3 + 2 loads instead of 3 for 4; bound by
+// FP32 issue (2 K^2 N x 3 multiply-adds); 112x112x1 x 60 images: 32.7 -> 18.3 us on one GB300.  FP64 is bound by its
+// pipe, which issues a multiply-add for a row that is not needed as slowly as for one that is: one row per thread and
+// pass, and only the rows that move (by eights and by ones: 14x22x3 x 130 images 530 and 424 us, 23x10x2 x 200 1113 and
+// 990, 22x9x3 x 5 12.2 and 8.1).  Dynamic shared
 // memory: the string's K images at the CTA's 32 sites, [K][3][32], then W, [q][row] at row stride a.w_stride (whole
-// vectors, off a multiple of 32 words), when w_on_chip (else W is read through L1).  The tile is loaded whole before any row is written back.  Bound by
-// FP32 issue (2 K^2 N x 3 multiply-adds); 112x112x1 x 60 images: 32.7 -> 18.3 us on one GB300.
+// vectors, off a multiple of 32 words), when w_on_chip (else W is read through L1).  The tile is loaded whole before any
+// row is written back.
 template <typename T>
 __global__ void __launch_bounds__(256) spline_apply_kernel(GroupArgs<T> g, ArcArgs a, int w_on_chip) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1952,30 +1956,35 @@ __global__ void __launch_bounds__(256) spline_apply_kernel(GroupArgs<T> g, ArcAr
     __syncthreads();
     if (i >= N) return;
     const T* Wr = w_on_chip ? Ws : Wg;
-    for (int k0 = kSplineRows * grp; k0 < K - 1; k0 += 8 * kSplineRows) {
-        T u[kSplineRows][3];
+    constexpr int R = sizeof(T) == 4 ? kSplineRows : 1, UNROLL = R == 1 ? 16 : 2;  // (loads in flight ahead of the chains)
+    for (int k0 = R * grp; k0 < K - 1; k0 += 8 * R) {
+        if (R == 1 && (k0 < 1 || wc[k0])) continue;  // kept in place
+        T u[R][3];
 #pragma unroll
-        for (int r = 0; r < kSplineRows; ++r) u[r][0] = u[r][1] = u[r][2] = T(0);
-#pragma unroll 2
+        for (int r = 0; r < R; ++r) u[r][0] = u[r][1] = u[r][2] = T(0);
+#pragma unroll UNROLL
         for (int q = 0; q < K; ++q) {
             const T y0 = y[q * 96 + lane], y1 = y[q * 96 + 32 + lane], y2 = y[q * 96 + 64 + lane];
-            constexpr int NV = kSplineRows * sizeof(T) / 16;
-            union {
-                int4 v[NV];
-                T t[kSplineRows];
-            } w;
-            const int4* wv = reinterpret_cast<const int4*>(Wr + (size_t)q * ws + k0);
+            T w[R];
+            if constexpr (R == 1) {
+                w[0] = Wr[(size_t)q * ws + k0];
+            } else {
+                const float4* wv = reinterpret_cast<const float4*>(Wr + (size_t)q * ws + k0);
 #pragma unroll
-            for (int v = 0; v < NV; ++v) w.v[v] = wv[v];
+                for (int v = 0; v < R / 4; ++v) {
+                    const float4 x = wv[v];
+                    w[4 * v] = x.x, w[4 * v + 1] = x.y, w[4 * v + 2] = x.z, w[4 * v + 3] = x.w;
+                }
+            }
 #pragma unroll
-            for (int r = 0; r < kSplineRows; ++r) {
-                u[r][0] += w.t[r] * y0;
-                u[r][1] += w.t[r] * y1;
-                u[r][2] += w.t[r] * y2;
+            for (int r = 0; r < R; ++r) {
+                u[r][0] += w[r] * y0;
+                u[r][1] += w[r] * y1;
+                u[r][2] += w[r] * y2;
             }
         }
 #pragma unroll
-        for (int r = 0; r < kSplineRows; ++r) {
+        for (int r = 0; r < R; ++r) {
             const int k = k0 + r;
             if (k < 1 || k >= K - 1 || wc[k]) continue;  // kept in place
             const T n = rsqrt_t<T>(u[r][0] * u[r][0] + u[r][1] * u[r][1] + u[r][2] * u[r][2]);
