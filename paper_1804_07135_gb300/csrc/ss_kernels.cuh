@@ -2194,39 +2194,53 @@ __global__ void interp_identity_kernel(InterpEntry* tab, int img0, int K) {
 
 // ------------------------------------------------------------------------------------------------
 // launchers
-// Launch with programmatic stream serialisation (see griddep_wait); errors surface through
-// cudaGetLastError like a <<<>>> launch.
-template <typename... KArgs, typename... Args>
-static inline void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                              Args&&... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+// The split of the SM's 256 KB between shared memory and L1 that every launch on a group's state asks for, as a
+// percentage of 228 KB (the sizes are 100, 132, 164, 196 and 228 KB; the percentage is rounded down so that the next
+// size up is not taken), or -1: the driver's choice.  One split for all of a group's kernels: an SM changes its split
+// only when it is empty, and with programmatic dependent launch and graph branches it never is, so a kernel that starts
+// on SMs split for another one keeps that split -- the y/z kernel of 384 points ran with one resident CTA behind an x
+// kernel that had asked for less shared memory.  164 KB hold two y/z CTAs of 384 points or three of 256 and leave 92 KB
+// of L1 to the stencil (the 20-string study on one GB300: 4078 us per iteration with each kernel's own split, 3526 with
+// this one); 196 and 228 hold two CTAs of the longer lengths.  FP64 lines are twice as long (52 KB for 128 points):
+// there every kernel asks for all of it.  With the runtime-plan y/z kernel the driver chooses, for all kernels of the
+// group: that kernel lives on L1, and x kernels that asked for 164 KB beside it took a third of its speed or more
+// (14x70x20 x 24 images 302 us per iteration, 195 without; 14x30x32 x 24 440 and 220).  The preference goes with the
+// launch and not with the kernel, since groups of both kinds share the x kernels.
+template <typename T> static inline int carve_pct(const GroupArgs<T>& g) {
+    if (g.spec && !yz2p_ok(g.Py, g.nz, g.Px)) return -1;
+    const int P = t2_length(g.Px) && g.Px > g.Py ? g.Px : g.Py;
+    const int kb = sizeof(T) == 8 ? 228 : P <= 384 ? 164 : P <= 448 ? 196 : 228;
+    return kb * 100 / 228;
 }
-
-// As launch_pdl, with programmatic stream serialisation only when pdl is set.
-template <typename... KArgs, typename... Args>
+// Launch on a group's state with its split and, when pdl is set, programmatic stream serialisation (see
+// griddep_wait); errors surface through cudaGetLastError like a <<<>>> launch.
+template <typename... KArgs, typename T, typename... Args>
 static inline void launch_ex(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool pdl,
-                             Args&&... args) {
+                             const GroupArgs<T>& g, const Args&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute attr[2];
+    int n = 0;
+    if (pdl) {
+        attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    const int carve = carve_pct(g);
+    if (carve >= 0) {
+        attr[n].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+        attr[n++].val.sharedMemCarveout = carve;
+    }
     cfg.attrs = attr;
-    cfg.numAttrs = pdl ? 1 : 0;
-    cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+    cfg.numAttrs = n;
+    cudaLaunchKernelEx(&cfg, kernel, g, args...);
+}
+template <typename... KArgs, typename T, typename... Args>
+static inline void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                              const GroupArgs<T>& g, const Args&... args) {
+    launch_ex(kernel, grid, block, smem, st, true, g, args...);
 }
 
 // Programmatic dependent launch of an iteration's transform kernels.  FP64 two-pass y/z kernels are bound by each
@@ -2319,11 +2333,10 @@ template <typename T>
 void launch_xinv_eval(const GroupArgs<T>& g, bool do_fft, T* hout, int nthr, size_t smem, cudaStream_t st) {
     dim3 grid((g.ny + g.ty_c - 1) / g.ty_c, g.nz, g.n_pairs);
     if (do_fft && launch_xinv2p<1>(g, T(0), hout, false, st)) return;
-    if (do_fft) {
-        xinv_kernel<T, true, 1><<<grid, nthr, smem, st>>>(g, T(0), hout);
-    } else {
-        xinv_kernel<T, false, 1><<<grid, nthr, smem, st>>>(g, T(0), hout);
-    }
+    if (do_fft)
+        launch_ex(xinv_kernel<T, true, 1>, grid, dim3(nthr), smem, st, false, g, T(0), hout);
+    else
+        launch_ex(xinv_kernel<T, false, 1>, grid, dim3(nthr), smem, st, false, g, T(0), hout);
 }
 
 #ifdef SS_COMMON_LAUNCHERS
@@ -2384,10 +2397,10 @@ template <typename T> void launch_dipole_direct(const GroupArgs<T>& g, T* hdir, 
     int M = 4;
     while (M > 1 && (long)sites * ((g.n_img + M - 1) / M) < 2 * 152) M /= 2;
     const dim3 grid(sites, (g.n_img + M - 1) / M), blk(32 * kDirWarps);
-#define SS_CASE(m)                                                                             \
-    if (M == m) {                                                                              \
-        if (film) dipole_direct_kernel<T, m, true><<<grid, blk, 0, st>>>(g, hdir, dtab);       \
-        else dipole_direct_kernel<T, m, false><<<grid, blk, 0, st>>>(g, hdir, dtab);           \
+#define SS_CASE(m)                                                                                     \
+    if (M == m) {                                                                                      \
+        if (film) launch_ex(dipole_direct_kernel<T, m, true>, grid, blk, 0, st, false, g, hdir, dtab); \
+        else launch_ex(dipole_direct_kernel<T, m, false>, grid, blk, 0, st, false, g, hdir, dtab);     \
     }
     SS_CASE(1) SS_CASE(2) SS_CASE(4)
 #undef SS_CASE
@@ -2455,53 +2468,23 @@ void launch_extract_octant(const double2* spec, T* dhat, int Px, int Py, int nz,
 }
 
 // Raises the dynamic shared-memory limit of every kernel that stages lines in shared memory to
-// `bytes` less the kernel's static shared memory (the two together may not exceed `bytes`).  carve_kb > 0 also
-// asks for that split of the SM's 256 KB between shared memory and L1 (the sizes are 100, 132, 164, 196 and
-// 228 KB; the percentage is rounded down so that the next size up is not taken).
-template <typename F> static inline void set_dyn_smem(F* kernel, int bytes, int carve_kb = 0) {
+// `bytes` less the kernel's static shared memory (the two together may not exceed `bytes`).
+template <typename F> static inline void set_dyn_smem(F* kernel, int bytes) {
     cudaFuncAttributes fa{};
     if (cudaFuncGetAttributes(&fa, kernel) != cudaSuccess) return;
     cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes - (int)fa.sharedSizeBytes);
-    if (carve_kb) cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, carve_kb * 100 / 228);
 }
-// One split for every kernel of an iteration (two-pass kernels of up to 384 points, arc, climbing image,
-// spline, direct sums, Runge-Kutta): an SM changes its split only when it is empty, and with programmatic dependent launch and graph
-// branches it never is, so a kernel that starts on SMs split for another one keeps that split -- the y/z kernel
-// of 384 points ran with one resident CTA behind an x kernel that had asked for less shared memory.  164 KB
-// hold two y/z CTAs of 384 points or three of 256 and leave 92 KB of L1 to the stencil.  The 20-string study on
-// one GB300: 4078 us per iteration with each kernel's own split, 3526 with this one.
-// FP64 lines are twice as long (52 KB for 128 points): there every kernel asks for all of it.
-template <typename T> constexpr int carve_kb() { return sizeof(T) == 8 ? 228 : 164; }
 
 template <typename T> void set_smem_limits(int bytes) {
-    constexpr int carve = carve_kb<T>();
     set_dyn_smem(xfwd_kernel<T, true>, bytes);
-    set_dyn_smem(xfwd_kernel<T, false>, bytes, carve);
     set_dyn_smem(yz_kernel<T, 0>, bytes);
-    set_dyn_smem(xinv_kernel<T, true, 0>, bytes);
-    set_dyn_smem(xinv_kernel<T, true, 1>, bytes);
-    set_dyn_smem(xinv_kernel<T, false, 0>, bytes, carve);
-    set_dyn_smem(xinv_kernel<T, false, 1>, bytes, carve);
-    set_dyn_smem(xinv_kernel<T, true, 2>, bytes);
-    set_dyn_smem(xinv_kernel<T, false, 2>, bytes, carve);
-    set_dyn_smem(xinv_kernel<T, true, 3>, bytes);
-    set_dyn_smem(xinv_kernel<T, false, 3>, bytes, carve);
-    set_dyn_smem(xinv_kernel<T, true, 4>, bytes);
-    set_dyn_smem(xinv_kernel<T, false, 4>, bytes, carve);
-    set_dyn_smem(xinv_kernel<T, true, 5>, bytes);
-    set_dyn_smem(xinv_kernel<T, false, 5>, bytes, carve);
-    set_dyn_smem(spline_apply_kernel<T>, bytes, carve);
-    set_dyn_smem(arc_kernel<T>, bytes, carve);
-    set_dyn_smem(climb_dot_kernel<T>, bytes, carve);
-#define SS_CASE(M)                                                  \
-    set_dyn_smem(dipole_direct_kernel<T, M, true>, bytes, carve);   \
-    set_dyn_smem(dipole_direct_kernel<T, M, false>, bytes, carve);
-    SS_CASE(1) SS_CASE(2) SS_CASE(4)
+#define SS_CASE(M)                                \
+    set_dyn_smem(xinv_kernel<T, true, M>, bytes); \
+    set_dyn_smem(xinv_kernel<T, false, M>, bytes);
+    SS_CASE(0) SS_CASE(1) SS_CASE(2) SS_CASE(3) SS_CASE(4) SS_CASE(5)
 #undef SS_CASE
-    set_dyn_smem(rk_finish_kernel<T>, bytes, carve);
-    set_dyn_smem(rk_control_kernel<T>, bytes, carve);
-    set_dyn_smem(rk_commit_kernel<T>, bytes, carve);
-    set_dyn_smem(climb_apply_kernel<T>, bytes, carve);
+    set_dyn_smem(spline_apply_kernel<T>, bytes);
+    set_dyn_smem(arc_kernel<T>, bytes);
     if constexpr (std::is_same<T, float>::value) {
 #define SS_CASE(Z) set_dyn_smem(yz_kernel<T, Z>, bytes);
         SS_FOR_NZ(SS_CASE)
