@@ -329,8 +329,9 @@ inline int padded_len(int n) {
 
 // The padded lengths of a lattice, Px first: the two-pass x kernels take every t2_length, but the two-pass y/z kernel
 // takes Py only together with a Px that its columns per CTA divide (yz2p_ok).  Where it does not (Px = 18 at one
-// layer, say), the runtime-plan kernel transforms y, and that one has stages of radix 2, 3, 4 and 8 alone: Py is then
-// padded_smooth(ny), never a two-pass length with a factor 5 or 7.
+// layer, say), the runtime-plan kernel transforms y, and that one has stages of radix 2, 3, 4 and 8 alone: a two-pass
+// length with a factor 5 or 7 is then exchanged for padded_smooth(ny).  The others stay, which have fewer radix-3 stages
+// (5x81x1 x 40 images, Py 192 and 162: 30.8 and 34.5 us per iteration on one GB300).
 //
 // FP64 kernels' time goes with the work they issue to the FP64 pipe.  The two-pass y/z kernel leaves lanes idle at
 // short lengths, which a grid of one or two CTAs per SM does not hide: up to kYz64Few of them the short lengths.  And
@@ -353,7 +354,7 @@ inline void padded_lengths(int real_bytes, int nx, int ny, int nz, int n_pairs, 
             *Px = sx;
         }
     }
-    if (!yz2p_ok(*Py, nz, *Px)) *Py = sy;
+    if (!yz2p_ok(*Py, nz, *Px) && (*Py % 5 == 0 || *Py % 7 == 0)) *Py = sy;
 }
 
 

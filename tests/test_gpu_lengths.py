@@ -13,7 +13,7 @@ from paper_1804_07135_gb300 import workloads as W
 pytestmark = pytest.mark.gpu
 
 # (nx, ny, nz, images); the last three have the image pairs that take FP64 past its rule for small grids
-CASES = [(9, 35, 1, 2), (9, 100, 1, 3), (6, 50, 1, 2), (5, 76, 3, 3), (2, 100, 4, 2), (3, 150, 2, 2), (350, 35, 1, 2),
+CASES = [(9, 35, 1, 2), (9, 100, 1, 3), (6, 50, 1, 2), (5, 76, 3, 3), (2, 100, 4, 2), (3, 150, 2, 2), (350, 35, 1, 2), (5, 81, 1, 3),
          (326, 33, 2, 2), (9, 33, 1, 240), (2, 40, 4, 140), (9, 50, 1, 240)]
 
 
