@@ -89,6 +89,7 @@ struct Group {
     void* hdir = nullptr; // [image][3][N] direct sums
     void* dtab = nullptr; // [6][N] tensor table of the direct sums
     FftPlan planx{}, plany{};
+    bool x2 = false;      // two-pass x kernels (x2_use)
     int lsx = 1, lsy = 1;
     int ty_a = 1, ty_c = 1, thr_a = 128, thr_b = 128, thr_c = 128, thr_arc = 256;
     int yz_kxb = 0;  // kx columns per CTA of the two-pass y/z kernel (0: default; autotuned)
@@ -241,6 +242,7 @@ template <typename T> GroupArgs<T> group_args(const ss_ctx* c, const Group& g) {
     a.m_hx = fast_div_m(g.nx / 2);
     a.lsx = g.lsx;
     a.lsy = g.lsy;
+    a.x2 = g.x2;
     a.s = (T*)g.s;
     a.sp = (T*)g.sp;
     a.spec = (cplx<T>*)g.spec;
@@ -270,7 +272,7 @@ template <typename T> GroupArgs<T> group_args(const ss_ctx* c, const Group& g) {
 // they need.
 void set_rows(Group& g, int ty_a, int ty_c, int thr_a = 256, int thr_c = 256) {
     const size_t cs = 2 * (size_t)g.rbytes;
-    const bool x2 = g.dipole && t2_length(g.Px);  // two-pass x kernels: fixed rows per CTA
+    const bool x2 = g.dipole && g.x2;  // two-pass x kernels: fixed rows per CTA
     if (x2) ty_a = ty_c = x2_rows(g.rbytes, g.Px);
     g.ty_a = ty_a;
     g.ty_c = ty_c;
@@ -502,7 +504,7 @@ template <typename T> ss_status tune_group(ss_ctx* c, Group& g) {
     }
     const size_t cs = 2 * real_size(c);
     std::vector<std::pair<int, int>> cands;  // (threads, rows)
-    if (g.dipole && t2_length(g.Px)) {
+    if (g.dipole && g.x2) {
         cands.push_back({g.thr_a, g.ty_a});  // one shape: nothing to tune
     } else {
         for (int thr : {256, 512})
@@ -1011,6 +1013,7 @@ ss_status ensure_ev64(ss_ctx* c) {
         e.dipole = g.dipole;
         e.Px = g.Px;
         e.Py = g.Py;
+        e.x2 = g.dipole && t2_length(g.Px);  // (its runtime-plan kernels would not be tuned)
         e.n_img = g.n_img;
         e.n_pairs = g.n_pairs;
         e.strs = g.strs;
@@ -1323,7 +1326,8 @@ ss_status ss_create_batch(int n_strings, const ss_string_desc* descs, const ss_o
         if (g.dipole) padded_lengths(g.rbytes, g.nx, g.ny, g.nz, g.n_pairs, &g.Px, &g.Py);
         g.planx = make_plan(g.Px);
         g.plany = make_plan(g.Py);
-        if (g.dipole && ((!t2_length(g.Px) && !fft_plan_2348(g.planx)) ||
+        g.x2 = g.dipole && x2_use(g.rbytes, g.Px, g.ny, g.nz, g.n_pairs);
+        if (g.dipole && ((!g.x2 && !fft_plan_2348(g.planx)) ||
                          (!yz2p_ok(g.Py, g.nz, g.Px) && !fft_plan_2348(g.plany))))  // padded_lengths never asks for it
             return bail(fail(c, SS_ERR_INVALID_ARG, "lattice %d x %d x %d: no kernel for the padded lengths %d x %d", g.nx,
                              g.ny, g.nz, g.Px, g.Py));

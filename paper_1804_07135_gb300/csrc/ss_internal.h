@@ -115,6 +115,7 @@ template <typename T> struct GroupArgs {
     RkNext<T> rk;          // force modes only
     int w_spec;            // evaluation: the dipole term per (column <= Px / 2, pair) is in the spectrum (FP64)
     int yz_kxb;            // kx columns per CTA of the two-pass y/z kernel (autotuned; 0: the default)
+    int x2;                // the x kernels are the two-pass ones (x2_use)
 };
 // Energy partials per image of the evaluation mode: the four terms of Eq. 1 (J, D, K, w with the constant
 // set to 1) and the squared norm of the dipole convolution (for the FP32 round-off bound of the w term).
@@ -293,6 +294,16 @@ inline int x2_launch_threads(int real_bytes, int P, int nx, long ctas) {
     const int hi = x2_threads(4, P), lo = P > 64 && P <= 256 ? hi - 64 : hi;
     const int items = nx % 2 == 0 ? 4 * nx : 8 * nx;
     return ctas < 10L * 152 && (items + hi - 1) / hi < (items + lo - 1) / lo ? hi : lo;
+}
+// Whether a group's x kernels are the two-pass ones: every length that has them, but for FP64 at 32 points on a large
+// grid.  There pass 1 has 12 roles per CTA (2 rows x 3 components x R2 = 2) and a warp's FP64 instruction takes as long
+// for 12 lanes as for 32, which shows once the grid is several CTAs per SM deep; the runtime-plan kernels at their tuned
+// rows fill their warps.  Per iteration on one GB300, two-pass and runtime-plan: 14x20x1 x 60 images (300 CTAs) 63.7 and
+// 63.7 us, 16x9x1 x 200 (500) 186 and 184, 16x60x1 x 40 (600) 92.3 and 82.1, 14x64x4 x 16 (1024) 129 and 113, 14x40x2 x
+// 100 (2000) 209 and 177, 14x22x3 x 130 (2145) 281 and 258.  (At 48 points neither is better by more than 6%.)
+constexpr long kX2Grid32 = 512;
+inline bool x2_use(int real_bytes, int Px, int ny, int nz, int n_pairs) {
+    return t2_length(Px) && !(real_bytes == 8 && Px == 32 && (long)((ny + 1) / 2) * nz * n_pairs > kX2Grid32);
 }
 // line stride of the x kernels: 16 / rows (mod 16)
 __host__ __device__ constexpr int x2_lsx(int real_bytes, int P) {

@@ -2208,7 +2208,7 @@ __global__ void interp_identity_kernel(InterpEntry* tab, int img0, int K) {
 // launch and not with the kernel, since groups of both kinds share the x kernels.
 template <typename T> static inline int carve_pct(const GroupArgs<T>& g) {
     if (g.spec && !yz2p_ok(g.Py, g.nz, g.Px)) return -1;
-    const int P = t2_length(g.Px) && g.Px > g.Py ? g.Px : g.Py;
+    const int P = g.x2 && g.Px > g.Py ? g.Px : g.Py;
     const int kb = sizeof(T) == 8 ? 228 : P <= 384 ? 164 : P <= 448 ? 196 : 228;
     return kb * 100 / 228;
 }
@@ -2251,11 +2251,11 @@ template <typename T> static inline bool pdl_fft(const GroupArgs<T>& g) {
     return sizeof(T) == 4 || !yz2p_ok(g.Py, g.nz, g.Px);
 }
 
-// The two-pass x-inverse kernel in mode MODE when Px is one of its lengths (rows per CTA x2_rows, set by
+// The two-pass x-inverse kernel in mode MODE where the group takes them (rows per CTA x2_rows, set by
 // the host); false otherwise.
 template <int MODE, typename T>
 static inline bool launch_xinv2p(const GroupArgs<T>& g, T dt, T* hout, bool pdl, cudaStream_t st) {
-    if (!t2_length(g.Px)) return false;
+    if (!g.x2) return false;
     switch (g.Px) {
 #define SS_CASE(P) \
     case P: t2_xinv<T, P>(g, MODE, dt, hout, pdl, st); break;
@@ -2281,7 +2281,7 @@ template <typename T> void launch_xfwd(const GroupArgs<T>& g, bool do_fft, int n
         launch_pdl(xfwd_kernel<T, false>, grid, dim3(nthr), 0, st, g);
         return;
     }
-    if (t2_length(g.Px)) {
+    if (g.x2) {
         switch (g.Px) {
 #define SS_CASE(P) \
     case P: t2_xfwd<T, P>(g, st); break;

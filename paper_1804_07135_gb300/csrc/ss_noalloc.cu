@@ -261,7 +261,8 @@ extern "C" ss_status ss_field_noalloc(int nx, int ny, int nz, double J, double D
     g.prm = prm;
     g.interp = interp;
     g.epart = nullptr;  // the field alone
-    g.ty_a = g.ty_c = dip && t2_length(Px) ? x2_rows(4, Px) : ty;  // the two-pass x kernels' own count
+    g.x2 = dip && t2_length(Px);
+    g.ty_a = g.ty_c = g.x2 ? x2_rows(4, Px) : ty;  // the two-pass x kernels' own count
     g.err = err;
     launch_xfwd<float>(g, dip, thr, smem_a, st);
     if (dip) launch_yz<float>(g, thr_b, smem_b, st);

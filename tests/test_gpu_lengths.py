@@ -36,3 +36,24 @@ def test_field_and_energies(case, precision):
     for k in some:
         ref = oracle.field(m, s[k])
         assert np.abs(field[k] - ref).max() <= (1e-12 if precision == "fp64" else 1e-5) * np.abs(ref).max(), k
+
+
+# FP64 at Px = 32: the two-pass x kernels (two rows per CTA, 128 threads) up to 512 CTAs, the runtime-plan ones beyond
+@pytest.mark.parametrize("case", [(16, 40, 2, 24), (16, 40, 2, 26), (14, 33, 1, 60), (13, 35, 3, 21)])
+def test_fp64_x_kernels_at_32_points(case):
+    nx, ny, nz, n = case
+    desc = (nx, ny, nz, 1.0, 0.3, 0.1, 0.03, n)
+    path = W.random_spins((n, nx * ny * nz, 3), seed=ny)
+    with binding.StringMethod([desc], precision=binding.SS_PREC_FP64) as sm:
+        cfg = sm.launch_config(0)
+        sm.set_path(0, path)
+        field, energies = sm.field(0), sm.energies(0)
+    assert cfg["Px"] == 32
+    two_pass = (ny + 1) // 2 * nz * ((n + 1) // 2) <= 512
+    assert ((cfg["rows_xfwd"], cfg["threads_xfwd"]) == (2, 128)) == two_pass
+    m = oracle.model(*desc[:7])
+    want = oracle.energies(m, path)
+    assert np.abs(energies - want).max() <= 1e-11 * (np.abs(want).max() + nx * ny * nz)
+    for k in (0, n // 2, n - 1):
+        ref = oracle.field(m, path[k])
+        assert np.abs(field[k] - ref).max() <= 1e-12 * np.abs(ref).max(), k
