@@ -349,8 +349,14 @@ inline int padded_len(int n) {
 // its time goes with Px: a two-pass Px more than a tenth above the short one does not pay where the y/z kernel is the
 // same with either.  Per iteration on one GB300, two-pass and short lengths: 13x17x2 x 11 images (192 CTAs) 68 and
 // 54 us, 14x22x3 x 10 (160) 74 and 60, 17x17x1 x 11 (144) 56 and 52, 50x26x1 x 8 (224) 64 and 77, 13x17x1 x 30 (240)
-// 56 and 64; short Px alone: 25x32x8 x 44 (64 or 54) 510 and 446, 25x25x8 x 40 430 and 399.
+// 56 and 64; short Px alone: 25x32x8 x 44 (64 or 54) 510 and 446, 25x25x8 x 40 430 and 399.  13 and 14 sites along y (27
+// or 32 points, where the two-pass kernel has 12 of 64 threads at work in two of its passes) take the short lengths
+// for longer: to about one round of the runtime-plan kernel, two CTAs per SM, with two layers, less with three and four,
+// whose lines take that kernel longer.  In sx n_pairs CTAs of it, two-pass and short: 14x14x2 x 16 (216) 68 and 51,
+// 8x14x2 x 36 (288) 64 and 55, 34x13x2 x 10 (360) 70 and 70; 14x14x3 x 18 (243) 70 and 60, 17x14x3 x 16 (288) 71 and
+// 74; 14x13x4 x 16 (216) 72 and 66, 10x14x4 x 20 (240) 70 and 75.
 constexpr long kYz64Few = 200;
+inline long yz64_few_27(int nz) { return nz == 2 ? 304 : nz == 3 ? 256 : nz == 4 ? 224 : 0; }
 inline void padded_lengths(int real_bytes, int nx, int ny, int nz, int n_pairs, int* Px, int* Py) {
     const int sx = padded_smooth(nx), sy = padded_smooth(ny);
     const int tx = padded_len(nx), ty = nz <= kT2MaxNz ? padded_len(ny) : sy;
@@ -358,7 +364,8 @@ inline void padded_lengths(int real_bytes, int nx, int ny, int nz, int n_pairs, 
     *Py = ty;
     if (real_bytes == 8) {
         const int kxb = yz2p_kxb_use(8, nz, 0);
-        if (kxb > 0 && (long)(tx / kxb) * n_pairs <= kYz64Few) {
+        if ((kxb > 0 && (long)(tx / kxb) * n_pairs <= kYz64Few) ||
+            (ty == 32 && sy == 27 && (long)sx * n_pairs <= yz64_few_27(nz))) {
             *Px = sx;
             *Py = sy;
         } else if (10 * tx > 11 * sx && yz2p_ok(ty, nz, sx) == yz2p_ok(ty, nz, tx)) {

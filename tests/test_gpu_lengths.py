@@ -57,3 +57,24 @@ def test_fp64_x_kernels_at_32_points(case):
     for k in (0, n // 2, n - 1):
         ref = oracle.field(m, path[k])
         assert np.abs(field[k] - ref).max() <= 1e-12 * np.abs(ref).max(), k
+
+
+# FP64 with 13 or 14 sites along y: short lengths up to the line of each layer count, two-pass lengths beyond it
+@pytest.mark.parametrize("case,Px,Py", [((14, 14, 2, 22), 27, 27), ((14, 14, 2, 24), 32, 32), ((10, 14, 3, 20), 24, 27),
+                                        ((10, 13, 3, 22), 24, 32), ((15, 13, 4, 14), 32, 27), ((15, 13, 4, 16), 32, 32),
+                                        ((15, 15, 3, 16), 32, 32), ((10, 14, 5, 18), 24, 32)])
+def test_fp64_lengths_at_13_and_14_sites(case, Px, Py):
+    nx, ny, nz, n = case
+    desc = (nx, ny, nz, 1.0, 0.3, 0.1, 0.03, n)
+    path = W.random_spins((n, nx * ny * nz, 3), seed=n)
+    with binding.StringMethod([desc], precision=binding.SS_PREC_FP64) as sm:
+        cfg = sm.launch_config(0)
+        sm.set_path(0, path)
+        field, energies = sm.field(0), sm.energies(0)
+    assert (cfg["Px"], cfg["Py"]) == (Px, Py)
+    m = oracle.model(*desc[:7])
+    want = oracle.energies(m, path)
+    assert np.abs(energies - want).max() <= 1e-11 * (np.abs(want).max() + nx * ny * nz)
+    for k in (0, n - 1):
+        ref = oracle.field(m, path[k])
+        assert np.abs(field[k] - ref).max() <= 1e-12 * np.abs(ref).max(), k
