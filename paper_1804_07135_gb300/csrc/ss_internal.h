@@ -343,6 +343,13 @@ inline int padded_len(int n) {
 // layer, say), the runtime-plan kernel transforms y, and that one has stages of radix 2, 3, 4 and 8 alone: a two-pass
 // length with a factor 5 or 7 is then exchanged for padded_smooth(ny).  The others stay, which have fewer radix-3 stages
 // (5x81x1 x 40 images, Py 192 and 162: 30.8 and 34.5 us per iteration on one GB300).
+// That kernel's time goes with its columns, in rounds of two CTAs per SM: with a two-pass Px a third longer (17 and 18
+// sites, 48 for 36 points) the x kernels gain less than it loses as soon as it takes more rounds (four or more with up to
+// eight layers, where a round is short), or two and more of long lines (400 sites and up per column), which share the
+// SM's L1 and issue.  FP32, per iteration on one GB300 with 36 and 48 points, rounds in brackets:
+// 18x12x1 x 40 images (3, 4) 35.0 and 33.9 us, x 64 (4, 6) 41.1 and 43.2, x 256 (16, 21) 104 and 119; 18x25x20 x 6 (1, 1)
+// 65.7 and 47.2, x 16 (1, 2) 71.8 and 86.8, x 24 (2, 2) 103 and 109, 18x40x9 x 24 (2, 2) 59.6 and 59.5.  A two-pass Px up to 1.19 times the short one (all
+// other lattices) gains 5 to 15%.
 //
 // FP64 kernels' time goes with the work they issue to the FP64 pipe.  The two-pass y/z kernel leaves lanes idle at
 // short lengths, which a grid of one or two CTAs per SM does not hide: up to kYz64Few of them the short lengths.  And
@@ -371,6 +378,9 @@ inline void padded_lengths(int real_bytes, int nx, int ny, int nz, int n_pairs, 
         } else if (10 * tx > 11 * sx && yz2p_ok(ty, nz, sx) == yz2p_ok(ty, nz, tx)) {
             *Px = sx;
         }
+    } else if (4 * tx > 5 * sx && !yz2p_ok(ty, nz, sx) && !yz2p_ok(ty, nz, tx)) {
+        const long round = 2 * 152, rs = (sx * (long)n_pairs + round - 1) / round, rt = (tx * (long)n_pairs + round - 1) / round;
+        if (rt > rs ? nz > kT2MaxNz || rs >= 4 : nz > kT2MaxNz && rs >= 2 && ny * nz >= 400) *Px = sx;
     }
     if (!yz2p_ok(*Py, nz, *Px) && (*Py % 5 == 0 || *Py % 7 == 0)) *Py = sy;
 }

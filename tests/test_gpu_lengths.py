@@ -78,3 +78,26 @@ def test_fp64_lengths_at_13_and_14_sites(case, Px, Py):
     for k in (0, n - 1):
         ref = oracle.field(m, path[k])
         assert np.abs(field[k] - ref).max() <= 1e-12 * np.abs(ref).max(), k
+
+
+# FP32 with 17 or 18 sites along x over the runtime-plan y/z kernel: 48 points until that kernel needs more rounds for them
+@pytest.mark.parametrize("case,Px", [((18, 12, 2, 40), 48), ((18, 12, 2, 64), 36), ((17, 5, 1, 130), 36), ((17, 9, 9, 6), 48),
+                                     ((18, 9, 9, 16), 36), ((17, 20, 12, 17), 48), ((17, 20, 12, 16), 36), ((18, 40, 10, 17), 36),
+                                     ((18, 13, 8, 64), 48)])
+def test_fp32_x_length_over_the_runtime_plan_kernel(case, Px):
+    nx, ny, nz, n = case
+    desc = (nx, ny, nz, 1.0, 0.3, 0.1, 0.03, n)
+    path = W.random_spins((n, nx * ny * nz, 3), seed=n).astype(np.float32)
+    with binding.StringMethod([desc]) as sm:
+        cfg = sm.launch_config(0)
+        sm.set_path(0, path)
+        s = sm.get_path(0)
+        field, energies = sm.field(0, dtype=np.float32), sm.energies(0)
+    assert cfg["Px"] == Px
+    s = s / np.linalg.norm(s, axis=-1, keepdims=True)
+    m = oracle.model(*desc[:7])
+    want = oracle.energies(m, s)
+    assert np.abs(energies - want).max() <= 1e-11 * (np.abs(want).max() + nx * ny * nz)
+    for k in (0, n - 1):
+        ref = oracle.field(m, s[k])
+        assert np.abs(field[k] - ref).max() <= 1e-5 * np.abs(ref).max(), k
