@@ -305,6 +305,11 @@ constexpr long kX2Grid32 = 512;
 inline bool x2_use(int real_bytes, int Px, int ny, int nz, int n_pairs) {
     return t2_length(Px) && !(real_bytes == 8 && Px == 32 && (long)((ny + 1) / 2) * nz * n_pairs > kX2Grid32);
 }
+// Whether SS_X_CONFIG may pin the x kernels to `thr` threads and `rows` rows per CTA: the runtime-plan kernels take 256 or
+// 512 threads; the two-pass ones have one shape per length, whatever it names.
+inline bool x_shape_ok(bool two_pass, int thr, int rows, int ny) {
+    return rows >= 1 && rows <= ny && (two_pass || thr == 256 || thr == 512);
+}
 // line stride of the x kernels: 16 / rows (mod 16)
 __host__ __device__ constexpr int x2_lsx(int real_bytes, int P) {
     const int v = t2_line(P) - 1;

@@ -1,4 +1,4 @@
-"""The padded lengths of every accepted lattice (no GPU): the rule of csrc/ss_internal.h compiled for the host.
+"""The padded lengths of every accepted lattice (no GPU): the rules of csrc/ss_internal.h compiled for the host.
 
 A length must hold the linear convolution (P >= 2n - 1), and a kernel of the runtime plans, whose stages are of
 radix 2, 3, 4 and 8, must never be handed a length with another prime factor: the y/z kernel is the two-pass one
@@ -42,6 +42,8 @@ int main() {
                         if (!ok && bad++ < 5) printf("bad %d %d %d real %d pairs %d: %d %d\n", nx, ny, nz, real, pairs, Px, Py);
                     }
             }
+    printf("shapes %d %d %d %d %d\n", x_shape_ok(true, 192, 4, 64), x_shape_ok(true, 384, 8, 64), x_shape_ok(false, 192, 4, 64),
+           x_shape_ok(false, 256, 4, 64), x_shape_ok(true, 192, 4, 3));
     printf("seen %ld bad %ld\n", seen, bad);
 }
 """
@@ -66,3 +68,8 @@ def test_no_length_reaches_a_kernel_that_cannot_transform_it(output):
 
 def test_the_build_compiles_every_two_pass_length(output):
     assert [int(v) for v in output[0].split()[1:]] == sorted(B.T2_LENGTHS)
+
+
+def test_pinned_x_shapes(output):
+    # the two-pass kernels of 128 points took any block size before they had one shape, and still do
+    assert output[-2] == "shapes 1 1 0 1 0"
