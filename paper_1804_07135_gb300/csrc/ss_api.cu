@@ -89,7 +89,7 @@ struct Group {
     void* hdir = nullptr; // [image][3][N] direct sums
     void* dtab = nullptr; // [6][N] tensor table of the direct sums
     FftPlan planx{}, plany{};
-    bool x2 = false;      // two-pass x kernels (x2_use)
+    bool x2 = false, yz2 = false;  // two-pass x kernels (x2_use) and y/z kernel (yz2_use)
     int lsx = 1, lsy = 1;
     int ty_a = 1, ty_c = 1, thr_a = 128, thr_b = 128, thr_c = 128, thr_arc = 256;
     int yz_kxb = 0;  // kx columns per CTA of the two-pass y/z kernel (0: default; autotuned)
@@ -243,6 +243,7 @@ template <typename T> GroupArgs<T> group_args(const ss_ctx* c, const Group& g) {
     a.lsx = g.lsx;
     a.lsy = g.lsy;
     a.x2 = g.x2;
+    a.yz2 = g.yz2;
     a.s = (T*)g.s;
     a.sp = (T*)g.sp;
     a.spec = (cplx<T>*)g.spec;
@@ -312,7 +313,7 @@ void configure_group(Group& g) {
     g.smem_b = (size_t)(g.Py + 3 * g.nz * g.lsy) * cs;
     const size_t slab = (size_t)(g.Py / 2 + 1) * g.nz * 6 * (size_t)g.rbytes;
     if (slab <= 24 * 1024) g.smem_b += slab;
-    if (g.dipole && yz2p_ok(g.Py, g.nz, g.Px)) {
+    if (g.dipole && g.yz2) {
         g.thr_b = yz2p_threads(g.rbytes, g.Py);
         g.smem_b = yz2p_smem(g.rbytes, g.Py, g.nz, yz2p_kxb_use(g.rbytes, g.nz, g.yz_kxb));
     }
@@ -320,7 +321,7 @@ void configure_group(Group& g) {
 
 // The two-pass y/z kernel's shared memory for the group's column count (after the autotuner's choice).
 void configure_yz_smem(Group& g) {
-    if (g.dipole && yz2p_ok(g.Py, g.nz, g.Px)) g.smem_b = yz2p_smem(g.rbytes, g.Py, g.nz, yz2p_kxb_use(g.rbytes, g.nz, g.yz_kxb));
+    if (g.dipole && g.yz2) g.smem_b = yz2p_smem(g.rbytes, g.Py, g.nz, yz2p_kxb_use(g.rbytes, g.nz, g.yz_kxb));
 }
 
 template <typename T> ss_status build_tensor_spectrum(ss_ctx* c, Group& g) {
@@ -352,7 +353,7 @@ template <typename T> ss_status build_tensor_spectrum(ss_ctx* c, Group& g) {
         // y: columns of length Py, stride Px
         launch_fft_strided_f64(d_data, d_twy, py, 6 * nz * Px, Px, Px, 1, (long)plane, c->cs);
         launch_extract_octant<T>(d_data, (T*)g.dhat, Px, Py, nz,
-                                 dhat_factor(Py, nz, Px) * 4.0 * M_PI / ((double)Px * Py), c->cs);
+                                 dhat_factor(g.yz2, nz) * 4.0 * M_PI / ((double)Px * Py), c->cs);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->cs);
@@ -513,7 +514,7 @@ template <typename T> ss_status tune_group(ss_ctx* c, Group& g) {
                     cands.push_back({thr, ty});
     }
     std::vector<int> kxbs;  // y/z columns per CTA
-    if (g.dipole && yz2p_ok(g.Py, g.nz, g.Px)) {
+    if (g.dipole && g.yz2) {
         const YzColumns k = yz2p_columns(g.nz);
         kxbs.assign(k.v, k.v + k.n);
     }
@@ -1013,6 +1014,7 @@ ss_status ensure_ev64(ss_ctx* c) {
         e.Px = g.Px;
         e.Py = g.Py;
         e.x2 = g.dipole && t2_length(g.Px);  // (its runtime-plan kernels would not be tuned)
+        e.yz2 = g.dipole && yz2p_ok(g.Py, g.nz, g.Px);
         e.n_img = g.n_img;
         e.n_pairs = g.n_pairs;
         e.strs = g.strs;
@@ -1325,9 +1327,10 @@ ss_status ss_create_batch(int n_strings, const ss_string_desc* descs, const ss_o
         if (g.dipole) padded_lengths(g.rbytes, g.nx, g.ny, g.nz, g.n_pairs, &g.Px, &g.Py);
         g.planx = make_plan(g.Px);
         g.plany = make_plan(g.Py);
+        g.yz2 = g.dipole && yz2_use(g.rbytes, g.Px, g.Py, g.nz, g.n_pairs);
         g.x2 = g.dipole && x2_use(g.rbytes, g.Px, g.ny, g.nz, g.n_pairs);
         if (g.dipole && ((!g.x2 && !fft_plan_2348(g.planx)) ||
-                         (!yz2p_ok(g.Py, g.nz, g.Px) && !fft_plan_2348(g.plany))))  // padded_lengths never asks for it
+                         (!g.yz2 && !fft_plan_2348(g.plany))))  // padded_lengths never asks for it
             return bail(fail(c, SS_ERR_INVALID_ARG, "lattice %d x %d x %d: no kernel for the padded lengths %d x %d", g.nx,
                              g.ny, g.nz, g.Px, g.Py));
         configure_group(g);

@@ -115,7 +115,7 @@ template <typename T> struct GroupArgs {
     RkNext<T> rk;          // force modes only
     int w_spec;            // evaluation: the dipole term per (column <= Px / 2, pair) is in the spectrum (FP64)
     int yz_kxb;            // kx columns per CTA of the two-pass y/z kernel (autotuned; 0: the default)
-    int x2;                // the x kernels are the two-pass ones (x2_use)
+    int x2, yz2;           // the x kernels and the y/z kernel are the two-pass ones (x2_use, yz2_use)
 };
 // Energy partials per image of the evaluation mode: the four terms of Eq. 1 (J, D, K, w with the constant
 // set to 1) and the squared norm of the dipole convolution (for the FP32 round-off bound of the w term).
@@ -268,9 +268,23 @@ inline int yz2p_kxb_use(int real_bytes, int nz, int tuned) {
         if (k.v[i] == tuned) return tuned;
     return k.n == 0 ? 0 : k.v[real_bytes == 8 ? k.n - 1 : 0];
 }
+// Whether a group's y/z kernel is the two-pass one: wherever it has a form, but for FP64 films of two to five layers on
+// a grid of little more than one round of the runtime-plan kernel (two CTAs per SM), at lengths that one can transform.
+// The two-pass kernel's roles leave lanes idle that the FP64 pipe still spends its time on, and its CTA takes 32 to 39 us
+// where the other's takes 18 to 30.  Per iteration on one GB300, two-pass and runtime-plan, Px n_pairs CTAs in brackets:
+// 15x15x2 x 8 images (128) 67 and 56 us, 16x24x2 x 4 (64) 66 and 51, 30x32x2 x 6 (192) 72 and 62, 21x15x2 x 12 (288) 68
+// and 66, 30x29x2 x 12 (384) 76 and 84; 15x16x3 x 8 (128) 70 and 56, 12x24x3 x 16 (192) 74 and 66, 12x24x3 x 24 (288) 76
+// and 88; with four and five layers at 32 points alone: 30x16x4 x 4 (128) 72 and 60, 4x16x5 x 50 (200) 74 and 70,
+// 12x15x4 x 22 (264) 72 and 74, but 48 points 21x21x4 x 8 (192) 78 and 80; one layer 12x24x1 x 24 (288) 51 and 57, eight
+// 12x16x8 x 4 (48) 78 and 90.
+inline bool yz2_use(int real_bytes, int Px, int Py, int nz, int n_pairs) {
+    if (!yz2p_ok(Py, nz, Px)) return false;
+    const bool few = nz == 2 ? (long)Px * n_pairs <= 256 : (nz == 3 || ((nz == 4 || nz == 5) && Py == 32)) && (long)Px * n_pairs <= 200;
+    return !(real_bytes == 8 && few && Py % 5 != 0 && Py % 7 != 0);
+}
 // Factor of the stored tensor spectrum besides 4 pi / (Px Py): the two-pass y/z kernel convolves sums and
 // differences of mirrored layers, which leaves a factor 2 to be taken out (exact)
-inline double dhat_factor(int Py, int nz, int Px) { return nz > 1 && yz2p_ok(Py, nz, Px) ? 0.5 : 1.0; }
+inline double dhat_factor(bool yz2, int nz) { return yz2 && nz > 1 ? 0.5 : 1.0; }
 // rows per CTA of the two-pass x kernels: 4, from 384 points on 8 (64-byte instead of 32-byte pieces of the spectrum,
 // fewer rows shared with neighbouring CTAs: 192x192x8 x 128 images x-forward 425 -> 382 us, step kernel 527 -> 480;
 // at 256 points the step kernel loses, 310 -> 322 on 128x128x4 x 384).  FP64: more, smaller CTAs, as for the y/z kernel
@@ -357,7 +371,8 @@ inline int padded_len(int n) {
 // other lattices) gains 5 to 15%.
 //
 // FP64 kernels' time goes with the work they issue to the FP64 pipe.  The two-pass y/z kernel leaves lanes idle at
-// short lengths, which a grid of one or two CTAs per SM does not hide: up to kYz64Few of them the short lengths.  And
+// short lengths, which a grid of one or two CTAs per SM does not hide: up to kYz64Few of them the short lengths (and
+// yz2_use).  And
 // its time goes with Px: a two-pass Px more than a tenth above the short one does not pay where the y/z kernel is the
 // same with either.  Per iteration on one GB300, two-pass and short lengths: 13x17x2 x 11 images (192 CTAs) 68 and
 // 54 us, 14x22x3 x 10 (160) 74 and 60, 17x17x1 x 11 (144) 56 and 52, 50x26x1 x 8 (224) 64 and 77, 13x17x1 x 30 (240)

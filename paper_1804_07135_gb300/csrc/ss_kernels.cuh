@@ -2207,7 +2207,7 @@ __global__ void interp_identity_kernel(InterpEntry* tab, int img0, int K) {
 // (14x70x20 x 24 images 302 us per iteration, 195 without; 14x30x32 x 24 440 and 220).  The preference goes with the
 // launch and not with the kernel, since groups of both kinds share the x kernels.
 template <typename T> static inline int carve_pct(const GroupArgs<T>& g) {
-    if (g.spec && !yz2p_ok(g.Py, g.nz, g.Px)) return -1;
+    if (g.spec && !g.yz2) return -1;
     const int P = g.x2 && g.Px > g.Py ? g.Px : g.Py;
     const int kb = sizeof(T) == 8 ? 228 : P <= 384 ? 164 : P <= 448 ? 196 : 228;
     return kb * 100 / 228;
@@ -2248,7 +2248,7 @@ static inline void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 // On one GB300 with and without: 40x50x3 x 16 images 223 and 210 us per iteration, 26x34x3 x 40 248 and 215,
 // 13x13x1 x 49 (less than one wave of CTAs) 55.9 and 54.1.
 template <typename T> static inline bool pdl_fft(const GroupArgs<T>& g) {
-    return sizeof(T) == 4 || !yz2p_ok(g.Py, g.nz, g.Px);
+    return sizeof(T) == 4 || !g.yz2;
 }
 
 // The two-pass x-inverse kernel in mode MODE where the group takes them (rows per CTA x2_rows, set by
@@ -2297,7 +2297,7 @@ template <typename T> void launch_yz(const GroupArgs<T>& g, int nthr, size_t sme
     dim3 grid(g.Px, g.n_pairs);
     const size_t base = (size_t)(g.Py + 3 * g.nz * g.lsy) * sizeof(cplx<T>);
     const int stage = smem >= base + (size_t)(g.Py / 2 + 1) * g.nz * 6 * sizeof(T);
-    if (yz2p_ok(g.Py, g.nz, g.Px)) {
+    if (g.yz2) {
         switch (g.Py) {
 #define SS_CASE(P) \
     case P: t2_yz<T, P>(g, st); break;

@@ -226,7 +226,7 @@ extern "C" ss_status ss_field_noalloc(int nx, int ny, int nz, double J, double D
         na_tensor_fill<<<(int)((cells + 255) / 256 < 4096 ? (cells + 255) / 256 : 4096), 256, 0, st>>>(tens, nx, ny, nz, Px, Py);
         launch_fft_strided_f64(tens, tw64x, px, 6 * nz * Py, 1, 1, 0, Px, st);
         launch_fft_strided_f64(tens, tw64y, py, 6 * nz * Px, Px, Px, 1, (long)Px * Py, st);
-        launch_extract_octant<float>(tens, dhat, Px, Py, nz, dhat_factor(Py, nz, Px) * 4.0 * M_PI / ((double)Px * Py), st);
+        launch_extract_octant<float>(tens, dhat, Px, Py, nz, dhat_factor(yz2p_ok(Py, nz, Px), nz) * 4.0 * M_PI / ((double)Px * Py), st);
     }
     ImgParam<float>* prm = reinterpret_cast<ImgParam<float>*>(base + o_prm);
     InterpEntry* interp = reinterpret_cast<InterpEntry*>(base + o_interp);
@@ -262,6 +262,7 @@ extern "C" ss_status ss_field_noalloc(int nx, int ny, int nz, double J, double D
     g.interp = interp;
     g.epart = nullptr;  // the field alone
     g.x2 = dip && t2_length(Px);
+    g.yz2 = dip && yz2p_ok(Py, nz, Px);
     g.ty_a = g.ty_c = g.x2 ? x2_rows(4, Px) : ty;  // the two-pass x kernels' own count
     g.err = err;
     launch_xfwd<float>(g, dip, thr, smem_a, st);

@@ -470,9 +470,9 @@ __global__ void __launch_bounds__(kYzqThreads, 2) yzq2p_kernel(GroupArgs<double>
         }
     }
     block_reduce_d<2>(q, red);
-    // -(1/2) times 1/4 (A and B doubled) times 2 (half of the form), once more for the column Px - kx; one layer's
-    // tensor comes without the factor of mirrored layers (dhat_factor)
-    const double f = (kx1 == kx ? -0.25 : -0.5) * (NZ == 1 ? 0.5 : 1.0);
+    // -(1/2) times 1/4 (A and B doubled) times 2 (half of the form), once more for the column Px - kx; a tensor without
+    // the factor of mirrored layers (dhat_factor) counts half
+    const double f = (kx1 == kx ? -0.25 : -0.5) * (NZ == 1 || !g.yz2 ? 0.5 : 1.0);
     if (tid == 0) blk0[0] = C{f * q[0], f * q[1]};
 }
 

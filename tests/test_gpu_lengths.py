@@ -101,3 +101,29 @@ def test_fp32_x_length_over_the_runtime_plan_kernel(case, Px):
     for k in (0, n - 1):
         ref = oracle.field(m, s[k])
         assert np.abs(field[k] - ref).max() <= 1e-5 * np.abs(ref).max(), k
+
+
+# FP64 on small grids at lengths both y/z kernels have: 64 to 256 threads of the two-pass one, 384 of the runtime plan's.
+# Energies come from the spectrum with either, whose tensor carries the two-pass kernel's factor or not.
+@pytest.mark.parametrize("case,two_pass", [((15, 15, 2, 16), False), ((15, 15, 2, 18), True), ((8, 29, 2, 3), False),
+                                           ((24, 16, 3, 8), False), ((24, 16, 3, 10), True), ((4, 46, 3, 7), False),
+                                           ((16, 15, 4, 12), False), ((16, 15, 4, 14), True), ((16, 24, 4, 4), True),
+                                           ((12, 16, 5, 16), False), ((12, 16, 5, 18), True), ((12, 24, 1, 4), True),
+                                           ((12, 16, 6, 4), True), ((8, 16, 8, 3), True)])
+def test_fp64_yz_kernel_of_small_grids(case, two_pass):
+    nx, ny, nz, n = case
+    desc = (nx, ny, nz, 1.0, 0.3, 0.1, 0.3, n)
+    path = W.random_spins((n, nx * ny * nz, 3), seed=ny + nz)
+    with binding.StringMethod([desc], precision=binding.SS_PREC_FP64) as sm:
+        cfg = sm.launch_config(0)
+        sm.set_path(0, path)
+        field, energies, terms = sm.field(0), sm.energies(0), sm.energy_terms(0)
+    assert (cfg["threads_yz"] != 384) == two_pass
+    m = oracle.model(*desc[:7])
+    want = oracle.energies(m, path)
+    scale = np.abs(want).max() + nx * ny * nz
+    assert np.abs(energies - want).max() <= 1e-11 * scale
+    assert np.abs(terms @ np.array(desc[3:7]) - want).max() <= 1e-11 * scale
+    for k in (0, n - 1):
+        ref = oracle.field(m, path[k])
+        assert np.abs(field[k] - ref).max() <= 1e-12 * np.abs(ref).max(), k
