@@ -1011,17 +1011,20 @@ ss_status ensure_ev64(ss_ctx* c) {
         e.nz = g.nz;
         e.N = g.N;
         e.dipole = g.dipole;
-        e.Px = g.Px;
-        e.Py = g.Py;
-        e.x2 = g.dipole && t2_length(g.Px);  // (its runtime-plan kernels would not be tuned)
+        // the group's lengths, but for the x length over a runtime-plan y/z kernel, whose time in FP64 outweighs the x
+        // kernels': the short one there (25x80x19 x 24 images, 54 instead of 64 points: energies 4722 -> 3997 us on one
+        // GB300, 13x120x12 x 40 2915 -> 2238, 81x30x9 x 24 1308 -> 1174)
         e.yz2 = g.dipole && yz2p_ok(g.Py, g.nz, g.Px);
+        e.Px = g.dipole && !e.yz2 ? padded_smooth(g.nx) : g.Px;
+        e.Py = g.Py;
+        e.x2 = g.dipole && t2_length(e.Px);  // (its runtime-plan kernels would not be tuned)
         e.n_img = g.n_img;
         e.n_pairs = g.n_pairs;
         e.strs = g.strs;
         e.str_img0 = g.str_img0;
         e.str_K = g.str_K;
         e.direct = g.direct;
-        e.planx = g.planx;
+        e.planx = make_plan(e.Px);
         e.plany = g.plany;
         configure_group(e);
         if (e.smem_a > 227 * 1024 || e.smem_b > 227 * 1024 || e.smem_c > 227 * 1024)

@@ -127,3 +127,21 @@ def test_fp64_yz_kernel_of_small_grids(case, two_pass):
     for k in (0, n - 1):
         ref = oracle.field(m, path[k])
         assert np.abs(field[k] - ref).max() <= 1e-12 * np.abs(ref).max(), k
+
+
+# An FP32 context's FP64 energies over the runtime-plan y/z kernel take an x length of their own
+@pytest.mark.parametrize("case", [(26, 30, 9, 3), (14, 5, 1, 4), (41, 12, 3, 2), (17, 4, 10, 5), (26, 14, 2, 3)])
+def test_energies_and_barrier_of_an_fp32_context(case):
+    nx, ny, nz, n = case
+    desc = (nx, ny, nz, 1.0, 0.3, 0.1, 0.3, n)
+    path = W.random_spins((n, nx * ny * nz, 3), seed=nx + nz).astype(np.float32)
+    with binding.StringMethod([desc]) as sm:
+        sm.set_path(0, path)
+        s = sm.get_path(0)
+        energies, terms, (barrier, k) = sm.energies(0), sm.energy_terms(0), sm.barrier(0)
+    s = s / np.linalg.norm(s, axis=-1, keepdims=True)
+    want = oracle.energies(oracle.model(*desc[:7]), s)
+    scale = np.abs(want).max() + nx * ny * nz
+    assert np.abs(energies - want).max() <= 1e-11 * scale
+    assert np.abs(terms @ np.array(desc[3:7]) - want).max() <= 1e-11 * scale
+    assert k == int(np.argmax(want)) and abs(barrier - (want.max() - want[0])) <= 2e-11 * scale
