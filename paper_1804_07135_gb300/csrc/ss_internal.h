@@ -367,8 +367,11 @@ inline int padded_len(int n) {
 // eight layers, where a round is short), or two and more of long lines (400 sites and up per column), which share the
 // SM's L1 and issue.  FP32, per iteration on one GB300 with 36 and 48 points, rounds in brackets:
 // 18x12x1 x 40 images (3, 4) 35.0 and 33.9 us, x 64 (4, 6) 41.1 and 43.2, x 256 (16, 21) 104 and 119; 18x25x20 x 6 (1, 1)
-// 65.7 and 47.2, x 16 (1, 2) 71.8 and 86.8, x 24 (2, 2) 103 and 109, 18x40x9 x 24 (2, 2) 59.6 and 59.5.  A two-pass Px up to 1.19 times the short one (all
-// other lattices) gains 5 to 15%.
+// 65.7 and 47.2, x 16 (1, 2) 71.8 and 86.8, x 24 (2, 2) 103 and 109, 18x40x9 x 24 (2, 2) 59.6 and 59.5.  A two-pass Px up to 1.19 times the short one (13,
+// 14, 25 to 27, 41, 81, 161, 162 sites) gains 5 to 15%, except on strips, where the x kernels have little to gain: about 5 us
+// a round for the columns it adds against 10 us and 60 per million sites that the x kernels save.  162x3x1 x 200 images,
+// 324 and 384 points: 553 and 643 us, 162x3x8 x 40 181 and 199, 162x12x8 x 100 545 and 533; 81x6x1 x 200 284 and 321,
+// 81x3x8 x 40 103 and 109, 81x30x9 x 24 142 and 122; 26x6x1 x 200 115 and 123, 26x12x8 x 100 115 and 101.
 //
 // FP64 kernels' time goes with the work they issue to the FP64 pipe.  The two-pass y/z kernel leaves lanes idle at
 // short lengths, which a grid of one or two CTAs per SM does not hide: up to kYz64Few of them the short lengths (and
@@ -398,9 +401,11 @@ inline void padded_lengths(int real_bytes, int nx, int ny, int nz, int n_pairs, 
         } else if (10 * tx > 11 * sx && yz2p_ok(ty, nz, sx) == yz2p_ok(ty, nz, tx)) {
             *Px = sx;
         }
-    } else if (4 * tx > 5 * sx && !yz2p_ok(ty, nz, sx) && !yz2p_ok(ty, nz, tx)) {
+    } else if (10 * tx > 11 * sx && !yz2p_ok(ty, nz, sx) && !yz2p_ok(ty, nz, tx)) {
         const long round = 2 * 152, rs = (sx * (long)n_pairs + round - 1) / round, rt = (tx * (long)n_pairs + round - 1) / round;
-        if (rt > rs ? nz > kT2MaxNz || rs >= 4 : nz > kT2MaxNz && rs >= 2 && ny * nz >= 400) *Px = sx;
+        const bool more = rt > rs ? nz > kT2MaxNz || rs >= 4 : nz > kT2MaxNz && rs >= 2 && ny * nz >= 400;
+        const bool strip = 5.0 * (tx - sx) * n_pairs / round > 10.0 + 60e-6 * 2.0 * n_pairs * nx * ny * nz;
+        if (strip || (4 * tx > 5 * sx && more)) *Px = sx;
     }
     if (!yz2p_ok(*Py, nz, *Px) && (*Py % 5 == 0 || *Py % 7 == 0)) *Py = sy;
 }

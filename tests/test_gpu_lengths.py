@@ -80,10 +80,13 @@ def test_fp64_lengths_at_13_and_14_sites(case, Px, Py):
         assert np.abs(field[k] - ref).max() <= 1e-12 * np.abs(ref).max(), k
 
 
-# FP32 with 17 or 18 sites along x over the runtime-plan y/z kernel: 48 points until that kernel needs more rounds for them
+# FP32 over the runtime-plan y/z kernel.  17 or 18 sites along x: 48 points until that kernel needs more rounds for them
 @pytest.mark.parametrize("case,Px", [((18, 12, 2, 40), 48), ((18, 12, 2, 64), 36), ((17, 5, 1, 130), 36), ((17, 9, 9, 6), 48),
                                      ((18, 9, 9, 16), 36), ((17, 20, 12, 17), 48), ((17, 20, 12, 16), 36), ((18, 40, 10, 17), 36),
-                                     ((18, 13, 8, 64), 48)])
+                                     ((18, 13, 8, 64), 48),
+                                     # strips: 324 (162) points instead of 384 (192) where the x kernels save too little
+                                     ((162, 3, 1, 40), 324), ((162, 3, 1, 16), 384), ((162, 12, 4, 40), 384), ((81, 2, 1, 60), 162),
+                                     ((81, 2, 1, 30), 192)])
 def test_fp32_x_length_over_the_runtime_plan_kernel(case, Px):
     nx, ny, nz, n = case
     desc = (nx, ny, nz, 1.0, 0.3, 0.1, 0.03, n)
