@@ -338,6 +338,17 @@ def group_keys(wl):
     return keys, imgs
 
 
+def group_lengths(sm, wl):
+    """Padded lengths (Px, Py) the library chose for each size group."""
+    out = {}
+    for i, s in enumerate(wl.strings):
+        k = (s.nx, s.ny, s.nz)
+        if k not in out:
+            cfg = sm.launch_config(i)
+            out[k] = (cfg["Px"], cfg["Py"])
+    return out
+
+
 def kernel_roofline(sm, wl, names_per_group, peaks, peak_kind, ms):
     """The dominant kernel's HBM roofline: algorithmic bytes per launch / event-timed mean duration."""
     keys, imgs = group_keys(wl)
@@ -351,8 +362,9 @@ def kernel_roofline(sm, wl, names_per_group, peaks, peak_kind, ms):
     (nx, ny, nz), dname = entries[dom]
     units = nx * ny * nz * imgs[(nx, ny, nz)]
     alg = BYTES_PER_SITE_IMAGE[dname] * units
+    px, py = group_lengths(sm, wl)[(nx, ny, nz)]
     if dname == "yz":
-        alg += 4 * 6 * nz * (padded(nx) // 2 + 1) * (padded(ny) // 2 + 1)
+        alg += 4 * 6 * nz * (px // 2 + 1) * (py // 2 + 1)
     achieved = alg / (ms[dom] * 1e-3) / 1e9
     tag = f"{dname}[{nx}x{ny}x{nz}]"
     total_alg = sum(BYTES_PER_SITE_IMAGE[n] * k[0] * k[1] * k[2] * imgs[k] for k, n in entries)
@@ -363,7 +375,7 @@ def kernel_roofline(sm, wl, names_per_group, peaks, peak_kind, ms):
         import torch
         sms = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
         peak_tf = sms * 128 * 2 * peaks.get("sm_max_mhz", 2070.0) * 1e6 / 1e12
-        flops = yz_flops_group(nx, ny, nz, imgs[(nx, ny, nz)])
+        flops = yz_flops_group(nx, ny, nz, imgs[(nx, ny, nz)], (px, py))
         ach_tf = flops / (ms[dom] * 1e-3) / 1e12
         secondary = {"kernel": tag, "bound": "alu", "achieved": ach_tf, "peak": peak_tf, "unit": "TFLOP/s",
                      "frac": ach_tf / peak_tf, "flops_per_launch": flops,
@@ -469,6 +481,7 @@ def main():
     peaks, peak_kind = measured_peaks()
     roofline = kernel_roofline(sm, wl, names, peaks, peak_kind, ms) if not climb else None
     keys, _ = group_keys(wl)
+    lengths = group_lengths(sm, wl)
     line = {
         "metric": "spin-updates/s", "value": value, "unit": "spin-updates/s", "n_gpus": world,
         "steps": args.steps, "warmup": args.warmup, "ms_per_step": step_s * 1e3, "higher_is_better": True,
@@ -476,7 +489,7 @@ def main():
         "config": {"workload": wl.name, "variant": args.variant, "strings": n_str,
                    "images": int(sum(s.n_images for s in wl.strings)),
                    "lattices": sorted({f"{s.nx}x{s.ny}x{s.nz}" for s in wl.strings}),
-                   "padded_xy": {f"{k[0]}x{k[1]}x{k[2]}": [padded(k[0]), padded(k[1])] for k in keys},
+                   "padded_xy": {f"{k[0]}x{k[1]}x{k[2]}": list(p) for k, p in lengths.items()},
                    "spin_updates_per_iteration": wl.spin_updates_per_iter,
                    "iterations_per_step": n_iter, "workload_iterations": wl.n_iter, "dt": wl.dt, "w": 0.01,
                    "precision": "fp32 spins, fields and FFTs; fp64 energy and arc-length reductions; "
@@ -755,9 +768,10 @@ def group_standalone(binding, wl, stream, iters=20, warm=3):
             "combined_vs_sum": combined / total}
 
 
-def yz_flops_group(nx, ny, nz, n_img):
-    """yz_flops for a size group of n_img images (image pairs formed over the group)."""
-    px, py = padded(nx), padded(ny)
+def yz_flops_group(nx, ny, nz, n_img, lengths=None):
+    """yz_flops for a size group of n_img images (image pairs formed over the group), at the padded lengths (Px, Py)
+    the library uses, or the nominal ones."""
+    px, py = lengths or (padded(nx), padded(ny))
     pairs = (n_img + 1) // 2
     fft = 2 * px * 3 * nz * 5 * py * math.log2(py)
     conv = px * py * 36 * nz * nz
@@ -776,8 +790,9 @@ def yz_flops(spec):
 
 
 def padded(n):
-    """The library's padded transform length: smallest 2^a 3^b >= 2n - 1, or the power of two >= 2n - 1
-    when that is at most 1/8 longer."""
+    """Nominal padded transform length: smallest 2^a 3^b >= 2n - 1, or the power of two >= 2n - 1 when that is at most
+    1/8 longer.  The library's choice (ss_launch_config) is the same at the workloads' sizes; it also depends on the
+    other extents, the layer count, the precision and the number of images."""
     m = max(1, 2 * n - 1)
     while True:
         q = m
