@@ -299,7 +299,7 @@ __global__ void __launch_bounds__(kMaxThreadsX, kMinBlocksX) xfwd_kernel(GroupAr
 // kYzItems (ky, z) results per thread in registers, so one shared buffer serves both transforms.
 constexpr int kYzItems = 4;
 
-// z-convolution for a compile-time layer count NZ: one thread per (output component a, ky), a uniform
+// z-convolution for a compile-time layer count NZ (FP32, launch_yz): one thread per (output component a, ky), a uniform
 // across a warp (nthr/3 a multiple of 32), both z loops unrolled so |z - z'| and the z-parity sign are
 // constants.  Row a of the tensor: a = x: (xx, xy, i xz); a = y: (xy, yy, i yz); a = z: (i xz, i yz, zz).
 // dslab holds the coefficient (kyo, |dz|, comp) at dslab[kyo*dk + (|dz|*6 + comp)*dq].
@@ -337,68 +337,37 @@ __device__ __forceinline__ void zconv_c(C* A, int lsy, int Py, int kx, int Px, c
             }
 #pragma unroll
             for (int z = 0; z < NZ; ++z) out[z] = C{T(0), T(0)};
-            if constexpr (std::is_same<T, float>::value) {
-                // paired FP32 form: out += (e, e) * S and (g, g) * (i S) with i S = (-S.y, S.x); the
-                // z-parity sign of the odd terms moves onto the operand, -(i S) = (S.y, -S.x)
-                if (a < 2) {
-#pragma unroll
-                    for (int zp = 0; zp < NZ; ++zp) {
-                        const float2 sx = A[(0 * NZ + zp) * lsy + pky];
-                        const float2 sy = A[(1 * NZ + zp) * lsy + pky];
-                        const float2 sz = A[(2 * NZ + zp) * lsy + pky];
-                        const float2 isz = make_float2(-sz.y, sz.x), nisz = make_float2(sz.y, -sz.x);
-#pragma unroll
-                        for (int z = 0; z < NZ; ++z) {
-                            const int q = z >= zp ? z - zp : zp - z;
-                            out[z] = __ffma2_rn(make_float2(e0[q], e0[q]), sx, out[z]);
-                            out[z] = __ffma2_rn(make_float2(e1[q], e1[q]), sy, out[z]);
-                            out[z] = __ffma2_rn(make_float2(e2[q], e2[q]), z >= zp ? isz : nisz, out[z]);
-                        }
-                    }
-                } else {
-#pragma unroll
-                    for (int zp = 0; zp < NZ; ++zp) {
-                        const float2 sx = A[(0 * NZ + zp) * lsy + pky];
-                        const float2 sy = A[(1 * NZ + zp) * lsy + pky];
-                        const float2 sz = A[(2 * NZ + zp) * lsy + pky];
-                        const float2 isx = make_float2(-sx.y, sx.x), nisx = make_float2(sx.y, -sx.x);
-                        const float2 isy = make_float2(-sy.y, sy.x), nisy = make_float2(sy.y, -sy.x);
-#pragma unroll
-                        for (int z = 0; z < NZ; ++z) {
-                            const int q = z >= zp ? z - zp : zp - z;
-                            out[z] = __ffma2_rn(make_float2(e0[q], e0[q]), z >= zp ? isx : nisx, out[z]);
-                            out[z] = __ffma2_rn(make_float2(e1[q], e1[q]), z >= zp ? isy : nisy, out[z]);
-                            out[z] = __ffma2_rn(make_float2(e2[q], e2[q]), sz, out[z]);
-                        }
-                    }
-                }
-            } else if (a < 2) {
+            // paired FP32 form: out += (e, e) * S and (g, g) * (i S) with i S = (-S.y, S.x); the
+            // z-parity sign of the odd terms moves onto the operand, -(i S) = (S.y, -S.x)
+            if (a < 2) {
 #pragma unroll
                 for (int zp = 0; zp < NZ; ++zp) {
-                    const C sx = A[(0 * NZ + zp) * lsy + pky];
-                    const C sy = A[(1 * NZ + zp) * lsy + pky];
-                    const C sz = A[(2 * NZ + zp) * lsy + pky];
+                    const float2 sx = A[(0 * NZ + zp) * lsy + pky];
+                    const float2 sy = A[(1 * NZ + zp) * lsy + pky];
+                    const float2 sz = A[(2 * NZ + zp) * lsy + pky];
+                    const float2 isz = make_float2(-sz.y, sz.x), nisz = make_float2(sz.y, -sz.x);
 #pragma unroll
                     for (int z = 0; z < NZ; ++z) {
                         const int q = z >= zp ? z - zp : zp - z;
-                        const T g2 = z >= zp ? e2[q] : -e2[q];  // odd in z
-                        out[z].x += e0[q] * sx.x + e1[q] * sy.x - g2 * sz.y;
-                        out[z].y += e0[q] * sx.y + e1[q] * sy.y + g2 * sz.x;
+                        out[z] = __ffma2_rn(make_float2(e0[q], e0[q]), sx, out[z]);
+                        out[z] = __ffma2_rn(make_float2(e1[q], e1[q]), sy, out[z]);
+                        out[z] = __ffma2_rn(make_float2(e2[q], e2[q]), z >= zp ? isz : nisz, out[z]);
                     }
                 }
             } else {
 #pragma unroll
                 for (int zp = 0; zp < NZ; ++zp) {
-                    const C sx = A[(0 * NZ + zp) * lsy + pky];
-                    const C sy = A[(1 * NZ + zp) * lsy + pky];
-                    const C sz = A[(2 * NZ + zp) * lsy + pky];
+                    const float2 sx = A[(0 * NZ + zp) * lsy + pky];
+                    const float2 sy = A[(1 * NZ + zp) * lsy + pky];
+                    const float2 sz = A[(2 * NZ + zp) * lsy + pky];
+                    const float2 isx = make_float2(-sx.y, sx.x), nisx = make_float2(sx.y, -sx.x);
+                    const float2 isy = make_float2(-sy.y, sy.x), nisy = make_float2(sy.y, -sy.x);
 #pragma unroll
                     for (int z = 0; z < NZ; ++z) {
                         const int q = z >= zp ? z - zp : zp - z;
-                        const T g0 = z >= zp ? e0[q] : -e0[q];  // odd in z
-                        const T g1 = z >= zp ? e1[q] : -e1[q];  // odd in z
-                        out[z].x += -g0 * sx.y - g1 * sy.y + e2[q] * sz.x;
-                        out[z].y += g0 * sx.x + g1 * sy.x + e2[q] * sz.y;
+                        out[z] = __ffma2_rn(make_float2(e0[q], e0[q]), z >= zp ? isx : nisx, out[z]);
+                        out[z] = __ffma2_rn(make_float2(e1[q], e1[q]), z >= zp ? isy : nisy, out[z]);
+                        out[z] = __ffma2_rn(make_float2(e2[q], e2[q]), sz, out[z]);
                     }
                 }
             }
