@@ -103,8 +103,8 @@ ss_status ss_get_path(ss_ctx* ctx, int string, void* out, int dtype, int on_devi
 ss_status ss_step(ss_ctx* ctx, int n_iter);
 
 /* Energy (Eq. 1 / Eq. 8) of every image of the current path of `string`, into host out[n_images]: a
- * fresh FP64 evaluation of the current path -- the stored spins renormalised in FP64, every term
- * (the dipole convolution included) in FP64.  On an SS_PREC_FP32 context this is the FP64 pipeline
+ * fresh FP64 evaluation of the current path -- the stored spins renormalised in FP64 (those of an SS_PREC_FP64
+ * context are unit vectors to rounding as stored), every term (the dipole convolution included) in FP64.  On an SS_PREC_FP32 context this is the FP64 pipeline
  * applied to the FP32 state widened to FP64, so the reported energies carry no FP32 round-off of
  * their own (only the FP32 trajectory's); its FP64 buffers (about twice the context's) are allocated
  * on the first call of this, ss_barrier, ss_energy_terms or ss_grad with dE_dJDKw.  Synchronises. */

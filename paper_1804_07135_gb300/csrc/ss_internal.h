@@ -286,7 +286,7 @@ inline bool yz2_use(int real_bytes, int Px, int Py, int nz, int n_pairs) {
 // differences of mirrored layers, which leaves a factor 2 to be taken out (exact)
 inline double dhat_factor(bool yz2, int nz) { return yz2 && nz > 1 ? 0.5 : 1.0; }
 // rows per CTA of the two-pass x kernels: 4, from 384 points on 8 (64-byte instead of 32-byte pieces of the spectrum,
-// fewer rows shared with neighbouring CTAs: 192x192x8 x 128 images x-forward 425 -> 382 us, step kernel 527 -> 480;
+// fewer rows shared with neighbouring CTAs: 192x192x8 x 128 images x-forward 425 -> 379 us, step kernel 527 -> 462;
 // at 256 points the step kernel loses, 310 -> 322 on 128x128x4 x 384).  FP64: more, smaller CTAs, as for the y/z kernel
 __host__ __device__ constexpr int x2_rows(int real_bytes, int P) { return real_bytes == 8 ? 2 : P >= 384 ? 8 : 4; }
 // x CTAs: pass 2 has 48 roles per row (up to P = 384), pass 1 has 3 P/16 per row, the sites of four rows take 4 nx

