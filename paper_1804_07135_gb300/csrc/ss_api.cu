@@ -310,9 +310,7 @@ void configure_group(Group& g) {
     // y/z kernel: all 3*nz lines of one (pair, kx) in shared memory, plus the kx slab of the tensor
     // spectrum when it is small enough to stage
     g.thr_b = kMaxThreadsYz;
-    g.smem_b = (size_t)(g.Py + 3 * g.nz * g.lsy) * cs;
-    const size_t slab = (size_t)(g.Py / 2 + 1) * g.nz * 6 * (size_t)g.rbytes;
-    if (slab <= 24 * 1024) g.smem_b += slab;
+    g.smem_b = yz_smem(g.rbytes, g.Py, g.nz);
     if (g.dipole && g.yz2) {
         g.thr_b = yz2p_threads(g.rbytes, g.Py);
         g.smem_b = yz2p_smem(g.rbytes, g.Py, g.nz, yz2p_kxb_use(g.rbytes, g.nz, g.yz_kxb));

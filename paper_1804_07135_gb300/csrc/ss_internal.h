@@ -113,9 +113,11 @@ template <typename T> struct GroupArgs {
     const T* hdir;         // [image][3][N] direct dipole sums (SS_DIPOLE_DIRECT), or null
     const int* pair_on;    // [n_pairs] evaluate only the pairs flagged here (generic kernels), or null: all
     RkNext<T> rk;          // force modes only
-    int w_spec;            // evaluation: the dipole term per (column <= Px / 2, pair) is in the spectrum (FP64)
+    unsigned char w_spec;  // evaluation: the dipole term per (column <= Px / 2, pair) is in the spectrum (FP64)
+    // the x kernels and the y/z kernel are the two-pass ones (x2_use, yz2_use); bytes, since eight more bytes of arguments
+    // cost the four launches of a 16x16x1 iteration 1% (13.60 and 13.73 us on one GB300)
+    unsigned char x2, yz2;
     int yz_kxb;            // kx columns per CTA of the two-pass y/z kernel (autotuned; 0: the default)
-    int x2, yz2;           // the x kernels and the y/z kernel are the two-pass ones (x2_use, yz2_use)
 };
 // Energy partials per image of the evaluation mode: the four terms of Eq. 1 (J, D, K, w with the constant
 // set to 1) and the squared norm of the dipole convolution (for the FP32 round-off bound of the w term).
@@ -267,6 +269,12 @@ inline int yz2p_kxb_use(int real_bytes, int nz, int tuned) {
     for (int i = 0; i < k.n; ++i)
         if (k.v[i] == tuned) return tuned;
     return k.n == 0 ? 0 : k.v[real_bytes == 8 ? k.n - 1 : 0];
+}
+// Dynamic shared memory of the runtime-plan y/z kernel: twiddles, the 3 nz lines of one kx, and the kx slab of the tensor
+// spectrum when it is small enough to stage.
+inline size_t yz_smem(int real_bytes, int Py, int nz) {
+    const size_t slab = (size_t)(Py / 2 + 1) * nz * 6 * real_bytes;
+    return (size_t)(Py + 3 * nz * fft_line_stride(Py)) * 2 * real_bytes + (slab <= 24 * 1024 ? slab : 0);
 }
 // Whether a group's y/z kernel is the two-pass one: wherever it has a form, but for FP64 films of two to five layers on
 // a grid of little more than one round of the runtime-plan kernel (two CTAs per SM), at lengths that one can transform.

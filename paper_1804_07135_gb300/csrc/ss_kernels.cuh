@@ -2164,26 +2164,30 @@ __global__ void interp_identity_kernel(InterpEntry* tab, int img0, int K) {
 
 // ------------------------------------------------------------------------------------------------
 // launchers
-// The split of the SM's 256 KB between shared memory and L1 that every launch on a group's state asks for, as a
-// percentage of 228 KB (the sizes are 100, 132, 164, 196 and 228 KB; the percentage is rounded down so that the next
-// size up is not taken), or -1: the driver's choice.  One split for all of a group's kernels: an SM changes its split
-// only when it is empty, and with programmatic dependent launch and graph branches it never is, so a kernel that starts
-// on SMs split for another one keeps that split -- the y/z kernel of 384 points ran with one resident CTA behind an x
-// kernel that had asked for less shared memory.  164 KB hold two y/z CTAs of 384 points or three of 256 and leave 92 KB
-// of L1 to the stencil (the 20-string study on one GB300: 4078 us per iteration with each kernel's own split, 3526 with
-// this one); 196 and 228 hold two CTAs of the longer lengths.  FP64 lines are twice as long (52 KB for 128 points):
-// there every kernel asks for all of it.  With the runtime-plan y/z kernel the driver chooses, for all kernels of the
-// group: that kernel lives on L1, and x kernels that asked for 164 KB beside it took a third of its speed or more
-// (14x70x20 x 24 images 302 us per iteration, 195 without; 14x30x32 x 24 440 and 220).  The preference goes with the
-// launch and not with the kernel, since groups of both kinds share the x kernels.
-template <typename T> static inline int carve_pct(const GroupArgs<T>& g) {
-    if (g.spec && !g.yz2) return -1;
-    const int P = g.x2 && g.Px > g.Py ? g.Px : g.Py;
-    const int kb = sizeof(T) == 8 ? 228 : P <= 384 ? 164 : P <= 448 ? 196 : 228;
-    return kb * 100 / 228;
+// One split for every kernel of an iteration (two-pass kernels of up to 384 points, arc, climbing image,
+// spline, direct sums, Runge-Kutta): an SM changes its split only when it is empty, and with programmatic dependent launch and graph
+// branches it never is, so a kernel that starts on SMs split for another one keeps that split -- the y/z kernel
+// of 384 points ran with one resident CTA behind an x kernel that had asked for less shared memory.  164 KB
+// hold two y/z CTAs of 384 points or three of 256 and leave 92 KB of L1 to the stencil.  The 20-string study on
+// one GB300: 4078 us per iteration with each kernel's own split, 3526 with this one.
+// FP64 lines are twice as long (52 KB for 128 points): there every kernel asks for all of it.
+template <typename T> constexpr int carve_kb() { return sizeof(T) == 8 ? 228 : 164; }
+// Launches on a group's state, with programmatic stream serialisation (see griddep_wait) or, launch_ex, only when pdl is
+// set; errors surface through cudaGetLastError like a <<<>>> launch.
+//
+// FP32 groups with the runtime-plan y/z kernel ask for one split of shared memory and L1 with every launch: the smallest of
+// 164, 196 and 228 KB that holds two of its CTAs (their registers allow no more) and what the two-pass x kernels of the
+// group ask for.  That kernel has no split of its own, and beside x kernels that have one it ended up with most of the SM's
+// L1 gone (14x70x20 x 24 images 303 us per iteration, 195 so; 14x30x32 x 24 436 and 221; others unchanged; a split with
+// room for one CTA costs 15 to 30%, 228 KB for all of them up to 2.7 times).  The other groups' splits are properties of the
+// kernels: given with the launch they cost 0.03 us each, 1% of an iteration of 16x16x1.
+template <typename T> static inline int carve_launch(const GroupArgs<T>& g) {
+    if (sizeof(T) == 8 || !g.spec || g.yz2) return -1;
+    const size_t one = yz_smem(4, g.Py, g.nz) + 1024, need = 2 * one <= 228 * 1024 ? 2 * one : one;
+    const int yz = need <= 164 * 1024 ? 164 : need <= 196 * 1024 ? 196 : 228;
+    const int x = !g.x2 || g.Px <= 384 ? 164 : g.Px <= 448 ? 196 : 228;
+    return std::max(x, yz) * 100 / 228;
 }
-// Launch on a group's state with its split and, when pdl is set, programmatic stream serialisation (see
-// griddep_wait); errors surface through cudaGetLastError like a <<<>>> launch.
 template <typename... KArgs, typename T, typename... Args>
 static inline void launch_ex(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool pdl,
                              const GroupArgs<T>& g, const Args&... args) {
@@ -2198,7 +2202,7 @@ static inline void launch_ex(void (*kernel)(KArgs...), dim3 grid, dim3 block, si
         attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[n++].val.programmaticStreamSerializationAllowed = 1;
     }
-    const int carve = carve_pct(g);
+    const int carve = carve_launch(g);
     if (carve >= 0) {
         attr[n].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
         attr[n++].val.sharedMemCarveout = carve;
@@ -2266,7 +2270,7 @@ template <typename T> void launch_xfwd(const GroupArgs<T>& g, bool do_fft, int n
 template <typename T> void launch_yz(const GroupArgs<T>& g, int nthr, size_t smem, cudaStream_t st) {
     dim3 grid(g.Px, g.n_pairs);
     const size_t base = (size_t)(g.Py + 3 * g.nz * g.lsy) * sizeof(cplx<T>);
-    const int stage = smem >= base + (size_t)(g.Py / 2 + 1) * g.nz * 6 * sizeof(T);
+    const int stage = smem >= base + (size_t)(g.Py / 2 + 1) * g.nz * 6 * sizeof(T);  // (yz_smem has room for the slab)
     if (g.yz2) {
         switch (g.Py) {
 #define SS_CASE(P) \
@@ -2438,23 +2442,45 @@ void launch_extract_octant(const double2* spec, T* dhat, int Px, int Py, int nz,
 }
 
 // Raises the dynamic shared-memory limit of every kernel that stages lines in shared memory to
-// `bytes` less the kernel's static shared memory (the two together may not exceed `bytes`).
-template <typename F> static inline void set_dyn_smem(F* kernel, int bytes) {
+// `bytes` less the kernel's static shared memory (the two together may not exceed `bytes`).  carve_kb > 0 also
+// asks for that split of the SM's 256 KB between shared memory and L1 (the sizes are 100, 132, 164, 196 and
+// 228 KB; the percentage is rounded down so that the next size up is not taken).
+template <typename F> static inline void set_dyn_smem(F* kernel, int bytes, int carve_kb = 0) {
     cudaFuncAttributes fa{};
     if (cudaFuncGetAttributes(&fa, kernel) != cudaSuccess) return;
     cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes - (int)fa.sharedSizeBytes);
+    if (carve_kb) cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, carve_kb * 100 / 228);
 }
 
 template <typename T> void set_smem_limits(int bytes) {
+    constexpr int carve = carve_kb<T>();
     set_dyn_smem(xfwd_kernel<T, true>, bytes);
+    set_dyn_smem(xfwd_kernel<T, false>, bytes, carve);
     set_dyn_smem(yz_kernel<T, 0>, bytes);
-#define SS_CASE(M)                                \
-    set_dyn_smem(xinv_kernel<T, true, M>, bytes); \
-    set_dyn_smem(xinv_kernel<T, false, M>, bytes);
-    SS_CASE(0) SS_CASE(1) SS_CASE(2) SS_CASE(3) SS_CASE(4) SS_CASE(5)
+    set_dyn_smem(xinv_kernel<T, true, 0>, bytes);
+    set_dyn_smem(xinv_kernel<T, true, 1>, bytes);
+    set_dyn_smem(xinv_kernel<T, false, 0>, bytes, carve);
+    set_dyn_smem(xinv_kernel<T, false, 1>, bytes, carve);
+    set_dyn_smem(xinv_kernel<T, true, 2>, bytes);
+    set_dyn_smem(xinv_kernel<T, false, 2>, bytes, carve);
+    set_dyn_smem(xinv_kernel<T, true, 3>, bytes);
+    set_dyn_smem(xinv_kernel<T, false, 3>, bytes, carve);
+    set_dyn_smem(xinv_kernel<T, true, 4>, bytes);
+    set_dyn_smem(xinv_kernel<T, false, 4>, bytes, carve);
+    set_dyn_smem(xinv_kernel<T, true, 5>, bytes);
+    set_dyn_smem(xinv_kernel<T, false, 5>, bytes, carve);
+    set_dyn_smem(spline_apply_kernel<T>, bytes, carve);
+    set_dyn_smem(arc_kernel<T>, bytes, carve);
+    set_dyn_smem(climb_dot_kernel<T>, bytes, carve);
+#define SS_CASE(M)                                                  \
+    set_dyn_smem(dipole_direct_kernel<T, M, true>, bytes, carve);   \
+    set_dyn_smem(dipole_direct_kernel<T, M, false>, bytes, carve);
+    SS_CASE(1) SS_CASE(2) SS_CASE(4)
 #undef SS_CASE
-    set_dyn_smem(spline_apply_kernel<T>, bytes);
-    set_dyn_smem(arc_kernel<T>, bytes);
+    set_dyn_smem(rk_finish_kernel<T>, bytes, carve);
+    set_dyn_smem(rk_control_kernel<T>, bytes, carve);
+    set_dyn_smem(rk_commit_kernel<T>, bytes, carve);
+    set_dyn_smem(climb_apply_kernel<T>, bytes, carve);
     if constexpr (std::is_same<T, float>::value) {
 #define SS_CASE(Z) set_dyn_smem(yz_kernel<T, Z>, bytes);
         SS_FOR_NZ(SS_CASE)

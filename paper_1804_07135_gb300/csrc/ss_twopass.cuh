@@ -628,16 +628,17 @@ template <typename T, int P> void t2_yzq(const GroupArgs<T>& g, cudaStream_t st)
 }
 
 template <typename T, int P> void t2_smem_limits(int bytes) {
-    set_dyn_smem(xfwd2p_kernel<T, P>, bytes);
-#define SS_CASE(M) set_dyn_smem(xinv2p_kernel<T, P, M>, bytes);
+    constexpr int carve = sizeof(T) == 8 || P <= 384 ? carve_kb<T>() : P <= 448 ? 196 : 228;  // two FP32 y/z CTAs
+    set_dyn_smem(xfwd2p_kernel<T, P>, bytes, carve);
+#define SS_CASE(M) set_dyn_smem(xinv2p_kernel<T, P, M>, bytes, carve);
     SS_CASE(0) SS_CASE(1) SS_CASE(2) SS_CASE(3) SS_CASE(4) SS_CASE(5)
 #undef SS_CASE
-#define SS_CASE(Z, B) set_dyn_smem(yz2p_kernel<T, P, Z, B>, bytes);
+#define SS_CASE(Z, B) set_dyn_smem(yz2p_kernel<T, P, Z, B>, bytes, carve);
     SS_T2_YZ(SS_CASE)
 #undef SS_CASE
     if constexpr (sizeof(T) == 8) {
 #define SS_CASE(Z) \
-    if constexpr (yzq2p_fits(P, Z)) set_dyn_smem(yzq2p_kernel<P, Z>, bytes);
+    if constexpr (yzq2p_fits(P, Z)) set_dyn_smem(yzq2p_kernel<P, Z>, bytes, carve);
         SS_CASE(1) SS_CASE(2) SS_CASE(3) SS_CASE(4) SS_CASE(5) SS_CASE(6) SS_CASE(7) SS_CASE(8)
 #undef SS_CASE
     }
