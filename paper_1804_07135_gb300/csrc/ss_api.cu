@@ -1009,11 +1009,13 @@ ss_status ensure_ev64(ss_ctx* c) {
         e.nz = g.nz;
         e.N = g.N;
         e.dipole = g.dipole;
-        // the group's lengths, but for the x length over a runtime-plan y/z kernel, whose time in FP64 outweighs the x
-        // kernels': the short one there (25x80x19 x 24 images, 54 instead of 64 points: energies 4722 -> 3997 us on one
-        // GB300, 13x120x12 x 40 2915 -> 2238, 81x30x9 x 24 1308 -> 1174)
+        // the group's lengths, but for an x length of thick films that is more than a tenth above the short one: the
+        // runtime-plan y/z kernel's time in FP64 outweighs the x kernels' there (25x80x19 x 24 images, 54 instead of 64
+        // points: energies 4722 -> 4008 us on one GB300, 13x120x12 x 40 2915 -> 2242, 81x30x9 x 24 1308 -> 1178).  Thin
+        // ones keep the two-pass x kernels, since the runtime-plan ones run here without tuned shapes (35x8x1 x 40, 80
+        // or 72 points: 129 and 154)
         e.yz2 = g.dipole && yz2p_ok(g.Py, g.nz, g.Px);
-        e.Px = g.dipole && !e.yz2 ? padded_smooth(g.nx) : g.Px;
+        e.Px = g.dipole && g.nz > kT2MaxNz && 10 * g.Px > 11 * padded_smooth(g.nx) ? padded_smooth(g.nx) : g.Px;
         e.Py = g.Py;
         e.x2 = g.dipole && t2_length(e.Px);  // (its runtime-plan kernels would not be tuned)
         e.n_img = g.n_img;
