@@ -320,10 +320,10 @@ inline int x2_launch_threads(int real_bytes, int P, int nx, long ctas) {
 // Whether a group's x kernels are the two-pass ones: every length that has them, but for FP64 at 32 points on a large
 // grid.  There pass 1 has 12 roles per CTA (2 rows x 3 components x R2 = 2) and a warp's FP64 instruction takes as long
 // for 12 lanes as for 32, which shows once the grid is several CTAs per SM deep; the runtime-plan kernels at their tuned
-// rows fill their warps.  Per iteration on one GB300, two-pass and runtime-plan: 14x20x1 x 60 images (300 CTAs) 63.7 and
-// 63.7 us, 16x9x1 x 200 (500) 186 and 184, 16x60x1 x 40 (600) 92.3 and 82.1, 14x64x4 x 16 (1024) 129 and 113, 14x40x2 x
-// 100 (2000) 209 and 177, 14x22x3 x 130 (2145) 281 and 258.  (At 48 points neither is better by more than 6%.)
-constexpr long kX2Grid32 = 512;
+// rows fill their warps.  Per iteration on one GB300, two-pass and runtime-plan: 16x60x1 x 40 images (600 CTAs) 90.3 and
+// 94.4 us, 15x40x1 x 80 (800) 109 and 105, 14x20x3 x 60 (900) 162 and 162, 14x64x4 x 16 (1024) 129 and 111, 14x40x2 x 100
+// (2000) 209 and 176, 14x22x3 x 130 (2145) 281 and 257.  (At 48 points neither is better by more than 6%.)
+constexpr long kX2Grid32 = 700;
 inline bool x2_use(int real_bytes, int Px, int ny, int nz, int n_pairs) {
     return t2_length(Px) && !(real_bytes == 8 && Px == 32 && (long)((ny + 1) / 2) * nz * n_pairs > kX2Grid32);
 }
